@@ -187,7 +187,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
     griddep_wait();          // the states are the preceding kernel's output
 
     if (warp == 0 || warp == kThreads / 32 - 1) {
-        if (lane == 0) {
+        if (elect_one()) {
             const int me = warp == 0 ? 0 : 1;
             int stage = 0, seq = 0;
             uint32_t phase = 0;
@@ -212,7 +212,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             if (!ok) abort_grace();
         }
     } else if (warp == 1) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0 && elect_one()) {
             const uint32_t idesc = make_instr_desc(kPairRows, j.block_n, false);
             const uint32_t desc_hi = (uint32_t)(make_smem_desc(0) >> 32);
             const uint32_t lo_base = (smem_u32(tiles) & 0x3ffffu) >> 4, lo_slot = p.slot_bytes >> 4;

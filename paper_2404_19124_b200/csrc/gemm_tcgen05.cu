@@ -48,12 +48,12 @@ __global__ void __launch_bounds__(kThreads, 1)
 gemm_tc_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     const Pipe pp = pipe_setup(smem_raw, p.stages, p.slot_bytes, p.tmem_cols, p.acc_stride, p.tbuf_bytes, p.err);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = threadIdx.x >> 5;
 
     griddep_launch();   // the next kernel in the stream may start its own set-up now
     if (warp == 0 || warp == kThreads / 32 - 1) {
         const int me = warp == 0 ? 0 : 1;
-        if (lane == 0 && me < p.producers) {
+        if (me < p.producers && elect_one()) {
             RingPos rp{0, 0u};
             int issued = 0;
             bool ok = true;
@@ -66,7 +66,7 @@ gemm_tc_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         griddep_wait();
     } else if (warp == 1) {
         griddep_wait();
-        if (lane == 0) {
+        if (elect_one()) {
             RingPos rp{0, 0u};
             AccPos ap{0, 0u};
             bool ok = true;

@@ -88,6 +88,22 @@ struct AccPos { int acc; uint32_t phase; };
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// True in one lane of a converged warp.  The single-thread roles (TMA issue, MMA issue) are entered through this and
+// not through "lane == 0": only then does the compiler know that one lane is active, and TMA, MMA and commit
+// instructions take their operands from warp-uniform registers.  With "lane == 0" the four MMAs of a K block took 255
+// cycles to issue instead of 50, a ring slot 580 cycles whatever its bytes, which is more than the weight stream
+// of a level of few nodes allows (single-candidate chain at the 13B widths 214.5 -> 193.6 us per draft, steps at the
+// 7B shape 192 -> 184, 13B 302 -> 291, 34B 536 -> 499, Llama3-8B 6518 -> 6128).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok));
+    return ok != 0;
+}
+
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count));
 }
@@ -327,7 +343,7 @@ __device__ __forceinline__ void advance(const Pipe &pp, RingPos &rp) {
 // opened) and the state operand of those slots follows.  A CTA without a tile in the job neither
 // loads nor waits.  `issued` counts slots filled since the kernel started (for the abort path).
 // Producer `me` of `n_prod` walks every slot like the others and fills the slots whose running number
-// `issued` (counted over all jobs of the launch) is congruent to `me`.
+// `issued` (counted over all jobs of the launch) is congruent to `me` (n_prod is a power of two).
 template <typename DepWait>
 __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, const CUtensorMap *tmap_a,
                                             const CUtensorMap *tmap_a_short, const CUtensorMap *tmap_b, RingPos &rp,
@@ -345,7 +361,7 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
         n_pre = min(pp.stages, t0.kb1 - t0.kb0);
         RingPos q = rp;
         for (int i = 0; i < n_pre; ++i) {
-            if ((issued + i) % n_prod == me) {
+            if (((issued + i) & (n_prod - 1)) == me) {
                 if (!mbar_wait(&bars->empty[q.stage], q.phase ^ 1u, bars, pp.err)) return false;
                 uint8_t *sa = pp.tiles + (size_t)q.stage * pp.slot_bytes;
                 mbar_arrive_expect_tx(&bars->full[q.stage], tx);
@@ -365,7 +381,7 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
             uint8_t *sa = pp.tiles + (size_t)rp.stage * pp.slot_bytes;
             uint8_t *sb = sa + kABytes;
             const bool prefetched = done < n_pre;   // the weights of this slot are already on their way
-            if (issued % n_prod == me) {
+            if ((issued & (n_prod - 1)) == me) {
                 if (!prefetched) {
                     if (!mbar_wait(&bars->empty[rp.stage], rp.phase ^ 1u, bars, pp.err)) return false;
                     mbar_arrive_expect_tx(&bars->full[rp.stage], tx);

@@ -149,6 +149,24 @@ __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, i
         : "memory");
 }
 
+// The weights are read once per launch (by all CTAs that share a box at about the same time) and are far larger than
+// L2 (126 MB), so their lines are marked to leave it first.  With the default policy 20 us of weight stream push out
+// everything else a draft touches again: the instructions of the row kernels above all (a merge spent 2-3 us waiting
+// for its own code), launch parameters, tensor maps, page-table entries.  Per pass: 7B-shaped step 184 -> 170.5 us,
+// batch-1 draft at the 7B widths 167 -> 152, single-candidate chain at the 13B widths 194 -> 177.  Not so on CTA pairs
+// (gemm_pair.cu), where up to 24 row tiles share a weight box: 34B step 484 -> 492, Llama3-8B 6150 -> 6250.
+__device__ __forceinline__ uint64_t evict_first_policy() {
+    uint64_t pol;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+    return pol;
+}
+__device__ __forceinline__ void tma_load_2d_once(void *dst, const CUtensorMap *map, int c0, int c1, uint64_t *bar, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;"
+        ::"r"(smem_u32(dst)), "l"((uint64_t)map), "r"(c0), "r"(c1), "r"(smem_u32(bar)), "l"(policy)
+        : "memory");
+}
+
 // Shared-memory matrix descriptor: K-major operand, 128-byte swizzle, rows at a 128-byte
 // pitch, groups of 8 rows 1024 bytes apart (stride byte offset), descriptor version 1.
 __device__ __forceinline__ uint64_t make_smem_desc(uint32_t saddr) {
@@ -353,6 +371,7 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
     const TileWalk w = walk_of(j);
     if (w.first >= w.end) return true;
     Barriers *bars = pp.bars;
+    const uint64_t once = evict_first_policy();
     int n_pre = 0;
     {
         const TilePos t0 = pos_of(j, w, w.first);
@@ -365,8 +384,8 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
                 if (!mbar_wait(&bars->empty[q.stage], q.phase ^ 1u, bars, pp.err)) return false;
                 uint8_t *sa = pp.tiles + (size_t)q.stage * pp.slot_bytes;
                 mbar_arrive_expect_tx(&bars->full[q.stage], tx);
-                if (j.w_is_a) tma_load_2d(sa, ma, (t0.kb0 + i) * ke, t0.a_row, &bars->full[q.stage]);
-                else tma_load_2d(sa + kABytes, tmap_b, (t0.kb0 + i) * ke, t0.b_row, &bars->full[q.stage]);
+                if (j.w_is_a) tma_load_2d_once(sa, ma, (t0.kb0 + i) * ke, t0.a_row, &bars->full[q.stage], once);
+                else tma_load_2d_once(sa + kABytes, tmap_b, (t0.kb0 + i) * ke, t0.b_row, &bars->full[q.stage], once);
             }
             advance(pp, q);
         }
@@ -386,8 +405,13 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
                     if (!mbar_wait(&bars->empty[rp.stage], rp.phase ^ 1u, bars, pp.err)) return false;
                     mbar_arrive_expect_tx(&bars->full[rp.stage], tx);
                 }
-                if (!prefetched || !j.w_is_a) tma_load_2d(sa, ma, kb * ke, t.a_row, &bars->full[rp.stage]);
-                if (!prefetched || j.w_is_a) tma_load_2d(sb, tmap_b, kb * ke, t.b_row, &bars->full[rp.stage]);
+                if (j.w_is_a) {
+                    if (!prefetched) tma_load_2d_once(sa, ma, kb * ke, t.a_row, &bars->full[rp.stage], once);
+                    tma_load_2d(sb, tmap_b, kb * ke, t.b_row, &bars->full[rp.stage]);
+                } else {
+                    tma_load_2d(sa, ma, kb * ke, t.a_row, &bars->full[rp.stage]);
+                    if (!prefetched) tma_load_2d_once(sb, tmap_b, kb * ke, t.b_row, &bars->full[rp.stage], once);
+                }
             }
             ++done;
             ++issued;

@@ -1,6 +1,6 @@
 // Stand-alone row kernels of the draft path (the row-wise steps themselves are in row_ops.cuh):
 //   mix_ln_gelu_kernel   one CTA of 256 threads per tree node
-//   merge_expand_kernel  one CTA of 128 threads per row of the vocabulary head
+//   merge_expand_kernel  one CTA of 160 threads per row of the vocabulary head
 //   prune_kernel         one CTA of 256 threads per sequence
 // Each is launched with programmatic stream serialization, so its CTAs are usually resident, waiting,
 // while the kernel before it still runs.
@@ -13,7 +13,7 @@ namespace {
 using namespace rows;
 
 constexpr int kRowThreads = 256;
-constexpr int kMergeThreads = 128;
+constexpr int kMergeThreads = 160;   // one list per thread up to V = 35000 (a CTA of the head GEMM leaves one)
 
 // Rows of up to 4096 elements: at most 128 registers, so that two CTAs fit beside a resident GEMM CTA.
 __global__ void __launch_bounds__(kRowThreads, 2) mix_ln_gelu_kernel(MixArgs m) {
@@ -97,13 +97,14 @@ __global__ void __launch_bounds__(256) draft_init_kernel(int32_t *hdr, int words
     for (int i = threadIdx.x; i < words; i += blockDim.x) hdr[i] = 0;
 }
 
+template <int kLen>
 __global__ void __launch_bounds__(kMergeThreads) merge_expand_kernel(MergeArgs g) {
     extern __shared__ LeafKey merge_keys[];   // [Lpad] when the prune is folded in, else nothing
     __shared__ Scratch sc;
     __shared__ int last_of_sequence;
     griddep_launch();
     griddep_wait();
-    merge_expand_row<kMergeThreads, BlockSync>(g, blockIdx.x, threadIdx.x, &sc);
+    merge_expand_row<kMergeThreads, kLen, BlockSync>(g, blockIdx.x, threadIdx.x, &sc);
     prune_if_last<kMergeThreads, BlockSync>(g, blockIdx.x, threadIdx.x, merge_keys, &last_of_sequence);
 }
 
@@ -125,12 +126,11 @@ __global__ void __launch_bounds__(kRowThreads, 2) merge_mix_kernel(MergeMixArgs 
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, tid = threadIdx.x;
-    merge_expand_row<kRowThreads, BlockSync>(a.merge, r, tid, &sc);
-    // sc.out_id[0 .. topk) now hold the children's tokens (valid for the whole CTA after merge_select's last barrier)
+    const int tok = merge_expand_row<kRowThreads, 4, BlockSync>(a.merge, r, tid, &sc).id;
     if (a.mix.d <= 8 * kRowThreads)
-        mix_children<kRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, sc.out_id, red_a, red_b, tid);
+        mix_children<kRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
     else
-        mix_children<kRowThreads, 2, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, sc.out_id, red_a, red_b, tid);
+        mix_children<kRowThreads, 2, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
 }
 
 // Rows of 2049 to 4096 elements: 512 threads, one 8-element group each, like mix_ln_gelu_512_kernel (single-
@@ -142,8 +142,8 @@ __global__ void __maxnreg__(72) merge_mix_512_kernel(MergeMixArgs a) {
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, tid = threadIdx.x;
-    merge_expand_row<kWideRowThreads, BlockSync>(a.merge, r, tid, &sc);
-    mix_children<kWideRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, sc.out_id, red_a, red_b, tid);
+    const int tok = merge_expand_row<kWideRowThreads, 4, BlockSync>(a.merge, r, tid, &sc).id;
+    mix_children<kWideRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
 }
 
 // Vocabulary-parallel head: one warp per row folds the n_ranks raw lists (see launch_merge_shards).
@@ -243,16 +243,18 @@ int launch_draft_init(int32_t *hdr, int words, cudaStream_t st) {
 
 int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st) {
     const size_t smem = g.seq_done ? sizeof(LeafKey) * (size_t)g.Lpad : 0;
-    SPEC_CUDA_TRY(launch_pdl(merge_expand_kernel, dim3(rows), dim3(kMergeThreads), smem, st, g));
+    const bool four = (g.list_len > 0 ? g.list_len : g.topk) <= 4;
+    SPEC_CUDA_TRY(launch_pdl(four ? merge_expand_kernel<4> : merge_expand_kernel<8>, dim3(rows), dim3(kMergeThreads), smem, st, g));
     return SPEC_OK;
 }
 
 // Returns SPEC_ERR_SHAPE when the fused form does not cover the shape (rows wider than 4096 elements, an e4m3
 // copy of the states wanted): the caller then launches the merge and the mix separately.
 int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_t st) {
-    if (m.d > 8 * kRowThreads * 2 || m.S8_out != nullptr || g.lse_out != nullptr || g.seq_done != nullptr)
+    if (m.d > 8 * kRowThreads * 2 || g.topk > 4 || m.S8_out != nullptr || g.lse_out != nullptr || g.seq_done != nullptr)
         return SPEC_ERR_SHAPE;
     MergeMixArgs a{g, m};
+    a.merge.next_emb = nullptr;   // the gather follows in the same CTA
     if (m.d > 8 * kRowThreads && m.d <= 8 * kWideRowThreads) {
         SPEC_CUDA_TRY(launch_pdl(merge_mix_512_kernel, dim3(rows), dim3(kWideRowThreads), 0, st, a));
         return SPEC_OK;

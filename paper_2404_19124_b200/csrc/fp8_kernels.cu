@@ -75,9 +75,10 @@ __global__ void __launch_bounds__(kRescoreThreads) merge_rescore_kernel(RescoreA
     const float base = (tid == 0 && a.merge.score_in) ? __ldcg(a.merge.score_in + r) : 0.0f;
     // short list: twice the branching factor plus two, at least 8, at most one per warp
     const int n_short = min(kShortList, max(8, 2 * a.merge.topk + 2));
-    merge_select<kRescoreThreads, BlockSync>(a.merge, r, tid, &sc, n_short);
+    const MergeOut o = merge_select<kRescoreThreads, 8, BlockSync>(a.merge, r, tid, &sc, n_short);
+    const int short_id = o.id;   // lane j: the j-th short-listed token
     // exact logit of short-listed token `warp`: dot product of two bf16 rows, fp32 accumulation
-    const int v = warp < n_short ? sc.out_id[warp] : -1;
+    const int v = warp < n_short ? __shfl_sync(0xffffffffu, short_id, warp) : -1;
     float acc = 0.0f;
     if (v >= 0 && v < a.V) {
         const uint16_t *w = a.W + (size_t)v * a.d, *s = a.S + (size_t)r * a.d;
@@ -112,8 +113,8 @@ __global__ void __launch_bounds__(kRescoreThreads) merge_rescore_kernel(RescoreA
     // warp 0: the top-k of the exact logits, (value desc, token id asc)
     if (warp == 0) {
         float val = lane < n_short ? exact[lane] : -INFINITY;
-        int id = lane < n_short ? sc.out_id[lane] : 0x7fffffff;
-        const float lse = sc.lse;
+        int id = lane < n_short ? short_id : 0x7fffffff;
+        const float lse = o.lse;
         const int topk = a.merge.topk;
         for (int j = 0; j < topk; ++j) {
             const uint32_t key = float_key(val);
@@ -122,6 +123,11 @@ __global__ void __launch_bounds__(kRescoreThreads) merge_rescore_kernel(RescoreA
             if (lane == 0) {
                 a.merge.tok_out[(size_t)r * topk + j] = (int)bi;
                 a.merge.score_out[(size_t)r * topk + j] = base + (key_float(bk) - lse);
+            }
+            if (a.merge.next_emb != nullptr && bi < (uint32_t)a.merge.next_emb_rows) {   // (see prefetch_embeddings)
+                const char *row = (const char *)a.merge.next_emb + (size_t)bi * a.merge.next_emb_bytes;
+                for (int i = lane * 128; i < a.merge.next_emb_bytes; i += 32 * 128)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(row + i));
             }
             if (key == bk && (uint32_t)id == bi) {   // taken
                 val = -INFINITY;

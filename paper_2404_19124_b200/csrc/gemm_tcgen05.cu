@@ -34,8 +34,7 @@ struct GemmParams {
     uint32_t slot_bytes;
     int producers;           // TMA-issuing threads: 1 or 2
     uint32_t tbuf_bytes;     // transposed accumulator tile of a mode-3 job (0: none in this launch)
-    int32_t *clear;          // words that the first kernel of a draft sets to zero (the workspace header) ...
-    int clear_words;         // ... by CTA 0, after the preceding grid has completed; 0: nothing
+    DraftStart start;        // first kernel of a draft only
     int32_t *err;
 };
 
@@ -80,9 +79,18 @@ gemm_tc_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         // First kernel of a draft: the header (error word, per-sequence counters) starts at zero.  Nothing of
         // this draft has reported or counted yet: the counters are first touched by the last level's merge,
         // and a wait that runs out does so millions of polls after this point.
-        if (p.clear_words > 0 && blockIdx.x == 0)
-            for (int i = (int)threadIdx.x - kEpilogueFirst; i < p.clear_words; i += kEpilogueThreads)
-                p.clear[i] = 0;
+        if (p.start.clear != nullptr) {
+            const int u = (int)threadIdx.x - kEpilogueFirst;
+            if (blockIdx.x == 0)
+                for (int i = u; i < p.start.clear_words; i += kEpilogueThreads) p.start.clear[i] = 0;
+            for (int b = blockIdx.x; b < p.start.n_tok; b += gridDim.x) {
+                const int t = __ldcg(p.start.tok + b);
+                if (t < 0 || t >= p.start.emb_rows) continue;   // (the mix reports it)
+                const char *row = (const char *)p.start.emb + (size_t)t * p.start.emb_row_bytes;
+                for (int i = u * 128; i < p.start.emb_row_bytes; i += kEpilogueThreads * 128)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(row + i));
+            }
+        }
         for (int q = 0; ok && q < p.n_jobs; ++q) ok = epilogue_job(pp, p.job[q], ap);
     }
     pipe_teardown(pp, p.tmem_cols);
@@ -256,15 +264,13 @@ void set_gemm_producers(int n) { g_gemm_producers = n >= 2 ? 2 : 1; }
 
 // One launch, one or two contractions.  The tiles of the second are dealt to the CTAs starting where
 // the first one's stopped, so a CTA that got no tile of the first starts on the second at once.
-int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaStream_t st, int32_t *clear,
-                        int clear_words) {
+int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaStream_t st, const DraftStart *start) {
     if (n_calls < 1 || n_calls > kMaxJobs) return SPEC_ERR_INVALID_ARG;
     GemmParams p{};
     GemmMaps maps{};
     p.n_jobs = n_calls;
     p.producers = g_gemm_producers;
-    p.clear = clear;
-    p.clear_words = clear ? clear_words : 0;
+    if (start) p.start = *start;
     int max_block_n = 32;
     long long total_tiles = 0;
     for (int q = 0; q < n_calls; ++q) {

@@ -30,13 +30,9 @@ struct BlockSync {
 constexpr int kMaxGroupWarps = 16;
 constexpr int kMaxRounds = 16;        // most entries a selection can return (top-k itself needs at most 8)
 struct Scratch {
-    float red[32];
     float red_m[kMaxGroupWarps], red_s[kMaxGroupWarps];
-    uint32_t cand_k[2][kMaxGroupWarps];
-    int cand_i[2][kMaxGroupWarps];
-    float out_val[kMaxRounds];        // result of merge_select: values, best first ...
-    int out_id[kMaxRounds];           // ... and their token ids
-    float lse;
+    uint32_t cand_k[kMaxGroupWarps][kMaxRounds];   // every warp's best entries, best first: value keys ...
+    int cand_i[kMaxGroupWarps][kMaxRounds];        // ... and token ids
 };
 
 template <int kThreads, typename Sync>
@@ -80,11 +76,10 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int tid
     constexpr int kSp = 4;                                        // partial projections fetched per batch
     constexpr int kGroup = kIters >= 8 ? 1 : (kIters < kDepth ? kIters : kDepth);
     const int t = __ldcg(m.tok + r);
-    const bool tok_ok = (t >= 0) && (t < m.V);
-    if (!tok_ok && tid == 0) report_error(m.err, SPEC_ERR_TOKEN_RANGE);
+    bool tok_ok = false;
     const int d = m.d;
     const float *p = m.P + (size_t)(r / m.parent_div) * d;
-    const uint16_t *e = m.emb + (size_t)(tok_ok ? t : 0) * d;
+    const uint16_t *e = nullptr;
 
     float h[kIters][8];
     float sum = 0.0f;
@@ -96,8 +91,6 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int tid
 #pragma unroll
         for (int q = 0; q < kGroup; ++q) {
             const int i = ((g0 + q) * kThreads + tid) * 8;
-            ev[q] = make_uint4(0u, 0u, 0u, 0u);
-            if (i < d && tok_ok) ev[q] = *(const uint4 *)(e + i);
 #pragma unroll
             for (int sp = 0; sp < kSp; ++sp) {
                 pa[q][sp] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -107,6 +100,17 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int tid
                     pb[q][sp] = __ldcg((const float4 *)(p + sp * m.p_split_stride + i + 4));
                 }
             }
+        }
+        if (g0 == 0) {   // (only now: everything above is in flight while the token arrives)
+            tok_ok = (t >= 0) && (t < m.V);
+            if (!tok_ok && tid == 0) report_error(m.err, SPEC_ERR_TOKEN_RANGE);
+            e = m.emb + (size_t)(tok_ok ? t : 0) * d;
+        }
+#pragma unroll
+        for (int q = 0; q < kGroup; ++q) {
+            const int i = ((g0 + q) * kThreads + tid) * 8;
+            ev[q] = make_uint4(0u, 0u, 0u, 0u);
+            if (i < d && tok_ok) ev[q] = *(const uint4 *)(e + i);
         }
 #pragma unroll
         for (int q = 0; q < kGroup; ++q) {
@@ -228,43 +232,24 @@ __device__ __forceinline__ float key_float(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
 }
 
-// Sorts one tile's list (8 slots, any order, slots >= topk ignored) best first with a fixed network and
-// folds it into the sorted list (tv, ti): with both lists sorted, "the better of a[i] and b[7 - i]" keeps
-// the best 8 of the 16 as a bitonic sequence, which three compare-exchange stages sort (depth 10 in all,
-// where an insertion chain has 64).
-__device__ __forceinline__ void fold_tile_list(float (&tv)[SPEC_MAX_TOPK], int (&ti)[SPEC_MAX_TOPK], const float4 &v0,
-                                               const float4 &v1, const int4 &i0, const int4 &i1, int topk, bool valid) {
-    constexpr int kT = SPEC_MAX_TOPK;
-    static_assert(kT == 8, "the networks are written for lists of 8");
-    float lv[kT] = {v0.x, v0.y, v0.z, v0.w, v1.x, v1.y, v1.z, v1.w};
-    int li[kT] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
-#pragma unroll
-    for (int j = 0; j < kT; ++j) {
-        const bool none = (j >= topk) | !valid;   // slots past the list's length hold nothing
-        lv[j] = none ? -INFINITY : lv[j];
-        li[j] = none ? 0x7fffffff : li[j];
+// Sorts a list of kLen (4 or 8) entries best first with a fixed network.
+template <int kLen>
+__device__ __forceinline__ void sort_list(float (&v)[kLen], int (&i)[kLen]) {
+    static_assert(kLen == 4 || kLen == 8, "networks for 4 and 8 entries");
+#define SPEC_CX(a, b) order_pair(v[a], i[a], v[b], i[b])
+    if constexpr (kLen == 8) {
+        SPEC_CX(0, 2); SPEC_CX(1, 3); SPEC_CX(4, 6); SPEC_CX(5, 7);
+        SPEC_CX(0, 4); SPEC_CX(1, 5); SPEC_CX(2, 6); SPEC_CX(3, 7);
+        SPEC_CX(0, 1); SPEC_CX(2, 3); SPEC_CX(4, 5); SPEC_CX(6, 7);
+        SPEC_CX(2, 4); SPEC_CX(3, 5);
+        SPEC_CX(1, 4); SPEC_CX(3, 6);
+        SPEC_CX(1, 2); SPEC_CX(3, 4); SPEC_CX(5, 6);
+    } else {
+        SPEC_CX(0, 2); SPEC_CX(1, 3);
+        SPEC_CX(0, 1); SPEC_CX(2, 3);
+        SPEC_CX(1, 2);
     }
-    // 19-comparator sorting network for 8 inputs
-#define SPEC_CX(a, b) order_pair(lv[a], li[a], lv[b], li[b])
-    SPEC_CX(0, 2); SPEC_CX(1, 3); SPEC_CX(4, 6); SPEC_CX(5, 7);
-    SPEC_CX(0, 4); SPEC_CX(1, 5); SPEC_CX(2, 6); SPEC_CX(3, 7);
-    SPEC_CX(0, 1); SPEC_CX(2, 3); SPEC_CX(4, 5); SPEC_CX(6, 7);
-    SPEC_CX(2, 4); SPEC_CX(3, 5);
-    SPEC_CX(1, 4); SPEC_CX(3, 6);
-    SPEC_CX(1, 2); SPEC_CX(3, 4); SPEC_CX(5, 6);
 #undef SPEC_CX
-#pragma unroll
-    for (int j = 0; j < kT; ++j) {
-        const bool take = better(lv[kT - 1 - j], li[kT - 1 - j], tv[j], ti[j]);
-        tv[j] = take ? lv[kT - 1 - j] : tv[j];
-        ti[j] = take ? li[kT - 1 - j] : ti[j];
-    }
-#pragma unroll
-    for (int stride = kT / 2; stride > 0; stride >>= 1) {
-#pragma unroll
-        for (int j = 0; j < kT; ++j)
-            if ((j & stride) == 0) order_pair(tv[j], ti[j], tv[j + stride], ti[j + stride]);
-    }
 }
 
 __device__ __forceinline__ void fold_max_sum(float &m, float &s, const float2 &ms) {
@@ -276,122 +261,192 @@ __device__ __forceinline__ void fold_max_sum(float &m, float &s, const float2 &m
     }
 }
 
-// Thread t folds the lists of tiles t, t + kThreads, ... into one sorted list of 8 in registers, two
-// tiles per trip with all ten loads issued before the first is used.  The group then extracts the
-// `rounds` best (rounds <= kMaxRounds) in as many rounds; a round is two warp-wide integer reductions
-// (redux.sync: maximum of the value keys, then minimum token id among the lanes that hold it) and one
-// shared-memory exchange between the warps.  Results: sc->out_val / out_id (best first; exhausted slots
-// hold -inf / 0x7fffffff) and sc->lse, valid for the whole group after the function returns.
-template <int kThreads, typename Sync>
-__device__ __forceinline__ void merge_select(const MergeArgs &g, int r, int tid, Scratch *sc, int rounds) {
+// One partial list as it was written by the head GEMM.
+template <int kLen>
+struct TileList {
+    float2 ms;
+    float4 v[kLen / 4];
+    int4 i[kLen / 4];
+};
+
+template <int kLen>
+__device__ __forceinline__ void load_list(TileList<kLen> &l, const MergeArgs &g, size_t tile, bool valid) {
+    l.ms = make_float2(-INFINITY, 0.0f);
+    if (valid) {
+        l.ms = __ldcg((const float2 *)g.part_ms + tile);
+#pragma unroll
+        for (int q = 0; q < kLen / 4; ++q) {
+            l.v[q] = __ldcg((const float4 *)g.part_val + 2 * tile + q);
+            l.i[q] = __ldcg((const int4 *)g.part_idx + 2 * tile + q);
+        }
+    }
+}
+
+// What merge_select leaves in every warp of the group: lane j < rounds holds the j-th best entry of the row
+// (-inf / 0x7fffffff when there are fewer), all lanes its log-sum-exp.
+struct MergeOut {
+    float val;
+    int id;
+    float lse;
+};
+
+// The `rounds` best entries (rounds <= kMaxRounds) of row r's partial lists and the row's log-sum-exp.  kLen is 4
+// when a list has at most four valid slots, else 8.
+// The step is a chain of latencies in a kernel that runs for a few microseconds, so it has one barrier and little
+// code: thread t takes the lists t, t + kThreads, ... one at a time, sorts the list in registers, and its warp extracts
+// its own `rounds` best with warp-wide integer reductions (redux.sync: maximum of the value keys, then minimum token id
+// among the lanes that hold it), carrying the winners of the lists so far as one more entry of lanes 0 .. rounds - 1.
+// After the barrier every warp merges the warps' sorted results, one head per lane, in `rounds` more rounds, so that
+// no second barrier is needed.  143 lists of a 16-row level: 5.2 us for the whole kernel with a running list of eight
+// folded per thread and block-wide rounds (three times the code), 3.6 now; the last level with its prune 10.4 -> 7.1 (7B
+// shape), 13.5 -> 9.3 (13B).
+template <int kThreads, int kLen, typename Sync>
+__device__ __forceinline__ MergeOut merge_select(const MergeArgs &g, int r, int tid, Scratch *sc, int rounds) {
     constexpr int kWarps = kThreads / 32;
-    constexpr int kT = SPEC_MAX_TOPK;
     static_assert(kWarps <= kMaxGroupWarps, "scratch arrays");
     const int lane = tid & 31, warp = tid >> 5;
-    const int n_tiles = g.n_tiles, topk = g.list_len > 0 ? g.list_len : g.topk;   // slots to read per list
-    const float4 *pv4 = (const float4 *)(g.part_val + (size_t)r * n_tiles * kT);
-    const int4 *pi4 = (const int4 *)(g.part_idx + (size_t)r * n_tiles * kT);
-    const float2 *pms = (const float2 *)(g.part_ms + (size_t)r * n_tiles * 2);
+    const int n_tiles = g.n_tiles, len = g.list_len > 0 ? g.list_len : g.topk;   // valid slots of every list
+    const size_t first = (size_t)r * n_tiles;
 
-    float tv[kT];
-    int ti[kT];
-#pragma unroll
-    for (int j = 0; j < kT; ++j) {
-        tv[j] = -INFINITY;
-        ti[j] = 0x7fffffff;
-    }
+    float cv = -INFINITY;   // the warp's winners so far: lane j the j-th
+    int ci = 0x7fffffff;
     float m = -INFINITY, s = 0.0f;
-    for (int t = tid; t < n_tiles; t += 2 * kThreads) {
-        const int t2 = t + kThreads;
-        const bool has2 = t2 < n_tiles;
-        const int tb = has2 ? t2 : t;
-        const float2 ms_a = __ldcg(pms + t), ms_b = __ldcg(pms + tb);
-        const float4 va0 = __ldcg(pv4 + 2 * t), va1 = __ldcg(pv4 + 2 * t + 1);
-        const int4 ia0 = __ldcg(pi4 + 2 * t), ia1 = __ldcg(pi4 + 2 * t + 1);
-        const float4 vb0 = __ldcg(pv4 + 2 * tb), vb1 = __ldcg(pv4 + 2 * tb + 1);
-        const int4 ib0 = __ldcg(pi4 + 2 * tb), ib1 = __ldcg(pi4 + 2 * tb + 1);
-        fold_max_sum(m, s, ms_a);
-        if (has2) fold_max_sum(m, s, ms_b);
-        fold_tile_list(tv, ti, va0, va1, ia0, ia1, topk, true);
-        fold_tile_list(tv, ti, vb0, vb1, ib0, ib1, topk, has2);
+    TileList<kLen> next;
+    load_list(next, g, first + tid, tid < n_tiles);
+    for (int t0 = warp * 32; t0 < n_tiles; t0 += kThreads) {   // (uniform over the warp)
+        const TileList<kLen> cur = next;
+        const bool valid = t0 + lane < n_tiles;
+        load_list(next, g, first + t0 + kThreads + lane, t0 + kThreads + lane < n_tiles);
+        fold_max_sum(m, s, cur.ms);
+        float tv[kLen];
+        int ti[kLen];
+#pragma unroll
+        for (int q = 0; q < kLen / 4; ++q) {
+            tv[4 * q] = cur.v[q].x; tv[4 * q + 1] = cur.v[q].y; tv[4 * q + 2] = cur.v[q].z; tv[4 * q + 3] = cur.v[q].w;
+            ti[4 * q] = cur.i[q].x; ti[4 * q + 1] = cur.i[q].y; ti[4 * q + 2] = cur.i[q].z; ti[4 * q + 3] = cur.i[q].w;
+        }
+#pragma unroll
+        for (int j = 0; j < kLen; ++j) {
+            const bool none = (j >= len) | !valid;   // slots past the list's length hold nothing
+            tv[j] = none ? -INFINITY : tv[j];
+            ti[j] = none ? 0x7fffffff : ti[j];
+        }
+        sort_list<kLen>(tv, ti);
+        float nv = -INFINITY;
+        int ni = 0x7fffffff;
+#pragma unroll 1
+        for (int j = 0; j < rounds; ++j) {
+            const bool carried = better(cv, ci, tv[0], ti[0]);
+            const float hv = carried ? cv : tv[0];
+            const int hi = carried ? ci : ti[0];
+            const uint32_t key = float_key(hv);
+            const uint32_t bk = __reduce_max_sync(0xffffffffu, key);
+            const int bi = (int)__reduce_min_sync(0xffffffffu, key == bk ? (uint32_t)hi : 0xffffffffu);
+            const bool mine = (key == bk) & (hi == bi);   // token ids are unique, so one lane owns a real entry
+            const bool pop = mine & !carried;
+            cv = mine & carried ? -INFINITY : cv;
+            ci = mine & carried ? 0x7fffffff : ci;
+#pragma unroll
+            for (int q = 0; q < kLen - 1; ++q) {
+                tv[q] = pop ? tv[q + 1] : tv[q];
+                ti[q] = pop ? ti[q + 1] : ti[q];
+            }
+            tv[kLen - 1] = pop ? -INFINITY : tv[kLen - 1];
+            ti[kLen - 1] = pop ? 0x7fffffff : ti[kLen - 1];
+            nv = lane == j ? key_float(bk) : nv;
+            ni = lane == j ? bi : ni;
+        }
+        cv = nv;
+        ci = ni;
     }
-    // log-sum-exp of the whole row
+    // the warp's (max, sum-exp)
     float wm = m;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xffffffffu, wm, off));
     float ws = (m > -INFINITY) ? s * __expf(m - wm) : 0.0f;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, off);
-    Sync::sync();   // the scratch may still be read by a previous call
+    if (lane < rounds) {
+        sc->cand_k[warp][lane] = float_key(cv);
+        sc->cand_i[warp][lane] = ci;
+    }
     if (lane == 0) {
         sc->red_m[warp] = wm;
         sc->red_s[warp] = ws;
     }
     Sync::sync();
-    if (warp == 0) {   // one lane per warp's (max, sum): a second shuffle reduction
+    MergeOut out;
+    {
         const float pm = lane < kWarps ? sc->red_m[lane] : -INFINITY;
         const float ps = lane < kWarps ? sc->red_s[lane] : 0.0f;
         float bm = pm;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, off));
+        for (int off = kMaxGroupWarps / 2; off > 0; off >>= 1) bm = fmaxf(bm, __shfl_xor_sync(0xffffffffu, bm, off));
         float bs = pm > -INFINITY ? ps * __expf(pm - bm) : 0.0f;
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) bs += __shfl_xor_sync(0xffffffffu, bs, off);
-        if (lane == 0) sc->lse = bm + logf(bs);
+        for (int off = kMaxGroupWarps / 2; off > 0; off >>= 1) bs += __shfl_xor_sync(0xffffffffu, bs, off);
+        out.lse = __shfl_sync(0xffffffffu, bm + logf(bs), 0);
     }
-
+    out.val = -INFINITY;
+    out.id = 0x7fffffff;
+    const uint32_t none_key = float_key(-INFINITY);
+    uint32_t hk = lane < kWarps ? sc->cand_k[lane][0] : none_key;
+    uint32_t hi = lane < kWarps ? (uint32_t)sc->cand_i[lane][0] : 0x7fffffffu;
+    int used = 0;
+#pragma unroll 1
     for (int j = 0; j < rounds; ++j) {
-        const uint32_t my_key = float_key(tv[0]);
-        const uint32_t wk = __reduce_max_sync(0xffffffffu, my_key);
-        const uint32_t wi = __reduce_min_sync(0xffffffffu, my_key == wk ? (uint32_t)ti[0] : 0xffffffffu);
-        if (lane == 0) {
-            sc->cand_k[j & 1][warp] = wk;
-            sc->cand_i[j & 1][warp] = (int)wi;
+        const uint32_t bk = __reduce_max_sync(0xffffffffu, hk);
+        const uint32_t bi = __reduce_min_sync(0xffffffffu, hk == bk ? hi : 0xffffffffu);
+        if (lane == j) {
+            out.val = key_float(bk);
+            out.id = (int)bi;
         }
-        Sync::sync();   // rounds alternate between two buffers, so one barrier per round is enough
-        // every warp reduces the warps' candidates again, one per lane: two more redux instead of a scan
-        const uint32_t ck = lane < kWarps ? sc->cand_k[j & 1][lane] : 0u;
-        const uint32_t ci = lane < kWarps ? (uint32_t)sc->cand_i[j & 1][lane] : 0xffffffffu;
-        const uint32_t bk = __reduce_max_sync(0xffffffffu, ck);
-        const int bi = (int)__reduce_min_sync(0xffffffffu, (lane < kWarps && ck == bk) ? ci : 0xffffffffu);
-        if (ti[0] == bi && my_key == bk) {   // token ids are unique, so exactly one thread owns a real entry
-#pragma unroll
-            for (int q = 0; q < kT - 1; ++q) {
-                tv[q] = tv[q + 1];
-                ti[q] = ti[q + 1];
-            }
-            tv[kT - 1] = -INFINITY;
-            ti[kT - 1] = 0x7fffffff;
-        }
-        if (tid == 0) {
-            sc->out_val[j] = key_float(bk);
-            sc->out_id[j] = bi;
+        if (lane < kWarps && hk == bk && hi == bi) {
+            ++used;
+            hk = used < rounds ? sc->cand_k[lane][used] : none_key;
+            hi = used < rounds ? (uint32_t)sc->cand_i[lane][used] : 0x7fffffffu;
         }
     }
-    Sync::sync();
+    return out;
+}
+
+// The rows of the next level's embedding table that the children's gather is about to read, requested into L2 as soon
+// as their tokens are known: the gather is the next kernel's first dependent load and goes to DRAM otherwise.
+template <int kThreads>
+__device__ __forceinline__ void prefetch_embeddings(const MergeArgs &g, const MergeOut &o, int tid) {
+    if (g.next_emb == nullptr) return;
+    for (int j = 0; j < g.topk; ++j) {
+        const int t = __shfl_sync(0xffffffffu, o.id, j);
+        if (t < 0 || t >= g.next_emb_rows) continue;
+        const char *row = (const char *)g.next_emb + (size_t)t * g.next_emb_bytes;
+        for (int i = tid * 128; i < g.next_emb_bytes; i += kThreads * 128)
+            asm volatile("prefetch.global.L2 [%0];" ::"l"(row + i));
+    }
 }
 
 // The row's top-k tokens and log-probabilities become its children.
-template <int kThreads, typename Sync>
-__device__ __forceinline__ void merge_expand_row(const MergeArgs &g, int r, int tid, Scratch *sc) {
+template <int kThreads, int kLen, typename Sync>
+__device__ __forceinline__ MergeOut merge_expand_row(const MergeArgs &g, int r, int tid, Scratch *sc) {
     const float base = (tid < g.topk && g.score_in && !g.lse_out) ? __ldcg(g.score_in + r) : 0.0f;   // in flight during the merge
-    merge_select<kThreads, Sync>(g, r, tid, sc, g.topk);
+    const MergeOut o = merge_select<kThreads, kLen, Sync>(g, r, tid, sc, g.topk);
     if (tid < g.topk) {
-        g.tok_out[(size_t)r * g.topk + tid] = sc->out_id[tid];
-        g.score_out[(size_t)r * g.topk + tid] = g.lse_out ? sc->out_val[tid] : base + (sc->out_val[tid] - sc->lse);
+        g.tok_out[(size_t)r * g.topk + tid] = o.id;
+        g.score_out[(size_t)r * g.topk + tid] = g.lse_out ? o.val : base + (o.val - o.lse);
     }
-    if (g.lse_out != nullptr && tid == 0) g.lse_out[r] = sc->lse;
+    if (g.lse_out != nullptr && tid == 0) g.lse_out[r] = o.lse;
+    prefetch_embeddings<kThreads>(g, o, tid);
+    return o;
 }
 
 // The children of one parent row, all at once: gather + mix + LayerNorm + exact GELU of up to kBatch child
 // nodes per trip (Sec. 3.1: siblings share the projected parent state and differ in the token embedding).
-// `tok` holds the children's tokens (shared memory, written by the merge just before), `first_child` is the
-// row of child 0 in the next level.  The projected parent state (sum of the split-K partials, added in
+// Lane j of every warp holds child j's token (`tok`, as merge_select returns it), `first_child` is the row of child 0
+// in the next level.  The projected parent state (sum of the split-K partials, added in
 // ascending order) and the LayerNorm parameters are loaded once; per trip the embedding rows of the batch
 // are requested together and the two LayerNorm reductions are done for the whole batch with one barrier
 // each (red_a / red_b: kThreads / 32 x kBatch floats each; kBatch children per trip).  d <= 8 * kThreads * kIters, d % 8 == 0.
 template <int kThreads, int kIters, int kBatch, typename Sync>
-__device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int first_child, int n_child, const int *tok,
+__device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int first_child, int n_child, int tok,
                                              float *red_a, float *red_b, int tid) {
     constexpr int kWarps = kThreads / 32;
     const int d = m.d, lane = tid & 31, warp = tid >> 5;
@@ -424,7 +479,7 @@ __device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int f
         uint4 ev[kBatch][kIters];
 #pragma unroll
         for (int q = 0; q < kBatch; ++q) {
-            const int t = c0 + q < n_child ? tok[c0 + q] : -1;
+            const int t = c0 + q < n_child ? __shfl_sync(0xffffffffu, tok, c0 + q) : -1;
             const bool tok_ok = t >= 0 && t < m.V;
             if (c0 + q < n_child && !tok_ok && tid == 0) report_error(m.err, SPEC_ERR_TOKEN_RANGE);
 #pragma unroll

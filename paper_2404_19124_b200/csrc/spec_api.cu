@@ -329,6 +329,18 @@ MixArgs make_mix_args(const spec_handle_s *h, const DraftPlan &p, char *ws, cons
     return mx;
 }
 
+DraftStart make_draft_start(const spec_handle_s *h, const DraftPlan &p, const int32_t *last_tok, int B, int32_t *header) {
+    DraftStart s{};
+    s.clear = header;
+    s.clear_words = p.header_words;
+    s.tok = last_tok;
+    s.n_tok = B;
+    s.emb = h->w.emb[0];
+    s.emb_rows = h->w.V;
+    s.emb_row_bytes = 2 * h->w.d_inner;
+    return s;
+}
+
 PruneArgs make_prune_args(const DraftPlan &p, char *ws, const int32_t *topk) {
     PruneArgs pa{};
     pa.n = p.n;
@@ -539,6 +551,7 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
     float *part_ms = (float *)(ws + p.lay.part_ms);
     float *logits_scratch = (float *)(ws + p.lay.logits);
 
+    const DraftStart start = make_draft_start(h, p, last_tok, B, err);
     auto proj_call = [&](int l) { return make_proj_call(h, p, ws, ctx_state, B, l); };
     const PruneArgs pa = make_prune_args(p, ws, topk);
     const bool fold_prune = !h->profile;
@@ -555,7 +568,7 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
         if (!proj_done) {
             if (h->gemm_impl == 0) {
                 const GemmCall c = proj_call(l);
-                rc = launch_gemm_tc_jobs(&c, 1, err, st, l == 0 ? err : nullptr, p.header_words);
+                rc = launch_gemm_tc_jobs(&c, 1, err, st, l == 0 ? &start : nullptr);
             } else {
                 rc = run_gemm_store(h, parent_states, w.proj[l], parent_rows, w.d_inner, d_in_of(w, l),
                                     p.proj_block_n[l], P, err, st);
@@ -612,6 +625,11 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
         g.score_in = score_l;
         g.tok_out = (int32_t *)(ws + p.lay.tok[l + 1]);
         g.score_out = (float *)(ws + p.lay.score[l + 1]);
+        if (l + 1 < p.n) {
+            g.next_emb = w.emb[l + 1];
+            g.next_emb_rows = w.V;
+            g.next_emb_bytes = 2 * w.d_inner;
+        }
         if (l == p.n - 1 && fold_prune) {
             g.seq_done = (int32_t *)(ws + p.seq_done);
             g.rows_per_seq = rows / B;
@@ -722,7 +740,8 @@ int spec_draft_vp_local(spec_handle_t h, int level, const void *ctx_state, const
     const int l = level, rows = p.N[l];
     if (l == 0) {   // the first step of a draft clears the header and projects the context states
         const GemmCall c = make_proj_call(h, p, ws, ctx_state, B, 0);
-        rc = launch_gemm_tc_jobs(&c, 1, err, st, err, p.header_words);
+        const DraftStart start = make_draft_start(h, p, last_tok, B, err);
+        rc = launch_gemm_tc_jobs(&c, 1, err, st, &start);
         if (rc != SPEC_OK) return rc;
     }
     const MixArgs mx = make_mix_args(h, p, ws, last_tok, B, topk, l, err);

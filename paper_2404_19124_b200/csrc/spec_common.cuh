@@ -125,10 +125,18 @@ struct GemmCall {
     int M, N, Kd, block_n;
     GemmEpilogue epi;
 };
-// `clear` / `clear_words`: int32 words that CTA 0 zeroes once the preceding grid has completed (the first
-// kernel of a draft clears the workspace header this way); null: nothing.
-int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaStream_t st, int32_t *clear = nullptr,
-                        int clear_words = 0);
+// What the first kernel of a draft does beside its contraction, once the preceding grid has completed: CTA 0 zeroes
+// the workspace header, and the embedding rows of the last tokens, which the next kernel gathers, are requested into L2.
+struct DraftStart {
+    int32_t *clear;            // `clear_words` int32 words; null: nothing is cleared and nothing requested
+    int clear_words;
+    const int32_t *tok;        // [n_tok]
+    int n_tok;
+    const void *emb;           // bf16 [emb_rows, emb_row_bytes / 2]
+    int emb_rows, emb_row_bytes;
+};
+int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaStream_t st,
+                        const DraftStart *start = nullptr);
 
 // ---- the tensor-bound head on CTA pairs (gemm_pair.cu) --------------------------------------------
 int pair_block_n(int rows, int vocab_rows);
@@ -172,6 +180,9 @@ struct MergeArgs {
     const float *score_in;     // [rows] or null (score 0)
     int32_t *tok_out;          // [rows, topk]
     float *score_out;          // [rows, topk]
+    // The next level's embedding table (null: not prefetched), its rows and the bytes of one.
+    const void *next_emb;
+    int next_emb_rows, next_emb_bytes;
     // Raw form (lse_out != null), for a vocabulary shard: score_out receives the logits themselves and
     // lse_out [rows] the log-sum-exp over this shard's columns; score_in is ignored.
     float *lse_out;

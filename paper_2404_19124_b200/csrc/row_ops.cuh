@@ -605,7 +605,7 @@ __device__ __forceinline__ void load_path(const PruneArgs &pa, int L, int b, int
 template <int kThreads, typename Sync>
 __device__ __forceinline__ void prune_sequence(const float *leaf_score, const PruneArgs &pa, int L, int Lpad, int K,
                                                int32_t *cand_tok, float *cand_logp, int b, int tid, LeafKey *keys) {
-    constexpr int kOwn = 256 / kThreads > 0 ? 256 / kThreads : 1;   // leaves per thread in the ranked form
+    constexpr int kOwn = (256 + kThreads - 1) / kThreads;   // leaves per thread in the ranked form
     int32_t path[kOwn][SPEC_MAX_HEADS];
     if (L <= 256) {
 #pragma unroll

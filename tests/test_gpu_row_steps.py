@@ -1,0 +1,79 @@
+"""The row-wise steps of a draft at the sizes where their thread counts matter: partial lists per row and leaves per
+sequence below, at and above the threads of a CTA."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2404_19124_b200 import synth
+from helpers import LOGIT_TOL, TIE_TOL, DraftChecker, small_cfg, to_oracle_weights, weights_to_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2404_19124_b200 import build
+    build.build()
+    from paper_2404_19124_b200 import binding
+    return binding
+
+
+@pytest.mark.parametrize("fp8", [False, True])
+@pytest.mark.parametrize("topk,K", [((8, 4, 5), 160), ((7, 7, 3), 100), ((8, 4, 3, 2), 64), ((8, 4, 3, 2), 192),
+                                    ((8, 8, 4), 255), ((8, 8, 4), 256)])
+def test_prune_leaves_round_the_thread_counts(B, topk, K, fp8):
+    """147 to 256 leaves: more and fewer than the 160 (or 512) threads of the CTA that ranks them."""
+    cfg = small_cfg(d_base=48, d_inner=64, V=96, topk=topk, K=K, B=3, seed=K)
+    sw = synth.make_weights(cfg)
+    ow, gw = to_oracle_weights(sw), weights_to_cuda(sw)
+    ctx, tok = synth.make_draft_inputs(cfg)
+    h = B.spec_create(gw)
+    if fp8:
+        B.spec_attach_fp8_heads(h)
+        B.spec_set_option(h, B.SPEC_OPT_FP8_MAX_ROWS, 4096)
+    ct = torch.full((cfg.B, K, cfg.n), -1, dtype=torch.int32, device="cuda")
+    lp = torch.full((cfg.B, K), 1.0, device="cuda")
+    _, _, ws = B.spec_draft(h, ctx.cuda(), tok.cuda(), topk, K, cand_tok=ct, cand_logp=lp)
+    assert B.spec_poll_error(ws) == 0
+    lay = B.spec_draft_layout(h, cfg.B, topk, K)
+    L = cfg.leaves
+    leaf = ws[lay.score[cfg.n]:lay.score[cfg.n] + 4 * cfg.B * L].view(torch.float32).view(cfg.B, L)
+    want = torch.sort(leaf, dim=1, descending=True, stable=True)
+    assert torch.equal(lp, want.values[:, :K])
+    last = ws[lay.tok[cfg.n]:lay.tok[cfg.n] + 4 * cfg.B * L].view(torch.int32).view(cfg.B, L)
+    assert torch.equal(ct[:, :, -1], torch.gather(last, 1, want.indices[:, :K]))
+    if not fp8:
+        chk = DraftChecker(ow, topk, K)
+        for b in range(cfg.B):
+            chk.check(synth.bf16_bits(ctx)[b], int(tok[b]), ct[b].cpu().numpy(), lp[b].cpu().numpy())
+    B.spec_destroy(h)
+
+
+@pytest.mark.parametrize("swap", [0, 128])
+@pytest.mark.parametrize("k", [1, 4, 5, 8])
+@pytest.mark.parametrize("V", [159 * 32, 160 * 32, 161 * 32, 320 * 32 + 1, 80000])
+def test_merge_lists_round_the_thread_counts(B, V, k, swap):
+    """Tiles 32 wide: 159 to 2500 partial lists per row for 160 threads (one, two, many lists per thread)."""
+    rows, d = 5, 64
+    cfg = small_cfg(d_base=d, d_inner=d, V=V, topk=(2, 2), seed=V % 97 + k)
+    sw = synth.make_weights(cfg)
+    ow, gw = to_oracle_weights(sw), weights_to_cuda(sw)
+    h = B.spec_create(gw)
+    if swap:
+        B.spec_set_option(h, B.SPEC_OPT_HEAD_SWAP_MAX_ROWS, swap)
+    else:
+        B.spec_set_option(h, B.SPEC_OPT_HEAD_BLOCK_N, 32)
+    g = torch.Generator().manual_seed(k)
+    S = torch.randn(rows, d, generator=g).to(torch.bfloat16)
+    tok, logp, ws = B.spec_head_topk(h, 0, S.cuda(), k)
+    assert B.spec_poll_error(ws) == 0
+    logits = oracle.stage_logits(ow, 0, S.to(torch.float32).numpy())
+    lse = torch.logsumexp(torch.from_numpy(logits).double(), 1).numpy()
+    got = tok.cpu().numpy()
+    for r in range(rows):
+        ids, _ = oracle.topk(logits[r], k)
+        near = np.abs(logits[r][got[r]] - logits[r][ids])      # (a near-tie may be ordered either way)
+        assert len(set(got[r].tolist())) == k and near.max() <= TIE_TOL
+        assert np.abs(logp[r].cpu().numpy() - (logits[r][got[r]] - lse[r])).max() <= LOGIT_TOL
+    B.spec_destroy(h)

@@ -62,8 +62,8 @@ enum spec_option {
     SPEC_OPT_HEAD_SWAP_MAX_ROWS = 5, /* levels with at most this many nodes (0 .. 128) run the head GEMM
                                   with the weight matrix on the 128-row side of the MMA and the nodes
                                   as columns, so the tensor work follows the number of nodes; 0 = never;
-                                  -1 (default) = automatic: up to 8 nodes, or up to 32 when the
-                                  vocabulary gives every CTA at least four 128-row tiles.  Ignored
+                                  -1 (default) = automatic: up to 32 nodes, up to 64 when the
+                                  vocabulary gives every CTA a full 128-row tile.  Ignored
                                   while SPEC_OPT_HEAD_BLOCK_N forces a tile width.              */
     SPEC_OPT_GEMM_PRODUCERS = 6, /* 1 or 2 (default) threads per CTA issue the TMA copies of the GEMM
                                   kernels; process-wide, not per handle                        */

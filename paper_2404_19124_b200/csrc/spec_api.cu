@@ -78,15 +78,17 @@ int head_block_n_for(const spec_handle_s *h, int rows) {
 }
 
 // Levels of few nodes run the head with the weights on the 128-row side of the MMA (epilogue mode 3).
-// Which levels: set explicitly, or by what measured faster inside whole drafts.  The swapped form costs fewer
-// TMA requests and MMA cycles per weight byte but ends every CTA with a longer epilogue (transposition, scan,
-// combination of the segment lists), which only a long weight stream pays back: up to 8 nodes at any
-// vocabulary, up to 32 nodes when every CTA streams at least four 128-row tiles (V = 128256: 121 against
-// 137 us at 16 nodes); at 16 nodes and V = 32000 the one-thread-per-node form is 2-3 us per level faster.
+// Which levels: set explicitly, or by what measured faster inside whole drafts.  The swapped form costs fewer TMA
+// requests and MMA cycles per weight byte, and up to eight threads share a node's selection, but every tile is transposed
+// through shared memory first.  Three single-candidate levels, one thread per node row -> swapped (us per draft):
+// d 1024, V 1500, 12 / 24 / 48 nodes 52.3 -> 48.9 / 50.3 / 52.0; V 4500 58.3, 58.2, 56.7 -> 50.9 / 52.7 / 54.6;
+// V 12000 62.8, 62.0, 60.3 -> 52.8 / 54.6 / 57.4; d 2048, V 12000, 64 / 96 nodes 72.1, 74.2 -> 72.7 / 79.6;
+// V 32000, 64 / 80 / 128 nodes 109.6, 112.5, 119.0 -> 106.7 / 114.4 / 128.8.
 bool head_swapped_for(const spec_handle_s *h, int rows) {
     if (h->gemm_impl != 0 || h->head_block_n != 0 || rows > 128) return false;
     if (h->swap_max_rows >= 0) return rows <= h->swap_max_rows;
-    return rows <= 8 || (rows <= 32 && h->head_rows >= 4 * 128 * num_sms());
+    const int rows_per_sm = h->head_rows / num_sms();
+    return rows <= (rows_per_sm >= 128 ? 64 : rows_per_sm >= 30 ? 48 : 32);
 }
 
 // Levels of more than 128 nodes (several 128-row tiles per weight tile) may run on CTA pairs.

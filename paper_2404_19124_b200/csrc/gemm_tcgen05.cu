@@ -43,7 +43,10 @@ struct GemmMaps {
     CUtensorMap a_short;   // mode 3 (job 0): the weight box of the last, shorter tile of every CTA
 };
 
-__global__ void __launch_bounds__(kThreads, 1)
+// 112 registers: registers are given out for four warps at a time, so the CTA counts as eight warps and 112 is what lets
+// it share an SM with a CTA of the widest row kernel (16 warps of 72): 8 * 32 * 112 + 16 * 32 * 72 = 65536.  With 118 the
+// head of a level of 96 nodes could not become resident, and request its first weights, before the mix had ended.
+__global__ void __maxnreg__(112)
 gemm_tc_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ GemmParams p) {
     extern __shared__ uint8_t smem_raw[];
     const Pipe pp = pipe_setup(smem_raw, p.stages, p.slot_bytes, p.tmem_cols, p.acc_stride, p.tbuf_bytes, p.err);
@@ -62,6 +65,10 @@ gemm_tc_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
                                  [] { griddep_wait(); return true; });
             if (!ok) producer_drain(pp, rp, issued);
         }
+        // The other lanes must not reach the dependency wait before the producing lane does: the instruction holds
+        // up the whole warp, so that without this barrier the weights were requested only once the preceding grid
+        // had completed.
+        __syncwarp();
         griddep_wait();
     } else if (warp == 1) {
         griddep_wait();

@@ -128,8 +128,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Bounded wait.  Returns false when it gave up (or another role already did).
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Barriers *bars, int32_t *err) {
+// Bounded wait.  Returns false when it gave up (or another role already did).  The polling loop is one copy out of line:
+// what a launch executes it fetches cold, so the roles are kept small.
+static __device__ __noinline__ bool mbar_poll(uint64_t *bar, uint32_t parity, Barriers *bars, int32_t *err) {
     for (uint32_t it = 0; it < kSpinMax; ++it) {
         if (mbar_try_wait(bar, parity)) return true;
         if (it > kSpinFast) {
@@ -140,6 +141,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Barrie
     bars->abort_flag = 1;
     report_error(err, SPEC_ERR_TIMEOUT);
     return false;
+}
+__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Barriers *bars, int32_t *err) {
+    return mbar_try_wait(bar, parity) || mbar_poll(bar, parity, bars, err);
 }
 
 __device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *map, int c0, int c1, uint64_t *bar) {
@@ -362,62 +366,60 @@ __device__ __forceinline__ void advance(const Pipe &pp, RingPos &rp) {
 // loads nor waits.  `issued` counts slots filled since the kernel started (for the abort path).
 // Producer `me` of `n_prod` walks every slot like the others and fills the slots whose running number
 // `issued` (counted over all jobs of the launch) is congruent to `me` (n_prod is a power of two).
+// One loop serves the first fill, its state operands and the rest, again to keep the code small.
 template <typename DepWait>
 __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, const CUtensorMap *tmap_a,
                                             const CUtensorMap *tmap_a_short, const CUtensorMap *tmap_b, RingPos &rp,
                                             int &issued, int me, int n_prod, DepWait dep_wait) {
-    const int ke = slab_elems(j);
-    const uint32_t b_bytes = (uint32_t)j.block_n * kSlabBytes;
     const TileWalk w = walk_of(j);
     if (w.first >= w.end) return true;
+    const int ke = slab_elems(j);
+    const uint32_t b_bytes = (uint32_t)j.block_n * kSlabBytes;
+    const uint32_t w_at = j.w_is_a ? 0u : (uint32_t)kABytes, s_at = j.w_is_a ? (uint32_t)kABytes : 0u;   // in the slot
+    const CUtensorMap *s_map = j.w_is_a ? tmap_b : tmap_a;
     Barriers *bars = pp.bars;
     const uint64_t once = evict_first_policy();
-    int n_pre = 0;
-    {
-        const TilePos t0 = pos_of(j, w, w.first);
-        const CUtensorMap *ma = t0.a_rows == kBlockM ? tmap_a : tmap_a_short;
-        const uint32_t tx = (uint32_t)t0.a_rows * kSlabBytes + b_bytes;
-        n_pre = min(pp.stages, t0.kb1 - t0.kb0);
-        RingPos q = rp;
-        for (int i = 0; i < n_pre; ++i) {
-            if (((issued + i) & (n_prod - 1)) == me) {
-                if (!mbar_wait(&bars->empty[q.stage], q.phase ^ 1u, bars, pp.err)) return false;
-                uint8_t *sa = pp.tiles + (size_t)q.stage * pp.slot_bytes;
-                mbar_arrive_expect_tx(&bars->full[q.stage], tx);
-                if (j.w_is_a) tma_load_2d_once(sa, ma, (t0.kb0 + i) * ke, t0.a_row, &bars->full[q.stage], once);
-                else tma_load_2d_once(sa + kABytes, tmap_b, (t0.kb0 + i) * ke, t0.b_row, &bars->full[q.stage], once);
+    int tile = w.first;
+    TilePos t = pos_of(j, w, tile);
+    const int n_pre = min(pp.stages, t.kb1 - t.kb0);   // slots of the first fill
+    bool first_fill = true;
+    RingPos q = rp;
+    int kb = t.kb0, done = 0;
+    for (;;) {
+        if (((issued + done) & (n_prod - 1)) == me) {
+            const bool fetched = !first_fill && done < n_pre;   // the weights of this slot are already on their way
+            uint8_t *slot = pp.tiles + (size_t)q.stage * pp.slot_bytes;
+            uint64_t *full = &bars->full[q.stage];
+            if (!fetched) {
+                if (!mbar_wait(&bars->empty[q.stage], q.phase ^ 1u, bars, pp.err)) {
+                    rp = q;
+                    issued += done;
+                    return false;
+                }
+                mbar_arrive_expect_tx(full, (uint32_t)t.a_rows * kSlabBytes + b_bytes);
+                const CUtensorMap *w_map = !j.w_is_a ? tmap_b : t.a_rows == kBlockM ? tmap_a : tmap_a_short;
+                tma_load_2d_once(slot + w_at, w_map, kb * ke, j.w_is_a ? t.a_row : t.b_row, full, once);
             }
-            advance(pp, q);
+            if (!first_fill) tma_load_2d(slot + s_at, s_map, kb * ke, j.w_is_a ? t.b_row : t.a_row, full);
+        }
+        advance(pp, q);
+        ++done;
+        ++kb;
+        if (first_fill && done == n_pre) {
+            if (!dep_wait()) return false;
+            first_fill = false;
+            q = rp;
+            done = 0;
+            kb = t.kb0;
+        } else if (kb == t.kb1) {
+            tile += w.step;
+            if (tile >= w.end) break;
+            t = pos_of(j, w, tile);
+            kb = t.kb0;
         }
     }
-    if (!dep_wait()) return false;
-    int done = 0;   // k blocks of this job handled so far
-    for (int tile = w.first; tile < w.end; tile += w.step) {
-        const TilePos t = pos_of(j, w, tile);
-        const CUtensorMap *ma = t.a_rows == kBlockM ? tmap_a : tmap_a_short;
-        const uint32_t tx = (uint32_t)t.a_rows * kSlabBytes + b_bytes;
-        for (int kb = t.kb0; kb < t.kb1; ++kb) {
-            uint8_t *sa = pp.tiles + (size_t)rp.stage * pp.slot_bytes;
-            uint8_t *sb = sa + kABytes;
-            const bool prefetched = done < n_pre;   // the weights of this slot are already on their way
-            if ((issued & (n_prod - 1)) == me) {
-                if (!prefetched) {
-                    if (!mbar_wait(&bars->empty[rp.stage], rp.phase ^ 1u, bars, pp.err)) return false;
-                    mbar_arrive_expect_tx(&bars->full[rp.stage], tx);
-                }
-                if (j.w_is_a) {
-                    if (!prefetched) tma_load_2d_once(sa, ma, kb * ke, t.a_row, &bars->full[rp.stage], once);
-                    tma_load_2d(sb, tmap_b, kb * ke, t.b_row, &bars->full[rp.stage]);
-                } else {
-                    tma_load_2d(sa, ma, kb * ke, t.a_row, &bars->full[rp.stage]);
-                    if (!prefetched) tma_load_2d_once(sb, tmap_b, kb * ke, t.b_row, &bars->full[rp.stage], once);
-                }
-            }
-            ++done;
-            ++issued;
-            advance(pp, rp);
-        }
-    }
+    rp = q;
+    issued += done;
     return true;
 }
 

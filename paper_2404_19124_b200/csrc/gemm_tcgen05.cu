@@ -253,12 +253,16 @@ int plan_job(tc::GemmJob *j, int M, int N, int Kd, int block_n, const GemmEpilog
     j->deal_ctas = 0;
     j->epi = epi;
     j->rows_per_cta = 0;
+    j->halves = 0;
     if (epi.mode == 3) {   // all nodes in one tile column; every CTA of the deal leaves one list per node
         if (N > kBlockM || j->n_tiles != 1 || fp8) return SPEC_ERR_SHAPE;
         j->epi.segs = swapped_head_segs(N);
         j->rows_per_cta = swapped_rows_per_cta(M);
         j->deal_ctas = (M + j->rows_per_cta - 1) / j->rows_per_cta;
         j->epi.n_parts = j->deal_ctas;
+        // Rows of a multiple of 4096 bytes only: the others gain nothing and pay 0.5 % for the second accumulator.  (Not in a
+        // vocabulary shard: shards whose sizes put them on different forms must agree on equal logits.)
+        j->halves = Kd % 2048 == 0 && !epi.sharded ? 1 : 0;
     }
     return SPEC_OK;
 }
@@ -278,7 +282,7 @@ int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaSt
     p.n_jobs = n_calls;
     p.producers = g_gemm_producers;
     if (start) p.start = *start;
-    int max_block_n = 32;
+    int max_block_n = 32, max_acc = 32;   // widest tile; most accumulator columns of one tile
     long long total_tiles = 0;
     for (int q = 0; q < n_calls; ++q) {
         const GemmCall &c = calls[q];
@@ -291,6 +295,7 @@ int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaSt
                        p.job[q].fp8 != 0);
         if (rc != SPEC_OK) return rc;
         if (c.block_n > max_block_n) max_block_n = c.block_n;
+        if (c.block_n << p.job[q].halves > max_acc) max_acc = c.block_n << p.job[q].halves;
         if (c.epi.mode == 3) {
             if (q != 0) return SPEC_ERR_INVALID_ARG;   // its CTAs are the first of the grid
             p.tbuf_bytes = (uint32_t)c.block_n * kTPitch * sizeof(float);
@@ -319,9 +324,9 @@ int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaSt
     if (p.stages > kMaxStages) p.stages = kMaxStages;
     if (p.stages < 2) return SPEC_ERR_SHAPE;
     int cols = 32;
-    while (cols < 2 * max_block_n) cols <<= 1;
+    while (cols < 2 * max_acc) cols <<= 1;
     p.tmem_cols = cols;
-    p.acc_stride = max_block_n;
+    p.acc_stride = max_acc;
     p.err = err;
 
     const size_t smem = 1024 + (size_t)p.stages * p.slot_bytes + p.tbuf_bytes + sizeof(Barriers);

@@ -270,6 +270,7 @@ GemmCall make_head_call(const spec_handle_s *h, const DraftPlan &p, char *ws, in
     c.epi.part_ms = (float *)(ws + p.lay.part_ms);
     c.epi.topk = topk_l;
     c.epi.idx_offset = h->vocab_offset;
+    c.epi.sharded = h->vp_ranks > 1;
     if (p.use_fp8[l]) {   // e4m3 operands; every tile keeps SPEC_MAX_TOPK candidates by approximate logit
         c.A = ws + p.lay.state8;
         c.B = h->head8[l];

@@ -68,6 +68,7 @@ struct GemmJob {
     int rows_per_cta;           // mode 3: A rows (vocabulary rows) of every CTA of the deal, a multiple of 8: CTA c
                                 // of the deal takes rows [c * rows_per_cta, (c + 1) * rows_per_cta) as 128-row tiles
                                 // plus one shorter tile, so that every CTA streams the same number of bytes
+    int halves;                 // mode 3: 1: the two halves of the K range have accumulators of their own (first_half)
     GemmEpilogue epi;
 };
 
@@ -304,7 +305,8 @@ __device__ __forceinline__ int num_k_blocks(const GemmJob &j) { return (j.Kd + s
 struct TileWalk { int first, end, step, rel; };
 struct TilePos {
     int a_row, b_row;    // first row of the A box and of the B box
-    int kb0, kb1;        // K blocks [kb0, kb1)
+    int kb0, kb1;        // K blocks [kb0, kb1) ...
+    int k_off;           // ... visited from kb0 + k_off on, wrapping round at the last one (see first_half)
     int a_rows;          // rows of the A box (mode 3: the last tile of a CTA may be shorter)
     int split, m_tile, n_tile;
 };
@@ -330,13 +332,23 @@ __device__ __forceinline__ TileWalk walk_of(const GemmJob &j) {
     return w;
 }
 
+// The CTAs of a launch walk their weight tiles in step, so that at any moment all of them read the same few columns.
+// When a row of the matrix is a power of two long those addresses differ only in their high bits and crowd on a part of
+// the memory channels.  In a job with `halves` every second weight tile therefore starts with the second half of the K
+// range.  Each half is summed in accumulator columns of its own and the epilogue adds the two, so that a logit does not
+// depend on which half came first (equal rows of the matrix give equal logits wherever they lie).  Rows of 8192 bytes:
+// single-candidate chain at the 13B widths 168.4 -> 161.6 us per draft, 64 sequences at the 34B widths 241 -> 234; more
+// groups of tiles than two are no better.
+__device__ __forceinline__ int first_half(int num_kb) { return num_kb / 2; }   // K blocks of the first half
+
 __device__ __forceinline__ TilePos pos_of(const GemmJob &j, const TileWalk &w, int t) {
     TilePos q;
-    const int num_kb = (j.Kd + (j.fp8 ? kSlabBytes : kSlabBytes / 2) - 1) / (j.fp8 ? kSlabBytes : kSlabBytes / 2);
+    const int num_kb = num_k_blocks(j);
     if (j.epi.mode == 3) {
         q.a_row = w.rel * j.rows_per_cta + t * kBlockM;
         q.b_row = 0;
         q.kb0 = 0; q.kb1 = num_kb;
+        q.k_off = j.halves && (w.rel & 1) ? first_half(num_kb) : 0;
         q.a_rows = (t + 1) * kBlockM <= j.rows_per_cta ? kBlockM : j.rows_per_cta - t * kBlockM;
         q.split = 0; q.m_tile = t; q.n_tile = 0;
     } else {
@@ -349,6 +361,7 @@ __device__ __forceinline__ TilePos pos_of(const GemmJob &j, const TileWalk &w, i
         q.b_row = q.n_tile * j.block_n;
         q.kb0 = q.split * j.kb_per_split;
         q.kb1 = min(num_kb, q.kb0 + j.kb_per_split);
+        q.k_off = 0;
         q.a_rows = kBlockM;
     }
     return q;
@@ -373,7 +386,7 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
                                             int &issued, int me, int n_prod, DepWait dep_wait) {
     const TileWalk w = walk_of(j);
     if (w.first >= w.end) return true;
-    const int ke = slab_elems(j);
+    const int ke = slab_elems(j), num_kb = num_k_blocks(j);
     const uint32_t b_bytes = (uint32_t)j.block_n * kSlabBytes;
     const uint32_t w_at = j.w_is_a ? 0u : (uint32_t)kABytes, s_at = j.w_is_a ? (uint32_t)kABytes : 0u;   // in the slot
     const CUtensorMap *s_map = j.w_is_a ? tmap_b : tmap_a;
@@ -384,7 +397,7 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
     const int n_pre = min(pp.stages, t.kb1 - t.kb0);   // slots of the first fill
     bool first_fill = true;
     RingPos q = rp;
-    int kb = t.kb0, done = 0;
+    int kb = t.kb0, kx = t.kb0 + t.k_off, done = 0;   // kx: the column block of slot kb
     for (;;) {
         if (((issued + done) & (n_prod - 1)) == me) {
             const bool fetched = !first_fill && done < n_pre;   // the weights of this slot are already on their way
@@ -398,12 +411,13 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
                 }
                 mbar_arrive_expect_tx(full, (uint32_t)t.a_rows * kSlabBytes + b_bytes);
                 const CUtensorMap *w_map = !j.w_is_a ? tmap_b : t.a_rows == kBlockM ? tmap_a : tmap_a_short;
-                tma_load_2d_once(slot + w_at, w_map, kb * ke, j.w_is_a ? t.a_row : t.b_row, full, once);
+                tma_load_2d_once(slot + w_at, w_map, kx * ke, j.w_is_a ? t.a_row : t.b_row, full, once);
             }
-            if (!first_fill) tma_load_2d(slot + s_at, s_map, kb * ke, j.w_is_a ? t.b_row : t.a_row, full);
+            if (!first_fill) tma_load_2d(slot + s_at, s_map, kx * ke, j.w_is_a ? t.b_row : t.a_row, full);
         }
         advance(pp, q);
         ++done;
+        if (++kx == num_kb) kx = 0;
         ++kb;
         if (first_fill && done == n_pre) {
             if (!dep_wait()) return false;
@@ -411,11 +425,13 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
             q = rp;
             done = 0;
             kb = t.kb0;
+            kx = t.kb0 + t.k_off;
         } else if (kb == t.kb1) {
             tile += w.step;
             if (tile >= w.end) break;
             t = pos_of(j, w, tile);
             kb = t.kb0;
+            kx = t.kb0 + t.k_off;
         }
     }
     rp = q;
@@ -489,13 +505,18 @@ __device__ __forceinline__ bool mma_job_kind(const Pipe &pp, const GemmJob &j, R
         const uint32_t tmem_d = pp.tmem_base + (uint32_t)(ap.acc * pp.acc_stride);
         const TilePos t = pos_of(j, w, tile);
         uint32_t acc = 0u;
+        // with `halves`: `left` blocks of this half to go; the other half's accumulator is `flip` columns away
+        uint32_t d = tmem_d + (t.k_off ? (uint32_t)j.block_n : 0u);
+        const uint32_t flip = t.k_off ? tmem_d : tmem_d + (uint32_t)j.block_n;
+        int left = j.halves ? (t.k_off ? t.kb1 - t.k_off : first_half(t.kb1)) : t.kb1;
         // (a short A box leaves the rest of the 128 rows as they were: those accumulator lanes are never read)
         for (int kb = t.kb0; kb < t.kb1; ++kb) {
             if (!mbar_wait(&bars->full[rp.stage], rp.phase, bars, pp.err)) return false;
             tc_fence_after();
             const uint32_t lo_a = lo_base + (uint32_t)rp.stage * lo_slot;
-            umma_k_block<kFp8>(tmem_d, lo_a, lo_a + (kABytes >> 4), desc_hi, idesc, acc);
+            umma_k_block<kFp8>(d, lo_a, lo_a + (kABytes >> 4), desc_hi, idesc, acc);
             acc = 1u;
+            if (--left == 0) { d = flip; acc = 0u; }
             umma_commit(&bars->empty[rp.stage]);   // frees the slot once these MMAs have read it
             advance(pp, rp);
         }
@@ -826,6 +847,12 @@ __device__ __forceinline__ bool epilogue_job_swapped(const Pipe &pp, const GemmJ
         for (int c = 0; c < nodes; c += 16) {
             float v[16];
             tmem_ld16(taddr + c, v);
+            if (j.halves) {
+                float v2[16];
+                tmem_ld16(taddr + j.block_n + c, v2);
+#pragma unroll
+                for (int i = 0; i < 16; ++i) v[i] += v2[i];
+            }
 #pragma unroll
             for (int i = 0; i < 16; ++i)
                 if (c + i < nodes) pp.tbuf[(c + i) * kTPitch + vrow] = v_ok ? v[i] : -INFINITY;

@@ -77,3 +77,28 @@ def test_merge_lists_round_the_thread_counts(B, V, k, swap):
         assert len(set(got[r].tolist())) == k and near.max() <= TIE_TOL
         assert np.abs(logp[r].cpu().numpy() - (logits[r][got[r]] - lse[r])).max() <= LOGIT_TOL
     B.spec_destroy(h)
+
+
+@pytest.mark.parametrize("rows", [1, 17, 48])
+@pytest.mark.parametrize("d", [2048, 4096, 2056])
+def test_equal_rows_give_equal_logits_in_every_tile(B, d, rows):
+    """Nodes as MMA columns, rows of 4096 and 8192 bytes: every second weight tile is summed with the halves of its K range
+    in the other order.  Copies of one head row in tiles of either kind must tie exactly, lower token first."""
+    V = 20000                                            # 136 rows per CTA: two tiles each
+    cfg = small_cfg(d_base=64, d_inner=d, V=V, topk=(8, 2), seed=rows + d)
+    sw = synth.make_weights(cfg)
+    copies = [5, 130, 140, 300, 4000, 4100, 9999, V - 1]
+    for c in copies[1:]:
+        sw.head[0][c] = sw.head[0][copies[0]]
+    h = B.spec_create(weights_to_cuda(sw))
+    B.spec_set_option(h, B.SPEC_OPT_HEAD_SWAP_MAX_ROWS, 128)
+    g = torch.Generator().manual_seed(rows)
+    scale = 1.0 + 0.5 * torch.rand(rows, 1, generator=g)
+    S = (sw.head[0][copies[0]].float()[None] * 40 * scale + 0.01 * torch.randn(rows, d, generator=g)).to(torch.bfloat16)
+    tok, logp, ws = B.spec_head_topk(h, 0, S.cuda(), 8)
+    assert B.spec_poll_error(ws) == 0
+    assert (tok.cpu() == torch.tensor(copies, dtype=torch.int32)).all()
+    assert (logp == logp[:, :1]).all()
+    want = torch.log_softmax(S.double() @ sw.head[0].double().t(), 1)[:, copies[0]]
+    assert (logp[:, 0].cpu().double() - want).abs().max() <= LOGIT_TOL
+    B.spec_destroy(h)

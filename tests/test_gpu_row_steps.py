@@ -102,3 +102,33 @@ def test_equal_rows_give_equal_logits_in_every_tile(B, d, rows):
     want = torch.log_softmax(S.double() @ sw.head[0].double().t(), 1)[:, copies[0]]
     assert (logp[:, 0].cpu().double() - want).abs().max() <= LOGIT_TOL
     B.spec_destroy(h)
+
+
+@pytest.mark.parametrize("d", [2048, 2056, 4096])
+@pytest.mark.parametrize("B_,topk", [(37, (4, 2)), (18, (8, 1, 2)), (149, (1, 2)), (74, (2, 1)), (75, (2, 1))])
+def test_merge_and_mix_round_one_child_per_sm(B, B_, topk, d):
+    """148 children and a few more or less (a level's merge and the next level's mix are one kernel up to one child per
+    SM), row widths round the two thread counts.  Every level is re-derived by the oracle from the GPU's parent level for
+    the first and the last sequence."""
+    K = int(np.prod(topk))
+    cfg = small_cfg(d_base=64, d_inner=d, V=600, topk=topk, K=K, B=B_, seed=B_ + d)
+    sw = synth.make_weights(cfg)
+    ow, gw = to_oracle_weights(sw), weights_to_cuda(sw)
+    ctx, tok = synth.make_draft_inputs(cfg)
+    h = B.spec_create(gw)
+    ct, lp, ws = B.spec_draft(h, ctx.cuda(), tok.cuda(), topk, K)
+    assert B.spec_poll_error(ws) == 0
+    lay = B.spec_draft_layout(h, B_, topk, K)
+    view = lambda off, n, dt: ws[off:off + n * torch.empty((), dtype=dt).element_size()].view(dt)
+    chk = DraftChecker(ow, topk, K)
+    for b in (0, B_ - 1):
+        st, tk, sc = [], [], []
+        for l in range(cfg.n):
+            N, N1 = cfg.nodes(l), cfg.nodes(l + 1)
+            S = view(lay.state[l], N * d, torch.bfloat16).view(B_, N // B_, d)
+            st.append(S[b].float().cpu().numpy())
+            tk.append(view(lay.tok[l + 1], N1, torch.int32).view(B_, -1)[b].cpu().numpy())
+            sc.append(view(lay.score[l + 1], N1, torch.float32).view(B_, -1)[b].cpu().numpy())
+        chk.check(synth.bf16_bits(ctx)[b], int(tok[b]), ct[b].cpu().numpy(), lp[b].cpu().numpy(),
+                  levels={"state": st, "tok": tk, "score": sc}, force_levels=True)
+    B.spec_destroy(h)

@@ -70,14 +70,10 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 // ---- verify (verify_kernels.cu) ----------------------------------------------------------
 struct VerifyPlan {
     int rows;          // B * K * (n + 1)
-    int chunk_elems;   // scalar fallback: elements of one (row, chunk) work unit
-    int chunks;        // scalar fallback: chunks per row
-    int vpr;           // streamed form: 16-byte vectors per row (0 when rows are not whole vectors)
-    int vec_per_warp;  // streamed form: vectors in one warp's contiguous range
-    int slots;         // partial slots reserved per row
+    int vec_per_warp;  // two-kernel form: 16-byte vectors in one warp's contiguous range
+    int slots;         // ... partial slots reserved per row
     size_t off_g;      // int32 [rows]
-    size_t off_pval;   // fp32 [rows, chunks]
-    size_t off_pidx;   // int32 [rows, chunks]
+    size_t off_part;   // (fp32 value, int32 index) [rows, slots]
     size_t total;
 };
 VerifyPlan make_verify_plan(int B, int K, int n, int V, int dtype);

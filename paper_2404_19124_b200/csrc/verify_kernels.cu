@@ -2,17 +2,18 @@
 // a bandwidth-bound streaming arg-max over every row of the base model's logits followed by
 // the longest-matching-prefix / best-candidate reduction.
 //
-// Kernel 1 (verify_stream_kernel): the whole tensor is one run of 16-byte vectors, cut into equal
-//   contiguous ranges, one per warp, sized so that the grid is a single wave of resident CTAs on
-//   every SM (no ragged second wave).  A warp walks the row segments inside its range with eight
-//   128-bit streaming loads in flight per lane.  For bf16 the running maximum is taken on packed
-//   pairs (max.bf16x2) and the element index is only resolved when a vector beats the lane's
-//   current best, so the common case costs about one ALU operation per element.  Each (row, warp)
-//   intersection writes one (value, index) partial into the row's slot list.
-//   (verify_argmax_kernel is the scalar fallback for unaligned tensors or odd row lengths: fixed
-//   chunks per row, one warp per chunk.)
-// Kernel 2 (verify_accept_kernel): one CTA per sequence folds the partials of its K*(n+1)
-//   rows into g[b,k,j], counts the matching prefix of every candidate and picks the best one.
+// Everywhere the tensor is one run of 16-byte vectors, whatever the row length and the alignment of its base: positions
+// are elements counted from the 16-byte boundary at or below the base, a row is a partial vector (read element by
+// element), a run of whole vectors, and another partial vector.  A lane keeps eight 128-bit streaming loads in flight.  For
+// bf16 the running maximum is taken on packed pairs (max.bf16x2) and the element index is only resolved when a vector
+// beats the lane's current best, so the common case costs about one ALU operation per element.
+//
+// Two forms (one_kernel_form chooses):
+//   verify_seq_kernel    one CTA per sequence does the whole job: its warps take equal contiguous ranges of the sequence's
+//                        vectors, fold them into a (value, index) key per row in shared memory, and the CTA accepts.
+//   verify_stream_kernel + verify_accept_kernel    all vectors cut into equal contiguous ranges, one per warp, a single
+//                        wave over the whole GPU; each (row, warp) intersection writes one (value, index) partial, which
+//                        one CTA per sequence folds and accepts.
 #include <float.h>
 
 #include <mutex>
@@ -26,6 +27,8 @@ namespace {
 constexpr int kArgmaxThreads = 256;
 constexpr int kWarpsPerBlock = kArgmaxThreads / 32;
 constexpr int kIdxNone = 0x7fffffff;
+constexpr int kSeqThreads = 1024;
+constexpr int kSeqMaxRows = 4000;   // 47 KB of keys and table
 
 __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
     uint32_t d;
@@ -83,82 +86,84 @@ __device__ __forceinline__ void warp_argmax(float &best, int &idx) {
 
 constexpr int kStreamUnroll = 8;
 
-// vec_per_warp vectors per warp; row r owns vectors [r * vpr, (r + 1) * vpr); the partial of the
-// (row, warp) intersection goes to slot  warp - first_warp(row)  of the row.
+// Elements per vector and its logarithm.
 template <bool kBf16>
-__global__ void __launch_bounds__(kArgmaxThreads, 4)
-verify_stream_kernel(const uint4 *__restrict__ logits, long long total_vec, int vpr, int vec_per_warp, int slots,
-                     float *pval, int32_t *pidx) {
-    griddep_launch();
-    griddep_wait();
-    constexpr int kEpv = kBf16 ? 8 : 4;
-    const int lane = threadIdx.x & 31;
-    const long long w = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    const long long beg = w * vec_per_warp;
-    if (beg >= total_vec) return;
-    const long long end = min(total_vec, beg + vec_per_warp);
-    long long sb = beg;
-    int row = (int)(beg / vpr);
-    while (sb < end) {
-        const long long row0 = (long long)row * vpr;
-        const long long se = min(end, row0 + vpr);   // end of this row's segment inside the range
-        float best = -INFINITY;
-        int idx = kIdxNone;
-        for (long long p0 = sb + lane; p0 < se; p0 += 32 * kStreamUnroll) {
-            uint4 q[kStreamUnroll];
+struct Elem {
+    static constexpr int kEpv = kBf16 ? 8 : 4, kShift = kBf16 ? 3 : 2;
+    static __device__ __forceinline__ float load(const char *base, long long i) {
+        return kBf16 ? bf16_bits_to_float(((const uint16_t *)base)[i]) : ((const float *)base)[i];
+    }
+};
+
+// The part of a row (elements [rs, re) of the run of vectors at `base`) that lies in vectors [a, e), read by `kGroup`
+// threads of which this is number `t`: the thread's maximum and its first index within the row.
+template <bool kBf16, int kGroup>
+__device__ __forceinline__ void scan_row(const char *base, long long rs, long long re, long long a, long long e, int t,
+                                         float &best, int &idx) {
+    using E = Elem<kBf16>;
+    const long long hv = rs >> E::kShift, body0 = (rs + E::kEpv - 1) >> E::kShift, body1 = re >> E::kShift;
+    if (body0 != hv && hv >= a && hv < e) {   // the row starts inside a vector
+        const long long i = rs + t, end = min(re, body0 << E::kShift);
+        const float x = i < end ? E::load(base, i) : -INFINITY;
+        if (x > best) {
+            best = x;
+            idx = t;
+        }
+    }
+    const long long p = max(body0, a), q = min(body1, e);
+    if (q > p) {
+        const uint4 *src = (const uint4 *)base + p;
+        const int n = (int)(q - p), col0 = (int)((p << E::kShift) - rs);
+        for (int i = t; i < n; i += kGroup * kStreamUnroll) {
+            uint4 v[kStreamUnroll];
 #pragma unroll
             for (int u = 0; u < kStreamUnroll; ++u)
-                if (p0 + 32 * u < se) q[u] = ld_stream(logits + p0 + 32 * u);
+                if (i + kGroup * u < n) v[u] = ld_stream(src + i + kGroup * u);
 #pragma unroll
             for (int u = 0; u < kStreamUnroll; ++u) {
-                if (p0 + 32 * u < se) {
-                    const int base = (int)(p0 + 32 * u - row0) * kEpv;
-                    if (kBf16) consume_bf16(q[u], base, best, idx);
-                    else consume_f32(q[u], base, best, idx);
+                if (i + kGroup * u < n) {
+                    const int col = col0 + (i + kGroup * u) * E::kEpv;
+                    if (kBf16) consume_bf16(v[u], col, best, idx);
+                    else consume_f32(v[u], col, best, idx);
                 }
             }
         }
-        warp_argmax(best, idx);
-        if (lane == 0) {
-            const long long first_w = row0 / vec_per_warp;
-            const size_t slot = (size_t)row * slots + (size_t)(w - first_w);
-            pval[slot] = best;
-            pidx[slot] = idx;
+    }
+    if (body1 >= body0 && body1 >= a && body1 < e && (re & (E::kEpv - 1)) != 0) {   // ... and ends inside another
+        const long long i = (body1 << E::kShift) + t;
+        const float x = i < re ? E::load(base, i) : -INFINITY;
+        if (x > best) {
+            best = x;
+            idx = (int)(i - rs);
         }
-        sb = se;
-        ++row;
     }
 }
 
-// Scalar fallback for tensors whose rows are not whole 16-byte vectors (or an unaligned base): fixed
-// chunks per row, one warp per (row, chunk).
+// vec_per_warp vectors per warp; row r is elements [skew + r * V, + V); the partial of the (row, warp) intersection goes to
+// slot  warp - first_warp(row)  of the row.
 template <bool kBf16>
-__global__ void __launch_bounds__(kArgmaxThreads)
-verify_argmax_kernel(const void *__restrict__ logits, int rows, int V, int chunk_elems, int chunks,
-                     float *__restrict__ pval, int32_t *__restrict__ pidx) {
+__global__ void __launch_bounds__(kArgmaxThreads, 4)
+verify_stream_kernel(const char *__restrict__ base, int skew, int rows, int V, long long total_vec, int vec_per_warp,
+                     int slots, float2 *part) {
     griddep_launch();
     griddep_wait();
+    using E = Elem<kBf16>;
     const int lane = threadIdx.x & 31;
-    const long long unit = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
-    if (unit >= (long long)rows * chunks) return;
-    const int row = (int)(unit / chunks), chunk = (int)(unit - (long long)row * chunks);
-    const int begin = chunk * chunk_elems;
-    const int count = min(chunk_elems, V - begin);
-    constexpr int kEsz = kBf16 ? 2 : 4;
-    const char *rp = (const char *)logits + ((size_t)row * V + begin) * kEsz;
-    float best = -INFINITY;
-    int idx = kIdxNone;
-    for (int i = lane; i < count; i += 32) {
-        const float x = kBf16 ? bf16_bits_to_float(((const uint16_t *)rp)[i]) : ((const float *)rp)[i];
-        if (x > best) {
-            best = x;
-            idx = begin + i;
+    const long long w = (long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5);
+    const long long beg = w * vec_per_warp, end = min(total_vec, beg + vec_per_warp);
+    if (beg >= end) return;
+    const long long first = (beg << E::kShift) - skew;
+    for (int row = first > 0 ? (int)(first / V) : 0; row < rows; ++row) {
+        const long long rs = skew + (long long)row * V;
+        if ((rs >> E::kShift) >= end) break;
+        float best = -INFINITY;
+        int idx = kIdxNone;
+        scan_row<kBf16, 32>(base, rs, rs + V, beg, end, lane, best, idx);
+        warp_argmax(best, idx);
+        if (lane == 0) {
+            const long long first_w = (rs >> E::kShift) / vec_per_warp;
+            part[(size_t)row * slots + (size_t)(w - first_w)] = make_float2(best, __int_as_float(idx));
         }
-    }
-    warp_argmax(best, idx);
-    if (lane == 0) {
-        pval[unit] = best;
-        pidx[unit] = idx;
     }
 }
 
@@ -167,70 +172,21 @@ verify_argmax_kernel(const void *__restrict__ logits, int rows, int V, int chunk
 // kernels start early under programmatic dependent launch and the same addresses are rewritten call after call.
 // base_logits itself is streamed with ld.global.nc: it must be complete before the call is enqueued behind
 // its producer on the stream, which stream order guarantees.)
-__global__ void __launch_bounds__(128)
-verify_accept_kernel(const int32_t *cand_tok, const float *pval, const int32_t *pidx, int K, int n, int slots, int vpr,
-                     int vec_per_warp, int32_t *g_out, int g_in_smem, int32_t *accept_len, int32_t *best_cand,
-                     int32_t *next_tok, int32_t *err) {
-    // The sequence's arg-max table is re-read by other threads for the prefix match: from shared memory
-    // when it fits the default 48 KB, otherwise from the copy in g_out this CTA has just written (global
-    // writes of a CTA are visible to its own threads after the barrier).
-    extern __shared__ int32_t g_s[];   // [K * (n + 1)] if g_in_smem
-    __shared__ unsigned int key_s;
-    const int b = blockIdx.x, rows_b = K * (n + 1);
-    griddep_launch();
-    griddep_wait();
-    if (threadIdx.x == 0) {
-        key_s = 0u;
-        if (b == 0 && err != nullptr) *err = 0;
-    }
-    // The step is a handful of dependent round trips to L2, so every load that does not depend on another is
-    // requested before the first one is used: the tokens of this thread's first candidate now, a row's partials
-    // (values and indices alike) eight slots at a time.
-    constexpr int kBatch = 8;
-    int32_t ctok[SPEC_MAX_HEADS];
-    {
-        const int k0 = threadIdx.x;
+// Tokens of one candidate, at most SPEC_MAX_HEADS of them, requested together.
+__device__ __forceinline__ void load_candidate(const int32_t *cand_tok, size_t c, int n, bool valid,
+                                               int32_t (&tok)[SPEC_MAX_HEADS]) {
 #pragma unroll
-        for (int j = 0; j < SPEC_MAX_HEADS; ++j)
-            ctok[j] = (k0 < K && j < n) ? __ldcg(cand_tok + ((size_t)b * K + k0) * n + j) : -1;
-    }
-    for (int r = threadIdx.x; r < rows_b; r += blockDim.x) {
-        const size_t gr = (size_t)b * rows_b + r;
-        const size_t u0 = gr * slots;
-        // streamed layout: the row's slots are the warps whose ranges intersect it
-        int chunks = slots;
-        if (vec_per_warp > 0)
-            chunks = (int)(((long long)(gr + 1) * vpr - 1) / vec_per_warp - ((long long)gr * vpr) / vec_per_warp) + 1;
-        float best = -INFINITY;
-        int arg = 0;   // a row without any value above -inf (all NaN) yields 0
-        for (int c0 = 0; c0 < chunks; c0 += kBatch) {
-            float v[kBatch];
-            int id[kBatch];
-#pragma unroll
-            for (int j = 0; j < kBatch; ++j) {
-                const bool in = c0 + j < chunks;
-                v[j] = in ? __ldcg(pval + u0 + c0 + j) : -INFINITY;
-                id[j] = in ? __ldcg(pidx + u0 + c0 + j) : 0;
-            }
-#pragma unroll
-            for (int j = 0; j < kBatch; ++j) {
-                const bool take = v[j] > best;   // chunks ascend, so the first maximum wins
-                best = take ? v[j] : best;
-                arg = take ? id[j] : arg;
-            }
-        }
-        if (g_in_smem) g_s[r] = arg;
-        g_out[(size_t)b * rows_b + r] = arg;
-    }
-    __syncthreads();
-    const int32_t *gtab = g_in_smem ? g_s : g_out + (size_t)b * rows_b;
+    for (int j = 0; j < SPEC_MAX_HEADS; ++j) tok[j] = valid && j < n ? __ldcg(cand_tok + c * n + j) : -1;
+}
+
+// Sequence b's acceptance from its arg-max table (K * (n + 1) entries, visible to the whole CTA), by a CTA whose threads
+// hold the tokens of their first candidate in `ctok`.  `key_s`: shared, zero.
+__device__ __forceinline__ void accept_sequence(const int32_t *cand_tok, const int32_t *gtab, int b, int K, int n,
+                                                int32_t (&ctok)[SPEC_MAX_HEADS], unsigned int *key_s,
+                                                int32_t *accept_len, int32_t *best_cand, int32_t *next_tok) {
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
         const int32_t *gk = gtab + k * (n + 1);
-        if (k != (int)threadIdx.x) {   // more candidates than threads: the later ones are fetched here
-#pragma unroll
-            for (int j = 0; j < SPEC_MAX_HEADS; ++j)
-                ctok[j] = j < n ? __ldcg(cand_tok + ((size_t)b * K + k) * n + j) : -1;
-        }
+        if (k != (int)threadIdx.x) load_candidate(cand_tok, (size_t)b * K + k, n, true, ctok);   // more candidates than threads
         int m = 0;
         bool open = true;
 #pragma unroll
@@ -243,15 +199,121 @@ verify_accept_kernel(const int32_t *cand_tok, const float *pval, const int32_t *
             while (m < n && __ldcg(c + m) == gk[m]) ++m;
         }
         // longest prefix first, then the lowest candidate index
-        atomicMax(&key_s, ((unsigned)m << 16) | (unsigned)(0xffff - k));
+        atomicMax(key_s, ((unsigned)m << 16) | (unsigned)(0xffff - k));
     }
     __syncthreads();
     if (threadIdx.x == 0) {
-        const int m = (int)(key_s >> 16), k = 0xffff - (int)(key_s & 0xffffu);
+        const int m = (int)(*key_s >> 16), k = 0xffff - (int)(*key_s & 0xffffu);
         accept_len[b] = m;
         best_cand[b] = k;
         next_tok[b] = gtab[k * (n + 1) + m];
     }
+}
+
+__global__ void __launch_bounds__(128)
+verify_accept_kernel(const int32_t *cand_tok, const float2 *part, int K, int n, int V, int skew, int shift, int slots,
+                     int vec_per_warp, int32_t *g_out, int g_in_smem, int32_t *accept_len, int32_t *best_cand,
+                     int32_t *next_tok, int32_t *err) {
+    // The sequence's arg-max table is re-read by other threads for the prefix match: from shared memory
+    // when it fits the default 48 KB, otherwise from the copy in g_out this CTA has just written (global
+    // writes of a CTA are visible to its own threads after the barrier).
+    extern __shared__ int32_t g_s[];   // [K * (n + 1)] if g_in_smem
+    __shared__ unsigned int key_s;
+    const int b = blockIdx.x, rows_b = K * (n + 1);
+    griddep_launch();
+    if (threadIdx.x == 0) key_s = 0u;
+    griddep_wait();
+    if (threadIdx.x == 0 && b == 0 && err != nullptr) *err = 0;
+    // The step is a handful of dependent round trips to L2, so every load that does not depend on another is
+    // requested before the first one is used: the tokens of this thread's first candidate now, a row's partials
+    // eight slots at a time.
+    constexpr int kBatch = 8;
+    int32_t ctok[SPEC_MAX_HEADS];
+    load_candidate(cand_tok, (size_t)b * K + threadIdx.x, n, (int)threadIdx.x < K, ctok);
+    for (int r = threadIdx.x; r < rows_b; r += blockDim.x) {
+        const size_t gr = (size_t)b * rows_b + r;
+        const float2 *pr = part + gr * slots;
+        // the row's slots are the warps whose ranges its vectors touch
+        const long long rs = skew + (long long)gr * V, v0 = rs >> shift, v1 = (rs + V - 1) >> shift;
+        const int chunks = (v1 >> 32) == 0 ? (int)((uint32_t)v1 / (uint32_t)vec_per_warp - (uint32_t)v0 / (uint32_t)vec_per_warp) + 1
+                                           : (int)(v1 / vec_per_warp - v0 / vec_per_warp) + 1;
+        float best = -INFINITY;
+        int arg = 0;   // a row without any value above -inf (all NaN) yields 0
+        for (int c0 = 0; c0 < chunks; c0 += kBatch) {
+            float2 v[kBatch];
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) v[j] = c0 + j < chunks ? __ldcg(pr + c0 + j) : make_float2(-INFINITY, 0.0f);
+#pragma unroll
+            for (int j = 0; j < kBatch; ++j) {
+                const bool take = v[j].x > best;   // chunks ascend, so the first maximum wins
+                best = take ? v[j].x : best;
+                arg = take ? __float_as_int(v[j].y) : arg;
+            }
+        }
+        if (g_in_smem) g_s[r] = arg;
+        g_out[gr] = arg;
+    }
+    __syncthreads();
+    accept_sequence(cand_tok, g_in_smem ? g_s : g_out + (size_t)b * rows_b, b, K, n, ctok, &key_s, accept_len, best_cand,
+                    next_tok);
+}
+
+// ---- one CTA per sequence ---------------------------------------------------------------------------
+// (value, first index) as one integer whose maximum is the arg-max: the order-preserving image of the value above the
+// complement of the index.  0 stands for "nothing above -inf".  (+ 0.0f: -0 and +0 are equal.)
+__device__ __forceinline__ unsigned long long argmax_key(float v, int idx) {
+    const uint32_t u = __float_as_uint(v + 0.0f);
+    const uint32_t hi = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    return idx == kIdxNone ? 0ull : ((unsigned long long)hi << 32) | (uint32_t)~idx;
+}
+
+template <bool kBf16>
+__global__ void __launch_bounds__(kSeqThreads, 1)
+verify_seq_kernel(const char *__restrict__ base, int skew, const int32_t *cand_tok, int K, int n, int V,
+                  int32_t *g_out, int32_t *accept_len, int32_t *best_cand, int32_t *next_tok, int32_t *err) {
+    extern __shared__ unsigned long long keys[];   // [K * (n + 1)], then the arg-max table, int32 [K * (n + 1)]
+    __shared__ unsigned int key_s;
+    using E = Elem<kBf16>;
+    const int rows_b = K * (n + 1), lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int b = blockIdx.x;
+    int32_t *g_s = (int32_t *)(keys + rows_b);
+    griddep_launch();
+    for (int r = threadIdx.x; r < rows_b; r += kSeqThreads) keys[r] = 0ull;
+    if (threadIdx.x == 0) key_s = 0u;
+    __syncthreads();
+    griddep_wait();
+    if (threadIdx.x == 0 && blockIdx.x == 0 && err != nullptr) *err = 0;
+    int32_t ctok[SPEC_MAX_HEADS];
+    load_candidate(cand_tok, (size_t)b * K + threadIdx.x, n, (int)threadIdx.x < K, ctok);
+    // the sequence as a run of vectors of its own
+    const long long s0 = skew + (long long)b * rows_b * V;
+    const char *seq = base + ((s0 >> E::kShift) << 4);
+    const int rel = (int)(s0 & (E::kEpv - 1));
+    const long long total = (rel + (long long)rows_b * V + E::kEpv - 1) >> E::kShift;
+    constexpr int kWarps = kSeqThreads / 32;
+    const long long per = (total + kWarps - 1) / kWarps;
+    const long long beg = (long long)warp * per, end = min(total, beg + per);
+    if (beg < end) {
+        const long long first = (beg << E::kShift) - rel;
+        for (int row = first > 0 ? (int)(first / V) : 0; row < rows_b; ++row) {
+            const long long rs = rel + (long long)row * V;
+            if ((rs >> E::kShift) >= end) break;
+            float best = -INFINITY;
+            int idx = kIdxNone;
+            scan_row<kBf16, 32>(seq, rs, rs + V, beg, end, lane, best, idx);
+            warp_argmax(best, idx);
+            if (lane == 0) atomicMax(&keys[row], argmax_key(best, idx));
+        }
+    }
+    __syncthreads();
+    for (int r = threadIdx.x; r < rows_b; r += kSeqThreads) {
+        const unsigned long long k = keys[r];
+        const int arg = k == 0ull ? 0 : (int)~(uint32_t)k;
+        g_s[r] = arg;
+        g_out[(size_t)b * rows_b + r] = arg;
+    }
+    __syncthreads();
+    accept_sequence(cand_tok, g_s, b, K, n, ctok, &key_s, accept_len, best_cand, next_tok);
 }
 
 // ---- early-exit form ------------------------------------------------------------------------------
@@ -262,34 +324,20 @@ verify_accept_kernel(const int32_t *cand_tok, const float *pval, const int32_t *
 // B K (n+1) V to sum over candidates of (m + 1) V elements; rows that were not read get g = -1.
 template <bool kBf16>
 __global__ void __launch_bounds__(kArgmaxThreads)
-verify_early_kernel(const uint4 *__restrict__ logits, const int32_t *cand_tok, int n, int vpr, int32_t *g,
+verify_early_kernel(const char *__restrict__ base, const int32_t *cand_tok, int n, int V, int32_t *g,
                     int32_t *match_len) {
     __shared__ float s_val[kWarpsPerBlock];
     __shared__ int s_idx[kWarpsPerBlock];
     __shared__ int s_arg;
     griddep_launch();
     griddep_wait();
-    constexpr int kEpv = kBf16 ? 8 : 4;
     const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int m = n, j = 0;
     for (; j <= n; ++j) {
-        const uint4 *rp = logits + ((size_t)c * (n + 1) + j) * vpr;
+        const long long rs = ((long long)c * (n + 1) + j) * V;
         float best = -INFINITY;
         int idx = kIdxNone;
-        for (int p0 = tid; p0 < vpr; p0 += kArgmaxThreads * kStreamUnroll) {
-            uint4 q[kStreamUnroll];
-#pragma unroll
-            for (int u = 0; u < kStreamUnroll; ++u)
-                if (p0 + kArgmaxThreads * u < vpr) q[u] = ld_stream(rp + p0 + kArgmaxThreads * u);
-#pragma unroll
-            for (int u = 0; u < kStreamUnroll; ++u) {
-                if (p0 + kArgmaxThreads * u < vpr) {
-                    const int base = (p0 + kArgmaxThreads * u) * kEpv;
-                    if (kBf16) consume_bf16(q[u], base, best, idx);
-                    else consume_f32(q[u], base, best, idx);
-                }
-            }
-        }
+        scan_row<kBf16, kArgmaxThreads>(base, rs, rs + V, 0, 1ll << 62, tid, best, idx);
         warp_argmax(best, idx);
         if (lane == 0) {
             s_val[warp] = best;
@@ -349,44 +397,31 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 }  // namespace
 
+// One kernel when a sequence is little enough for one CTA to read in less time than a second kernel costs.  One CTA reads
+// about 65 GB/s: 64 KB 7.5 us per call against 9.5 us in two kernels (both bound by the host), 256 KB 7.6 against 9.5 alone
+// but 65.0 against 63.6 us inside a decoding step, 512 KB 11.6 against 9.7, 1 MB 15.3 against 9.5.
+constexpr long long kSeqMaxBytes = 128 << 10;
+bool one_kernel_form(int rows_b, int V, int dtype) {
+    return rows_b <= kSeqMaxRows && (long long)rows_b * V * (dtype == SPEC_BF16 ? 2 : 4) <= kSeqMaxBytes;
+}
+
 // Resident CTAs per SM of the streaming kernel (launch bound above) times the SM count gives the
 // number of warps of one full wave; every warp gets an equal range of at least one unrolled trip.
 VerifyPlan make_verify_plan(int B, int K, int n, int V, int dtype) {
     VerifyPlan p{};
     p.rows = B * K * (n + 1);
-    const int esz = dtype == SPEC_BF16 ? 2 : 4;
-    const int epv = 16 / esz;
-    // scalar fallback layout (also the upper bound used for the workspace when V % epv != 0)
-    {
-        const int gran = 32 * 4 * epv;
-        const long long target_units = (long long)num_sms() * 64 * 2;
-        int chunks = (int)((target_units + p.rows - 1) / p.rows);
-        const int max_chunks = (V + gran - 1) / gran;
-        if (chunks > max_chunks) chunks = max_chunks;
-        if (chunks < 1) chunks = 1;
-        const int per = (V + chunks - 1) / chunks;
-        p.chunk_elems = (per + gran - 1) / gran * gran;
-        p.chunks = (V + p.chunk_elems - 1) / p.chunk_elems;
-    }
-    p.vpr = 0;
-    p.vec_per_warp = 0;
-    p.slots = p.chunks;
-    if (V % epv == 0) {
-        p.vpr = V / epv;
-        const long long total = (long long)p.rows * p.vpr;
-        const long long wave_warps = (long long)num_sms() * 4 * kWarpsPerBlock;
-        long long c = (total + wave_warps - 1) / wave_warps;
-        const long long min_c = 32 * kStreamUnroll;
-        if (c < min_c) c = min_c;
-        if (c > (1ll << 30)) c = 1ll << 30;
-        p.vec_per_warp = (int)c;
-        const int stream_slots = (int)((p.vpr + c - 1) / c) + 1;
-        if (stream_slots > p.slots) p.slots = stream_slots;
-    }
+    const int epv = dtype == SPEC_BF16 ? 8 : 4;
+    const long long total = ((long long)p.rows * V + 2 * epv - 2) / epv;   // vectors, the base at its least aligned
+    const long long wave_warps = (long long)num_sms() * 4 * kWarpsPerBlock;
+    long long c = (total + wave_warps - 1) / wave_warps;
+    if (c < 32 * kStreamUnroll) c = 32 * kStreamUnroll;
+    if (c > (1ll << 30)) c = 1ll << 30;
+    p.vec_per_warp = (int)c;
+    const long long row_vec = (V + epv - 1) / epv + 1;   // most vectors that one row touches
+    p.slots = (int)((row_vec + c - 2) / c + 1);
     p.off_g = kWsAlign;
-    p.off_pval = align_up(p.off_g + sizeof(int32_t) * (size_t)p.rows, kWsAlign);
-    p.off_pidx = align_up(p.off_pval + sizeof(float) * (size_t)p.rows * p.slots, kWsAlign);
-    p.total = align_up(p.off_pidx + sizeof(int32_t) * (size_t)p.rows * p.slots, kWsAlign);
+    p.off_part = align_up(p.off_g + sizeof(int32_t) * (size_t)p.rows, kWsAlign);
+    p.total = align_up(p.off_part + sizeof(float2) * (size_t)p.rows * p.slots, kWsAlign);
     return p;
 }
 
@@ -396,40 +431,27 @@ int launch_verify(const int32_t *cand_tok, const void *base_logits, int dtype, i
     char *w = (char *)ws;
     int32_t *err = (int32_t *)w;
     int32_t *g = (int32_t *)(w + plan.off_g);
-    float *pval = (float *)(w + plan.off_pval);
-    int32_t *pidx = (int32_t *)(w + plan.off_pidx);
-    const bool stream = plan.vec_per_warp > 0 && ((uintptr_t)base_logits % 16 == 0);
-    int vec_per_warp = 0;
-    if (stream) {
-        vec_per_warp = plan.vec_per_warp;
-        const long long total = (long long)plan.rows * plan.vpr;
-        const long long warps = (total + vec_per_warp - 1) / vec_per_warp;
-        const unsigned grid = (unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
-        const uint4 *lp = (const uint4 *)base_logits;
-        if (dtype == SPEC_BF16)
-            SPEC_CUDA_TRY(launch_pdl(verify_stream_kernel<true>, dim3(grid), dim3(kArgmaxThreads), 0, st, lp, total,
-                                     plan.vpr, vec_per_warp, plan.slots, pval, pidx));
-        else
-            SPEC_CUDA_TRY(launch_pdl(verify_stream_kernel<false>, dim3(grid), dim3(kArgmaxThreads), 0, st, lp, total,
-                                     plan.vpr, vec_per_warp, plan.slots, pval, pidx));
-    } else {
-        // scalar fallback; its partials use the first plan.chunks slots of every row, laid out with
-        // plan.chunks as the row pitch
-        const long long units = (long long)plan.rows * plan.chunks;
-        const unsigned grid = (unsigned)((units + kWarpsPerBlock - 1) / kWarpsPerBlock);
-        if (dtype == SPEC_BF16)
-            SPEC_CUDA_TRY(launch_pdl(verify_argmax_kernel<true>, dim3(grid), dim3(kArgmaxThreads), 0, st,
-                                     base_logits, plan.rows, V, plan.chunk_elems, plan.chunks, pval, pidx));
-        else
-            SPEC_CUDA_TRY(launch_pdl(verify_argmax_kernel<false>, dim3(grid), dim3(kArgmaxThreads), 0, st,
-                                     base_logits, plan.rows, V, plan.chunk_elems, plan.chunks, pval, pidx));
+    const bool bf16 = dtype == SPEC_BF16;
+    const int shift = bf16 ? 3 : 2, esz = bf16 ? 2 : 4;
+    const char *base = (const char *)((uintptr_t)base_logits & ~(uintptr_t)15);
+    const int skew = (int)(((uintptr_t)base_logits & 15) / esz), rows_b = K * (n + 1);
+    if (one_kernel_form(rows_b, V, dtype)) {
+        const size_t smem = (sizeof(unsigned long long) + sizeof(int32_t)) * (size_t)rows_b;
+        SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_seq_kernel<true> : verify_seq_kernel<false>, dim3((unsigned)B), dim3(kSeqThreads),
+                                 smem, st, base, skew, cand_tok, K, n, V, g, accept_len, best_cand, next_tok, err));
+        return SPEC_OK;
     }
-    size_t smem = sizeof(int32_t) * (size_t)K * (n + 1);
+    float2 *part = (float2 *)(w + plan.off_part);
+    const long long total = (skew + (long long)plan.rows * V + (1 << shift) - 1) >> shift;
+    const long long warps = (total + plan.vec_per_warp - 1) / plan.vec_per_warp;
+    const unsigned grid = (unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
+    SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_stream_kernel<true> : verify_stream_kernel<false>, dim3(grid), dim3(kArgmaxThreads),
+                             0, st, base, skew, plan.rows, V, total, plan.vec_per_warp, plan.slots, part));
+    size_t smem = sizeof(int32_t) * (size_t)rows_b;
     const int g_in_smem = smem <= 40 * 1024;
     if (!g_in_smem) smem = 0;
-    SPEC_CUDA_TRY(launch_pdl(verify_accept_kernel, dim3(B), dim3(128), smem, st, cand_tok, (const float *)pval,
-                             (const int32_t *)pidx, K, n, stream ? plan.slots : plan.chunks, plan.vpr, vec_per_warp,
-                             g, g_in_smem, accept_len, best_cand, next_tok, err));
+    SPEC_CUDA_TRY(launch_pdl(verify_accept_kernel, dim3(B), dim3(128), smem, st, cand_tok, (const float2 *)part, K, n, V, skew,
+                             shift, plan.slots, plan.vec_per_warp, g, g_in_smem, accept_len, best_cand, next_tok, err));
     return SPEC_OK;
 }
 
@@ -438,18 +460,14 @@ int launch_verify(const int32_t *cand_tok, const void *base_logits, int dtype, i
 int launch_verify_early(const int32_t *cand_tok, const void *base_logits, int dtype, int B, int K, int n, int V,
                         int32_t *accept_len, int32_t *best_cand, int32_t *next_tok, void *ws, const VerifyPlan &plan,
                         cudaStream_t st) {
-    if (plan.vpr <= 0 || ((uintptr_t)base_logits % 16) != 0) return SPEC_ERR_SHAPE;
+    const bool bf16 = dtype == SPEC_BF16;
+    if (V % (bf16 ? 8 : 4) != 0 || ((uintptr_t)base_logits % 16) != 0) return SPEC_ERR_SHAPE;
     char *w = (char *)ws;
     int32_t *err = (int32_t *)w;
     int32_t *g = (int32_t *)(w + plan.off_g);
-    int32_t *match_len = (int32_t *)(w + plan.off_pval);   // B * K words; the partial-maxima area is not used here
-    const uint4 *lp = (const uint4 *)base_logits;
-    if (dtype == SPEC_BF16)
-        SPEC_CUDA_TRY(launch_pdl(verify_early_kernel<true>, dim3(B * K), dim3(kArgmaxThreads), 0, st, lp, cand_tok, n,
-                                 plan.vpr, g, match_len));
-    else
-        SPEC_CUDA_TRY(launch_pdl(verify_early_kernel<false>, dim3(B * K), dim3(kArgmaxThreads), 0, st, lp, cand_tok, n,
-                                 plan.vpr, g, match_len));
+    int32_t *match_len = (int32_t *)(w + plan.off_part);   // B * K words; the partial maxima's area is not used here
+    SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_early_kernel<true> : verify_early_kernel<false>, dim3(B * K), dim3(kArgmaxThreads), 0,
+                             st, (const char *)base_logits, cand_tok, n, V, g, match_len));
     SPEC_CUDA_TRY(launch_pdl(verify_accept_early_kernel, dim3(B), dim3(128), 0, st, (const int32_t *)g,
                              (const int32_t *)match_len, K, n, accept_len, best_cand, next_tok, err));
     return SPEC_OK;

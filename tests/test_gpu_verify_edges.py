@@ -1,0 +1,73 @@
+"""Verification where rows start and end inside 16-byte vectors, at the borders between the warps that share a row, and
+on both sides of the size up to which one kernel does the whole job.  Integer results: compared exactly."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2404_19124_b200 import synth
+from helpers import ws_view
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def B():
+    from paper_2404_19124_b200 import build
+    build.build()
+    from paper_2404_19124_b200 import binding
+    return binding
+
+
+def _check(B, cand, logits):
+    Bn, K, n = cand.shape
+    bf16 = logits.dtype == torch.bfloat16
+    host = logits.cpu().contiguous()
+    acc, best, nxt, ws = B.spec_verify(cand.cuda(), logits)
+    o = oracle.verify(cand.numpy(), synth.bf16_bits(host) if bf16 else host.numpy(), oracle.BF16 if bf16 else oracle.F32,
+                      want_g=True)
+    assert B.spec_poll_error(ws) == 0
+    g = ws_view(ws, 256, Bn * K * (n + 1), torch.int32).cpu().numpy().reshape(Bn, K, n + 1)
+    assert np.array_equal(g, o[3])
+    for got, want in zip((acc, best, nxt), o):
+        assert np.array_equal(got.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("shape", [(5, 11, 3, 32003), (2, 4, 2, 8191), (1, 3, 1, 65537), (3, 7, 2, 9), (4, 5, 3, 17),
+                                   (2, 30, 1, 1093), (70, 2, 1, 4001), (1, 2, 3, 8192), (1, 2, 3, 8193), (1, 1000, 2, 21),
+                                   (1, 1334, 2, 5)])
+def test_rows_that_are_not_whole_vectors(B, shape, dtype):
+    """Random rows, one planted maximum each at the places where a partial vector, a warp's range or the row begins or
+    ends, and for every third row a second equal maximum further right (the first must win)."""
+    Bn, K, n, V = shape
+    g = torch.Generator().manual_seed(V)
+    x = torch.randn(Bn, K, n + 1, V, generator=g).to(dtype)
+    rows = x.view(-1, V)
+    epv = 8 if dtype == torch.bfloat16 else 4
+    for r in range(rows.shape[0]):
+        start = r * V
+        places = [0, V - 1, min(V - 1, -start % epv), max(0, V - 1 - (start + V) % epv), r * 37 % V, V // 2]
+        p = places[r % len(places)]
+        rows[r, p] = 9.0
+        if r % 3 == 0:
+            rows[r, p + (V - 1 - p) // 2:][-1] = 9.0
+    cand = torch.randint(0, V, (Bn, K, n), generator=g, dtype=torch.int64).to(torch.int32)
+    am = x.float().argmax(-1)
+    for k in range(K):
+        cand[:, k, :k % (n + 1)] = am[:, k, :k % (n + 1)].to(torch.int32)
+    _check(B, cand, x.cuda())
+
+
+@pytest.mark.parametrize("V", [1000, 30001])
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+def test_every_alignment_of_the_base(B, V, dtype):
+    Bn, K, n = 2, 3, 2
+    g = torch.Generator().manual_seed(V)
+    size = Bn * K * (n + 1) * V
+    buf = torch.randn(size + 8, generator=g).to(dtype).cuda()
+    cand = torch.randint(0, V, (Bn, K, n), generator=g, dtype=torch.int64).to(torch.int32)
+    for off in range(8 if dtype == torch.bfloat16 else 4):
+        buf[:off] = 50.0                                  # what lies before and behind the tensor must not be seen
+        buf[off + size:] = 50.0
+        _check(B, cand, buf[off:off + size].view(Bn, K, n + 1, V))

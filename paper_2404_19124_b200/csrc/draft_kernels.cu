@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(kRowThreads) mix_ln_gelu_wide_kernel(MixArgs m
         const float c = h_s[i] - mean;
         sq += c * c;
     }
-    const float var = group_sum<kRowThreads, BlockSync>(sq, red, tid) / (float)d;
+    const float var = group_sum<kRowThreads, BlockSync>(sq, red + kMaxGroupWarps, tid) / (float)d;
     const float rstd = rsqrtf(var + m.eps);
     for (int i = tid; i < d; i += kRowThreads)
         m.S_out[(size_t)r * d + i] = (uint16_t)float_to_bf16_bits(gelu_erf((h_s[i] - mean) * rstd * m.gamma[i] + m.beta[i]));

@@ -35,12 +35,12 @@ struct Scratch {
     int cand_i[kMaxGroupWarps][kMaxRounds];        // ... and token ids
 };
 
+// (`red`: one float per warp, not read by anybody else until the next barrier behind the call)
 template <int kThreads, typename Sync>
 __device__ __forceinline__ float group_sum(float v, float *red, int tid) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     const int w = tid >> 5, l = tid & 31;
-    Sync::sync();   // red may still be read from a previous call
     if (l == 0) red[w] = v;
     Sync::sync();
     float t = (l < kThreads / 32) ? red[l] : 0.0f;
@@ -63,9 +63,12 @@ __device__ __forceinline__ float group_max(float v, float *red, int tid) {
     return t;
 }
 
-// Exact (erf) GELU.  erff is kept out of line: inlined it would be the bulk of the row step's code.
-static __device__ __noinline__ float erf_call(float x) { return erff(x); }
-__device__ __forceinline__ float gelu_erf(float y) { return 0.5f * y * (1.0f + erf_call(y * 0.70710678118654752440f)); }
+// Exact (erf) GELU.  erff is kept out of line: inlined it would be the bulk of the row step's code.  Four at a time, whose
+// latency chains overlap (one by one the eight evaluations of a thread were a third of the step).
+__device__ __forceinline__ float gelu_erf(float y) { return 0.5f * y * (1.0f + erff(y * 0.70710678118654752440f)); }
+static __device__ __noinline__ float4 gelu_erf4(float4 y) {
+    return make_float4(gelu_erf(y.x), gelu_erf(y.y), gelu_erf(y.z), gelu_erf(y.w));
+}
 
 // Node r of the level, whose token is t and whose projected parent state is row `parent` of P.
 // h = a * P[parent] + b * E[t].  The row lives in registers: thread t owns the 8-element groups
@@ -167,7 +170,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
             }
         }
     }
-    const float var = group_sum<kThreads, Sync>(sq, red, tid) / (float)d;
+    const float var = group_sum<kThreads, Sync>(sq, red + kMaxGroupWarps, tid) / (float)d;
     const float rstd = rsqrtf(var + m.eps);
     float amax = 0.0f;   // largest magnitude of the bf16-rounded state (for the e4m3 copy); h is reused for it
 #pragma unroll
@@ -185,13 +188,21 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
         const float bv[8] = {bq[hq][0].x, bq[hq][0].y, bq[hq][0].z, bq[hq][0].w, bq[hq][1].x, bq[hq][1].y, bq[hq][1].z, bq[hq][1].w};
         uint32_t packed[4];
 #pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-            const float s0 = gelu_erf((h[it][j] - mean) * rstd * gv[j] + bv[j]);
-            const float s1 = gelu_erf((h[it][j + 1] - mean) * rstd * gv[j + 1] + bv[j + 1]);
-            packed[j >> 1] = float_to_bf16_bits(s0) | (float_to_bf16_bits(s1) << 16);
-            h[it][j] = i < d ? __uint_as_float(packed[j >> 1] << 16) : 0.0f;
-            h[it][j + 1] = i < d ? __uint_as_float(packed[j >> 1] & 0xffff0000u) : 0.0f;
-            amax = fmaxf(amax, fmaxf(fabsf(h[it][j]), fabsf(h[it][j + 1])));
+        for (int j = 0; j < 8; j += 4) {
+            float4 y;
+            y.x = (h[it][j] - mean) * rstd * gv[j] + bv[j];
+            y.y = (h[it][j + 1] - mean) * rstd * gv[j + 1] + bv[j + 1];
+            y.z = (h[it][j + 2] - mean) * rstd * gv[j + 2] + bv[j + 2];
+            y.w = (h[it][j + 3] - mean) * rstd * gv[j + 3] + bv[j + 3];
+            y = gelu_erf4(y);
+            packed[j >> 1] = float_to_bf16_bits(y.x) | (float_to_bf16_bits(y.y) << 16);
+            packed[(j >> 1) + 1] = float_to_bf16_bits(y.z) | (float_to_bf16_bits(y.w) << 16);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const uint32_t w = packed[(j + q) >> 1];
+                h[it][j + q] = i < d ? __uint_as_float((q & 1) ? w & 0xffff0000u : w << 16) : 0.0f;
+                amax = fmaxf(amax, fabsf(h[it][j + q]));
+            }
         }
         if (i < d) *(uint4 *)(m.S_out + (size_t)r * d + i) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
     }
@@ -549,10 +560,15 @@ __device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int f
                 const int i = (it * kThreads + tid) * 8;
                 uint32_t packed[4];
 #pragma unroll
-                for (int j = 0; j < 8; j += 2) {
-                    const float s0 = gelu_erf((h[q][it][j] - mean[q]) * rstd[q] * gv[it][j] + bv[it][j]);
-                    const float s1 = gelu_erf((h[q][it][j + 1] - mean[q]) * rstd[q] * gv[it][j + 1] + bv[it][j + 1]);
-                    packed[j >> 1] = float_to_bf16_bits(s0) | (float_to_bf16_bits(s1) << 16);
+                for (int j = 0; j < 8; j += 4) {
+                    float4 y;
+                    y.x = (h[q][it][j] - mean[q]) * rstd[q] * gv[it][j] + bv[it][j];
+                    y.y = (h[q][it][j + 1] - mean[q]) * rstd[q] * gv[it][j + 1] + bv[it][j + 1];
+                    y.z = (h[q][it][j + 2] - mean[q]) * rstd[q] * gv[it][j + 2] + bv[it][j + 2];
+                    y.w = (h[q][it][j + 3] - mean[q]) * rstd[q] * gv[it][j + 3] + bv[it][j + 3];
+                    y = gelu_erf4(y);
+                    packed[j >> 1] = float_to_bf16_bits(y.x) | (float_to_bf16_bits(y.y) << 16);
+                    packed[(j >> 1) + 1] = float_to_bf16_bits(y.z) | (float_to_bf16_bits(y.w) << 16);
                 }
                 if (i < d) *(uint4 *)(m.S_out + row * d + i) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
             }

@@ -224,15 +224,6 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
 // 8-entry list took 2000-6000 cycles to fold instead of a few hundred.
 __device__ __forceinline__ bool better(float v, int i, float w, int j) { return (v > w) | ((v == w) & (i < j)); }
 
-// The pair at (va, ia) and the pair at (vb, ib) swap places unless the first is already the better one.
-__device__ __forceinline__ void order_pair(float &va, int &ia, float &vb, int &ib) {
-    const bool sw = better(vb, ib, va, ia);
-    const float hv = sw ? vb : va, lv = sw ? va : vb;
-    const int hi = sw ? ib : ia, li = sw ? ia : ib;
-    va = hv; vb = lv;
-    ia = hi; ib = li;
-}
-
 // Order-preserving map of a float (no NaN) onto unsigned integers, and back.
 __device__ __forceinline__ uint32_t float_key(float v) {
     const uint32_t u = __float_as_uint(v);
@@ -240,26 +231,6 @@ __device__ __forceinline__ uint32_t float_key(float v) {
 }
 __device__ __forceinline__ float key_float(uint32_t k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
-
-// Sorts a list of kLen (4 or 8) entries best first with a fixed network.
-template <int kLen>
-__device__ __forceinline__ void sort_list(float (&v)[kLen], int (&i)[kLen]) {
-    static_assert(kLen == 4 || kLen == 8, "networks for 4 and 8 entries");
-#define SPEC_CX(a, b) order_pair(v[a], i[a], v[b], i[b])
-    if constexpr (kLen == 8) {
-        SPEC_CX(0, 2); SPEC_CX(1, 3); SPEC_CX(4, 6); SPEC_CX(5, 7);
-        SPEC_CX(0, 4); SPEC_CX(1, 5); SPEC_CX(2, 6); SPEC_CX(3, 7);
-        SPEC_CX(0, 1); SPEC_CX(2, 3); SPEC_CX(4, 5); SPEC_CX(6, 7);
-        SPEC_CX(2, 4); SPEC_CX(3, 5);
-        SPEC_CX(1, 4); SPEC_CX(3, 6);
-        SPEC_CX(1, 2); SPEC_CX(3, 4); SPEC_CX(5, 6);
-    } else {
-        SPEC_CX(0, 2); SPEC_CX(1, 3);
-        SPEC_CX(0, 1); SPEC_CX(2, 3);
-        SPEC_CX(1, 2);
-    }
-#undef SPEC_CX
 }
 
 __device__ __forceinline__ void fold_max_sum(float &m, float &s, const float2 &ms) {
@@ -271,7 +242,7 @@ __device__ __forceinline__ void fold_max_sum(float &m, float &s, const float2 &m
     }
 }
 
-// One partial list as it was written by the head GEMM.
+// One partial list as it was written by the head GEMM, best first.
 template <int kLen>
 struct TileList {
     float2 ms;
@@ -303,7 +274,7 @@ struct MergeOut {
 // The `rounds` best entries (rounds <= kMaxRounds) of row r's partial lists and the row's log-sum-exp.  kLen is 4
 // when a list has at most four valid slots, else 8.
 // The step is a chain of latencies in a kernel that runs for a few microseconds, so it has one barrier and little
-// code: thread t takes the lists t, t + kThreads, ... one at a time, sorts the list in registers, and its warp extracts
+// code: thread t takes the lists t, t + kThreads, ... one at a time (they are sorted best first), and its warp extracts
 // its own `rounds` best with warp-wide integer reductions (redux.sync: maximum of the value keys, then minimum token id
 // among the lanes that hold it), carrying the winners of the lists so far as one more entry of lanes 0 .. rounds - 1.
 // After the barrier every warp merges the warps' sorted results, one head per lane, in `rounds` more rounds, so that
@@ -341,7 +312,6 @@ __device__ __forceinline__ MergeOut merge_select(const MergeArgs &g, int r, int 
             tv[j] = none ? -INFINITY : tv[j];
             ti[j] = none ? 0x7fffffff : ti[j];
         }
-        sort_list<kLen>(tv, ti);
         float nv = -INFINITY;
         int ni = 0x7fffffff;
 #pragma unroll 1

@@ -169,7 +169,7 @@ struct PruneArgs {
 };
 
 struct MergeArgs {
-    const float *part_val;     // [rows, n_tiles, SPEC_MAX_TOPK] (first `topk` of each list valid, any order)
+    const float *part_val;     // [rows, n_tiles, SPEC_MAX_TOPK] (first `topk` of each list valid, best first)
     const int32_t *part_idx;   // same shape
     const float *part_ms;      // [rows, n_tiles, 2] = (max, sum of exp(x - max))
     int n_tiles, topk;

@@ -542,11 +542,14 @@ __device__ __forceinline__ bool mma_job(const Pipe &pp, const GemmJob &j, RingPo
 
 // ---- epilogue, mode 1 -----------------------------------------------------------------------------
 // One thread owns one accumulator row.  Data-dependent insertion into a sorted list diverges in
-// every warp (each lane inserts at different columns), so the selection is done branch-free:
-//   pass 1  streams the tile once: online (max, sum-exp) and the kCap largest VALUES of the row,
-//           kept sorted by a min/max network (new_v[j] = max(v[j], min(v[j-1], x)));
-//   pass 2  re-reads the tile from TMEM and emits the columns whose value reaches the topk-th
-//           largest; equal values are taken in ascending column order, exactly `topk` entries.
+// every warp (each lane inserts at different columns), so the bulk of the selection is branch-free:
+//   pass 1  streams the tile once: online (max, sum-exp) and the kCap largest of the maxima of four neighbouring
+//           columns each, kept sorted by a min/max network (new_v[j] = max(v[j], min(v[j-1], x))).  The maxima are by-products
+//           of the chunk's maximum, and the network, the largest part of the pass, sees a quarter of the columns;
+//   pass 2  re-reads the tile from TMEM.  The topk-th largest of those maxima bounds the topk-th largest column from
+//           below, so the few columns that reach it hold the answer: they are inserted, in ascending column order, into a
+//           sorted list of kCap.
+// The list leaves the kernel best first (value desc, column asc).
 // e4m3 operands: accumulator -> logit, v[i] * row_scale * col_scale[col0 + c + i] (columns past N untouched).
 __device__ __forceinline__ void scale_chunk(float (&v)[32], float rs, const float *cs, int valid) {
     if (valid >= 32 && (((uintptr_t)cs) & 15) == 0) {
@@ -581,13 +584,10 @@ __device__ __forceinline__ void epilogue_topk(const GemmJob &p, uint32_t taddr, 
             for (int i = 0; i < 32; ++i)
                 if (i >= valid) v[i] = -INFINITY;
         }
-        float cm0 = fmaxf(v[0], v[1]), cm1 = fmaxf(v[2], v[3]);
+        float g[8];
 #pragma unroll
-        for (int i = 4; i < 32; i += 2) {
-            cm0 = fmaxf(cm0, v[i]);
-            cm1 = fmaxf(cm1, v[i + 1]);
-        }
-        const float cm = fmaxf(cm0, cm1);
+        for (int i = 0; i < 8; ++i) g[i] = fmaxf(fmaxf(v[4 * i], v[4 * i + 1]), fmaxf(v[4 * i + 2], v[4 * i + 3]));
+        const float cm = fmaxf(fmaxf(fmaxf(g[0], g[1]), fmaxf(g[2], g[3])), fmaxf(fmaxf(g[4], g[5]), fmaxf(g[6], g[7])));
         if (cm > run_m) {
             run_s *= ex2_approx((run_m - cm) * kLog2e);
             run_m = cm;
@@ -603,28 +603,25 @@ __device__ __forceinline__ void epilogue_topk(const GemmJob &p, uint32_t taddr, 
         }
         if (run_m > -INFINITY) run_s += (s0 + s1) + (s2 + s3);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-            const float x = v[i];
+        for (int i = 0; i < 8; ++i) {
+            const float x = g[i];
 #pragma unroll
             for (int j = kCap - 1; j > 0; --j) best[j] = fmaxf(best[j], fminf(best[j - 1], x));
             best[0] = fmaxf(best[0], x);
         }
     }
-    // threshold = topk-th largest value of the row in this tile; how many entries lie strictly above it
     const int topk = p.epi.topk;
     float thr = best[0];
 #pragma unroll
     for (int j = 1; j < kCap; ++j)
         if (j < topk) thr = best[j];
-    int above = 0;
+    float lv[kCap];
+    int li[kCap];
 #pragma unroll
-    for (int j = 0; j < kCap; ++j)
-        if (j < topk && best[j] > thr) ++above;
-    int eq_left = topk - above;
-    const size_t u = (size_t)row * p.n_tiles + n_tile;
-    float *pv = p.epi.part_val + u * SPEC_MAX_TOPK;
-    int32_t *pi = p.epi.part_idx + u * SPEC_MAX_TOPK;
-    int cnt = 0;
+    for (int j = 0; j < kCap; ++j) {
+        lv[j] = -INFINITY;
+        li[j] = 0x7fffffff;
+    }
     for (int c = 0; c < p.block_n; c += 32) {
         float v[32];
         tmem_ld32(taddr + c, v);
@@ -650,24 +647,30 @@ __device__ __forceinline__ void epilogue_topk(const GemmJob &p, uint32_t taddr, 
 #pragma unroll
             for (int i = 0; i < 2; ++i) t2[i] = (bpos & 8) ? t4[2 * i + 1] : t4[2 * i];
             const float x = (bpos & 16) ? t2[1] : t2[0];
-            const bool gt = x > thr;
-            if (gt || eq_left > 0) {
-                if (!gt) --eq_left;
-                if (cnt < topk) {
-                    pv[cnt] = x;
-                    pi[cnt] = col0 + c + bpos + p.epi.idx_offset;
-                }
-                ++cnt;
+            const int id = col0 + c + bpos + p.epi.idx_offset;
+            // equal values: the earlier column stays in front; an entry of -inf counts only where none is left
+            bool beats[kCap];
+#pragma unroll
+            for (int j = 0; j < kCap; ++j) beats[j] = (x > lv[j]) | ((x == lv[j]) & (id < li[j]));
+#pragma unroll
+            for (int j = kCap - 1; j > 0; --j) {
+                lv[j] = beats[j - 1] ? lv[j - 1] : (beats[j] ? x : lv[j]);
+                li[j] = beats[j - 1] ? li[j - 1] : (beats[j] ? id : li[j]);
             }
+            lv[0] = beats[0] ? x : lv[0];
+            li[0] = beats[0] ? id : li[0];
         }
     }
     if (row_ok) {
-        for (; cnt < topk; ++cnt) {   // fewer than topk comparable values (NaN rows, tiny tiles)
-            pv[cnt] = -INFINITY;
-            pi[cnt] = 0x7fffffff;
+        const size_t u = (size_t)row * p.n_tiles + n_tile;
+        float4 *pv = (float4 *)(p.epi.part_val + u * SPEC_MAX_TOPK);
+        int4 *pi = (int4 *)(p.epi.part_idx + u * SPEC_MAX_TOPK);
+#pragma unroll
+        for (int q = 0; q < kCap / 4; ++q) {
+            pv[q] = make_float4(lv[4 * q], lv[4 * q + 1], lv[4 * q + 2], lv[4 * q + 3]);
+            pi[q] = make_int4(li[4 * q], li[4 * q + 1], li[4 * q + 2], li[4 * q + 3]);
         }
-        p.epi.part_ms[2 * u] = run_m;
-        p.epi.part_ms[2 * u + 1] = run_s;
+        *(float2 *)(p.epi.part_ms + 2 * u) = make_float2(run_m, run_s);
     }
 }
 
@@ -702,9 +705,9 @@ __device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, %0;" 
 
 // One thread scans `len` (a multiple of 16) consecutive logits of one node in the transposed tile: `col`
 // points at the first, `valid` of them are real vocabulary rows (the rest hold -inf), `idx0` is the token id
-// of the first.  Pass 1: online (max, sum-exp) and the kCap largest values (min/max network).  Pass 2: the
-// entries that reach the topk-th largest value, ties in ascending token order, exactly topk of them, are
-// inserted into the running list.
+// of the first.  As in epilogue_topk, but with the values themselves (a thread has only 16 to 128 of them): pass 1 takes the
+// online (max, sum-exp) and the kCap largest values, pass 2 inserts the entries that reach the topk-th largest of them, and
+// the topk-th entry of the running list, into that list.
 template <int kCap>
 __device__ __forceinline__ void swap_scan_tile(const float *col, int len, int valid, int idx0, int topk, SwapRun &r) {
     constexpr float kLog2e = 1.4426950408889634f;
@@ -718,13 +721,10 @@ __device__ __forceinline__ void swap_scan_tile(const float *col, int len, int va
             const float4 f = *(const float4 *)(col + c + 4 * q);
             v[4 * q] = f.x; v[4 * q + 1] = f.y; v[4 * q + 2] = f.z; v[4 * q + 3] = f.w;
         }
-        float cm0 = fmaxf(v[0], v[1]), cm1 = fmaxf(v[2], v[3]);
+        float g[8];
 #pragma unroll
-        for (int i = 4; i < 16; i += 2) {
-            cm0 = fmaxf(cm0, v[i]);
-            cm1 = fmaxf(cm1, v[i + 1]);
-        }
-        const float cm = fmaxf(cm0, cm1);
+        for (int i = 0; i < 8; ++i) g[i] = fmaxf(v[2 * i], v[2 * i + 1]);
+        const float cm = fmaxf(fmaxf(fmaxf(g[0], g[1]), fmaxf(g[2], g[3])), fmaxf(fmaxf(g[4], g[5]), fmaxf(g[6], g[7])));
         if (cm > r.m) {
             r.s *= ex2_approx((r.m - cm) * kLog2e);
             r.m = cm;
@@ -747,15 +747,13 @@ __device__ __forceinline__ void swap_scan_tile(const float *col, int len, int va
             best[0] = fmaxf(best[0], x);
         }
     }
-    float thr = best[0];
+    float thr = best[0], worst = r.tv[0];
 #pragma unroll
-    for (int j = 1; j < kCap; ++j)
-        if (j < topk) thr = best[j];
-    int above = 0;
-#pragma unroll
-    for (int j = 0; j < kCap; ++j)
-        if (j < topk && best[j] > thr) ++above;
-    int eq_left = topk - above;
+    for (int j = 1; j < kCap; ++j) {
+        thr = j < topk ? best[j] : thr;
+        worst = j < topk ? r.tv[j] : worst;
+    }
+    thr = fmaxf(thr, worst);
     for (int c = 0; c < len; c += 16) {
         uint32_t mask = 0;
 #pragma unroll
@@ -771,12 +769,7 @@ __device__ __forceinline__ void swap_scan_tile(const float *col, int len, int va
         while (mask) {   // ascending token ids; a handful of iterations per tile
             const int bpos = __ffs(mask) - 1;
             mask &= mask - 1;
-            const float x = col[c + bpos];
-            const bool gt = x > thr;
-            if (gt || eq_left > 0) {
-                if (!gt) --eq_left;
-                list_insert(r, x, idx0 + c + bpos);
-            }
+            list_insert(r, col[c + bpos], idx0 + c + bpos);
         }
     }
 }

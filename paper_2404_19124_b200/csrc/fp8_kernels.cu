@@ -154,7 +154,7 @@ int launch_merge_rescore(const MergeArgs &g, const void *W, const void *S, int r
     a.S = (const uint16_t *)S;
     a.d = d;
     a.V = V;
-    const size_t smem = g.seq_done ? sizeof(LeafKey) * (size_t)g.Lpad : 0;
+    const size_t smem = g.seq_done ? prune_smem_bytes(g.L, g.Lpad) : 0;
     SPEC_CUDA_TRY(launch_pdl(merge_rescore_kernel, dim3(rows), dim3(kRescoreThreads), smem, st, a));
     return SPEC_OK;
 }

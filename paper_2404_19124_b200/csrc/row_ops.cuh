@@ -36,14 +36,14 @@ struct Scratch {
 };
 
 // (`red`: one float per warp, not read by anybody else until the next barrier behind the call)
-template <int kThreads, typename Sync>
+template <int kThreads, typename Sync>   // (kThreads 0: blockDim.x)
 __device__ __forceinline__ float group_sum(float v, float *red, int tid) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     const int w = tid >> 5, l = tid & 31;
     if (l == 0) red[w] = v;
     Sync::sync();
-    float t = (l < kThreads / 32) ? red[l] : 0.0f;
+    float t = l < (kThreads > 0 ? kThreads : (int)blockDim.x) / 32 ? red[l] : 0.0f;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
     return t;
@@ -57,7 +57,7 @@ __device__ __forceinline__ float group_max(float v, float *red, int tid) {
     Sync::sync();
     if (l == 0) red[w] = v;
     Sync::sync();
-    float t = (l < kThreads / 32) ? red[l] : 0.0f;   // used for magnitudes only
+    float t = l < (kThreads > 0 ? kThreads : (int)blockDim.x) / 32 ? red[l] : 0.0f;   // used for magnitudes only
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) t = fmaxf(t, __shfl_xor_sync(0xffffffffu, t, off));
     return t;
@@ -72,13 +72,14 @@ static __device__ __noinline__ float4 gelu_erf4(float4 y) {
 
 // Node r of the level, whose token is t and whose projected parent state is row `parent` of P.
 // h = a * P[parent] + b * E[t].  The row lives in registers: thread t owns the 8-element groups
-// t, t + kThreads, ... (kIters of them; d <= 8 * kThreads * kIters, d % 8 == 0).  kDepth of those
-// groups have their loads in flight together (registers against latency).
-template <int kThreads, int kIters, int kDepth, typename Sync>
+// t, t + kThreads, ... (kIters of them; d <= 8 * kThreads * kIters, d % 8 == 0; kThreads 0: as many as the CTA has).
+// kDepth of those groups, and kSp partial projections of each, have their loads in flight together (registers against
+// latency).
+template <int kThreads, int kIters, int kDepth, typename Sync, int kSp = 4>
 __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int parent, int t, int tid, float *red) {
-    constexpr int kSp = 4;                                        // partial projections fetched per batch
     constexpr int kGroup = kIters >= 8 ? 1 : (kIters < kDepth ? kIters : kDepth);
     bool tok_ok = false;
+    const int nt = kThreads > 0 ? kThreads : (int)blockDim.x;
     const int d = m.d;
     const float *p = m.P + (size_t)parent * d;
     const uint16_t *e = nullptr;
@@ -92,7 +93,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
         float4 pa[kGroup][kSp], pb[kGroup][kSp];
 #pragma unroll
         for (int q = 0; q < kGroup; ++q) {
-            const int i = ((g0 + q) * kThreads + tid) * 8;
+            const int i = ((g0 + q) * nt + tid) * 8;
 #pragma unroll
             for (int sp = 0; sp < kSp; ++sp) {
                 pa[q][sp] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -110,14 +111,14 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
         }
 #pragma unroll
         for (int q = 0; q < kGroup; ++q) {
-            const int i = ((g0 + q) * kThreads + tid) * 8;
+            const int i = ((g0 + q) * nt + tid) * 8;
             ev[q] = make_uint4(0u, 0u, 0u, 0u);
             if (i < d && tok_ok) ev[q] = *(const uint4 *)(e + i);
         }
 #pragma unroll
         for (int q = 0; q < kGroup; ++q) {
             const int it = g0 + q;
-            const int i = (it * kThreads + tid) * 8;
+            const int i = (it * nt + tid) * 8;
             float pv[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
             for (int sp = 0; sp < kSp; ++sp) {      // partials are added in ascending order: reproducible
@@ -149,7 +150,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
     if (kHoist) {
 #pragma unroll
         for (int it = 0; it < kHeld; ++it) {
-            const int i = (it * kThreads + tid) * 8;
+            const int i = (it * nt + tid) * 8;
             const int ic = i < d ? i : 0;
             gq[it][0] = *(const float4 *)(m.gamma + ic);
             gq[it][1] = *(const float4 *)(m.gamma + ic + 4);
@@ -161,7 +162,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
     float sq = 0.0f;
 #pragma unroll
     for (int it = 0; it < kIters; ++it) {
-        const int i = (it * kThreads + tid) * 8;
+        const int i = (it * nt + tid) * 8;
         if (i < d) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -175,7 +176,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
     float amax = 0.0f;   // largest magnitude of the bf16-rounded state (for the e4m3 copy); h is reused for it
 #pragma unroll
     for (int it = 0; it < kIters; ++it) {
-        const int i = (it * kThreads + tid) * 8;
+        const int i = (it * nt + tid) * 8;
         const int hq = kHoist ? it : 0;
         if (!kHoist) {
             const int ic = i < d ? i : 0;
@@ -211,7 +212,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
         const float inv = 1.0f / scale;
 #pragma unroll
         for (int it = 0; it < kIters; ++it) {
-            const int i = (it * kThreads + tid) * 8;
+            const int i = (it * nt + tid) * 8;
             if (i < d) *(uint2 *)(m.S8_out + (size_t)r * d + i) = e4m3x8(h[it], inv);
         }
         if (tid == 0) m.s8_scale[r] = scale;
@@ -546,7 +547,7 @@ __device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int f
     }
 }
 
-struct LeafKey {
+struct __align__(8) LeafKey {
     float score;
     int leaf;
 };
@@ -582,11 +583,81 @@ __device__ __forceinline__ void load_path(const PruneArgs &pa, int L, int b, int
     }
 }
 
+// Leaves of one sequence as integers: the order-preserving image of the score above 4095 - leaf, so that the greater key
+// is the better leaf and no two are equal.  (+ 0.0f: -0 and +0 are equal.)
+static_assert(SPEC_MAX_LEAVES <= 4096, "twelve bits for the leaf");
+__device__ __forceinline__ uint64_t leaf_key(float score, int leaf) {
+    return ((uint64_t)float_key(score + 0.0f) << 12) | (uint32_t)(4095 - leaf);
+}
+
+// The K best (K <= kSelectMax) of the L keys in shared memory, to `sel` in any order: a radix selection from the top, eight
+// bits a pass, until the keys of the bin that holds the K-th are wanted all or none.  `hist`: 256 words, `state`: 4 words.
+constexpr int kSelectMax = 256;
+constexpr int kSelectWords = 256 + 4 + 2 * kSelectMax;   // 32-bit words behind the keys: histogram, state, selection
+template <int kThreads, typename Sync>
+__device__ __forceinline__ void select_leaves(const uint64_t *keys, int L, int K, uint32_t *hist, uint32_t *state,
+                                              uint64_t *sel, int tid) {
+    const int lane = tid & 31, warp = tid >> 5;
+    uint64_t prefix = 0;   // the keys still in question are those whose bits from `top` on equal it
+    int top = 44, need = K;
+    while (true) {
+        const int shift = top > 8 ? top - 8 : 0;
+        for (int i = tid; i < 256; i += kThreads) hist[i] = 0;
+        if (tid == 0) state[3] = 0;
+        Sync::sync();
+        for (int i0 = warp * 32; i0 < L; i0 += kThreads) {   // (uniform over the warp)
+            const uint64_t k = i0 + lane < L ? keys[i0 + lane] : 0;
+            const bool in = i0 + lane < L && (k >> top) == prefix;
+            // scores crowd in few bins: one addition per bin and warp
+            const uint32_t bin = in ? (uint32_t)(k >> shift) & ((1u << (top - shift)) - 1u) : 256u;
+            const uint32_t peers = __match_any_sync(0xffffffffu, bin);
+            if (in && lane == __ffs(peers) - 1) atomicAdd(hist + bin, __popc(peers));
+        }
+        Sync::sync();
+        if (warp == 0) {   // lane l: bins 255 - 8 l downwards
+            uint32_t c[8], sum = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                c[q] = hist[255 - 8 * lane - q];
+                sum += c[q];
+            }
+            uint32_t upto = sum;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t o = __shfl_up_sync(0xffffffffu, upto, off);
+                if (lane >= off) upto += o;
+            }
+            uint32_t above = upto - sum;
+            if (above < (uint32_t)need && upto >= (uint32_t)need) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q) {
+                    if (above < (uint32_t)need && above + c[q] >= (uint32_t)need) {
+                        state[0] = 255 - 8 * lane - q;
+                        state[1] = need - above;
+                        state[2] = c[q];
+                    }
+                    above += c[q];
+                }
+            }
+        }
+        Sync::sync();
+        prefix = (prefix << (top - shift)) | state[0];
+        top = shift;
+        need = (int)state[1];
+        if (need == (int)state[2] || top == 0) break;
+    }
+    const uint64_t least = prefix << top;
+    for (int i = tid; i < L; i += kThreads)
+        if (keys[i] >= least) sel[atomicAdd(state + 3, 1u)] = keys[i];
+    Sync::sync();
+}
+
 // Sequence b: the K best leaves by (score desc, leaf index asc), traced back to the root.  `keys`:
-// shared memory for Lpad entries, Lpad the power of two >= max(L, 2).  Up to 256 leaves every thread
-// counts how many leaves precede its own (that is its rank; no barriers) and has requested the tokens of its
-// own leaves' paths together with the scores, so a kept leaf is written out without another trip to memory;
-// longer lists are sorted bitonically.
+// shared memory for Lpad entries, Lpad the power of two >= max(L, 2), and kSelectWords more when L > 256.  Up to 256 leaves
+// every thread counts how many leaves precede its own (that is its rank; no barriers) and has requested the tokens of its
+// own leaves' paths together with the scores, so a kept leaf is written out without another trip to memory.  Of longer lists
+// the K best are selected first and then ranked among themselves (2016 rows, 1512 leaves, K = 3: the last kernel 63 us with a
+// sort, 15.8 so); only when more than 256 are kept the whole list is sorted.
 template <int kThreads, typename Sync>
 __device__ __forceinline__ void prune_sequence(const float *leaf_score, const PruneArgs &pa, int L, int Lpad, int K,
                                                int32_t *cand_tok, float *cand_logp, int b, int tid, LeafKey *keys) {
@@ -596,6 +667,26 @@ __device__ __forceinline__ void prune_sequence(const float *leaf_score, const Pr
 #pragma unroll
         for (int q = 0; q < kOwn; ++q)
             if (tid + q * kThreads < L) load_path(pa, L, b, tid + q * kThreads, path[q]);
+    }
+    if (L > 256 && K <= kSelectMax) {
+        uint64_t *k64 = (uint64_t *)keys;
+        uint32_t *hist = (uint32_t *)(keys + Lpad), *state = hist + 256;
+        uint64_t *sel = (uint64_t *)(state + 4);
+        for (int i = tid; i < L; i += kThreads) k64[i] = leaf_key(__ldcg(leaf_score + (size_t)b * L + i), i);
+        select_leaves<kThreads, Sync>(k64, L, K, hist, state, sel, tid);   // (begins with a barrier)
+        for (int i = tid; i < K; i += kThreads) {
+            const uint64_t mine = sel[i];
+            const int leaf = 4095 - (int)(mine & 4095u);
+            int32_t own[SPEC_MAX_HEADS];
+            load_path(pa, L, b, leaf, own);
+            int rank = 0;
+            for (int j = 0; j < K; ++j) rank += sel[j] > mine ? 1 : 0;
+            cand_logp[(size_t)b * K + rank] = __ldcg(leaf_score + (size_t)b * L + leaf);
+#pragma unroll
+            for (int l = 0; l < SPEC_MAX_HEADS; ++l)
+                if (l < pa.n) cand_tok[((size_t)b * K + rank) * pa.n + l] = own[l];
+        }
+        return;
     }
     Sync::sync();   // a previous call may still be reading the keys
     for (int i = tid; i < Lpad; i += kThreads) {
@@ -638,6 +729,11 @@ __device__ __forceinline__ void prune_sequence(const float *leaf_score, const Pr
     }
     for (int k = tid; k < K; k += kThreads)
         emit_candidate(pa, L, K, cand_tok, cand_logp, b, k, keys[k].score, keys[k].leaf);
+}
+
+// Shared memory of prune_sequence.
+inline size_t prune_smem_bytes(int L, int Lpad) {
+    return sizeof(LeafKey) * (size_t)Lpad + (L > 256 ? sizeof(uint32_t) * kSelectWords : 0);
 }
 
 // Prune folded into the kernel that writes the last level.  Every row's CTA makes its children visible

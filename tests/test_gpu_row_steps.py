@@ -21,9 +21,12 @@ def B():
 
 @pytest.mark.parametrize("fp8", [False, True])
 @pytest.mark.parametrize("topk,K", [((8, 4, 5), 160), ((7, 7, 3), 100), ((8, 4, 3, 2), 64), ((8, 4, 3, 2), 192),
-                                    ((8, 8, 4), 255), ((8, 8, 4), 256)])
+                                    ((8, 8, 4), 255), ((8, 8, 4), 256), ((7, 5, 8), 1), ((8, 8, 8), 1),
+                                    ((8, 8, 8), 64), ((8, 8, 8), 255), ((8, 8, 8), 256), ((8, 8, 8), 257),
+                                    ((8, 8, 8, 8), 5), ((8, 8, 8, 8), 256)])
 def test_prune_leaves_round_the_thread_counts(B, topk, K, fp8):
-    """147 to 256 leaves: more and fewer than the 160 (or 512) threads of the CTA that ranks them."""
+    """147 to 256 leaves: more and fewer than the 160 (or 512) threads of the CTA that ranks them; more leaves: up to 256
+    kept are selected, more are sorted."""
     cfg = small_cfg(d_base=48, d_inner=64, V=96, topk=topk, K=K, B=3, seed=K)
     sw = synth.make_weights(cfg)
     ow, gw = to_oracle_weights(sw), weights_to_cuda(sw)
@@ -43,7 +46,7 @@ def test_prune_leaves_round_the_thread_counts(B, topk, K, fp8):
     assert torch.equal(lp, want.values[:, :K])
     last = ws[lay.tok[cfg.n]:lay.tok[cfg.n] + 4 * cfg.B * L].view(torch.int32).view(cfg.B, L)
     assert torch.equal(ct[:, :, -1], torch.gather(last, 1, want.indices[:, :K]))
-    if not fp8:
+    if not fp8 and L <= 256:
         chk = DraftChecker(ow, topk, K)
         for b in range(cfg.B):
             chk.check(synth.bf16_bits(ctx)[b], int(tok[b]), ct[b].cpu().numpy(), lp[b].cpu().numpy())
@@ -131,4 +134,57 @@ def test_merge_and_mix_round_one_child_per_sm(B, B_, topk, d):
             sc.append(view(lay.score[l + 1], N1, torch.float32).view(B_, -1)[b].cpu().numpy())
         chk.check(synth.bf16_bits(ctx)[b], int(tok[b]), ct[b].cpu().numpy(), lp[b].cpu().numpy(),
                   levels={"state": st, "tok": tk, "score": sc}, force_levels=True)
+    B.spec_destroy(h)
+
+
+@pytest.mark.parametrize("values", [1, 2, 5])
+@pytest.mark.parametrize("K", [1, 100, 256])
+def test_selection_among_equal_scores(B, K, values):
+    """All heads zero but for the last, whose rows repeat: 512 leaves with `values` distinct scores each; equal scores are
+    kept in ascending leaf order."""
+    topk = (8, 8, 8)
+    cfg = small_cfg(d_base=48, d_inner=64, V=96, topk=topk, K=K, B=2, seed=values)
+    sw = synth.make_weights(cfg)
+    for l in range(2):
+        sw.head[l].zero_()
+    sw.head[2][:] = sw.head[2][:1]
+    if values > 1:
+        sw.head[2][:4] *= 2.0
+    if values > 2:
+        sw.emb[2][:] = 0.0
+    h = B.spec_create(weights_to_cuda(sw))
+    ctx, tok = synth.make_draft_inputs(cfg)
+    ct, lp, ws = B.spec_draft(h, ctx.cuda(), tok.cuda(), topk, K)
+    assert B.spec_poll_error(ws) == 0
+    lay = B.spec_draft_layout(h, cfg.B, topk, K)
+    leaf = ws[lay.score[3]:lay.score[3] + 4 * cfg.B * 512].view(torch.float32).view(cfg.B, 512)
+    last = ws[lay.tok[3]:lay.tok[3] + 4 * cfg.B * 512].view(torch.int32).view(cfg.B, 512)
+    want = torch.sort(leaf, dim=1, descending=True, stable=True)
+    assert torch.equal(lp, want.values[:, :K])
+    assert torch.equal(ct[:, :, -1], torch.gather(last, 1, want.indices[:, :K]))
+    first = ws[lay.tok[1]:lay.tok[1] + 4 * cfg.B * 8].view(torch.int32).view(cfg.B, 8)
+    assert torch.equal(ct[:, :, 0], torch.gather(first, 1, want.indices[:, :K] // 64))
+    B.spec_destroy(h)
+
+
+@pytest.mark.parametrize("d", [264, 512, 520, 1024, 1032, 2304, 4096])
+@pytest.mark.parametrize("parents", [40, 74, 75, 150])
+def test_mix_of_many_rows_round_the_thread_counts(B, d, parents):
+    """More nodes than SMs, with the parents' projection split (up to 128 rows) and whole; states against the oracle."""
+    topk = (4, 1)
+    cfg = small_cfg(d_base=64, d_inner=d, V=64, topk=topk, K=4, B=parents, seed=d)
+    sw = synth.make_weights(cfg)
+    ow, gw = to_oracle_weights(sw), weights_to_cuda(sw)
+    ctx, tok = synth.make_draft_inputs(cfg)
+    h = B.spec_create(gw)
+    B.spec_set_option(h, B.SPEC_OPT_HEAD_PAIR, 0)
+    _, _, ws = B.spec_draft(h, ctx.cuda(), tok.cuda(), topk, 4)
+    assert B.spec_poll_error(ws) == 0
+    lay = B.spec_draft_layout(h, parents, topk, 4)
+    s0 = ws[lay.state[0]:lay.state[0] + 2 * parents * d].view(torch.bfloat16).view(parents, d).float().cpu().numpy()
+    s1 = ws[lay.state[1]:lay.state[1] + 8 * parents * d].view(torch.bfloat16).view(4 * parents, d).float().cpu().numpy()
+    t1 = ws[lay.tok[1]:lay.tok[1] + 16 * parents].view(torch.int32).cpu().numpy()
+    for r in (0, 1, 2 * parents + 1, 4 * parents - 1):
+        want = oracle.stage_state(ow, 1, s0[r // 4], int(t1[r]))
+        assert np.allclose(s1[r], want, rtol=0.008, atol=2e-4)
     B.spec_destroy(h)

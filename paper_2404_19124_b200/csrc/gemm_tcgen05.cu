@@ -242,6 +242,9 @@ int plan_job(tc::GemmJob *j, int M, int N, int Kd, int block_n, const GemmEpilog
     j->block_n = block_n;
     j->m_tiles = (M + kBlockM - 1) / kBlockM;
     j->n_tiles = (N + block_n - 1) / block_n;
+    const int m8 = (M + 7) / 8 * 8, n8 = (N + 7) / 8 * 8;
+    j->a_box_rows = m8 < kBlockM ? m8 : kBlockM;
+    j->b_box_rows = n8 < block_n ? n8 : block_n;
     j->fp8 = fp8;
     const int ke = fp8 ? kSlabBytes : kSlabBytes / 2;
     const int num_kb = (Kd + ke - 1) / ke;
@@ -259,6 +262,7 @@ int plan_job(tc::GemmJob *j, int M, int N, int Kd, int block_n, const GemmEpilog
         j->epi.segs = swapped_head_segs(N);
         j->rows_per_cta = swapped_rows_per_cta(M);
         j->deal_ctas = (M + j->rows_per_cta - 1) / j->rows_per_cta;
+        j->a_box_rows = j->rows_per_cta < kBlockM ? j->rows_per_cta : kBlockM;
         j->epi.n_parts = j->deal_ctas;
         // Rows of a multiple of 4096 bytes only: the others gain nothing and pay 0.5 % for the second accumulator.  (Not in a
         // vocabulary shard: shards whose sizes put them on different forms must agree on equal logits.)
@@ -282,6 +286,7 @@ int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaSt
     p.n_jobs = n_calls;
     p.producers = g_gemm_producers;
     if (start) p.start = *start;
+    int max_rows = 0, max_reach = 0;      // rows of a slot's boxes, and of what its MMAs read
     int max_block_n = 32, max_acc = 32;   // widest tile; most accumulator columns of one tile
     long long total_tiles = 0;
     for (int q = 0; q < n_calls; ++q) {
@@ -289,18 +294,23 @@ int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaSt
         int rc = plan_job(&p.job[q], c.M, c.N, c.Kd, c.block_n, c.epi);
         if (rc != SPEC_OK) return rc;
         if (((uintptr_t)c.A & 15) || ((uintptr_t)c.B & 15)) return SPEC_ERR_INVALID_ARG;
-        rc = make_tmap(&maps.a[q], c.A, (uint64_t)c.M, (uint64_t)c.Kd, kBlockM, p.job[q].w_is_a != 0, p.job[q].fp8 != 0);
+        rc = make_tmap(&maps.a[q], c.A, (uint64_t)c.M, (uint64_t)c.Kd, (uint32_t)p.job[q].a_box_rows, p.job[q].w_is_a != 0, p.job[q].fp8 != 0);
         if (rc != SPEC_OK) return rc;
-        rc = make_tmap(&maps.b[q], c.B, (uint64_t)c.N, (uint64_t)c.Kd, (uint32_t)c.block_n, p.job[q].w_is_a == 0,
+        rc = make_tmap(&maps.b[q], c.B, (uint64_t)c.N, (uint64_t)c.Kd, (uint32_t)p.job[q].b_box_rows, p.job[q].w_is_a == 0,
                        p.job[q].fp8 != 0);
         if (rc != SPEC_OK) return rc;
         if (c.block_n > max_block_n) max_block_n = c.block_n;
+        const int box_rows = p.job[q].a_box_rows + p.job[q].b_box_rows;
+        if (box_rows > max_rows) max_rows = box_rows;
+        // (what the MMAs of a slot read from its start on)
+        const int reach = kBlockM > p.job[q].a_box_rows + c.block_n ? kBlockM : p.job[q].a_box_rows + c.block_n;
+        if (reach > max_reach) max_reach = reach;
         if (c.block_n << p.job[q].halves > max_acc) max_acc = c.block_n << p.job[q].halves;
         if (c.epi.mode == 3) {
             if (q != 0) return SPEC_ERR_INVALID_ARG;   // its CTAs are the first of the grid
             p.tbuf_bytes = (uint32_t)c.block_n * kTPitch * sizeof(float);
             const int short_rows = p.job[q].rows_per_cta % kBlockM;
-            if (short_rows > 0) {
+            if (short_rows > 0 && p.job[q].rows_per_cta > kBlockM) {
                 rc = make_tmap(&maps.a_short, c.A, (uint64_t)c.M, (uint64_t)c.Kd, (uint32_t)short_rows, true, false);
                 if (rc != SPEC_OK) return rc;
             }
@@ -318,9 +328,10 @@ int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaSt
         offset += p.job[q].epi.mode == 3 ? (long long)p.job[q].deal_ctas
                                          : (long long)p.job[q].m_tiles * p.job[q].n_tiles * p.job[q].splits;
     }
-    p.slot_bytes = (uint32_t)kABytes + (uint32_t)max_block_n * kSlabBytes;
+    p.slot_bytes = (uint32_t)max_rows * kSlabBytes;
+    const int overhang = (max_reach - max_rows) * kSlabBytes;   // of the last slot's reads
     const int budget = kSmemLimit - 1024 - (int)sizeof(Barriers) - 64 - (int)p.tbuf_bytes;
-    p.stages = budget / (int)p.slot_bytes;
+    p.stages = (budget - (overhang > 0 ? overhang : 0)) / (int)p.slot_bytes;
     if (p.stages > kMaxStages) p.stages = kMaxStages;
     if (p.stages < 2) return SPEC_ERR_SHAPE;
     int cols = 32;
@@ -329,7 +340,8 @@ int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaSt
     p.acc_stride = max_acc;
     p.err = err;
 
-    const size_t smem = 1024 + (size_t)p.stages * p.slot_bytes + p.tbuf_bytes + sizeof(Barriers);
+    const size_t smem = 1024 + (size_t)p.stages * p.slot_bytes + p.tbuf_bytes + sizeof(Barriers) +
+                        (overhang > 0 ? (size_t)overhang : 0);
     int dev = 0;
     SPEC_CUDA_TRY(cudaGetDevice(&dev));
     {

@@ -258,7 +258,7 @@ int plan_job(tc::GemmJob *j, int M, int N, int Kd, int block_n, const GemmEpilog
     j->rows_per_cta = 0;
     j->halves = 0;
     if (epi.mode == 3) {   // all nodes in one tile column; every CTA of the deal leaves one list per node
-        if (N > kBlockM || j->n_tiles != 1 || fp8) return SPEC_ERR_SHAPE;
+        if (N > kBlockM || j->n_tiles != 1) return SPEC_ERR_SHAPE;
         j->epi.segs = swapped_head_segs(N);
         j->rows_per_cta = swapped_rows_per_cta(M);
         j->deal_ctas = (M + j->rows_per_cta - 1) / j->rows_per_cta;
@@ -266,7 +266,7 @@ int plan_job(tc::GemmJob *j, int M, int N, int Kd, int block_n, const GemmEpilog
         j->epi.n_parts = j->deal_ctas;
         // Rows of a multiple of 4096 bytes only: the others gain nothing and pay 0.5 % for the second accumulator.  (Not in a
         // vocabulary shard: shards whose sizes put them on different forms must agree on equal logits.)
-        j->halves = Kd % 2048 == 0 && !epi.sharded ? 1 : 0;
+        j->halves = Kd % 2048 == 0 && !fp8 && !epi.sharded ? 1 : 0;
     }
     return SPEC_OK;
 }
@@ -311,7 +311,7 @@ int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaSt
             p.tbuf_bytes = (uint32_t)c.block_n * kTPitch * sizeof(float);
             const int short_rows = p.job[q].rows_per_cta % kBlockM;
             if (short_rows > 0 && p.job[q].rows_per_cta > kBlockM) {
-                rc = make_tmap(&maps.a_short, c.A, (uint64_t)c.M, (uint64_t)c.Kd, (uint32_t)short_rows, true, false);
+                rc = make_tmap(&maps.a_short, c.A, (uint64_t)c.M, (uint64_t)c.Kd, (uint32_t)short_rows, true, p.job[q].fp8 != 0);
                 if (rc != SPEC_OK) return rc;
             }
             total_tiles += p.job[q].deal_ctas;   // what counts for the grid: the CTAs it occupies

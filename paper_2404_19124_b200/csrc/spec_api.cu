@@ -82,11 +82,13 @@ int head_block_n_for(const spec_handle_s *h, int rows) {
 // d 1024, V 1500, 12 / 24 / 48 nodes 52.3 -> 48.9 / 50.3 / 52.0; V 4500 58.3, 58.2, 56.7 -> 50.9 / 52.7 / 54.6;
 // V 12000 62.8, 62.0, 60.3 -> 52.8 / 54.6 / 57.4; d 2048, V 12000, 64 / 96 nodes 72.1, 74.2 -> 72.7 / 79.6;
 // V 32000, 64 / 80 / 128 nodes 109.6, 112.5, 119.0 -> 106.7 / 114.4 / 128.8.
-bool head_swapped_for(const spec_handle_s *h, int rows) {
+// e4m3 heads (lists of eight whatever the branching): V 32000, d 4096, two levels of 60 nodes 98.8 -> 88.3; V 27408,
+// d 3584, 7 nodes 55.3 -> 47.7; V 5000, d 2048, 40 nodes 46.5 -> 48.7; the 13B step 251 -> 243.
+bool head_swapped_for(const spec_handle_s *h, int rows, bool fp8 = false) {
     if (h->gemm_impl != 0 || h->head_block_n != 0 || rows > 128) return false;
     if (h->swap_max_rows >= 0) return rows <= h->swap_max_rows;
     const int rows_per_sm = h->head_rows / num_sms();
-    return rows <= (rows_per_sm >= 128 ? 64 : rows_per_sm >= 30 ? 48 : 32);
+    return rows <= (rows_per_sm >= 128 ? 64 : rows_per_sm >= 30 && !fp8 ? 48 : 32);
 }
 
 // Levels of more than 128 nodes (several 128-row tiles per weight tile) may run on CTA pairs.
@@ -185,7 +187,7 @@ int make_draft_plan(const spec_handle_s *h, int B, const int32_t *topk, int K, D
         p->use_fp8[l] = h->gemm_impl == 0 && !h->profile && h->head8[l] != nullptr && p->N[l] <= h->fp8_max_rows &&
                         w.d_inner <= 16384 && h->vp_ranks == 1;
         if (p->use_fp8[l] && p->N[l] > max_fp8_rows) max_fp8_rows = p->N[l];
-        p->swapped[l] = !p->use_fp8[l] && head_swapped_for(h, p->N[l]);
+        p->swapped[l] = head_swapped_for(h, p->N[l], p->use_fp8[l]);
         p->paired[l] = !p->use_fp8[l] && !h->profile && head_paired_for(h, p->N[l]);
     }
     for (int l = 0; l < p->n; ++l) {
@@ -276,9 +278,11 @@ GemmCall make_head_call(const spec_handle_s *h, const DraftPlan &p, char *ws, in
         c.epi.topk = SPEC_MAX_TOPK;
         c.epi.row_scale = (const float *)(ws + p.lay.state8_scale);
         c.epi.col_scale = h->head8_scale[l];
-    } else if (p.swapped[l]) {
-        c.A = w.head[l]; c.M = h->head_rows;
-        c.B = ws + p.lay.state[l]; c.N = p.N[l];
+    }
+    if (p.swapped[l]) {
+        const void *states = c.A;
+        c.A = c.B; c.M = h->head_rows;
+        c.B = states; c.N = p.N[l];
         c.block_n = (p.N[l] + 15) / 16 * 16;
         c.epi.mode = 3;
     }

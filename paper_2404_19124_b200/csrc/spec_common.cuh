@@ -101,8 +101,8 @@ struct GemmEpilogue {
     int32_t *part_idx; // mode 1: [M, n_tiles, SPEC_MAX_TOPK]
     float *part_ms;    // mode 1: [M, n_tiles, 2]
     int topk;          // mode 1
-    int fp8;           // operands are e4m3 bytes instead of bf16; mode 1 then multiplies every accumulator by
-                       // row_scale[m] * col_scale[n] before the selection
+    int fp8;           // operands are e4m3 bytes instead of bf16; the logit of node m and vocabulary row n is then
+                       // the accumulator times row_scale[m] * col_scale[n]
     const float *row_scale, *col_scale;
     int sharded;       // the weights are a vocabulary shard
     int idx_offset;    // mode 1 / 3: added to every token id written to part_idx (first vocabulary row of a shard)

@@ -713,12 +713,14 @@ __device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, %0;" 
 
 // One thread scans `len` (a multiple of 16) consecutive logits of one node in the transposed tile: `col`
 // points at the first, `valid` of them are real vocabulary rows (the rest hold -inf), `idx0` is the token id
-// of the first.  As in epilogue_topk, but with the values themselves (a thread has only 16 to 128 of them): pass 1 takes the
+// of the first.  The node's logits are `scale` > 0 times what is stored (and what the running list holds).  As in
+// epilogue_topk, but with the values themselves (a thread has only 16 to 128 of them): pass 1 takes the
 // online (max, sum-exp) and the kCap largest values, pass 2 inserts the entries that reach the topk-th largest of them, and
 // the topk-th entry of the running list, into that list.
 template <int kCap>
-__device__ __forceinline__ void swap_scan_tile(const float *col, int len, int valid, int idx0, int topk, SwapRun &r) {
-    constexpr float kLog2e = 1.4426950408889634f;
+__device__ __forceinline__ void swap_scan_tile(const float *col, int len, int valid, int idx0, int topk, float scale,
+                                               SwapRun &r) {
+    const float kLog2e = 1.4426950408889634f * scale;
     float best[kCap];
 #pragma unroll
     for (int j = 0; j < kCap; ++j) best[j] = -INFINITY;
@@ -837,6 +839,8 @@ __device__ __forceinline__ bool epilogue_job_swapped(const Pipe &pp, const GemmJ
     }
     const TileWalk w = walk_of(j);
     const int row_end = min(j.M, (w.rel + 1) * j.rows_per_cta);   // the next CTA's rows start here
+    // e4m3: a vocabulary row's scale is applied on the way to shared memory, the node's in the end: it orders nothing
+    const float node_scale = j.fp8 && scans ? __ldcg(j.epi.row_scale + node) : 1.0f;
     for (int tile = w.first; tile < w.end; tile += w.step) {
         if (u == 0) bars->epi_ok = mbar_wait(&bars->acc_full[ap.acc], ap.phase, bars, pp.err) ? 1 : 0;
         epi_bar_sync();
@@ -845,6 +849,7 @@ __device__ __forceinline__ bool epilogue_job_swapped(const Pipe &pp, const GemmJ
         const uint32_t taddr = pp.tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ap.acc * pp.acc_stride);
         const int row0 = w.rel * j.rows_per_cta + tile * kBlockM;   // vocabulary row of TMEM lane 0
         const bool v_ok = row0 + vrow < row_end;
+        const float v_scale = j.fp8 && v_ok ? j.epi.col_scale[row0 + vrow] : 1.0f;
         for (int c = 0; c < nodes; c += 16) {
             float v[16];
             tmem_ld16(taddr + c, v);
@@ -856,7 +861,7 @@ __device__ __forceinline__ bool epilogue_job_swapped(const Pipe &pp, const GemmJ
             }
 #pragma unroll
             for (int i = 0; i < 16; ++i)
-                if (c + i < nodes) pp.tbuf[(c + i) * kTPitch + vrow] = v_ok ? v[i] : -INFINITY;
+                if (c + i < nodes) pp.tbuf[(c + i) * kTPitch + vrow] = v_ok ? v[i] * v_scale : -INFINITY;
         }
         tc_fence_before();
         epi_bar_sync();
@@ -867,11 +872,14 @@ __device__ __forceinline__ bool epilogue_job_swapped(const Pipe &pp, const GemmJ
             int valid = row_end - seg_row;
             valid = valid < 0 ? 0 : (valid > len ? len : valid);
             const float *col = pp.tbuf + node * kTPitch + seg * len;
-            if (topk <= 4) swap_scan_tile<4>(col, len, valid, seg_row + j.epi.idx_offset, topk, run);
-            else swap_scan_tile<SPEC_MAX_TOPK>(col, len, valid, seg_row + j.epi.idx_offset, topk, run);
+            if (topk <= 4) swap_scan_tile<4>(col, len, valid, seg_row + j.epi.idx_offset, topk, node_scale, run);
+            else swap_scan_tile<SPEC_MAX_TOPK>(col, len, valid, seg_row + j.epi.idx_offset, topk, node_scale, run);
         }
     }
     if (w.first >= w.end) return true;
+    run.m *= node_scale;
+#pragma unroll
+    for (int q = 0; q < SPEC_MAX_TOPK; ++q) run.tv[q] *= node_scale;
     // the P neighbouring lanes of a node fold their results (every lane of the warp takes part in the shuffles)
     for (int off = 1; off < P; off <<= 1) {
         float ov[SPEC_MAX_TOPK];

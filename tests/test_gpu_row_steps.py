@@ -111,14 +111,32 @@ def test_equal_rows_give_equal_logits_in_every_tile(B, d, rows):
 @pytest.mark.parametrize("B_,topk", [(37, (4, 2)), (18, (8, 1, 2)), (149, (1, 2)), (74, (2, 1)), (75, (2, 1))])
 def test_merge_and_mix_round_one_child_per_sm(B, B_, topk, d):
     """148 children and a few more or less (a level's merge and the next level's mix are one kernel up to one child per
-    SM), row widths round the two thread counts.  Every level is re-derived by the oracle from the GPU's parent level for
-    the first and the last sequence."""
-    K = int(np.prod(topk))
-    cfg = small_cfg(d_base=64, d_inner=d, V=600, topk=topk, K=K, B=B_, seed=B_ + d)
+    SM), row widths round the two thread counts."""
+    _check_every_level(B, small_cfg(d_base=64, d_inner=d, V=600, topk=topk, K=int(np.prod(topk)), B=B_, seed=B_ + d))
+
+
+@pytest.mark.parametrize("swap", [0, 128])
+@pytest.mark.parametrize("B_,topk,V,d", [(37, (4, 1), 600, 2048), (37, (4, 1), 600, 4096), (37, (4, 1), 600, 4112),
+                                         (75, (2, 1), 600, 512), (2, (4, 3, 2), 4805, 272), (1, (8, 1, 2), 19000, 1040),
+                                         (17, (1, 7), 37900, 128)])
+def test_e4m3_levels_with_and_without_swapped_operands(B, B_, topk, V, d, swap):
+    """Both operand orders of the e4m3 head, with one and several weight tiles per CTA and short last ones; children of a
+    re-scored level below, at and above one per SM and row widths round what one CTA covers."""
+    _check_every_level(B, small_cfg(d_base=64, d_inner=d, V=V, topk=topk, K=int(np.prod(topk)), B=B_, seed=B_ + d),
+                       e4m3=True, swap=swap)
+
+
+def _check_every_level(B, cfg, e4m3=False, swap=None):
+    """Every level is re-derived by the oracle from the GPU's parent level for the first and the last sequence."""
+    B_, topk, K, d = cfg.B, cfg.topk, cfg.K, cfg.d_inner
     sw = synth.make_weights(cfg)
     ow, gw = to_oracle_weights(sw), weights_to_cuda(sw)
     ctx, tok = synth.make_draft_inputs(cfg)
     h = B.spec_create(gw)
+    if e4m3:
+        B.spec_attach_fp8_heads(h)
+    if swap is not None:
+        B.spec_set_option(h, B.SPEC_OPT_HEAD_SWAP_MAX_ROWS, swap)
     ct, lp, ws = B.spec_draft(h, ctx.cuda(), tok.cuda(), topk, K)
     assert B.spec_poll_error(ws) == 0
     lay = B.spec_draft_layout(h, B_, topk, K)

@@ -63,19 +63,15 @@ struct RescoreArgs {
     int d, V;
 };
 
-// One CTA per row.
-__global__ void __launch_bounds__(kRescoreThreads) merge_rescore_kernel(RescoreArgs a) {
-    extern __shared__ LeafKey rescore_keys[];   // [Lpad] when the prune is folded in, else nothing
-    __shared__ Scratch sc;
-    __shared__ float exact[kShortList];
-    __shared__ int last_of_sequence;
-    griddep_launch();
-    griddep_wait();
-    const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+// Row r's children: the top-k of the exactly recomputed logits of its short list, written if `writer`.  Every warp finds
+// them all; the token of child `pick` is returned to every thread.  `exact`: shared, kShortList floats.
+__device__ __forceinline__ int rescore_row(const RescoreArgs &a, int r, int tid, Scratch *sc, float *exact, bool writer,
+                                           int pick) {
+    const int lane = tid & 31, warp = tid >> 5;
     const float base = (tid == 0 && a.merge.score_in) ? __ldcg(a.merge.score_in + r) : 0.0f;
     // short list: twice the branching factor plus two, at least 8, at most one per warp
     const int n_short = min(kShortList, max(8, 2 * a.merge.topk + 2));
-    const MergeOut o = merge_select<kRescoreThreads, 8, BlockSync>(a.merge, r, tid, &sc, n_short);
+    const MergeOut o = merge_select<kRescoreThreads, 8, BlockSync>(a.merge, r, tid, sc, n_short);
     const int short_id = o.id;   // lane j: the j-th short-listed token
     // exact logit of short-listed token `warp`: dot product of two bf16 rows, fp32 accumulation
     const int v = warp < n_short ? __shfl_sync(0xffffffffu, short_id, warp) : -1;
@@ -110,32 +106,61 @@ __global__ void __launch_bounds__(kRescoreThreads) merge_rescore_kernel(RescoreA
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
     if (lane == 0) exact[warp] = (v >= 0 && v < a.V) ? acc : -INFINITY;
     __syncthreads();
-    // warp 0: the top-k of the exact logits, (value desc, token id asc)
-    if (warp == 0) {
-        float val = lane < n_short ? exact[lane] : -INFINITY;
-        int id = lane < n_short ? short_id : 0x7fffffff;
-        const float lse = o.lse;
-        const int topk = a.merge.topk;
-        for (int j = 0; j < topk; ++j) {
-            const uint32_t key = float_key(val);
-            const uint32_t bk = __reduce_max_sync(0xffffffffu, key);
-            const uint32_t bi = __reduce_min_sync(0xffffffffu, key == bk ? (uint32_t)id : 0xffffffffu);
-            if (lane == 0) {
-                a.merge.tok_out[(size_t)r * topk + j] = (int)bi;
-                a.merge.score_out[(size_t)r * topk + j] = base + (key_float(bk) - lse);
-            }
-            if (a.merge.next_emb != nullptr && bi < (uint32_t)a.merge.next_emb_rows) {   // (see prefetch_embeddings)
-                const char *row = (const char *)a.merge.next_emb + (size_t)bi * a.merge.next_emb_bytes;
-                for (int i = lane * 128; i < a.merge.next_emb_bytes; i += 32 * 128)
-                    asm volatile("prefetch.global.L2 [%0];" ::"l"(row + i));
-            }
-            if (key == bk && (uint32_t)id == bi) {   // taken
-                val = -INFINITY;
-                id = 0x7fffffff;
-            }
+    // the top-k of the exact logits, (value desc, token id asc)
+    float val = lane < n_short ? exact[lane] : -INFINITY;
+    int id = lane < n_short ? short_id : 0x7fffffff;
+    const int topk = a.merge.topk;
+    int picked = -1;
+    for (int j = 0; j < topk; ++j) {
+        const uint32_t key = float_key(val);
+        const uint32_t bk = __reduce_max_sync(0xffffffffu, key);
+        const uint32_t bi = __reduce_min_sync(0xffffffffu, key == bk ? (uint32_t)id : 0xffffffffu);
+        if (j == pick) picked = (int)bi;
+        if (writer && tid == 0) {
+            a.merge.tok_out[(size_t)r * topk + j] = (int)bi;
+            a.merge.score_out[(size_t)r * topk + j] = base + (key_float(bk) - o.lse);
+        }
+        if (warp == 0 && a.merge.next_emb != nullptr && bi < (uint32_t)a.merge.next_emb_rows) {   // (see prefetch_embeddings)
+            const char *row = (const char *)a.merge.next_emb + (size_t)bi * a.merge.next_emb_bytes;
+            for (int i = lane * 128; i < a.merge.next_emb_bytes; i += 32 * 128)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(row + i));
+        }
+        if (key == bk && (uint32_t)id == bi) {   // taken
+            val = -INFINITY;
+            id = 0x7fffffff;
         }
     }
-    prune_if_last<kRescoreThreads, BlockSync>(a.merge, r, tid, rescore_keys, &last_of_sequence);
+    return picked;
+}
+
+// One CTA per row.
+__global__ void __launch_bounds__(kRescoreThreads) merge_rescore_kernel(RescoreArgs a) {
+    extern __shared__ LeafKey rescore_keys[];   // prune_smem_bytes when the prune is folded in, else nothing
+    __shared__ Scratch sc;
+    __shared__ float exact[kShortList];
+    __shared__ int last_of_sequence;
+    griddep_launch();
+    griddep_wait();
+    rescore_row(a, blockIdx.x, threadIdx.x, &sc, exact, true, -1);
+    prune_if_last<kRescoreThreads, BlockSync>(a.merge, blockIdx.x, threadIdx.x, rescore_keys, &last_of_sequence);
+}
+
+// One CTA per child, up to one per SM: re-scores its parent's short list (the siblings find the weight rows in L2) and
+// computes the child's state, as merge_mix_child_kernel does for bf16 heads.  One launch, one barrier between grids and one
+// round trip of the token through memory less per level: the 13B step with e4m3 heads 243 -> 240 us, two levels of 60
+// nodes 88.3 -> 87.2, 16 sequences times 8 nodes 96.1 -> 94.3.  More children than SMs would take turns on them.
+struct RescoreMixArgs {
+    RescoreArgs rescore;
+    MixArgs mix;
+};
+__global__ void __maxnreg__(72) rescore_mix_child_kernel(RescoreMixArgs a) {
+    __shared__ Scratch sc;
+    __shared__ float exact[kShortList], red[2 * kMaxGroupWarps];
+    griddep_launch();
+    griddep_wait();
+    const int c = blockIdx.x, topk = a.rescore.merge.topk, r = c / topk;
+    const int t = rescore_row(a.rescore, r, threadIdx.x, &sc, exact, c == r * topk, c - r * topk);
+    mix_ln_gelu_row<kRescoreThreads, 1, 1, BlockSync>(a.mix, c, r, t, threadIdx.x, red);
 }
 
 }  // namespace
@@ -156,6 +181,21 @@ int launch_merge_rescore(const MergeArgs &g, const void *W, const void *S, int r
     a.V = V;
     const size_t smem = g.seq_done ? prune_smem_bytes(g.L, g.Lpad) : 0;
     SPEC_CUDA_TRY(launch_pdl(merge_rescore_kernel, dim3(rows), dim3(kRescoreThreads), smem, st, a));
+    return SPEC_OK;
+}
+
+int launch_rescore_mix(const MergeArgs &g, const void *W, const void *S, const MixArgs &m, int rows, int d, int V,
+                       cudaStream_t st) {
+    if (m.d > 8 * kRescoreThreads || rows * g.topk > num_sms() || g.seq_done != nullptr) return SPEC_ERR_SHAPE;
+    RescoreMixArgs a{};
+    a.rescore.merge = g;
+    a.rescore.merge.next_emb = nullptr;   // the gather follows in the same CTA
+    a.rescore.W = (const uint16_t *)W;
+    a.rescore.S = (const uint16_t *)S;
+    a.rescore.d = d;
+    a.rescore.V = V;
+    a.mix = m;
+    SPEC_CUDA_TRY(launch_pdl(rescore_mix_child_kernel, dim3(rows * g.topk), dim3(kRescoreThreads), 0, st, a));
     return SPEC_OK;
 }
 

@@ -650,7 +650,12 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
         if (fp8) {
             // short list by approximate logit, exact re-scoring from the bf16 weights, then the children
             g.list_len = SPEC_MAX_TOPK;
-            rc = launch_merge_rescore(g, w.head[l], S, rows, w.d_inner, w.V, st);
+            rc = SPEC_ERR_SHAPE;
+            if (proj_done) {
+                rc = launch_rescore_mix(g, w.head[l], S, mix_args(l + 1), rows, w.d_inner, w.V, st);
+                mix_done = rc == SPEC_OK;
+            }
+            if (rc == SPEC_ERR_SHAPE) rc = launch_merge_rescore(g, w.head[l], S, rows, w.d_inner, w.V, st);
         } else {
             rc = SPEC_ERR_SHAPE;
             if (proj_done) {

@@ -197,6 +197,9 @@ struct MergeArgs {
 int launch_quantize_rows(const void *X, int rows, int d, void *Q, float *scale, cudaStream_t st);
 // merge of approximate partial lists + exact re-scoring of the short list + expansion (fp8_kernels.cu)
 int launch_merge_rescore(const MergeArgs &g, const void *W, const void *S, int rows, int d, int V, cudaStream_t st);
+// the same with the children's states; SPEC_ERR_SHAPE: shape not covered, launch the two separately
+int launch_rescore_mix(const MergeArgs &g, const void *W, const void *S, const MixArgs &m, int rows, int d, int V,
+                       cudaStream_t st);
 
 int launch_draft_init(int32_t *hdr, int words, cudaStream_t st);
 int launch_mix_ln_gelu(const MixArgs &m, int rows, cudaStream_t st);

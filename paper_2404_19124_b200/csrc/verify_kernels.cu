@@ -95,6 +95,25 @@ struct Elem {
     }
 };
 
+// The n vectors at `src`, the first of which is element col0 of its row, read by `kGroup` threads of which this is number t.
+template <bool kBf16, int kGroup>
+__device__ __forceinline__ void scan_vectors(const uint4 *src, int n, int col0, int t, float &best, int &idx) {
+    for (int i = t; i < n; i += kGroup * kStreamUnroll) {
+        uint4 v[kStreamUnroll];
+#pragma unroll
+        for (int u = 0; u < kStreamUnroll; ++u)
+            if (i + kGroup * u < n) v[u] = ld_stream(src + i + kGroup * u);
+#pragma unroll
+        for (int u = 0; u < kStreamUnroll; ++u) {
+            if (i + kGroup * u < n) {
+                const int col = col0 + (i + kGroup * u) * Elem<kBf16>::kEpv;
+                if (kBf16) consume_bf16(v[u], col, best, idx);
+                else consume_f32(v[u], col, best, idx);
+            }
+        }
+    }
+}
+
 // The part of a row (elements [rs, re) of the run of vectors at `base`) that lies in vectors [a, e), read by `kGroup`
 // threads of which this is number `t`: the thread's maximum and its first index within the row.
 template <bool kBf16, int kGroup>
@@ -112,22 +131,7 @@ __device__ __forceinline__ void scan_row(const char *base, long long rs, long lo
     }
     const long long p = max(body0, a), q = min(body1, e);
     if (q > p) {
-        const uint4 *src = (const uint4 *)base + p;
-        const int n = (int)(q - p), col0 = (int)((p << E::kShift) - rs);
-        for (int i = t; i < n; i += kGroup * kStreamUnroll) {
-            uint4 v[kStreamUnroll];
-#pragma unroll
-            for (int u = 0; u < kStreamUnroll; ++u)
-                if (i + kGroup * u < n) v[u] = ld_stream(src + i + kGroup * u);
-#pragma unroll
-            for (int u = 0; u < kStreamUnroll; ++u) {
-                if (i + kGroup * u < n) {
-                    const int col = col0 + (i + kGroup * u) * E::kEpv;
-                    if (kBf16) consume_bf16(v[u], col, best, idx);
-                    else consume_f32(v[u], col, best, idx);
-                }
-            }
-        }
+        scan_vectors<kBf16, kGroup>((const uint4 *)base + p, (int)(q - p), (int)((p << E::kShift) - rs), t, best, idx);
     }
     if (body1 >= body0 && body1 >= a && body1 < e && (re & (E::kEpv - 1)) != 0) {   // ... and ends inside another
         const long long i = (body1 << E::kShift) + t;
@@ -318,55 +322,74 @@ verify_seq_kernel(const char *__restrict__ base, int skew, const int32_t *cand_t
 
 // ---- early-exit form ------------------------------------------------------------------------------
 // The rows of a candidate matter only up to its first mismatch (Sec. 1: the tokens after a rejected
-// one are discarded), so reading them is optional work: one CTA per candidate walks its rows in order,
-// takes the arg-max of a row with the whole CTA (eight 128-bit loads in flight per thread) and stops
+// one are discarded), so reading them is optional work: one CTA or a cluster of them per candidate walks its rows in order,
+// takes the arg-max of a row together (a contiguous part each, eight 128-bit loads in flight per thread) and stops
 // after the first row whose arg-max differs from the speculated token.  Bytes read fall from
 // B K (n+1) V to sum over candidates of (m + 1) V elements; rows that were not read get g = -1.
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+constexpr int kMaxEarlyCtas = 8;
+
 template <bool kBf16>
 __global__ void __launch_bounds__(kArgmaxThreads)
-verify_early_kernel(const char *__restrict__ base, const int32_t *cand_tok, int n, int V, int32_t *g,
+verify_early_kernel(const char *__restrict__ base, const int32_t *cand_tok, int n, int V, int ctas, int32_t *g,
                     int32_t *match_len) {
-    __shared__ float s_val[kWarpsPerBlock];
-    __shared__ int s_idx[kWarpsPerBlock];
-    __shared__ int s_arg;
+    // One barrier per row: every warp hands its key to every CTA of the cluster, in one of two sets of slots by turns (a set
+    // is written again only after the next row's barrier, when all its readers have arrived).
+    __shared__ unsigned long long keys[2][kMaxEarlyCtas * kWarpsPerBlock];
+    using E = Elem<kBf16>;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = ctas > 1 ? (int)cluster_rank() : 0, c = blockIdx.x / ctas, slots = ctas * kWarpsPerBlock;
     griddep_launch();
+    if (ctas > 1) cluster_barrier();   // the other CTAs' shared memory is there
     griddep_wait();
-    const int c = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int row_vec = V >> E::kShift, per = (row_vec + ctas - 1) / ctas;   // a row is a run of whole vectors
+    const int first = rank * per, count = min(row_vec - first, per);
     int m = n, j = 0;
     for (; j <= n; ++j) {
-        const long long rs = ((long long)c * (n + 1) + j) * V;
+        const long long row = (long long)c * (n + 1) + j;
+        const int tok = j < n ? __ldcg(cand_tok + (size_t)c * n + j) : -1;
         float best = -INFINITY;
         int idx = kIdxNone;
-        scan_row<kBf16, kArgmaxThreads>(base, rs, rs + V, 0, 1ll << 62, tid, best, idx);
+        scan_vectors<kBf16, kArgmaxThreads>((const uint4 *)base + row * row_vec + first, count, first * E::kEpv, tid, best, idx);
         warp_argmax(best, idx);
-        if (lane == 0) {
-            s_val[warp] = best;
-            s_idx[warp] = idx;
-        }
-        __syncthreads();
-        if (tid == 0) {
-            float bv = -INFINITY;
-            int arg = 0;   // a row without any value above -inf (all NaN) yields 0
-            int bi = kIdxNone;
-            for (int w = 0; w < kWarpsPerBlock; ++w) {
-                if (s_val[w] > bv || (s_val[w] == bv && s_idx[w] < bi)) {   // the lowest index among equal maxima
-                    bv = s_val[w];
-                    bi = s_idx[w];
-                }
+        unsigned long long *set = keys[j & 1];
+        if (lane < ctas) {
+            const unsigned long long key = argmax_key(best, idx);
+            if (ctas > 1) {
+                uint32_t there;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                             : "=r"(there)
+                             : "r"((uint32_t)__cvta_generic_to_shared(set + rank * kWarpsPerBlock + warp)), "r"(lane));
+                asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(there), "l"(key) : "memory");
+            } else {
+                set[warp] = key;
             }
-            if (bi != kIdxNone && bv > -INFINITY) arg = bi;
-            s_arg = arg;
-            g[(size_t)c * (n + 1) + j] = arg;
         }
-        __syncthreads();
-        const int arg = s_arg;
-        if (j < n && __ldcg(cand_tok + (size_t)c * n + j) != arg) {   // uniform over the CTA
+        if (ctas > 1) cluster_barrier();
+        else __syncthreads();
+        unsigned long long k = lane < slots ? set[lane] : 0ull;
+        if (slots > 32) k = max(k, set[lane + 32 < slots ? lane + 32 : lane]);
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) k = max(k, __shfl_xor_sync(0xffffffffu, k, off));
+        const int arg = k == 0ull ? 0 : (int)~(uint32_t)k;   // a row without any value above -inf (all NaN) yields 0
+        if (rank == 0 && tid == 0) g[row] = arg;
+        if (j < n && tok != arg) {   // uniform over the cluster
             m = j;
             break;
         }
     }
-    for (int jj = j + 1 + tid; jj <= n; jj += kArgmaxThreads) g[(size_t)c * (n + 1) + jj] = -1;
-    if (tid == 0) match_len[c] = m;
+    if (rank == 0) {
+        for (int jj = j + 1 + tid; jj <= n; jj += kArgmaxThreads) g[(size_t)c * (n + 1) + jj] = -1;
+        if (tid == 0) match_len[c] = m;
+    }
 }
 
 // One CTA per sequence: the candidate with the longest match (lowest index among equals) and its bonus token.
@@ -455,6 +478,20 @@ int launch_verify(const int32_t *cand_tok, const void *base_logits, int dtype, i
     return SPEC_OK;
 }
 
+// CTAs per candidate of the early-exit form: as many as the GPU holds at once (four per SM), up to eight, and no more than
+// leave each of them three 16-byte vectors per thread of a row.  One CTA reads a row at 30 GB/s, whatever else the GPU does.
+// us per call for 1 / 2 / 4 / 8 CTAs, bf16, match lengths uniform: V 128256, 8 candidates 43.2 / 27.8 / 18.9 / 14.0,
+// 128 candidates 57.2 / 43.2 / 32.8 / 36.4, 256 candidates 56.4 / 42.1 / 44.1 / 51.5, 512 candidates 66.4 / 68.4 / 71.3 / 90.7
+// (50 for the bytes; 69.2 with two barriers per row), 2048 candidates of two rows 120.0 / 127.0 / 153.5 / 215.7 (118.6 with
+// two barriers); V 32000, 32 candidates 18.6 / 15.3 / 14.0 / 13.8; V 8000, 128 candidates 9.6 / 11.7 / 12.5 / 19.3.
+int early_ctas(int candidates, int row_vec) {
+    int ctas = 1;
+    while (2 * ctas <= kMaxEarlyCtas && (long long)candidates * 2 * ctas <= 4ll * num_sms() &&
+           row_vec >= 3 * kArgmaxThreads * 2 * ctas)
+        ctas *= 2;
+    return ctas;
+}
+
 // Early-exit form; returns SPEC_ERR_SHAPE when the rows are not whole 16-byte vectors (the caller then
 // uses the streaming form).
 int launch_verify_early(const int32_t *cand_tok, const void *base_logits, int dtype, int B, int K, int n, int V,
@@ -466,8 +503,10 @@ int launch_verify_early(const int32_t *cand_tok, const void *base_logits, int dt
     int32_t *err = (int32_t *)w;
     int32_t *g = (int32_t *)(w + plan.off_g);
     int32_t *match_len = (int32_t *)(w + plan.off_part);   // B * K words; the partial maxima's area is not used here
-    SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_early_kernel<true> : verify_early_kernel<false>, dim3(B * K), dim3(kArgmaxThreads), 0,
-                             st, (const char *)base_logits, cand_tok, n, V, g, match_len));
+    const int ctas = early_ctas(B * K, V / (bf16 ? 8 : 4));
+    SPEC_CUDA_TRY(launch_pdl_cluster(bf16 ? verify_early_kernel<true> : verify_early_kernel<false>, dim3(B * K * ctas),
+                                     dim3(kArgmaxThreads), 0, ctas, st, (const char *)base_logits, cand_tok, n, V, ctas, g,
+                                     match_len));
     SPEC_CUDA_TRY(launch_pdl(verify_accept_early_kernel, dim3(B), dim3(128), 0, st, (const int32_t *)g,
                              (const int32_t *)match_len, K, n, accept_len, best_cand, next_tok, err));
     return SPEC_OK;

@@ -71,3 +71,37 @@ def test_every_alignment_of_the_base(B, V, dtype):
         buf[:off] = 50.0                                  # what lies before and behind the tensor must not be seen
         buf[off + size:] = 50.0
         _check(B, cand, buf[off:off + size].view(Bn, K, n + 1, V))
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("Bn,K,n,vectors", [(1, 2, 3, 6143), (1, 2, 3, 6144), (1, 3, 1, 6145), (2, 37, 2, 6150),
+                                            (3, 25, 2, 6151), (4, 37, 1, 3073), (149, 1, 1, 3073), (16, 37, 1, 1535),
+                                            (16, 37, 1, 1536), (593, 1, 1, 1536), (1, 1, 9, 1537), (7, 3, 3, 1)])
+def test_early_exit_rows_shared_by_the_ctas_of_a_cluster(B, Bn, K, n, vectors, dtype):
+    """Row lengths and candidate counts at which 1, 2, 4 and 8 CTAs share a candidate, the maxima at the ends of the parts
+    and, for every third row, an equal one in a later part (the first must win)."""
+    V = vectors * (8 if dtype == torch.bfloat16 else 4)
+    g = torch.Generator().manual_seed(V + Bn)
+    x = torch.randn(Bn, K, n + 1, V, generator=g, dtype=torch.float32).to(dtype)
+    rows = x.view(-1, V)
+    for r in range(rows.shape[0]):
+        parts = 1 << r % 4
+        end = min(V, -(-vectors // parts) * (V // vectors) * (1 + r // 4 % parts))
+        p = (end - 1, end % V)[r % 2]
+        rows[r, p] = 9.0
+        if r % 3 == 0:
+            rows[r, p + (V - 1 - p) // 2] = 9.0
+    cand = torch.randint(0, V, (Bn, K, n), generator=g, dtype=torch.int64).to(torch.int32)
+    am = x.float().argmax(-1)
+    for k in range(Bn * K):
+        m = k % (n + 1)
+        cand.view(-1, n)[k, :m] = am.view(-1, n + 1)[k, :m].to(torch.int32)
+    host = synth.bf16_bits(x) if dtype == torch.bfloat16 else x.numpy()
+    o = oracle.verify(cand.numpy(), host, oracle.BF16 if dtype == torch.bfloat16 else oracle.F32, want_g=True)
+    acc, best, nxt, ws = B.spec_verify(cand.cuda(), x.cuda(), early_exit=True)
+    assert B.spec_poll_error(ws) == 0
+    for got, want in zip((acc, best, nxt), o):
+        assert np.array_equal(got.cpu().numpy(), want)
+    got = ws_view(ws, 256, Bn * K * (n + 1), torch.int32).cpu().numpy().reshape(Bn, K, n + 1)
+    read = np.cumprod(np.concatenate([np.ones((Bn, K, 1), bool), cand.numpy() == o[3][:, :, :n]], 2), 2) > 0
+    assert np.array_equal(got, np.where(read, o[3], -1))

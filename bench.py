@@ -758,8 +758,11 @@ def main():
                              f"{t_d + t_v:.1f} s of oracle time; `draft` and `verify` are the two parts timed apart, `value` both"}
 
     # per step: level-0 projection (clears the header), then per level mix, head GEMM (the next level's
-    # projection rides in the same launch) and merge (the last one also prunes); verify = streaming arg-max + accept
-    launches_per_step = 1 + 3 * n + 2
+    # projection rides in the same launch) and merge (the last one also prunes), merge and next mix in one kernel for
+    # levels with at most one child per SM or two per node; verify = streaming arg-max + accept
+    sms = torch.cuda.get_device_properties(dev).multi_processor_count
+    fused = sum(cfg.nodes(l + 1) <= sms or cfg.topk[l] <= 2 for l in range(n - 1))
+    launches_per_step = 1 + 3 * n - fused + 2
     out = {
         "metric": METRIC, "value": shard.whole_job_rate(Bn, world, ms_step * 1e-3), "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",

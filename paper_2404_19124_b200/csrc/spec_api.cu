@@ -65,6 +65,7 @@ struct DraftPlan {
     bool swapped[SPEC_MAX_HEADS];      // the level's head runs with the operands swapped (few nodes: weight stream)
     bool paired[SPEC_MAX_HEADS];       // the level's head runs on CTA pairs (more than 128 nodes: tensor-bound)
     size_t seq_done;                   // byte offset of the per-sequence counters of the folded prune
+    bool small;                        // the whole draft is one kernel
     int header_words;                  // int32 words cleared at the start of a draft
     size_t xchg;                       // vocabulary-parallel heads: byte offset of the rank slots
     size_t slot_bytes[SPEC_MAX_HEADS]; // bytes of one rank's slot at each level
@@ -205,6 +206,10 @@ int make_draft_plan(const spec_handle_s *h, int B, const int32_t *topk, int K, D
         if (p->N[l] > max_rows) max_rows = p->N[l];
         p->proj_block_n[l] = proj_block_n_for(h, parent_rows);
     }
+    // (options that choose between forms of the kernel chain ask for the chain)
+    p->small = h->gemm_impl == 0 && !h->profile && h->head_block_n == 0 && h->proj_block_n == 0 && h->swap_max_rows < 0 &&
+               h->head_pair < 0 && h->vp_ranks == 1 && max_fp8_rows == 0 && small_draft_fits(w, B, topk);
+    if (p->small && small_draft_proj_floats(w) > max_proj_floats) max_proj_floats = small_draft_proj_floats(w);
     y.proj = off;
     off = align_up(off + sizeof(float) * max_proj_floats, kWsAlign);
     y.state8 = off;
@@ -567,6 +572,19 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
         return mx;
     };
     const PruneArgs pa = make_prune_args(p, ws, topk);
+    if (p.small) {
+        MixArgs mixes[SPEC_MAX_HEADS];
+        int32_t *toks[SPEC_MAX_HEADS + 1] = {};
+        float *scores[SPEC_MAX_HEADS + 1] = {};
+        for (int l = 0; l < p.n; ++l) {
+            mixes[l] = mix_args(l);
+            toks[l + 1] = (int32_t *)(ws + p.lay.tok[l + 1]);
+            scores[l + 1] = (float *)(ws + p.lay.score[l + 1]);
+        }
+        rc = launch_draft_small(w, ctx_state, B, topk, K, mixes, toks, scores, P, err, p.header_words, pa, p.L, cand_tok,
+                                cand_logp, st);
+        if (rc != SPEC_ERR_SHAPE) return rc;
+    }
     const bool fold_prune = !h->profile;
     bool proj_done = false;   // the projection of the level about to start ran with the previous head
     bool mix_done = false;    // the states of the level about to start were written by the previous level's merge

@@ -38,8 +38,8 @@ UNIT = "sequences/s"
 DEFAULT_STEPS, DEFAULT_WARMUP = 2000, 50
 
 NCU_TRAFFIC_BYTES = {
-    ("llama2-13b", "head_gemm_384_rows"): 279.2e6,     # profiles/gemm_tc_kernel_head_llama2-13b.md
-    ("llama2-13b", "verify_stream"): 134.9e6,          # profiles/verify_stream_kernel_llama2-13b.md
+    ("llama2-13b", "head_gemm_384_rows"): 274.6e6,     # profiles/gemm_tc_kernel_head_llama2-13b.md
+    ("llama2-13b", "verify_stream"): 135.2e6,          # profiles/verify_stream_kernel_llama2-13b.md
 }
 
 
@@ -762,7 +762,9 @@ def main():
     # levels with at most one child per SM or two per node; verify = streaming arg-max + accept
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     fused = sum(cfg.nodes(l + 1) <= sms or cfg.topk[l] <= 2 for l in range(n - 1))
-    launches_per_step = 1 + 3 * n - fused + 2
+    small = cfg.d_inner <= 512 and cfg.d_base <= 2048 and all(cfg.nodes(l) <= 16 for l in range(n)) and \
+        sum(V * cfg.d_inner * (16 + cfg.nodes(l)) for l in range(n)) <= n * (23 << 20)      # the whole draft is one kernel
+    launches_per_step = (1 if small else 1 + 3 * n - fused) + 2
     out = {
         "metric": METRIC, "value": shard.whole_job_rate(Bn, world, ms_step * 1e-3), "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",

@@ -169,9 +169,11 @@ __global__ void __maxnreg__(72) merge_mix_512_kernel(MergeMixArgs a) {
 template <int kThreads, int kLen>
 __device__ __forceinline__ void merge_mix_child(const MergeMixArgs &a, Scratch *sc, float *red) {
     const int c = blockIdx.x, topk = a.merge.topk, r = c / topk, tid = threadIdx.x;
-    const MergeOut o = merge_expand_row<kThreads, kLen, BlockSync>(a.merge, r, tid, sc, c == r * topk);
+    float pre[1][8];
+    const MergeOut o = merge_expand_row<kThreads, kLen, BlockSync>(a.merge, r, tid, sc, c == r * topk,
+                                                                   [&] { parent_state<kThreads>(a.mix, r, tid, pre); });
     const int t = __shfl_sync(0xffffffffu, o.id, c - r * topk);
-    mix_ln_gelu_row<kThreads, 1, 1, BlockSync>(a.mix, c, r, t, tid, red);
+    mix_ln_gelu_row<kThreads, 1, 1, BlockSync>(a.mix, c, r, t, tid, red, pre);
 }
 template <int kLen>
 __global__ void __launch_bounds__(kRowThreads, 2) merge_mix_child_kernel(MergeMixArgs a) {

@@ -64,14 +64,16 @@ struct RescoreArgs {
 };
 
 // Row r's children: the top-k of the exactly recomputed logits of its short list, written if `writer`.  Every warp finds
-// them all; the token of child `pick` is returned to every thread.  `exact`: shared, kShortList floats.
+// them all; the token of child `pick` is returned to every thread.  `exact`: shared, kShortList floats.  `meanwhile`: see
+// merge_select.
+template <typename Meanwhile = Nothing>
 __device__ __forceinline__ int rescore_row(const RescoreArgs &a, int r, int tid, Scratch *sc, float *exact, bool writer,
-                                           int pick) {
+                                           int pick, Meanwhile meanwhile = Meanwhile()) {
     const int lane = tid & 31, warp = tid >> 5;
     const float base = (tid == 0 && a.merge.score_in) ? __ldcg(a.merge.score_in + r) : 0.0f;
     // short list: twice the branching factor plus two, at least 8, at most one per warp
     const int n_short = min(kShortList, max(8, 2 * a.merge.topk + 2));
-    const MergeOut o = merge_select<kRescoreThreads, 8, BlockSync>(a.merge, r, tid, sc, n_short);
+    const MergeOut o = merge_select<kRescoreThreads, 8, BlockSync>(a.merge, r, tid, sc, n_short, meanwhile);
     const int short_id = o.id;   // lane j: the j-th short-listed token
     // exact logit of short-listed token `warp`: dot product of two bf16 rows, fp32 accumulation
     const int v = warp < n_short ? __shfl_sync(0xffffffffu, short_id, warp) : -1;
@@ -159,8 +161,10 @@ __global__ void __maxnreg__(72) rescore_mix_child_kernel(RescoreMixArgs a) {
     griddep_launch();
     griddep_wait();
     const int c = blockIdx.x, topk = a.rescore.merge.topk, r = c / topk;
-    const int t = rescore_row(a.rescore, r, threadIdx.x, &sc, exact, c == r * topk, c - r * topk);
-    mix_ln_gelu_row<kRescoreThreads, 1, 1, BlockSync>(a.mix, c, r, t, threadIdx.x, red);
+    float pre[1][8];
+    const int t = rescore_row(a.rescore, r, threadIdx.x, &sc, exact, c == r * topk, c - r * topk,
+                              [&] { parent_state<kRescoreThreads>(a.mix, r, threadIdx.x, pre); });
+    mix_ln_gelu_row<kRescoreThreads, 1, 1, BlockSync>(a.mix, c, r, t, threadIdx.x, red, pre);
 }
 
 }  // namespace

@@ -70,13 +70,43 @@ static __device__ __noinline__ float4 gelu_erf4(float4 y) {
     return make_float4(gelu_erf(y.x), gelu_erf(y.y), gelu_erf(y.z), gelu_erf(y.w));
 }
 
+// The projected parent state (the sum of its partials, added in ascending order) of the groups that thread `tid` owns in
+// mix_ln_gelu_row with one group per thread.
+template <int kThreads>
+__device__ __forceinline__ void parent_state(const MixArgs &m, int parent, int tid, float (&pre)[1][8]) {
+    const int i = tid * 8;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) pre[0][j] = 0.0f;
+    if (i >= m.d) return;
+    const float *p = m.P + (size_t)parent * m.d + i;
+    for (int s0 = 0; s0 < m.p_splits; s0 += 4) {
+        float4 a[4], b[4];
+#pragma unroll
+        for (int sp = 0; sp < 4; ++sp) {
+            a[sp] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            b[sp] = a[sp];
+            if (s0 + sp < m.p_splits) {
+                a[sp] = __ldcg((const float4 *)(p + (s0 + sp) * m.p_split_stride));
+                b[sp] = __ldcg((const float4 *)(p + (s0 + sp) * m.p_split_stride + 4));
+            }
+        }
+#pragma unroll
+        for (int sp = 0; sp < 4; ++sp) {
+            pre[0][0] += a[sp].x; pre[0][1] += a[sp].y; pre[0][2] += a[sp].z; pre[0][3] += a[sp].w;
+            pre[0][4] += b[sp].x; pre[0][5] += b[sp].y; pre[0][6] += b[sp].z; pre[0][7] += b[sp].w;
+        }
+    }
+}
+
 // Node r of the level, whose token is t and whose projected parent state is row `parent` of P.
 // h = a * P[parent] + b * E[t].  The row lives in registers: thread t owns the 8-element groups
 // t, t + kThreads, ... (kIters of them; d <= 8 * kThreads * kIters, d % 8 == 0; kThreads 0: as many as the CTA has).
 // kDepth of those groups, and kSp partial projections of each, have their loads in flight together (registers against
 // latency).
+// `pre`: the projected parent state of this thread's groups (parent_state), if the caller has it already.
 template <int kThreads, int kIters, int kDepth, typename Sync, int kSp = 4>
-__device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int parent, int t, int tid, float *red) {
+__device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int parent, int t, int tid, float *red,
+                                                const float (*pre)[8] = nullptr) {
     constexpr int kGroup = kIters >= 8 ? 1 : (kIters < kDepth ? kIters : kDepth);
     bool tok_ok = false;
     const int nt = kThreads > 0 ? kThreads : (int)blockDim.x;
@@ -98,7 +128,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
             for (int sp = 0; sp < kSp; ++sp) {
                 pa[q][sp] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
                 pb[q][sp] = pa[q][sp];
-                if (i < d && sp < m.p_splits) {
+                if (pre == nullptr && i < d && sp < m.p_splits) {
                     pa[q][sp] = __ldcg((const float4 *)(p + sp * m.p_split_stride + i));
                     pb[q][sp] = __ldcg((const float4 *)(p + sp * m.p_split_stride + i + 4));
                 }
@@ -125,7 +155,10 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
                 pv[0] += pa[q][sp].x; pv[1] += pa[q][sp].y; pv[2] += pa[q][sp].z; pv[3] += pa[q][sp].w;
                 pv[4] += pb[q][sp].x; pv[5] += pb[q][sp].y; pv[6] += pb[q][sp].z; pv[7] += pb[q][sp].w;
             }
-            if (i < d) {
+            if (pre != nullptr) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) pv[j] = pre[it][j];
+            } else if (i < d) {
                 for (int sp = kSp; sp < m.p_splits; ++sp) {   // more partials than one batch holds (rare)
                     const float4 p0 = __ldcg((const float4 *)(p + sp * m.p_split_stride + i));
                     const float4 p1 = __ldcg((const float4 *)(p + sp * m.p_split_stride + i + 4));
@@ -282,8 +315,13 @@ struct MergeOut {
 // no second barrier is needed.  143 lists of a 16-row level: 5.2 us for the whole kernel with a running list of eight
 // folded per thread and block-wide rounds (three times the code), 3.6 now; the last level with its prune 10.4 -> 7.1 (7B
 // shape), 13.5 -> 9.3 (13B).
-template <int kThreads, int kLen, typename Sync>
-__device__ __forceinline__ MergeOut merge_select(const MergeArgs &g, int r, int tid, Scratch *sc, int rounds) {
+// `meanwhile` runs while the first lists are in flight.
+struct Nothing {
+    __device__ __forceinline__ void operator()() const {}
+};
+template <int kThreads, int kLen, typename Sync, typename Meanwhile = Nothing>
+__device__ __forceinline__ MergeOut merge_select(const MergeArgs &g, int r, int tid, Scratch *sc, int rounds,
+                                                 Meanwhile meanwhile = Meanwhile()) {
     constexpr int kWarps = kThreads / 32;
     static_assert(kWarps <= kMaxGroupWarps, "scratch arrays");
     const int lane = tid & 31, warp = tid >> 5;
@@ -295,6 +333,7 @@ __device__ __forceinline__ MergeOut merge_select(const MergeArgs &g, int r, int 
     float m = -INFINITY, s = 0.0f;
     TileList<kLen> next;
     load_list(next, g, first + tid, tid < n_tiles);
+    meanwhile();
     for (int t0 = warp * 32; t0 < n_tiles; t0 += kThreads) {   // (uniform over the warp)
         const TileList<kLen> cur = next;
         const bool valid = t0 + lane < n_tiles;
@@ -406,10 +445,11 @@ __device__ __forceinline__ void prefetch_embeddings(const MergeArgs &g, const Me
 }
 
 // The row's top-k tokens and log-probabilities become its children.  `writer` = false: another CTA writes them.
-template <int kThreads, int kLen, typename Sync>
-__device__ __forceinline__ MergeOut merge_expand_row(const MergeArgs &g, int r, int tid, Scratch *sc, bool writer = true) {
+template <int kThreads, int kLen, typename Sync, typename Meanwhile = Nothing>
+__device__ __forceinline__ MergeOut merge_expand_row(const MergeArgs &g, int r, int tid, Scratch *sc, bool writer = true,
+                                                     Meanwhile meanwhile = Meanwhile()) {
     const float base = (tid < g.topk && g.score_in && !g.lse_out) ? __ldcg(g.score_in + r) : 0.0f;   // in flight during the merge
-    const MergeOut o = merge_select<kThreads, kLen, Sync>(g, r, tid, sc, g.topk);
+    const MergeOut o = merge_select<kThreads, kLen, Sync>(g, r, tid, sc, g.topk, meanwhile);
     if (writer && tid < g.topk) {
         g.tok_out[(size_t)r * g.topk + tid] = o.id;
         g.score_out[(size_t)r * g.topk + tid] = g.lse_out ? o.val : base + (o.val - o.lse);

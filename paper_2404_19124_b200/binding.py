@@ -103,7 +103,6 @@ _lib.spec_head_partials.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.
 _lib.spec_head_topk.argtypes = [C.c_void_p, C.c_int, C.c_void_p, C.c_int, C.c_int, C.c_void_p, C.c_void_p,
                                 C.c_void_p, C.c_size_t, C.c_void_p]
 
-
 class SpecError(RuntimeError):
     def __init__(self, status: int, where: str):
         msg = _lib.spec_status_str(status).decode()
@@ -120,13 +119,28 @@ def _check(status: int, where: str) -> None:
 # The calls of a decoding step take a few microseconds of GPU time at small shapes, so what marshalling costs is visible:
 # addresses go to ctypes as plain integers, the raw stream is asked for without building a Stream object (0.3 instead of
 # 3.2 us), the current device is switched only when it has to be (2.5 us).  Host time of one step of the smallest
-# shape: 66 -> 41 us, of spec_verify 19 -> 12.5, spec_next_ctx 14.5 -> 7.5, spec_draft 34 -> 26.
+# shape: 66 -> 41 us, of spec_verify 19 -> 12.5, spec_next_ctx 14.5 -> 7.5, spec_draft 34 -> 26 (with fewer kernels and
+through csrc/pycall.c now: spec_verify 4.7, spec_draft 5.4, a 7B step 34).
 def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 
 
 _current_device = getattr(torch._C, "_cuda_getDevice", None)
 _current_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+# The calls of a decoding step with every tensor given are marshalled in C (csrc/pycall.c).  Without that module, or where it
+# answers None, the Python code below does the same, with checks that say what is wrong.
+try:
+    from . import _pycall
+except ImportError:
+    _pycall = None
+if _current_device is None or _current_raw_stream is None:
+    _pycall = None
+if _pycall is not None:
+    _pycall.bind(*(C.cast(f, C.c_void_p).value for f in (_lib.spec_verify, _lib.spec_verify_early, _lib.spec_next_ctx,
+                                                         _lib.spec_draft)),
+                 torch.int32, torch.bfloat16, torch.float32, _current_device, _current_raw_stream)
 
 
 def _stream_ptr(stream: Optional[torch.cuda.Stream]):
@@ -250,6 +264,13 @@ def spec_draft(h: SpecHandle, ctx_state: torch.Tensor, last_tok: torch.Tensor, t
                cand_tok: Optional[torch.Tensor] = None, cand_logp: Optional[torch.Tensor] = None,
                workspace: Optional[torch.Tensor] = None, stream: Optional[torch.cuda.Stream] = None):
     """Enqueues one draft; returns (cand_tok [B,K,n] int32, cand_logp [B,K] fp32, workspace)."""
+    if _pycall is not None and cand_tok is not None and cand_logp is not None and workspace is not None:
+        status = _pycall.draft(h._h.value, h.n_heads, h.d_base, ctx_state, last_tok, topk, K, cand_tok, cand_logp, workspace,
+                               stream)
+        if status is not None:
+            if status != SPEC_OK:
+                raise SpecError(status, "spec_draft")
+            return cand_tok, cand_logp, workspace
     B = ctx_state.shape[0]
     _dev(ctx_state, torch.bfloat16, (B, h.d_base), "ctx_state")
     _dev(last_tok, torch.int32, (B,), "last_tok")
@@ -335,6 +356,12 @@ def spec_verify(cand_tok: torch.Tensor, base_logits: torch.Tensor, accept_len: O
                 early_exit: bool = False):
     """Enqueues one verification; returns (accept_len, best_cand, next_tok, workspace), int32 [B] each.
     early_exit: the form that stops reading a candidate's rows at its first mismatch (spec_verify_early)."""
+    if _pycall is not None and workspace is not None:
+        status = _pycall.verify(cand_tok, base_logits, accept_len, best_cand, next_tok, workspace, stream, early_exit)
+        if status is not None:
+            if status != SPEC_OK:
+                raise SpecError(status, "spec_verify")
+            return accept_len, best_cand, next_tok, workspace
     B, K, n = cand_tok.shape
     _dev(cand_tok, torch.int32, name="cand_tok")
     if base_logits.dtype == torch.bfloat16:
@@ -396,6 +423,12 @@ def spec_next_ctx(base_state: torch.Tensor, best_cand: torch.Tensor, accept_len:
                   stream: Optional[torch.cuda.Stream] = None) -> torch.Tensor:
     """ctx_state[b] = base_state[b, best_cand[b], accept_len[b]]: the state the next spec_draft starts from.
     `err_workspace` (e.g. the verify workspace) receives SPEC_ERR_INDEX_RANGE at offset 0 on a bad index."""
+    if _pycall is not None and ctx_state is not None:
+        status = _pycall.next_ctx(base_state, best_cand, accept_len, ctx_state, err_workspace, stream)
+        if status is not None:
+            if status != SPEC_OK:
+                raise SpecError(status, "spec_next_ctx")
+            return ctx_state
     B, K, n1, d = base_state.shape
     _dev(base_state, torch.bfloat16, name="base_state")
     _dev(best_cand, torch.int32, (B,), "best_cand")

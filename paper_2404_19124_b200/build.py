@@ -1,16 +1,21 @@
-"""Builds libspec_b200.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension)."""
+"""Builds libspec_b200.so in-tree with nvcc for sm_100a (no JIT cache, no torch extension), and beside it the CPython module
+_pycall.so that marshals the calls of a decoding step (the binding does without where the interpreter's headers are not
+installed)."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 _ROOT = os.path.dirname(_PKG)
 CSRC = os.path.join(_PKG, "csrc")
 INCLUDE = os.path.join(_ROOT, "include")
 LIB_PATH = os.path.join(_PKG, "libspec_b200.so")
-SOURCES = ["spec_api.cu", "verify_kernels.cu", "draft_kernels.cu", "draft_small.cu", "fp8_kernels.cu", "gemm_tcgen05.cu", "gemm_pair.cu", "gemm_simt.cu"]
+PYCALL_PATH = os.path.join(_PKG, "_pycall.so")
+SOURCES = ["spec_api.cu", "verify_kernels.cu", "draft_kernels.cu", "draft_small.cu", "fp8_kernels.cu", "gemm_tcgen05.cu",
+           "gemm_pair.cu", "gemm_simt.cu"]
 
 
 def _newest_source_mtime() -> float:
@@ -18,7 +23,22 @@ def _newest_source_mtime() -> float:
     return max(os.path.getmtime(p) for p in paths)
 
 
+def _build_pycall(force: bool) -> None:
+    source = os.path.join(CSRC, "pycall.c")
+    newest = max(os.path.getmtime(source), os.path.getmtime(os.path.join(INCLUDE, "spec_b200.h")))
+    headers = sysconfig.get_paths()["include"]
+    if not os.path.exists(os.path.join(headers, "Python.h")):
+        return
+    if not force and os.path.exists(PYCALL_PATH) and os.path.getmtime(PYCALL_PATH) >= newest:
+        return
+    tmp = PYCALL_PATH + f".tmp{os.getpid()}"
+    subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-std=c11", "-Wall", "-shared", "-fPIC", "-I", headers,
+                           "-I", INCLUDE, source, "-o", tmp])
+    os.replace(tmp, PYCALL_PATH)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    _build_pycall(force)
     if not force and os.path.exists(LIB_PATH) and os.path.getmtime(LIB_PATH) >= _newest_source_mtime():
         return LIB_PATH
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")

@@ -421,7 +421,7 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 }  // namespace
 
 // One kernel when a sequence is little enough for one CTA to read in less time than a second kernel costs.  One CTA reads
-// about 65 GB/s: 64 KB 7.5 us per call against 9.5 us in two kernels (both bound by the host), 256 KB 7.6 against 9.5 alone
+// about 65 GB/s: 64 KB 4.9 us per call against 6.8 us in two kernels (both bound by the host), 256 KB 7.6 against 9.5 alone
 // but 65.0 against 63.6 us inside a decoding step, 512 KB 11.6 against 9.7, 1 MB 15.3 against 9.5.
 constexpr long long kSeqMaxBytes = 128 << 10;
 bool one_kernel_form(int rows_b, int V, int dtype) {

@@ -120,7 +120,7 @@ def _check(status: int, where: str) -> None:
 # addresses go to ctypes as plain integers, the raw stream is asked for without building a Stream object (0.3 instead of
 # 3.2 us), the current device is switched only when it has to be (2.5 us).  Host time of one step of the smallest
 # shape: 66 -> 41 us, of spec_verify 19 -> 12.5, spec_next_ctx 14.5 -> 7.5, spec_draft 34 -> 26 (with fewer kernels and
-through csrc/pycall.c now: spec_verify 4.7, spec_draft 5.4, a 7B step 34).
+# through csrc/pycall.c now: spec_verify 4.7, spec_draft 5.4, a 7B step 34).
 def _ptr(t: Optional[torch.Tensor]):
     return None if t is None else t.data_ptr()
 

@@ -763,7 +763,7 @@ def main():
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     fused = sum(cfg.nodes(l + 1) <= sms or cfg.topk[l] <= 2 for l in range(n - 1))
     small = cfg.d_inner <= 512 and cfg.d_base <= 2048 and all(cfg.nodes(l) <= 16 for l in range(n)) and \
-        sum(V * cfg.d_inner * (16 + cfg.nodes(l)) for l in range(n)) <= n * (23 << 20)      # the whole draft is one kernel
+        sum(V * cfg.d_inner * (16 + cfg.nodes(l)) for l in range(n)) <= n * (30 << 20)      # the whole draft is one kernel
     launches_per_step = (1 if small else 1 + 3 * n - fused) + 2
     out = {
         "metric": METRIC, "value": shard.whole_job_rate(Bn, world, ms_step * 1e-3), "unit": UNIT, "n_gpus": world, "steps": args.steps,

@@ -10,10 +10,12 @@
 //
 //   P_0 | mix_0, P_1 + head_0 | merge_0, mix_1, P_2 + head_1 | ... | merge_last, prune      ("|": a cluster barrier)
 //
-// What bounds it: the latency of every step.  Per level of the smallest shape (V 1024, d 256, 1 / 4 / 12 nodes) mix 2.1 - 2.7,
-// projection and head 1.6 - 2.3, selection 1.0 - 1.3, barrier 0.5, merge 0.9 us; 8 instead of 16 CTAs are 0.5 us faster there
-// and 5 to 6 us slower at V 4096; 256 instead of 512 threads 2.5 us slower; requesting the level's weights into L1 before the
-// mix gains nothing.
+// What bounds it: the latency of every step.  Per level of the smallest shape (V 1024, d 256, 1 / 4 / 12 nodes) mix 1.7 - 2.4,
+// projection and head 1.0 - 1.2, selection 1.4 - 2.0, barrier 0.5, merge 0.9 us, the prune 0.9.  8 instead of 16 CTAs are
+// 0.5 us faster there and 5 to 6 us slower at V 4096; 256 instead of 512 threads 2.5 us slower; requesting the level's weights
+// into L1 before the mix gains nothing, nor do the arguments in shared memory; sums and lists of the selection in separate
+// warps, which must then leave the logits as they are, cost it 2 us.  (Loads without predicates and the LayerNorm parameters,
+// the tokens and the leaves in shared memory: 31.5 -> 28.2 us for the step.)
 #include <mutex>
 
 #include "row_ops.cuh"
@@ -22,8 +24,6 @@ namespace spec {
 
 namespace {
 
-using rows::BlockSync;
-using rows::LeafKey;
 using rows::float_key;
 using rows::key_float;
 
@@ -48,13 +48,12 @@ struct SmallArgs {
     int32_t topk[SPEC_MAX_HEADS];
     int32_t *header;
     int header_words;
-    int B, K, L, Lpad;
+    int B, K, L;
     int32_t *cand_tok;
     float *cand_logp;
-    PruneArgs prune;
     int pitch_base, pitch;              // bytes between the rows of the operand in shared memory: 64 modulo 128
     int off_logits, logit_pitch;        // byte offset of the logits, floats between the nodes
-    int off_lists, off_nodes, off_keys; // byte offsets of the partial lists (two sets), the nodes' tokens and scores, the leaves
+    int off_lists, off_nodes, off_ln;   // byte offsets of the partial lists (two sets), the nodes, the LayerNorm parameters
 };
 
 // Partial list of one (node, CTA).
@@ -92,34 +91,55 @@ __device__ __forceinline__ void mma16816(float (&c)[4], uint32_t a0, uint32_t a1
 // 32 of rows g and g + 8 and of node g: one 16-byte load each, two MMAs.  (The order of k inside a group is the same
 // permutation on both sides.)  c[q]: nodes 8 q + 2 t, + 1 of row g, then of row g + 8.
 constexpr int kGroups = kMaxNodes / 8;
-constexpr int kAhead = 4;   // groups of 32 elements whose loads are in flight together
+constexpr int kAhead = 8;   // groups of 32 elements whose loads are in flight together
 __device__ __forceinline__ void tile_times_nodes(const uint16_t *W, int rows, int Kd, int row0, int k0, int k1,
                                                  const char *x, int pitch, int nodes, int lane, float (&c)[kGroups][4]) {
     const int g = lane >> 2, t = lane & 3;
 #pragma unroll
     for (int q = 0; q < kGroups; ++q) c[q][0] = c[q][1] = c[q][2] = c[q][3] = 0.0f;
-    const bool ok0 = row0 + g < rows, ok1 = row0 + g + 8 < rows;
-    const uint16_t *w0 = W + (size_t)(row0 + g) * Kd + 8 * t, *w1 = w0 + (size_t)8 * Kd;
-    const char *xg = x + g * pitch + 16 * t;
-    for (int k = k0; k < k1; k += 32 * kAhead) {
+    // (a row past the last one is read as the first: its results go nowhere)
+    const uint16_t *w0 = W + (size_t)(row0 + g < rows ? row0 + g : 0) * Kd + k0 + 8 * t;
+    const uint16_t *w1 = W + (size_t)(row0 + g + 8 < rows ? row0 + g + 8 : 0) * Kd + k0 + 8 * t;
+    const char *xg = x + g * pitch + 2 * k0 + 16 * t;
+    const bool second = nodes > 8;
+    auto multiply = [&](const uint4 &p, const uint4 &q, const char *at) {
+        // (rows past the last node hold something finite and their results go nowhere either)
+        const uint4 b = *(const uint4 *)at;
+        mma16816(c[0], p.x, q.x, p.y, q.y, b.x, b.y);
+        mma16816(c[0], p.z, q.z, p.w, q.w, b.z, b.w);
+        if (second) {
+            const uint4 e = *(const uint4 *)(at + 8 * pitch);
+            mma16816(c[1], p.x, q.x, p.y, q.y, e.x, e.y);
+            mma16816(c[1], p.z, q.z, p.w, q.w, e.z, e.w);
+        }
+    };
+    static_assert(kGroups == 2, "multiply");
+    int left = k1 - k0;
+    for (; left >= 32 * kAhead; left -= 32 * kAhead) {
         uint4 a0[kAhead], a1[kAhead];
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
-            const bool in = k + 32 * u + 8 * t < k1;
-            a0[u] = ld_weights(w0 + k + 32 * u, in && ok0);
-            a1[u] = ld_weights(w1 + k + 32 * u, in && ok1);
+            a0[u] = ld_weights(w0 + 32 * u, true);
+            a1[u] = ld_weights(w1 + 32 * u, true);
+        }
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) multiply(a0[u], a1[u], xg + 64 * u);
+        w0 += 32 * kAhead;
+        w1 += 32 * kAhead;
+        xg += 64 * kAhead;
+    }
+    if (left > 0) {
+        uint4 a0[kAhead], a1[kAhead];
+#pragma unroll
+        for (int u = 0; u < kAhead; ++u) {
+            const bool in = 32 * u + 8 * t < left;
+            a0[u] = ld_weights(w0 + 32 * u, in);
+            a1[u] = ld_weights(w1 + 32 * u, in);
         }
 #pragma unroll
         for (int u = 0; u < kAhead; ++u) {
-            if (k + 32 * u >= k1) break;   // (uniform)
-#pragma unroll
-            for (int q = 0; q < kGroups; ++q) {
-                if (8 * q >= nodes) break;
-                // (rows past the last node hold something finite and their results go nowhere)
-                const uint4 b = *(const uint4 *)(xg + 8 * q * pitch + 2 * (k + 32 * u));
-                mma16816(c[q], a0[u].x, a1[u].x, a0[u].y, a1[u].y, b.x, b.y);
-                mma16816(c[q], a0[u].z, a1[u].z, a0[u].w, a1[u].w, b.z, b.w);
-            }
+            if (32 * u >= left) break;   // (uniform)
+            multiply(a0[u], a1[u], xg + 64 * u);
         }
     }
 }
@@ -154,9 +174,14 @@ __global__ void __launch_bounds__(kSmallThreads, 1) draft_small_kernel(const __g
     char *x = smem;
     float *logits = (float *)(smem + a.off_logits);
     SmallList *lists = (SmallList *)(smem + a.off_lists);           // [2][kMaxNodes][kCtas]
-    int *node_tok = (int *)(smem + a.off_nodes);                    // [kMaxNodes * SPEC_MAX_TOPK]: nodes of the level ...
-    float *node_score = (float *)(node_tok + kMaxNodes * SPEC_MAX_TOPK);   // ... their scores, two sets by turns
+    constexpr int kLevel = kMaxNodes * SPEC_MAX_TOPK;               // most nodes of a level
+    int *node_tok = (int *)(smem + a.off_nodes);                    // [n + 1][kLevel]: the nodes' tokens, every level's ...
+    float *node_score = (float *)(node_tok + (n + 1) * kLevel);     // ... their scores, two sets by turns
     griddep_launch();
+    float *ln = (float *)(smem + a.off_ln);   // [n][2][d]: the LayerNorm parameters
+    for (int l = 0; l < n; ++l)
+        for (int i = tid; i < 2 * d; i += kSmallThreads)
+            ln[l * 2 * d + i] = i < d ? a.w.ln_gamma[l][i] : a.w.ln_beta[l][i - d];
     for (int i = tid * 16; i < a.off_logits; i += kSmallThreads * 16) *(uint4 *)(smem + i) = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     griddep_wait();
@@ -188,9 +213,11 @@ __global__ void __launch_bounds__(kSmallThreads, 1) draft_small_kernel(const __g
         uint16_t *S = m.S_out;
         for (int i = warp; i < nodes; i += kSmallWarps) {
             m.S_out = (uint16_t *)(x + i * a.pitch);
+            m.gamma = ln + l * 2 * d;
+            m.beta = m.gamma + d;
             m.err = rank == 0 ? a.mix[l].err : nullptr;
-            if (d <= 256) rows::mix_ln_gelu_row<32, 1, 1, WarpSync, kMaxSplits>(m, 0, i / parent_div, node_tok[i], lane, red[warp]);
-            else rows::mix_ln_gelu_row<32, 2, 1, WarpSync, kMaxSplits>(m, 0, i / parent_div, node_tok[i], lane, red[warp]);
+            if (d <= 256) rows::mix_ln_gelu_row<32, 1, 1, WarpSync, kMaxSplits>(m, 0, i / parent_div, node_tok[l * kLevel + i], lane, red[warp]);
+            else rows::mix_ln_gelu_row<32, 2, 1, WarpSync, kMaxSplits>(m, 0, i / parent_div, node_tok[l * kLevel + i], lane, red[warp]);
         }
         __syncthreads();
         // the next level's projection and this level's head
@@ -292,9 +319,8 @@ __global__ void __launch_bounds__(kSmallThreads, 1) draft_small_kernel(const __g
         }
         small_barrier();
         // the nodes' children, in every CTA
-        const float *score_in = node_score + (l & 1) * kMaxNodes * SPEC_MAX_TOPK;
-        float *score_out = node_score + ((l + 1) & 1) * kMaxNodes * SPEC_MAX_TOPK;
-        const bool write = rank == 0 || l == n - 1;   // (the last level's by all, with the same values: each prunes some of it)
+        const float *score_in = node_score + (l & 1) * kLevel;
+        float *score_out = node_score + ((l + 1) & 1) * kLevel;
         for (int i = warp; i < nodes; i += kSmallWarps) {
             const SmallList *li = set + i * kCtas + (lane < kCtas ? lane : 0);
             const float pm = lane < kCtas ? li->m : -INFINITY, ps = lane < kCtas ? li->s : 0.0f;
@@ -314,9 +340,9 @@ __global__ void __launch_bounds__(kSmallThreads, 1) draft_small_kernel(const __g
                 if (lane == 0) {
                     const int child = i * topk + j;
                     const float score = base + (key_float(bk) - lse);
-                    node_tok[child] = bi;
+                    node_tok[(l + 1) * kLevel + child] = bi;
                     score_out[child] = score;
-                    if (write) {
+                    if (rank == 0) {
                         a.tok[l + 1][child] = bi;
                         a.score[l + 1][child] = score;
                     }
@@ -331,9 +357,23 @@ __global__ void __launch_bounds__(kSmallThreads, 1) draft_small_kernel(const __g
         __syncthreads();
         nodes *= topk;
     }
-    for (int b = rank; b < a.B; b += kCtas)
-        rows::prune_sequence<kSmallThreads, BlockSync>(a.score[n], a.prune, a.L, a.Lpad, a.K, a.cand_tok, a.cand_logp, b, tid,
-                                                       (LeafKey *)(smem + a.off_keys));
+    // the K best leaves of every sequence by (score desc, leaf asc): a thread's rank is the leaves that precede its own
+    if (rank == 0 && tid < nodes) {
+        const float *score = node_score + (n & 1) * kLevel;
+        const int b = tid / a.L, leaf = tid - b * a.L;
+        const rows::LeafKey mine = {score[tid], leaf};
+        int before = 0;
+        for (int j = 0; j < a.L; ++j) before += rows::leaf_before({score[b * a.L + j], j}, mine) ? 1 : 0;
+        if (before < a.K) {
+            const size_t out = (size_t)b * a.K + before;
+            a.cand_logp[out] = mine.score;
+            int idx = tid;
+            for (int l = n; l > 0; --l) {
+                a.cand_tok[out * n + l - 1] = node_tok[l * kLevel + idx];
+                idx /= a.topk[l - 1];
+            }
+        }
+    }
 }
 
 int pitch_of(int elems) { return (2 * elems + 127) / 128 * 128 + 64; }
@@ -342,11 +382,12 @@ int pitch_of(int elems) { return (2 * elems + 127) / 128 * 128 + 64; }
 
 // Which drafts run as one kernel: those whose levels read little for the sixteen CTAs (a megabyte each way costs 2 to 3 us,
 // in the kernel chain a fifth of that), the less the more nodes every CTA has to mix and to select for.  us per draft, kernel
-// chain -> one kernel, d_base 512, branching 4, 3, 2 unless stated: V 1000, d 256 39.7 -> 27; V 4096, d 256 39.5 -> 29.7;
-// V 2000, d 512 41.5 -> 35.2; V 3000, d 512 41.9 -> 40.0; V 6000, d 512 42.6 -> 52.7; V 16000, d 256 41.1 -> 56.3; branching
-// 6, 2 for two sequences, V 1500, d 504 31.6 -> 25.6; one level, V 1200, d 256 16.8 -> 11.4; chains of three for 16
-// sequences, V 1000, d 256 38.0 -> 30.0, V 2000, d 512 39.6 -> 42.3; a chain of five for one, V 4000, d 512 59.5 -> 60.7.
-// (32 nodes, with room for them: V 2000, d 256 40.8 -> 47.4.)  The smallest decoding step 45.7 -> 31.5.
+// chain -> one kernel, d_base 512, branching 4, 3, 2 unless stated: V 1000, d 256 39.7 -> 23; V 4096, d 256 39.5 -> 27.0;
+// V 5400, d 256 40.4 -> 30.3; V 2000, d 512 41.5 -> 30.4; V 2700, d 512 41.6 -> 33.2; branching 6, 2 for two sequences, V 1500,
+// d 504 31.6 -> 22.5; one level, V 1200, d 256 16.8 -> 9.7; chains of three for 16 sequences, V 1000, d 256 38.0 -> 26.2,
+// V 3600, d 256 38.1 -> 31.8, V 1800, d 512 39.6 -> 38.2; a chain of five for one, V 3400, d 512 61.1 -> 50.1.  Far beyond
+// the line (3 us more per draft then): V 6000, d 512 42.6 -> 52.7; V 16000, d 256 41.1 -> 56.3; 32 nodes, with room for
+// them, V 2000, d 256 40.8 -> 47.4.  The smallest decoding step 45.7 -> 28.2.
 bool small_draft_fits(const spec_weights_t &w, int B, const int32_t *topk) {
     if (w.d_inner > 512 || w.d_base > 2048) return false;
     long long nodes = B, cost = 0;
@@ -355,7 +396,7 @@ bool small_draft_fits(const spec_weights_t &w, int B, const int32_t *topk) {
         cost += (long long)w.V * w.d_inner * (16 + nodes);
         nodes *= topk[l];
     }
-    return cost <= (23ll << 20) * w.n_heads;
+    return cost <= (30ll << 20) * w.n_heads;
 }
 
 // Floats of the two projection buffers together.
@@ -363,7 +404,7 @@ size_t small_draft_proj_floats(const spec_weights_t &w) { return (size_t)2 * kMa
 
 int launch_draft_small(const spec_weights_t &w, const void *ctx, int B, const int32_t *topk, int K, const MixArgs *mix,
                        int32_t *const *tok, float *const *score, float *proj, int32_t *header, int header_words,
-                       const PruneArgs &prune, int L, int32_t *cand_tok, float *cand_logp, cudaStream_t st) {
+                       int L, int32_t *cand_tok, float *cand_logp, cudaStream_t st) {
     SmallArgs a{};
     a.w = w;
     a.ctx = (const uint16_t *)ctx;
@@ -392,11 +433,8 @@ int launch_draft_small(const spec_weights_t &w, const void *ctx, int B, const in
     a.header = header;
     a.header_words = header_words;
     a.B = B; a.K = K; a.L = L;
-    a.Lpad = 2;
-    while (a.Lpad < L) a.Lpad <<= 1;
     a.cand_tok = cand_tok;
     a.cand_logp = cand_logp;
-    a.prune = prune;
     a.pitch_base = pitch_of(w.d_base);
     a.pitch = pitch_of(w.d_inner);
     const int node_rows = (max_nodes + 7) / 8 * 8;
@@ -409,9 +447,9 @@ int launch_draft_small(const spec_weights_t &w, const void *ctx, int B, const in
     a.off_lists = (off + 127) / 128 * 128;
     off = a.off_lists + 2 * kMaxNodes * kCtas * (int)sizeof(SmallList);
     a.off_nodes = (off + 127) / 128 * 128;
-    off = a.off_nodes + 3 * 4 * kMaxNodes * SPEC_MAX_TOPK;
-    a.off_keys = (off + 127) / 128 * 128;
-    off = a.off_keys + (int)rows::prune_smem_bytes(L, a.Lpad);
+    off = a.off_nodes + (n + 3) * 4 * kMaxNodes * SPEC_MAX_TOPK;
+    a.off_ln = (off + 127) / 128 * 128;
+    off = a.off_ln + n * 2 * 4 * w.d_inner;
     if (off > kMaxSmem) return SPEC_ERR_SHAPE;
     int dev = 0;
     SPEC_CUDA_TRY(cudaGetDevice(&dev));

@@ -40,6 +40,7 @@ template <int kThreads, typename Sync>   // (kThreads 0: blockDim.x)
 __device__ __forceinline__ float group_sum(float v, float *red, int tid) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    if (kThreads == 32) return v;
     const int w = tid >> 5, l = tid & 31;
     if (l == 0) red[w] = v;
     Sync::sync();

@@ -581,7 +581,7 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
             toks[l + 1] = (int32_t *)(ws + p.lay.tok[l + 1]);
             scores[l + 1] = (float *)(ws + p.lay.score[l + 1]);
         }
-        rc = launch_draft_small(w, ctx_state, B, topk, K, mixes, toks, scores, P, err, p.header_words, pa, p.L, cand_tok,
+        rc = launch_draft_small(w, ctx_state, B, topk, K, mixes, toks, scores, P, err, p.header_words, p.L, cand_tok,
                                 cand_logp, st);
         if (rc != SPEC_ERR_SHAPE) return rc;
     }

@@ -215,7 +215,7 @@ bool small_draft_fits(const spec_weights_t &w, int B, const int32_t *topk);
 size_t small_draft_proj_floats(const spec_weights_t &w);
 int launch_draft_small(const spec_weights_t &w, const void *ctx, int B, const int32_t *topk, int K, const MixArgs *mix,
                        int32_t *const *tok, float *const *score, float *proj, int32_t *header, int header_words,
-                       const PruneArgs &prune, int L, int32_t *cand_tok, float *cand_logp, cudaStream_t st);
+                       int L, int32_t *cand_tok, float *cand_logp, cudaStream_t st);
 
 int launch_draft_init(int32_t *hdr, int words, cudaStream_t st);
 int launch_mix_ln_gelu(const MixArgs &m, int rows, cudaStream_t st);

@@ -131,7 +131,7 @@ def test_e4m3_levels_with_and_without_swapped_operands(B, B_, topk, V, d, swap):
                                                  (2, (8, 8), 2047, 8, 128), (1, (8, 2, 8), 600, 2048, 8),
                                                  (2, (8,), 16, 72, 504), (5, (3, 1, 2), 257, 1000, 248),
                                                  (1, (4, 2, 2, 2), 2048, 256, 512), (9, (1, 1, 4), 129, 2040, 40),
-                                                 (1, (4, 3), 2100, 64, 512), (1, (4, 3), 2600, 64, 512)])
+                                                 (1, (4, 3), 3100, 64, 512), (1, (4, 3), 3300, 64, 512)])
 def test_small_drafts_are_one_kernel(B, B_, topk, V, d_base, d):
     """Node counts, widths and vocabularies at the edges of what one cluster takes: 16 and 17 nodes, fewer rows than warps,
     CTAs without any vocabulary row, K ranges that end inside a group of 32, sizes on both sides of the limit."""

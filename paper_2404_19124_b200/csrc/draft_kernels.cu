@@ -166,6 +166,9 @@ __global__ void __maxnreg__(72) merge_mix_512_kernel(MergeMixArgs a) {
 // parent's merge (a few KB from L2) and computes its own state, so no parallelism is lost and a kernel boundary is saved.
 // Levels 0 -> 1 -> 2 of the 7B shape (8 -> 32 -> 96 nodes): 10.2 us a level as two kernels, 8.0 as one; the step 160.8 ->
 // 158.9 us, smallest shape 51.2 -> 48.4, ragged step 131.2 -> 129.3, single-candidate chain 163.6 -> 161.5.
+// With one or two children per row the LayerNorm sums are added in the order of merge_mix_kernel, which takes such levels beyond
+// one child per SM, so that a level's states are the same bits on both sides of that line.  (In a tree a sum's last bit
+// differs, now and then a state rounds to the other bf16 neighbour and a score moves by up to 1e-3.)
 template <int kThreads, int kLen>
 __device__ __forceinline__ void merge_mix_child(const MergeMixArgs &a, Scratch *sc, float *red) {
     const int c = blockIdx.x, topk = a.merge.topk, r = c / topk, tid = threadIdx.x;
@@ -173,7 +176,8 @@ __device__ __forceinline__ void merge_mix_child(const MergeMixArgs &a, Scratch *
     const MergeOut o = merge_expand_row<kThreads, kLen, BlockSync>(a.merge, r, tid, sc, c == r * topk,
                                                                    [&] { parent_state<kThreads>(a.mix, r, tid, pre); });
     const int t = __shfl_sync(0xffffffffu, o.id, c - r * topk);
-    mix_ln_gelu_row<kThreads, 1, 1, BlockSync>(a.mix, c, r, t, tid, red, pre);
+    const bool in_order = topk <= kFusedMixMaxChildren && a.mix.S8_out == nullptr;
+    mix_ln_gelu_row<kThreads, 1, 1, BlockSync>(a.mix, c, r, t, tid, red, pre, in_order);
 }
 template <int kLen>
 __global__ void __launch_bounds__(kRowThreads, 2) merge_mix_child_kernel(MergeMixArgs a) {

@@ -35,16 +35,24 @@ struct Scratch {
     int cand_i[kMaxGroupWarps][kMaxRounds];        // ... and token ids
 };
 
-// (`red`: one float per warp, not read by anybody else until the next barrier behind the call)
+// (`red`: one float per warp, not read by anybody else until the next barrier behind the call.  `in_order`: the warps' sums are
+// added one after the other, as mix_children adds them, instead of in a tree.)
 template <int kThreads, typename Sync>   // (kThreads 0: blockDim.x)
-__device__ __forceinline__ float group_sum(float v, float *red, int tid) {
+__device__ __forceinline__ float group_sum(float v, float *red, int tid, bool in_order = false) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     if (kThreads == 32) return v;
     const int w = tid >> 5, l = tid & 31;
     if (l == 0) red[w] = v;
     Sync::sync();
-    float t = l < (kThreads > 0 ? kThreads : (int)blockDim.x) / 32 ? red[l] : 0.0f;
+    const int warps = (kThreads > 0 ? kThreads : (int)blockDim.x) / 32;
+    if (in_order) {   // (uniform)
+        float t = 0.0f;
+#pragma unroll
+        for (int q = 0; q < warps; ++q) t += red[q];
+        return t;
+    }
+    float t = l < warps ? red[l] : 0.0f;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
     return t;
@@ -70,6 +78,10 @@ __device__ __forceinline__ float gelu_erf(float y) { return 0.5f * y * (1.0f + e
 static __device__ __noinline__ float4 gelu_erf4(float4 y) {
     return make_float4(gelu_erf(y.x), gelu_erf(y.y), gelu_erf(y.z), gelu_erf(y.w));
 }
+
+// An element of the mixed row.  Which of the two products is rounded before the sum is spelt out: left to the compiler it
+// differed from one kernel to the next, and with it, now and then, the bf16 value that a state is rounded to.
+__device__ __forceinline__ float mix_element(const MixArgs &m, float p, float z) { return fmaf(m.b, z, __fmul_rn(m.a, p)); }
 
 // The projected parent state (the sum of its partials, added in ascending order) of the groups that thread `tid` owns in
 // mix_ln_gelu_row with one group per thread.
@@ -104,10 +116,11 @@ __device__ __forceinline__ void parent_state(const MixArgs &m, int parent, int t
 // t, t + kThreads, ... (kIters of them; d <= 8 * kThreads * kIters, d % 8 == 0; kThreads 0: as many as the CTA has).
 // kDepth of those groups, and kSp partial projections of each, have their loads in flight together (registers against
 // latency).
-// `pre`: the projected parent state of this thread's groups (parent_state), if the caller has it already.
+// `pre`: the projected parent state of this thread's groups (parent_state), if the caller has it already.  `in_order`: see
+// group_sum.
 template <int kThreads, int kIters, int kDepth, typename Sync, int kSp = 4>
 __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int parent, int t, int tid, float *red,
-                                                const float (*pre)[8] = nullptr) {
+                                                const float (*pre)[8] = nullptr, bool in_order = false) {
     constexpr int kGroup = kIters >= 8 ? 1 : (kIters < kDepth ? kIters : kDepth);
     bool tok_ok = false;
     const int nt = kThreads > 0 ? kThreads : (int)blockDim.x;
@@ -171,7 +184,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const float z = (j & 1) ? __uint_as_float(ew[j >> 1] & 0xffff0000u) : __uint_as_float(ew[j >> 1] << 16);
-                h[it][j] = i < d ? m.a * pv[j] + m.b * z : 0.0f;
+                h[it][j] = i < d ? mix_element(m, pv[j], z) : 0.0f;
                 sum += h[it][j];
             }
         }
@@ -192,7 +205,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
             bq[it][1] = *(const float4 *)(m.beta + ic + 4);
         }
     }
-    const float mean = group_sum<kThreads, Sync>(sum, red, tid) / (float)d;
+    const float mean = group_sum<kThreads, Sync>(sum, red, tid, in_order) / (float)d;
     float sq = 0.0f;
 #pragma unroll
     for (int it = 0; it < kIters; ++it) {
@@ -205,7 +218,7 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
             }
         }
     }
-    const float var = group_sum<kThreads, Sync>(sq, red + kMaxGroupWarps, tid) / (float)d;
+    const float var = group_sum<kThreads, Sync>(sq, red + kMaxGroupWarps, tid, in_order) / (float)d;
     const float rstd = rsqrtf(var + m.eps);
     float amax = 0.0f;   // largest magnitude of the bf16-rounded state (for the e4m3 copy); h is reused for it
 #pragma unroll
@@ -521,7 +534,7 @@ __device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int f
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     const float z = (j & 1) ? __uint_as_float(ew[j >> 1] & 0xffff0000u) : __uint_as_float(ew[j >> 1] << 16);
-                    h[q][it][j] = i < d ? m.a * pv[it][j] + m.b * z : 0.0f;
+                    h[q][it][j] = i < d ? mix_element(m, pv[it][j], z) : 0.0f;
                     part[q] += h[q][it][j];
                 }
             }

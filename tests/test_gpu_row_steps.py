@@ -218,3 +218,25 @@ def test_mix_of_many_rows_round_the_thread_counts(B, d, parents):
         want = oracle.stage_state(ow, 1, s0[r // 4], int(t1[r]))
         assert np.allclose(s1[r], want, rtol=0.008, atol=2e-4)
     B.spec_destroy(h)
+
+
+@pytest.mark.parametrize("k,d", [(2, 1032), (2, 2048), (2, 2056), (2, 4096), (4, 1032), (4, 2048)])
+def test_states_are_the_same_bits_in_every_kernel(B, k, d):
+    """148 children have one CTA each; with one parent more they are computed one CTA per parent (two children per row) or by a
+    kernel of their own (four).  The children that both batches have get the same states, so that a sequence's result does not
+    hang on the batch it is in."""
+    topk, n0 = (k, 1), 148 // k
+    cfg = small_cfg(d_base=64, d_inner=d, V=600, topk=topk, K=k, B=n0 + 1, seed=d)
+    sw = synth.make_weights(cfg)
+    ctx, tok = synth.make_draft_inputs(cfg)
+    h = B.spec_create(weights_to_cuda(sw))
+    got = []
+    for n in (n0, n0 + 1):
+        ct, lp, ws = B.spec_draft(h, ctx[:n].cuda(), tok[:n].cuda(), topk, k)
+        assert B.spec_poll_error(ws) == 0
+        lay = B.spec_draft_layout(h, n, topk, k)
+        got.append([ws[lay.state[l]:lay.state[l] + 2 * rows * d].view(torch.int16) for l, rows in ((0, n0), (1, 148))] +
+                   [ws[lay.tok[1]:lay.tok[1] + 4 * 148].view(torch.int32)])
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    B.spec_destroy(h)

@@ -244,8 +244,11 @@ int spec_verify_static(const int32_t *cand_tok, const void *base_logits, int log
  *                                    copies): afterwards every rank holds all n_ranks slots
  *     spec_draft_vp_merge(level l)   folds the slots into the level's children; at the last level also
  *                                    prunes to the K candidates
- * and every rank ends with the same cand_tok / cand_logp as spec_draft on unsplit weights (token sets and
- * order identical; log-probabilities equal up to the rounding of a two-stage log-sum-exp).
+ * and every rank ends with the same cand_tok / cand_logp as spec_draft on unsplit weights: a logit is the same
+ * sum whether the head is split or not, so a node's children are the same tokens in the same order;
+ * log-probabilities are equal up to the rounding of a two-stage log-sum-exp.  Two exceptions, both of near-ties
+ * only (scores that fp32 rounding separates): a draft that spec_draft runs as one kernel sums its logits in
+ * another order, and so do the LayerNorms behind a level of one or two children per node.
  *   spec_set_vocab_shard     declares that the head[] matrices given to spec_create hold `head_rows` rows
  *                            starting at token `vocab_offset` (weights.V stays the full vocabulary).
  *                            n_ranks <= 8, n_ranks * topk[l] <= 64.  On such a handle spec_draft, the

@@ -85,10 +85,12 @@ int head_block_n_for(const spec_handle_s *h, int rows) {
 // V 32000, 64 / 80 / 128 nodes 109.6, 112.5, 119.0 -> 106.7 / 114.4 / 128.8.
 // e4m3 heads (lists of eight whatever the branching): V 32000, d 4096, two levels of 60 nodes 98.8 -> 88.3; V 27408,
 // d 3584, 7 nodes 55.3 -> 47.7; V 5000, d 2048, 40 nodes 46.5 -> 48.7; the 13B step 251 -> 243.
+// A shard of the vocabulary takes the form that the whole one takes: a logit is then the same sum, and the split and the
+// unsplit draft order the same tokens the same way.
 bool head_swapped_for(const spec_handle_s *h, int rows, bool fp8 = false) {
     if (h->gemm_impl != 0 || h->head_block_n != 0 || rows > 128) return false;
     if (h->swap_max_rows >= 0) return rows <= h->swap_max_rows;
-    const int rows_per_sm = h->head_rows / num_sms();
+    const int rows_per_sm = h->w.V / num_sms();
     return rows <= (rows_per_sm >= 128 ? 64 : rows_per_sm >= 30 && !fp8 ? 48 : 32);
 }
 
@@ -275,7 +277,6 @@ GemmCall make_head_call(const spec_handle_s *h, const DraftPlan &p, char *ws, in
     c.epi.part_ms = (float *)(ws + p.lay.part_ms);
     c.epi.topk = topk_l;
     c.epi.idx_offset = h->vocab_offset;
-    c.epi.sharded = h->vp_ranks > 1;
     if (p.use_fp8[l]) {   // e4m3 operands; every tile keeps SPEC_MAX_TOPK candidates by approximate logit
         c.A = ws + p.lay.state8;
         c.B = h->head8[l];

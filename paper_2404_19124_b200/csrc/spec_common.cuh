@@ -113,7 +113,6 @@ struct GemmEpilogue {
     int fp8;           // operands are e4m3 bytes instead of bf16; the logit of node m and vocabulary row n is then
                        // the accumulator times row_scale[m] * col_scale[n]
     const float *row_scale, *col_scale;
-    int sharded;       // the weights are a vocabulary shard
     int idx_offset;    // mode 1 / 3: added to every token id written to part_idx (first vocabulary row of a shard)
     int segs;          // mode 3: threads that share one node's column (swapped_head_segs)
     int n_parts;       // mode 3: partial lists per node = CTAs the tiles are dealt to * segs (swapped_head_parts)

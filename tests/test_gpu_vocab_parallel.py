@@ -23,8 +23,8 @@ def B():
     return binding
 
 
-def _run_ranks(B, gw, cfg, world, ctx, tok):
-    """Emulates `world` ranks; returns their (cand_tok, cand_logp) and the handles' workspaces."""
+def _run_ranks(B, gw, cfg, world, ctx, tok, keep=False):
+    """Emulates `world` ranks; returns their (cand_tok, cand_logp), with `keep` also their workspaces and layouts."""
     parts = shard.split_vocab(cfg.V, world)
     hs = []
     for r, (lo, cnt) in enumerate(parts):
@@ -49,6 +49,8 @@ def _run_ranks(B, gw, cfg, world, ctx, tok):
     for ws in wss:
         assert B.spec_poll_error(ws) == 0
     out = [(c.cpu().numpy(), lp.cpu().numpy()) for c, lp in zip(cands, logps)]
+    if keep:
+        out = [o + (ws, B.spec_draft_layout(h, cfg.B, cfg.topk, cfg.K)) for o, ws, h in zip(out, wss, hs)]
     for h in hs:
         B.spec_destroy(h)
     return out
@@ -95,6 +97,37 @@ def test_vocab_parallel_full_width_two_ranks(B):
     for b in range(cfg.B):
         chk.check(ctx_bits[b], int(tok[b]), results[0][0][b], results[0][1][b])
     assert chk.exact + chk.tolerated == cfg.B
+
+
+@pytest.mark.parametrize("world", [2, 3])
+@pytest.mark.parametrize("Bn,topk,V,d", [(1, (6, 8), 4099, 2048), (4, (8, 8), 4096, 4096), (5, (8, 3), 20000, 2048),
+                                         (32, (8, 3), 4096, 2048), (3, (4, 4), 4099, 2056), (1, (8, 3), 1024, 512)])
+def test_split_and_unsplit_heads_order_near_ties_alike(B, world, Bn, topk, V, d):
+    """Every logit has a twin further up the vocabulary that is the same sum in another order (states whose halves are equal,
+    head rows with their halves exchanged): which of the two is larger hangs on the rounding alone, and the split draft has
+    to see it as the unsplit one does.  1 to 256 nodes, one to many tiles per CTA, widths with and without halves of their own."""
+    cfg = small_cfg(d_base=64, d_inner=d, V=V, topk=topk, K=topk[0], B=Bn, seed=d + Bn)
+    w, hd, hv = synth.make_weights(cfg), d // 2, V // 2
+    for l in range(cfg.n):
+        w.emb[l][:, hd:] = w.emb[l][:, :hd]
+        w.proj[l][hd:] = w.proj[l][:hd]
+        w.ln_gamma[l][hd:] = w.ln_gamma[l][:hd]
+        w.ln_beta[l][hd:] = w.ln_beta[l][:hd]
+        w.head[l][hv:2 * hv, :hd] = w.head[l][:hv, hd:]
+        w.head[l][hv:2 * hv, hd:] = w.head[l][:hv, :hd]
+    gw = weights_to_cuda(w)
+    ctx, tok = (t.cuda() for t in synth.make_draft_inputs(cfg))
+    h = B.spec_create(gw)
+    if d <= 512:
+        B.spec_set_option(h, B.SPEC_OPT_HEAD_PAIR, 0)      # (no draft in one kernel: its sums are its own)
+    _, _, ws = B.spec_draft(h, ctx, tok, topk, cfg.K)
+    assert B.spec_poll_error(ws) == 0
+    lay = B.spec_draft_layout(h, Bn, topk, cfg.K)
+    for _, _, rws, rlay in _run_ranks(B, gw, cfg, world, ctx, tok, keep=True):
+        for l in range(1, cfg.n + 1):
+            n = 4 * cfg.nodes(l)
+            assert torch.equal(ws[lay.tok[l]:lay.tok[l] + n].view(torch.int32), rws[rlay.tok[l]:rlay.tok[l] + n].view(torch.int32))
+    B.spec_destroy(h)
 
 
 def test_sharded_handle_refuses_the_unsplit_calls(B):

@@ -1,5 +1,11 @@
 """The natively marshalled calls: on tensors that are not what a call takes they stand aside for the Python checks, and on the
-GPU both ways of marshalling give the same results and the same errors."""
+GPU both ways of marshalling give the same results and the same errors.  The module itself: named for one interpreter, never
+older than its source, and not needed."""
+import os
+import shutil
+import sys
+import sysconfig
+
 import pytest
 import torch
 
@@ -26,6 +32,40 @@ def test_anything_unusual_is_left_to_the_python_checks(B):
     assert B._pycall.draft(1, 3, 8, i32, i32, (1, 1), 1, i32, i32, i32, None) is None
     with pytest.raises(ValueError, match="cand_tok"):
         B.spec_verify(i32, torch.zeros(2, 3, 2, 8), workspace=i32)
+
+
+def _private_tree(tmp_path, monkeypatch):
+    """The build of the module alone, in a package directory of its own."""
+    pkg = tmp_path / "pkg"
+    pkg.mkdir()
+    monkeypatch.setattr(build, "_PKG", str(pkg))
+    monkeypatch.setattr(build, "PYCALL_PATH", str(pkg / os.path.basename(build.PYCALL_PATH)))
+    return pkg
+
+
+def test_the_module_is_named_for_this_interpreter(tmp_path, monkeypatch):
+    assert sys.implementation.cache_tag in os.path.basename(build.PYCALL_PATH)
+    assert build.PYCALL_PATH.endswith(sysconfig.get_config_var("EXT_SUFFIX"))
+    pkg = _private_tree(tmp_path, monkeypatch)
+    (pkg / "_pycall.so").write_bytes(b"of another interpreter")
+    build._build_pycall(False)
+    assert not (pkg / "_pycall.so").exists()
+
+
+@pytest.mark.parametrize("missing", ["headers", "compiler", "working compiler"])
+def test_a_module_that_cannot_be_built_is_left_out(tmp_path, monkeypatch, missing):
+    pkg = _private_tree(tmp_path, monkeypatch)
+    stale = pkg / os.path.basename(build.PYCALL_PATH)
+    stale.write_bytes(b"of an older source")
+    os.utime(stale, (1, 1))
+    if missing == "headers":
+        monkeypatch.setattr(build.sysconfig, "get_paths", lambda: {"include": str(tmp_path)})
+        build._build_pycall(False)
+    else:
+        monkeypatch.setenv("CC", str(tmp_path / "none") if missing == "compiler" else shutil.which("false"))
+        with pytest.warns(UserWarning, match="marshalled in Python"):
+            build._build_pycall(False)
+    assert os.listdir(pkg) == []
 
 
 @pytest.mark.gpu

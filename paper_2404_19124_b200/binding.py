@@ -165,12 +165,12 @@ def _dev(t: torch.Tensor, dtype: torch.dtype, shape=None, name: str = "tensor") 
 
 @functools.lru_cache(maxsize=256)
 def _topk_const(topk: Tuple[int, ...]):
-    return (C.c_int32 * len(topk))(*[int(x) for x in topk])
+    return (C.c_int32 * len(topk))(*topk)
 
 
 def _topk_arr(topk: Sequence[int]):
-    """The branching factors as a C array (read-only for every callee)."""
-    return _topk_const(topk if type(topk) is tuple else tuple(topk))
+    """The branching factors as a C array (read-only for every callee), kept by their values: what comes in may be tensors."""
+    return _topk_const(tuple([int(x) for x in topk]))
 
 
 def spec_version() -> int:

@@ -99,3 +99,15 @@ def test_choose_k_follows_the_callers_batch_table(binding):
         assert e.value.status == binding.SPEC_ERR_INVALID_ARG
     with pytest.raises(binding.SpecError):
         binding.spec_choose_k(0, 3, rules)
+
+
+def test_branching_factors_are_taken_by_value(binding):
+    import numpy as np
+    import torch
+    t = (torch.tensor(4), torch.tensor(3))
+    assert list(binding._topk_arr(t)) == [4, 3]
+    t[0].fill_(2)                                       # the same objects with another value
+    assert list(binding._topk_arr(t)) == [2, 3]
+    a = np.array(5)
+    assert list(binding._topk_arr((a, 1))) == [5, 1]    # not hashable
+    assert list(binding._topk_arr(torch.tensor([6, 2]))) == [6, 2] and list(binding._topk_arr([7.0, 1])) == [7, 1]

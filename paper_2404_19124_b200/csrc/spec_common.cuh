@@ -80,9 +80,9 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 struct VerifyPlan {
     int rows;          // B * K * (n + 1)
     int vec_per_warp;  // two-kernel form: 16-byte vectors in one warp's contiguous range
-    int slots;         // ... partial slots reserved per row
+    int warps;         // ... ranges, at most (the base at its least aligned)
     size_t off_g;      // int32 [rows]
-    size_t off_part;   // (fp32 value, int32 index) [rows, slots]
+    size_t off_part;   // (fp32 value, int32 index) [warps + min(rows, warps)], see first_piece; early exit: int32 [B * K]
     size_t total;
 };
 VerifyPlan make_verify_plan(int B, int K, int n, int V, int dtype);

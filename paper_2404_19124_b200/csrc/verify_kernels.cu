@@ -12,8 +12,8 @@
 //   verify_seq_kernel    one CTA per sequence does the whole job: its warps take equal contiguous ranges of the sequence's
 //                        vectors, fold them into a (value, index) key per row in shared memory, and the CTA accepts.
 //   verify_stream_kernel + verify_accept_kernel    all vectors cut into equal contiguous ranges, one per warp, a single
-//                        wave over the whole GPU; each (row, warp) intersection writes one (value, index) partial, which
-//                        one CTA per sequence folds and accepts.
+//                        wave over the whole GPU; a row that lies in one range is finished there, of the others every
+//                        piece leaves a (value, index) partial; one CTA per sequence folds those and accepts.
 #include <float.h>
 
 #include <mutex>
@@ -143,12 +143,17 @@ __device__ __forceinline__ void scan_row(const char *base, long long rs, long lo
     }
 }
 
-// vec_per_warp vectors per warp; row r is elements [skew + r * V, + V); the partial of the (row, warp) intersection goes to
-// slot  warp - first_warp(row)  of the row.
+// Places of the partials.  A border between two warps is crossed by one row at most, so the pieces behind a border are
+// numbered by their warp; a row's first piece goes to a place of its row or of its warp behind those, whichever are fewer.
+__host__ __device__ __forceinline__ long long first_piece(long long warps, int rows, int row, long long w) {
+    return warps + (rows < warps ? row : w);
+}
+
+// vec_per_warp vectors per warp, `warps` of them at most; row r is elements [skew + r * V, + V).
 template <bool kBf16>
 __global__ void __launch_bounds__(kArgmaxThreads, 4)
 verify_stream_kernel(const char *__restrict__ base, int skew, int rows, int V, long long total_vec, int vec_per_warp,
-                     int slots, float2 *part) {
+                     int warps, int32_t *g_out, float2 *part) {
     griddep_launch();
     griddep_wait();
     using E = Elem<kBf16>;
@@ -165,8 +170,9 @@ verify_stream_kernel(const char *__restrict__ base, int skew, int rows, int V, l
         scan_row<kBf16, 32>(base, rs, rs + V, beg, end, lane, best, idx);
         warp_argmax(best, idx);
         if (lane == 0) {
-            const long long first_w = (rs >> E::kShift) / vec_per_warp;
-            part[(size_t)row * slots + (size_t)(w - first_w)] = make_float2(best, __int_as_float(idx));
+            const bool begins = (rs >> E::kShift) >= beg, ends = ((rs + V - 1) >> E::kShift) < end;   // in this range
+            if (begins && ends) g_out[row] = idx == kIdxNone ? 0 : idx;   // (nothing above -inf, all NaN: 0)
+            else part[begins ? first_piece(warps, rows, row, w) : w] = make_float2(best, __int_as_float(idx));
         }
     }
 }
@@ -215,7 +221,7 @@ __device__ __forceinline__ void accept_sequence(const int32_t *cand_tok, const i
 }
 
 __global__ void __launch_bounds__(128)
-verify_accept_kernel(const int32_t *cand_tok, const float2 *part, int K, int n, int V, int skew, int shift, int slots,
+verify_accept_kernel(const int32_t *cand_tok, const float2 *part, int K, int n, int V, int skew, int shift, int rows, int warps,
                      int vec_per_warp, int32_t *g_out, int g_in_smem, int32_t *accept_len, int32_t *best_cand,
                      int32_t *next_tok, int32_t *err) {
     // The sequence's arg-max table is re-read by other threads for the prefix match: from shared memory
@@ -236,17 +242,22 @@ verify_accept_kernel(const int32_t *cand_tok, const float2 *part, int K, int n, 
     load_candidate(cand_tok, (size_t)b * K + threadIdx.x, n, (int)threadIdx.x < K, ctok);
     for (int r = threadIdx.x; r < rows_b; r += blockDim.x) {
         const size_t gr = (size_t)b * rows_b + r;
-        const float2 *pr = part + gr * slots;
-        // the row's slots are the warps whose ranges its vectors touch
+        // the row's pieces are the warps whose ranges its vectors touch
         const long long rs = skew + (long long)gr * V, v0 = rs >> shift, v1 = (rs + V - 1) >> shift;
-        const int chunks = (v1 >> 32) == 0 ? (int)((uint32_t)v1 / (uint32_t)vec_per_warp - (uint32_t)v0 / (uint32_t)vec_per_warp) + 1
-                                           : (int)(v1 / vec_per_warp - v0 / vec_per_warp) + 1;
+        const bool narrow = (v1 >> 32) == 0;
+        const long long w0 = narrow ? (uint32_t)v0 / (uint32_t)vec_per_warp : v0 / vec_per_warp;
+        const int chunks = (int)((narrow ? (uint32_t)v1 / (uint32_t)vec_per_warp : v1 / vec_per_warp) - w0) + 1;
+        const float2 *first = part + first_piece(warps, rows, (int)gr, w0), *rest = part + w0;
+        if (chunks == 1) {   // finished by its warp
+            if (g_in_smem) g_s[r] = __ldcg(g_out + gr);
+            continue;
+        }
         float best = -INFINITY;
         int arg = 0;   // a row without any value above -inf (all NaN) yields 0
         for (int c0 = 0; c0 < chunks; c0 += kBatch) {
             float2 v[kBatch];
 #pragma unroll
-            for (int j = 0; j < kBatch; ++j) v[j] = c0 + j < chunks ? __ldcg(pr + c0 + j) : make_float2(-INFINITY, 0.0f);
+            for (int j = 0; j < kBatch; ++j) v[j] = c0 + j < chunks ? __ldcg(c0 + j == 0 ? first : rest + c0 + j) : make_float2(-INFINITY, 0.0f);
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
                 const bool take = v[j].x > best;   // chunks ascend, so the first maximum wins
@@ -446,11 +457,14 @@ VerifyPlan make_verify_plan(int B, int K, int n, int V, int dtype) {
     if (c < 32 * kStreamUnroll) c = 32 * kStreamUnroll;
     if (c > (1ll << 30)) c = 1ll << 30;
     p.vec_per_warp = (int)c;
-    const long long row_vec = (V + epv - 1) / epv + 1;   // most vectors that one row touches
-    p.slots = (int)((row_vec + c - 2) / c + 1);
+    p.warps = (int)((total + c - 1) / c);
     p.off_g = kWsAlign;
     p.off_part = align_up(p.off_g + sizeof(int32_t) * (size_t)p.rows, kWsAlign);
-    p.total = align_up(p.off_part + sizeof(float2) * (size_t)p.rows * p.slots, kWsAlign);
+    // at most a partial behind every border and a first piece for every row that crosses one.  Never less than 4 bytes per
+    // candidate, the early-exit form's match lengths.
+    const size_t partials = sizeof(float2) * ((size_t)p.warps + (p.rows < p.warps ? p.rows : p.warps));
+    const size_t lengths = sizeof(int32_t) * (size_t)B * K;
+    p.total = align_up(p.off_part + (partials > lengths ? partials : lengths), kWsAlign);
     return p;
 }
 
@@ -475,12 +489,12 @@ int launch_verify(const int32_t *cand_tok, const void *base_logits, int dtype, i
     const long long warps = (total + plan.vec_per_warp - 1) / plan.vec_per_warp;
     const unsigned grid = (unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
     SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_stream_kernel<true> : verify_stream_kernel<false>, dim3(grid), dim3(kArgmaxThreads),
-                             0, st, base, skew, plan.rows, V, total, plan.vec_per_warp, plan.slots, part));
+                             0, st, base, skew, plan.rows, V, total, plan.vec_per_warp, plan.warps, g, part));
     size_t smem = sizeof(int32_t) * (size_t)rows_b;
     const int g_in_smem = smem <= 40 * 1024;
     if (!g_in_smem) smem = 0;
     SPEC_CUDA_TRY(launch_pdl(verify_accept_kernel, dim3(B), dim3(128), smem, st, cand_tok, (const float2 *)part, K, n, V, skew,
-                             shift, plan.slots, plan.vec_per_warp, g, g_in_smem, accept_len, best_cand, next_tok, err));
+                             shift, plan.rows, plan.warps, plan.vec_per_warp, g, g_in_smem, accept_len, best_cand, next_tok, err));
     return SPEC_OK;
 }
 

@@ -46,6 +46,11 @@ def test_verify_host_side_validation(binding):
     assert lib.spec_verify_workspace_bytes(2, 4, 3, 100, 7) == 0
     need = lib.spec_verify_workspace_bytes(2, 4, 3, 1000, 0)
     assert need >= 256 + 4 * 2 * 4 * 4 and need % 256 == 0
+    # twelve bytes a row are enough wherever rows are many or short
+    for dtype in (0, 1):
+        for shape in ((5437, 4, 3, 1001), (21, 1024, 3, 21), (21840, 1, 3, 1023), (1, 4096, 2, 5), (7, 1365, 8, 9)):
+            rows = shape[0] * shape[1] * (shape[2] + 1)
+            assert lib.spec_verify_workspace_bytes(*shape, dtype) <= 1024 + 12 * rows
     # null pointers and bad shapes are rejected before anything is enqueued
     assert lib.spec_verify(None, None, 0, 1, 1, 1, 8, None, None, None, None, C.c_size_t(0), None) == binding.SPEC_ERR_INVALID_ARG
     one = C.c_void_p(256)

@@ -53,6 +53,13 @@ def test_two_calls_in_a_row_match_the_workspace_entry_point(B):
     _both(B, *_case((3, 16, 3, 8000), 1, torch.bfloat16))
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("shape", [(21, 1024, 3, 21), (7, 1365, 8, 9), (28, 768, 3, 1001)])
+def test_as_many_rows_of_odd_length_as_twelve_bytes_each_leave_room_for(B, shape, dtype):
+    """86000 rows that are not whole vectors, among them sequences whose arg-max table is too long for shared memory."""
+    assert _both(B, *_case(shape, 3, dtype)).max().item() > 0
+
+
 def test_benchmark_shape_fits_and_oversized_problem_is_refused(B):
     cfg = synth.CONFIGS["llama2-13b"]
     assert B.spec_verify_workspace_bytes(cfg.B, cfg.K, cfg.n, cfg.V, B.SPEC_BF16) <= B.SPEC_VERIFY_STATIC_SCRATCH_BYTES

@@ -440,9 +440,16 @@ size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 // One kernel when a sequence is little enough for one CTA to read in less time than a second kernel costs.  One CTA reads
 // about 65 GB/s: 64 KB 4.9 us per call against 6.8 us in two kernels (both bound by the host), 256 KB 7.6 against 9.5 alone
 // but 65.0 against 63.6 us inside a decoding step, 512 KB 11.6 against 9.7, 1 MB 15.3 against 9.5.
+// Its CTA has an SM to itself, so that more sequences than SMs take turns of about 3.3 us, while the two-kernel form reads them all
+// in one wave; that one walks the rows of a warp's range one by one, about 0.8 us each (256 vectors hold 8 * 256 / V rows of bf16),
+// and is the slower the shorter the rows.  us per call, one kernel / two, four candidates of four rows: V 64, 444 sequences
+// 10.6 / 39.7, 1000 23.9 / 41.9, 3000 69 / 44; V 256, 256 7.2 / 13.1, 444 10.6 / 11.2, 1000 24 / 16; V 1024, 148 4.6 / 6.5,
+// 149 7.3 / 6.4, 1000 25.8 / 13.9; V 4096, 148 5.8 / 8.5, 149 10.1 / 8.4, 1000 40.6 / 24.8.
 constexpr long long kSeqMaxBytes = 128 << 10;
-bool one_kernel_form(int rows_b, int V, int dtype) {
-    return rows_b <= kSeqMaxRows && (long long)rows_b * V * (dtype == SPEC_BF16 ? 2 : 4) <= kSeqMaxBytes;
+bool one_kernel_form(int B, int rows_b, int V, int dtype) {
+    const long long turns = ((long long)B + num_sms() - 1) / num_sms();
+    return rows_b <= kSeqMaxRows && (long long)rows_b * V * (dtype == SPEC_BF16 ? 2 : 4) <= kSeqMaxBytes &&
+           (turns - 1) * V <= 64 * (dtype == SPEC_BF16 ? Elem<true>::kEpv : Elem<false>::kEpv);
 }
 
 // Resident CTAs per SM of the streaming kernel (launch bound above) times the SM count gives the
@@ -478,7 +485,7 @@ int launch_verify(const int32_t *cand_tok, const void *base_logits, int dtype, i
     const int shift = bf16 ? 3 : 2, esz = bf16 ? 2 : 4;
     const char *base = (const char *)((uintptr_t)base_logits & ~(uintptr_t)15);
     const int skew = (int)(((uintptr_t)base_logits & 15) / esz), rows_b = K * (n + 1);
-    if (one_kernel_form(rows_b, V, dtype)) {
+    if (one_kernel_form(B, rows_b, V, dtype)) {
         const size_t smem = (sizeof(unsigned long long) + sizeof(int32_t)) * (size_t)rows_b;
         SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_seq_kernel<true> : verify_seq_kernel<false>, dim3((unsigned)B), dim3(kSeqThreads),
                                  smem, st, base, skew, cand_tok, K, n, V, g, accept_len, best_cand, next_tok, err));

@@ -39,6 +39,19 @@ def ws_view(ws: torch.Tensor, offset: int, count: int, dtype: torch.dtype) -> to
     return ws[offset:offset + nbytes].view(dtype)
 
 
+def kernels_launched(call) -> int:
+    """Kernels that `call` enqueues on the current stream (all its tensors made beforehand), counted in a captured graph."""
+    from cuda.bindings import runtime
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        call()
+    raw = runtime.cudaGraph_t(graph.raw_cuda_graph())
+    count = runtime.cudaGraphGetNodes(raw)[2]
+    nodes = runtime.cudaGraphGetNodes(raw, count)[1]
+    types = [runtime.cudaGraphNodeGetType(node)[1] for node in nodes]
+    return types.count(runtime.cudaGraphNodeType.cudaGraphNodeTypeKernel)
+
+
 LOGIT_TOL = 2e-2      # max-abs tolerance on head logits (bf16 operands, fp32 accumulation)
 TIE_TOL = 1e-3        # logits closer than this may be ordered either way
 

@@ -6,7 +6,7 @@ import torch
 
 import oracle
 from paper_2404_19124_b200 import synth
-from helpers import ws_view
+from helpers import kernels_launched, ws_view
 
 pytestmark = pytest.mark.gpu
 
@@ -57,6 +57,26 @@ def test_rows_that_are_not_whole_vectors(B, shape, dtype):
     for k in range(K):
         cand[:, k, :k % (n + 1)] = am[:, k, :k % (n + 1)].to(torch.int32)
     _check(B, cand, x.cuda())
+
+
+@pytest.mark.parametrize("shape,dtype,kernels", [((148, 2, 1, 8192), torch.bfloat16, 1), ((149, 2, 1, 8192), torch.bfloat16, 2),
+                                                 ((149, 3, 2, 512), torch.bfloat16, 1), ((149, 3, 2, 513), torch.bfloat16, 2),
+                                                 ((296, 2, 1, 256), torch.float32, 1), ((296, 2, 1, 257), torch.float32, 2),
+                                                 ((1332, 2, 1, 64), torch.bfloat16, 1), ((1333, 2, 1, 64), torch.bfloat16, 2)])
+def test_many_short_sequences(B, shape, dtype, kernels):
+    """More sequences than SMs: one kernel only while the turns they take are few for the length of a row."""
+    Bn, K, n, V = shape
+    g = torch.Generator().manual_seed(V)
+    x = torch.randn(Bn, K, n + 1, V, generator=g).to(dtype)
+    cand = torch.randint(0, V, (Bn, K, n), generator=g, dtype=torch.int64).to(torch.int32)
+    am = x.float().argmax(-1).to(torch.int32)
+    cand[::2, -1] = am[::2, -1, :n]
+    _check(B, cand, x.cuda())
+    cand, x = cand.cuda(), x.cuda()
+    out = [torch.empty(Bn, dtype=torch.int32, device="cuda") for _ in range(3)]
+    ws = torch.empty(B.spec_verify_workspace_bytes(*shape, B.SPEC_BF16 if dtype == torch.bfloat16 else B.SPEC_F32),
+                     dtype=torch.uint8, device="cuda")
+    assert kernels_launched(lambda: B.spec_verify(cand, x, *out, workspace=ws)) == kernels
 
 
 @pytest.mark.parametrize("V", [1000, 30001])

@@ -10,6 +10,11 @@
  *     the stream has finished.
  *   - spec_draft / spec_verify only enqueue work on `cuda_stream` (a cudaStream_t passed
  *     as void*; NULL = default stream) and never synchronise.
+ *   - weights (spec_weights_t, and the e4m3 copies of heads) are read ahead of stream order: kernels start, and
+ *     request weights, once the kernel before them has ended or has allowed its dependents to start (programmatic
+ *     dependent launch).  An ordinary kernel or copy that rewrites weights earlier on the stream has ended by then.
+ *     One that lets its dependents start early (the kernels of this library do) must not write them, unless the
+ *     stream is synchronised before the next call that reads them.
  *   - errors found on the host (bad pointers, shapes, workspace too small) are returned
  *     at once and nothing is enqueued.  Errors found on the device (token id outside
  *     [0, V), a bounded wait that ran out) are recorded in an error word at the start of

@@ -179,9 +179,6 @@ __global__ void __launch_bounds__(kSmallThreads, 1) draft_small_kernel(const __g
     float *node_score = (float *)(node_tok + (n + 1) * kLevel);     // ... their scores, two sets by turns
     griddep_launch();
     float *ln = (float *)(smem + a.off_ln);   // [n][2][d]: the LayerNorm parameters
-    for (int l = 0; l < n; ++l)
-        for (int i = tid; i < 2 * d; i += kSmallThreads)
-            ln[l * 2 * d + i] = i < d ? a.w.ln_gamma[l][i] : a.w.ln_beta[l][i - d];
     for (int i = tid * 16; i < a.off_logits; i += kSmallThreads * 16) *(uint4 *)(smem + i) = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
     griddep_wait();
@@ -199,6 +196,17 @@ __global__ void __launch_bounds__(kSmallThreads, 1) draft_small_kernel(const __g
     for (int i = gw; i < tiles_d * a.mix[0].p_splits; i += kWarpsAll)
         project((const uint16_t *)a.w.proj[0], d, a.w.d_base, a.mix[0].p_splits, i, x, a.pitch_base, a.B, (float *)a.mix[0].P,
                 a.mix[0].p_split_stride, lane);
+    // The LayerNorm parameters, like everything else not before the wait: a kernel earlier in the stream may have written them.
+    // Loaded by the warps that the projection leaves idle (32 tiles times four splits are half of the cluster's warps) and only
+    // behind its code: ahead of it, or by all warps, the smallest step took 0.4 us longer.
+    if (warp >= kSmallWarps / 2) {
+        const int u = tid - kSmallThreads / 2;
+#pragma unroll 1
+        for (int i = u; i < n * d / 2; i += kSmallThreads / 2) {
+            const int l = i / (d / 2), j = 4 * (i - l * (d / 2));
+            *(float4 *)(ln + l * 2 * d + j) = __ldcg((const float4 *)(j < d ? a.w.ln_gamma[l] + j : a.w.ln_beta[l] + (j - d)));
+        }
+    }
     small_barrier();   // (also: every CTA of the cluster runs, its shared memory may be written)
 
     int nodes = a.B;

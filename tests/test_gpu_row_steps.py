@@ -240,3 +240,36 @@ def test_states_are_the_same_bits_in_every_kernel(B, k, d):
     for a, b in zip(*got):
         assert torch.equal(a, b)
     B.spec_destroy(h)
+
+
+@pytest.mark.parametrize("d,what", [(256, "ln_gamma"), (256, "ln_beta"), (512, "ln_gamma"), (40, "ln_beta"), (256, "proj"), (256, "head")])
+def test_a_small_draft_reads_its_weights_in_stream_order(B, d, what):
+    """spec_next_ctx, whose kernel lets its dependents start at once and waits behind a long verification itself, writes into
+    the weights of the draft that follows it."""
+    cfg = small_cfg(d_base=256, d_inner=d, V=600, topk=(3, 2), K=6, B=1, seed=d)
+    gw = weights_to_cuda(synth.make_weights(cfg))
+    ctx, tok = (t.cuda() for t in synth.make_draft_inputs(cfg))
+    h = B.spec_create(gw)
+    target = getattr(gw, what)[0].view(torch.bfloat16).reshape(1, -1)
+    old = target.clone()
+    new = (getattr(gw, what)[0] * -0.75).view(torch.bfloat16).reshape(1, -1)
+    state = new.view(1, 1, 1, -1).expand(1, 1, 2, -1).contiguous()
+    zero = torch.zeros(1, dtype=torch.int32, device="cuda")
+    logits = torch.zeros((16, 8, 4, 128256), dtype=torch.bfloat16, device="cuda")
+    cand = torch.zeros((16, 8, 3), dtype=torch.int32, device="cuda")
+    res = [torch.empty(16, dtype=torch.int32, device="cuda") for _ in range(3)]
+    vws = B.spec_verify(cand, logits)[3]
+    ct, lp, ws = B.spec_draft(h, ctx, tok, cfg.topk, cfg.K)
+    before = lp.clone()
+    for _ in range(5):
+        target.copy_(old)
+        torch.cuda.synchronize()
+        B.spec_verify(cand, logits, *res, workspace=vws)
+        B.spec_next_ctx(state, zero, zero, ctx_state=target)
+        B.spec_draft(h, ctx, tok, cfg.topk, cfg.K, cand_tok=ct, cand_logp=lp, workspace=ws)
+        torch.cuda.synchronize()
+        got = ct.clone(), lp.clone()
+        B.spec_draft(h, ctx, tok, cfg.topk, cfg.K, cand_tok=ct, cand_logp=lp, workspace=ws)
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], ct) and torch.equal(got[1], lp) and not torch.equal(lp, before)
+    B.spec_destroy(h)

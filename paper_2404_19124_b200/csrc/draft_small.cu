@@ -16,8 +16,6 @@
 // into L1 before the mix gains nothing, nor do the arguments in shared memory; sums and lists of the selection in separate
 // warps, which must then leave the logits as they are, cost it 2 us.  (Loads without predicates and the LayerNorm parameters,
 // the tokens and the leaves in shared memory: 31.5 -> 28.2 us for the step.)
-#include <mutex>
-
 #include "row_ops.cuh"
 
 namespace spec {
@@ -459,30 +457,24 @@ int launch_draft_small(const spec_weights_t &w, const void *ctx, int B, const in
     a.off_ln = (off + 127) / 128 * 128;
     off = a.off_ln + n * 2 * 4 * w.d_inner;
     if (off > kMaxSmem) return SPEC_ERR_SHAPE;
-    int dev = 0;
-    SPEC_CUDA_TRY(cudaGetDevice(&dev));
-    {
-        static std::mutex mutex;
-        static int clusters[64] = {};   // per device: 1 + the clusters that fit, 0: not asked yet
-        std::lock_guard<std::mutex> lock(mutex);
-        int fit = dev >= 0 && dev < 64 ? clusters[dev] - 1 : -1;
-        if (fit < 0) {
-            SPEC_CUDA_TRY(cudaFuncSetAttribute(draft_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
-            SPEC_CUDA_TRY(cudaFuncSetAttribute(draft_small_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(kCtas);
-            cfg.blockDim = dim3(kSmallThreads);
-            cfg.dynamicSmemBytes = kMaxSmem;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = kCtas;
-            attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            SPEC_CUDA_TRY(cudaOccupancyMaxActiveClusters(&fit, draft_small_kernel, &cfg));
-            if (dev >= 0 && dev < 64) clusters[dev] = fit + 1;
-        }
-        if (fit < 1) return SPEC_ERR_SHAPE;   // (a context with fewer SMs than a cluster wants)
+    // Asked for on every call (0.3 us), for the stream and the context that it is made in: another one may have fewer SMs.
+    SPEC_CUDA_TRY(cudaFuncSetAttribute(draft_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
+    SPEC_CUDA_TRY(cudaFuncSetAttribute(draft_small_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kCtas);
+    cfg.blockDim = dim3(kSmallThreads);
+    cfg.dynamicSmemBytes = (size_t)off;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kCtas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int fit = 0;
+    if (cudaOccupancyMaxActiveClusters(&fit, draft_small_kernel, &cfg) != cudaSuccess || fit < 1) {
+        (void)cudaGetLastError();
+        return SPEC_ERR_SHAPE;   // fewer SMs side by side than a cluster wants
     }
     SPEC_CUDA_TRY(launch_pdl_cluster(draft_small_kernel, dim3(kCtas), dim3(kSmallThreads), (size_t)off, kCtas, st, a));
     return SPEC_OK;

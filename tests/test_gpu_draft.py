@@ -132,7 +132,7 @@ def test_head_topk_exact_ties_prefer_lower_token_id(B, swapped):
 
 
 def _draft_and_check(B, cfg, seqs=None, impl=0, check_levels=False, tie_weights=False, fp8=False, fp8_rows=None,
-                     swap=None):
+                     swap=None, chain=False):
     """Runs spec_draft at the config's full batch and compares the sequences in `seqs`
     (default: all) with the oracle, one sequence at a time (sequences are independent).
     tie_weights: every head after the first aliases the second head's tensors (the weight-tied
@@ -154,6 +154,8 @@ def _draft_and_check(B, cfg, seqs=None, impl=0, check_levels=False, tie_weights=
     if swap is not None:   # levels of up to `swap` nodes run the head with the nodes as MMA columns (0: none)
         B.spec_set_option(h, B.SPEC_OPT_HEAD_SWAP_MAX_ROWS, swap)
         B.spec_set_option(h, B.SPEC_OPT_HEAD_PAIR, 1 if swap else 0)   # and levels of > 128 nodes on CTA pairs / not
+    if chain:    # one kernel per step also where the whole draft would be one
+        B.spec_set_option(h, B.SPEC_OPT_HEAD_PAIR, 0)
     if fp8:      # levels of up to 128 nodes multiply in e4m3 and re-score a short list exactly
         B.spec_attach_fp8_heads(h)
         if fp8_rows is not None:   # also levels with more than the default 128 nodes
@@ -202,9 +204,9 @@ def _draft_and_check(B, cfg, seqs=None, impl=0, check_levels=False, tie_weights=
     return chk
 
 
-@pytest.mark.parametrize("impl", [0, 1])
-def test_draft_tiny_config(B, impl):
-    chk = _draft_and_check(B, synth.CONFIGS["tiny"], impl=impl, check_levels=True)
+@pytest.mark.parametrize("impl,chain", [(0, False), (0, True), (1, False)])
+def test_draft_tiny_config(B, impl, chain):
+    chk = _draft_and_check(B, synth.CONFIGS["tiny"], impl=impl, check_levels=True, chain=chain)
     assert chk.tolerated == 0
 
 
@@ -255,11 +257,12 @@ def test_draft_single_candidate_at_production_width(B, name, Bn):
     assert chk.tolerated <= 1
 
 
+@pytest.mark.parametrize("chain", [False, True])
 @pytest.mark.parametrize("topk,K", [((2, 2, 2), 5), ((2, 1, 2, 1), 3), ((1, 2, 1), 2)])
-def test_draft_one_or_two_children_per_node(B, topk, K):
+def test_draft_one_or_two_children_per_node(B, topk, K, chain):
     """Branching factors of one and two: the merge of a level writes the children's states in the same launch."""
     cfg = small_cfg(d_base=96, d_inner=160, V=3000, topk=topk, K=K, B=5, seed=11 + len(topk))
-    chk = _draft_and_check(B, cfg, check_levels=True)
+    chk = _draft_and_check(B, cfg, check_levels=True, chain=chain)
     assert chk.tolerated <= 1
 
 
@@ -383,13 +386,16 @@ def test_draft_is_deterministic_and_stream_ordered(B):
     B.spec_destroy(h)
 
 
-def test_draft_token_out_of_range_sets_error_word_without_trapping(B):
+@pytest.mark.parametrize("chain", [False, True])
+def test_draft_token_out_of_range_sets_error_word_without_trapping(B, chain):
     cfg = synth.CONFIGS["tiny"]
     sw, ow, gw = _setup(cfg)
     ctx, tok = synth.make_draft_inputs(cfg)
     bad = tok.clone()
     bad[0] = cfg.V + 5
     h = B.spec_create(gw)
+    if chain:
+        B.spec_set_option(h, B.SPEC_OPT_HEAD_PAIR, 0)
     _, _, ws = B.spec_draft(h, ctx.cuda(), bad.cuda(), cfg.topk, cfg.K)
     assert B.spec_poll_error(ws) == B.SPEC_ERR_TOKEN_RANGE
     assert B.spec_poll_error(ws) == 0                       # cleared by the poll

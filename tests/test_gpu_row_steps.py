@@ -6,7 +6,7 @@ import torch
 
 import oracle
 from paper_2404_19124_b200 import synth
-from helpers import LOGIT_TOL, TIE_TOL, DraftChecker, small_cfg, to_oracle_weights, weights_to_cuda
+from helpers import LOGIT_TOL, TIE_TOL, DraftChecker, kernels_launched, small_cfg, to_oracle_weights, weights_to_cuda
 
 pytestmark = pytest.mark.gpu
 
@@ -126,20 +126,26 @@ def test_e4m3_levels_with_and_without_swapped_operands(B, B_, topk, V, d, swap):
                        e4m3=True, swap=swap)
 
 
-@pytest.mark.parametrize("B_,topk,V,d_base,d", [(1, (4, 3, 2), 1024, 256, 256), (16, (1, 1, 1), 1000, 64, 512),
-                                                 (17, (1, 1), 1000, 64, 512), (3, (5, 1, 2), 1003, 40, 264),
-                                                 (2, (8, 8), 2047, 8, 128), (1, (8, 2, 8), 600, 2048, 8),
-                                                 (2, (8,), 16, 72, 504), (5, (3, 1, 2), 257, 1000, 248),
-                                                 (1, (4, 2, 2, 2), 2048, 256, 512), (9, (1, 1, 4), 129, 2040, 40),
-                                                 (1, (4, 3), 3100, 64, 512), (1, (4, 3), 3300, 64, 512)])
-def test_small_drafts_are_one_kernel(B, B_, topk, V, d_base, d):
+@pytest.mark.parametrize("chain", [False, True])
+@pytest.mark.parametrize("B_,topk,V,d_base,d,one", [(1, (4, 3, 2), 1024, 256, 256, True), (16, (1, 1, 1), 1000, 64, 512, True),
+                                                     (17, (1, 1), 1000, 64, 512, False), (3, (5, 1, 2), 1003, 40, 264, True),
+                                                     (2, (8, 8), 2047, 8, 128, True), (1, (8, 2, 8), 600, 2048, 8, True),
+                                                     (2, (8,), 16, 72, 504, True), (5, (3, 1, 2), 257, 1000, 248, True),
+                                                     (1, (4, 2, 2, 2), 2048, 256, 512, True), (9, (1, 1, 4), 129, 2040, 40, True),
+                                                     (1, (4, 3), 3100, 64, 512, True), (1, (4, 3), 3300, 64, 512, True),
+                                                     (1, (4, 3), 3322, 64, 512, False), (1, (2, 2), 1000, 64, 520, False),
+                                                     (1, (2, 2), 1000, 2056, 64, False), (16, (1, 1), 100000, 64, 8, False)])
+def test_small_drafts_are_one_kernel(B, B_, topk, V, d_base, d, one, chain):
     """Node counts, widths and vocabularies at the edges of what one cluster takes: 16 and 17 nodes, fewer rows than warps,
-    CTAs without any vocabulary row, K ranges that end inside a group of 32, sizes on both sides of the limit."""
-    _check_every_level(B, small_cfg(d_base=d_base, d_inner=d, V=V, topk=topk, K=int(np.prod(topk)), B=B_, seed=B_ + d))
+    CTAs without any vocabulary row, K ranges that end inside a group of 32, sizes on both sides of the limits, and logits of
+    16 nodes that do not fit its shared memory.  Each also as the chain of kernels that an option asks for."""
+    _check_every_level(B, small_cfg(d_base=d_base, d_inner=d, V=V, topk=topk, K=int(np.prod(topk)), B=B_, seed=B_ + d),
+                       pair=0 if chain else None, one_kernel=one and not chain)
 
 
-def _check_every_level(B, cfg, e4m3=False, swap=None):
-    """Every level is re-derived by the oracle from the GPU's parent level for the first and the last sequence."""
+def _check_every_level(B, cfg, e4m3=False, swap=None, pair=None, one_kernel=None):
+    """Every level is re-derived by the oracle from the GPU's parent level for the first and the last sequence; one_kernel:
+    whether the draft is to be a single kernel."""
     B_, topk, K, d = cfg.B, cfg.topk, cfg.K, cfg.d_inner
     sw = synth.make_weights(cfg)
     ow, gw = to_oracle_weights(sw), weights_to_cuda(sw)
@@ -149,7 +155,12 @@ def _check_every_level(B, cfg, e4m3=False, swap=None):
         B.spec_attach_fp8_heads(h)
     if swap is not None:
         B.spec_set_option(h, B.SPEC_OPT_HEAD_SWAP_MAX_ROWS, swap)
-    ct, lp, ws = B.spec_draft(h, ctx.cuda(), tok.cuda(), topk, K)
+    if pair is not None:
+        B.spec_set_option(h, B.SPEC_OPT_HEAD_PAIR, pair)
+    gctx, gtok = ctx.cuda(), tok.cuda()
+    ct, lp, ws = B.spec_draft(h, gctx, gtok, topk, K)
+    if one_kernel is not None:
+        assert one_kernel == (kernels_launched(lambda: B.spec_draft(h, gctx, gtok, topk, K, ct, lp, ws)) == 1)
     assert B.spec_poll_error(ws) == 0
     lay = B.spec_draft_layout(h, B_, topk, K)
     view = lambda off, n, dt: ws[off:off + n * torch.empty((), dtype=dt).element_size()].view(dt)

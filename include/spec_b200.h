@@ -67,9 +67,10 @@ enum spec_option {
     SPEC_OPT_HEAD_SWAP_MAX_ROWS = 5, /* levels with at most this many nodes (0 .. 128) run the head GEMM
                                   with the weight matrix on the 128-row side of the MMA and the nodes
                                   as columns, so the tensor work follows the number of nodes; 0 = never;
-                                  -1 (default) = automatic: up to 32 nodes, up to 64 when the
-                                  vocabulary gives every CTA a full 128-row tile.  Ignored
-                                  while SPEC_OPT_HEAD_BLOCK_N forces a tile width.              */
+                                  -1 (default) = automatic: up to 32 nodes, up to 48 (bf16 heads)
+                                  when the vocabulary has 30 rows per SM, up to 64 when it has
+                                  128.  e4m3 levels follow it too.  Ignored while
+                                  SPEC_OPT_HEAD_BLOCK_N forces a tile width.                    */
     SPEC_OPT_GEMM_PRODUCERS = 6, /* 1 or 2 (default) threads per CTA issue the TMA copies of the GEMM
                                   kernels; process-wide, not per handle                        */
     SPEC_OPT_HEAD_PAIR = 7       /* 1: levels of more than 128 nodes run the head GEMM on pairs of CTAs
@@ -96,7 +97,9 @@ typedef struct {
     float ln_eps;
 } spec_weights_t;
 
-/* Byte offsets into a draft workspace (for tests and debugging; N_l = B * prod_{j<l} topk[j]). */
+/* Byte offsets into a draft workspace (for tests and debugging; N_l = B * prod_{j<l} topk[j]).  A draft that runs as one
+ * kernel (see spec_draft) writes tok, score and state; it leaves part_* unwritten, proj holds two buffers in turns,
+ * and block_n / n_tiles are what the chain of kernels would use. */
 typedef struct {
     uint64_t total_bytes;
     uint64_t error_word;                  /* int32                                            */
@@ -137,6 +140,11 @@ int spec_set_option(spec_handle_t h, int option, int value);
  *   workspace  dev, 256-byte aligned, >= spec_draft_workspace_bytes(...).  Need not be zeroed: the
  *              first kernel of the call clears the header (error word at byte 0, one int32
  *              counter per sequence from byte 256 on).
+ * The draft of a small speculator (d_inner <= 512, d_base <= 2048, at most 16 nodes on every level that has a head, one or
+ * two million head elements per level) runs as one kernel, a cluster of 16 CTAs that need 16 free SMs of one GPC at the
+ * same time; beside long kernels on other streams it starts once they leave that room.  Setting any of SPEC_OPT_GEMM_IMPL,
+ * _HEAD_BLOCK_N, _PROJ_BLOCK_N, _PROFILE, _HEAD_SWAP_MAX_ROWS or _HEAD_PAIR away from its default asks for the chain of
+ * kernels instead, whatever the value changes otherwise.
  */
 size_t spec_draft_workspace_bytes(spec_handle_t h, int B, const int32_t *topk, int K);
 int spec_draft_layout(spec_handle_t h, int B, const int32_t *topk, int K, spec_draft_layout_t *out /*host*/);
@@ -184,8 +192,8 @@ int spec_verify(const int32_t *cand_tok, const void *base_logits, int logits_dty
 
 /* Early-exit form of spec_verify (Sec. 1: everything after a candidate's first rejected token is
  * discarded, so the base model's logits behind it need not be looked at).  Same arguments, same
- * three results.  One thread block per candidate reads its rows in order and stops after the first
- * row whose arg-max differs from the speculated token: the bytes read fall from B K (n+1) V elements
+ * three results.  One thread block, or a cluster of up to eight, per candidate reads its rows in order and stops after
+ * the first row whose arg-max differs from the speculated token: the bytes read fall from B K (n+1) V elements
  * to sum over the candidates of (m[b,k] + 1) V.  In the workspace, g holds -1 for rows that were not
  * read.  Worth it when many candidates fail early or the tensor is large; when nearly all rows are
  * needed the one-pass streaming form is faster.  Rows must be whole 16-byte vectors and base_logits

@@ -16,14 +16,13 @@ constexpr int kRowThreads = 256;
 constexpr int kFusedMixMaxChildren = 2;
 constexpr int kMergeThreads = 160;   // one list per thread up to V = 35000 (a CTA of the head GEMM leaves one)
 
-// Rows of up to 4096 elements: at most 128 registers, so that two CTAs fit beside a resident GEMM CTA.
+// Rows of up to 2048 elements: at most 128 registers, so that two CTAs fit beside a resident GEMM CTA.
 __global__ void __launch_bounds__(kRowThreads, 2) mix_ln_gelu_kernel(MixArgs m) {
     __shared__ float red[32];
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, t = __ldcg(m.tok + r);
-    if (m.d <= 8 * kRowThreads) mix_ln_gelu_row<kRowThreads, 1, 2, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
-    else mix_ln_gelu_row<kRowThreads, 2, 2, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
+    mix_ln_gelu_row<kRowThreads, 1, 2, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
 }
 
 // Rows of 2049 to 4096 elements in levels of at most one CTA per SM: 512 threads, one 8-element group each.  The
@@ -115,7 +114,7 @@ __global__ void __launch_bounds__(256) draft_init_kernel(int32_t *hdr, int words
 
 template <int kLen>
 __global__ void __launch_bounds__(kMergeThreads) merge_expand_kernel(MergeArgs g) {
-    extern __shared__ LeafKey merge_keys[];   // [Lpad] when the prune is folded in, else nothing
+    extern __shared__ LeafKey merge_keys[];   // prune_smem_bytes when the prune is folded in, else nothing
     __shared__ Scratch sc;
     __shared__ int last_of_sequence;
     griddep_launch();
@@ -143,10 +142,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) merge_mix_kernel(MergeMixArgs 
     griddep_wait();
     const int r = blockIdx.x, tid = threadIdx.x;
     const int tok = merge_expand_row<kRowThreads, 4, BlockSync>(a.merge, r, tid, &sc).id;
-    if (a.mix.d <= 8 * kRowThreads)
-        mix_children<kRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
-    else
-        mix_children<kRowThreads, 2, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
+    mix_children<kRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
 }
 
 // Rows of 2049 to 4096 elements: 512 threads, one 8-element group each, like mix_ln_gelu_512_kernel (single-
@@ -257,7 +253,7 @@ merge_shards_kernel(const char *slots, size_t slot_bytes, int n_ranks, int rows,
 
 __global__ void __launch_bounds__(kRowThreads)
 prune_kernel(const float *leaf_score, PruneArgs pa, int L, int Lpad, int K, int32_t *cand_tok, float *cand_logp) {
-    extern __shared__ LeafKey keys[];   // [Lpad]
+    extern __shared__ LeafKey keys[];   // prune_smem_bytes
     griddep_launch();
     griddep_wait();
     prune_sequence<kRowThreads, BlockSync>(leaf_score, pa, L, Lpad, K, cand_tok, cand_logp, blockIdx.x, threadIdx.x,
@@ -272,10 +268,10 @@ int launch_mix_ln_gelu(const MixArgs &m, int rows, cudaStream_t st) {
         SPEC_CUDA_TRY(launch_pdl(mix_ln_gelu_waves_kernel, dim3(rows), dim3((d_inner + 511) / 512 * 32), 0, st, m));
     } else if (d_inner <= 8 * kRowThreads * 2 && rows > num_sms()) {
         SPEC_CUDA_TRY(launch_pdl(mix_ln_gelu_many_kernel, dim3(rows), dim3(kRowThreads), 0, st, m));
-    } else if (d_inner <= 8 * kWideRowThreads && d_inner > 8 * kRowThreads) {
-        SPEC_CUDA_TRY(launch_pdl(mix_ln_gelu_512_kernel, dim3(rows), dim3(kWideRowThreads), 0, st, m));
-    } else if (d_inner <= 8 * kRowThreads * 2) {
+    } else if (d_inner <= 8 * kRowThreads) {
         SPEC_CUDA_TRY(launch_pdl(mix_ln_gelu_kernel, dim3(rows), dim3(kRowThreads), 0, st, m));
+    } else if (d_inner <= 8 * kWideRowThreads) {
+        SPEC_CUDA_TRY(launch_pdl(mix_ln_gelu_512_kernel, dim3(rows), dim3(kWideRowThreads), 0, st, m));
     } else if (d_inner <= 8 * kRowThreads * 8) {
         SPEC_CUDA_TRY(launch_pdl(mix_ln_gelu_mid_kernel, dim3(rows), dim3(kRowThreads), 0, st, m));
     } else {
@@ -300,8 +296,9 @@ int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st) {
     return SPEC_OK;
 }
 
-// Returns SPEC_ERR_SHAPE when the fused form does not cover the shape (rows wider than 4096 elements, an e4m3
-// copy of the states wanted): the caller then launches the merge and the mix separately.
+// Returns SPEC_ERR_SHAPE when no fused form covers the shape (rows wider than 4096 elements; beyond one child per SM also
+// more than two children per row, or an e4m3 copy of the states wanted): the caller then launches the merge and the mix
+// separately.
 int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_t st) {
     if (m.d > 8 * kRowThreads * 2 || g.lse_out != nullptr || g.seq_done != nullptr) return SPEC_ERR_SHAPE;
     MergeMixArgs a{g, m};
@@ -318,7 +315,7 @@ int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_
         return SPEC_OK;
     }
     if (g.topk > kFusedMixMaxChildren || m.S8_out != nullptr) return SPEC_ERR_SHAPE;
-    if (m.d > 8 * kRowThreads && m.d <= 8 * kWideRowThreads) {
+    if (m.d > 8 * kRowThreads) {
         SPEC_CUDA_TRY(launch_pdl(merge_mix_512_kernel, dim3(rows), dim3(kWideRowThreads), 0, st, a));
         return SPEC_OK;
     }

@@ -3,16 +3,18 @@
 // with one scale per vocabulary row, half the bytes of the bf16 matrix.  Per level:
 //   mix step            also writes the states as e4m3 (row_ops.cuh)
 //   head GEMM           kind::f8f6f4 on the two e4m3 operands; the epilogue rescales the accumulators
-//                       and keeps, per vocabulary tile, 8 candidates by APPROXIMATE logit and the
-//                       (max, sum-exp) of the approximate logits
-//   merge_rescore       folds the tiles' lists into a short list of 8 to 16 tokens per row and the
-//                       row's log-sum-exp, recomputes the short-listed logits EXACTLY from the bf16
-//                       weights and states (fp32 accumulation, as the bf16 head does), and takes the
-//                       top-k of those
-// The tokens and their logits are therefore those of the bf16 path whenever the true top-k are among
-// the 16 best approximate logits (the approximation error is a few hundredths of the logits' standard
-// deviation; the k-th and the 16th best of tens of thousands of logits are much further apart); only the
-// normaliser comes from approximate logits (error of order 1e-3, tolerance 2e-2).
+//                       and keeps 8 candidates by APPROXIMATE logit and the (max, sum-exp) of the
+//                       approximate logits: per vocabulary tile with the nodes as MMA rows, per CTA
+//                       (all its vocabulary rows, 872 of 128256) with the nodes as columns
+//   merge_rescore       folds those lists into a short list of max(8, 2 topk + 2), at most 16, tokens per
+//                       row and the row's log-sum-exp, recomputes the short-listed logits EXACTLY from the
+//                       bf16 weights and states (fp32 accumulation, as the bf16 head does), and takes
+//                       the top-k of those
+// The tokens and their logits are therefore those of the bf16 path whenever the true top-k are in the short
+// list, which takes that no more than eight of its tokens lie in one list (the approximation error is a few
+// hundredths of the logits' standard deviation; the k-th best of tens of thousands of logits and the last of the
+// short list are much further apart); only the normaliser comes from approximate logits (error of order
+// 1e-3, tolerance 2e-2).
 #include "row_ops.cuh"
 
 namespace spec {

@@ -115,7 +115,7 @@ struct GemmEpilogue {
     const float *row_scale, *col_scale;
     int idx_offset;    // mode 1 / 3: added to every token id written to part_idx (first vocabulary row of a shard)
     int segs;          // mode 3: threads that share one node's column (swapped_head_segs)
-    int n_parts;       // mode 3: partial lists per node = CTAs the tiles are dealt to * segs (swapped_head_parts)
+    int n_parts;       // mode 3: partial lists per node = CTAs the tiles are dealt to (swapped_head_parts)
 };
 // Mode 3 bookkeeping, the same on the host (workspace sizing, merge) and in the launch.
 int swapped_head_segs(int nodes);

@@ -53,6 +53,14 @@ def load_peaks():
     return {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0, "source": "fallback"}
 
 
+def kernels_in_graph(graph) -> int:
+    """Kernel nodes of a captured graph that was kept."""
+    from cuda.bindings import runtime
+    raw = runtime.cudaGraph_t(graph.raw_cuda_graph())
+    nodes = runtime.cudaGraphGetNodes(raw, runtime.cudaGraphGetNodes(raw)[2])[1]
+    return [runtime.cudaGraphNodeGetType(node)[1] for node in nodes].count(runtime.cudaGraphNodeType.cudaGraphNodeTypeKernel)
+
+
 class ClockSampler:
     """Samples SM clocks and throttle reasons with nvidia-smi while the timed region runs."""
     Q = ("clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.hw_slowdown,"
@@ -219,11 +227,12 @@ class Workload:
         when stream capture is not available; the steps are then launched call by call."""
         torch, c = self.torch, self.cfg
         self.graph = None
+        self.kernels_per_step = 2        # (the least that a draft and a verification can be, if they cannot be counted)
         try:
             cur = torch.cuda.current_stream()
             gs = torch.cuda.Stream()
             gs.wait_stream(cur)
-            g = torch.cuda.CUDAGraph()
+            g = torch.cuda.CUDAGraph(keep_graph=True)
             with torch.cuda.stream(gs):
                 # (thread-local capture mode: CUDA calls of other threads, e.g. a process group's watchdog, are
                 # none of this capture's business)
@@ -234,8 +243,10 @@ class Workload:
                         self.B.spec_verify(self.cand, self.rot[i], accept_len=self.acc, best_cand=self.best,
                                            next_tok=self.nxt, workspace=self.vws, stream=gs)
             cur.wait_stream(gs)
+            self.kernels_per_step = kernels_in_graph(g) // self.n_rot
+            g.instantiate()
             self.graph = g
-        except RuntimeError as e:
+        except (RuntimeError, ImportError) as e:
             sys.stderr.write(f"CUDA graph capture not available, steps are launched call by call: {e}\n")
         return self.graph is not None
 
@@ -505,7 +516,7 @@ def main():
     for i in range(args.warmup):
         step(i)
     W.capture()                  # (after the warm-up: every tensor map and attribute the launches need exists)
-    launch_form = W.launch_form()
+    launch_form, kernels_per_step = W.launch_form(), W.kernels_per_step
     W.run_steps(n_rot)
     ms_step, clocks = timed_region(args.steps)
     assert B.spec_poll_error(ws) == 0
@@ -757,14 +768,6 @@ def main():
                    "sample": f"{seqs} of {Bn} sequences of {cfg.name} (full draft tree + verify) x {len(times)} passes, "
                              f"{t_d + t_v:.1f} s of oracle time; `draft` and `verify` are the two parts timed apart, `value` both"}
 
-    # per step: level-0 projection (clears the header), then per level mix, head GEMM (the next level's
-    # projection rides in the same launch) and merge (the last one also prunes), merge and next mix in one kernel for
-    # levels with at most one child per SM or two per node; verify = streaming arg-max + accept
-    sms = torch.cuda.get_device_properties(dev).multi_processor_count
-    fused = sum(cfg.nodes(l + 1) <= sms or cfg.topk[l] <= 2 for l in range(n - 1))
-    small = cfg.d_inner <= 512 and cfg.d_base <= 2048 and all(cfg.nodes(l) <= 16 for l in range(n)) and \
-        sum(V * cfg.d_inner * (16 + cfg.nodes(l)) for l in range(n)) <= n * (30 << 20)      # the whole draft is one kernel
-    launches_per_step = (1 if small else 1 + 3 * n - fused) + 2
     out = {
         "metric": METRIC, "value": shard.whole_job_rate(Bn, world, ms_step * 1e-3), "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
@@ -791,7 +794,7 @@ def main():
                 "what": "pinned host buffers in, spec_draft + spec_verify call by call, candidates and results back, "
                         "a stream synchronize per step; the logits go up on a second stream in groups of sequences beside the draft, "
                         "each group verified on arrival"},
-        "gpu_launches": launches_per_step * args.steps,
+        "gpu_launches": kernels_per_step * args.steps,
         "clocks": clocks, "synthetic_tokens_per_step": tau,
     }
     print(json.dumps(out), flush=True)

@@ -339,11 +339,11 @@ __device__ __forceinline__ TileWalk walk_of(const GemmJob &j) {
 
 // The CTAs of a launch walk their weight tiles in step, so that at any moment all of them read the same few columns.
 // When a row of the matrix is a power of two long those addresses differ only in their high bits and crowd on a part of
-// the memory channels.  In a job with `halves` every second weight tile therefore starts with the second half of the K
+// the memory channels.  In a job with `halves` every second CTA therefore starts its tiles with the second half of the K
 // range.  Each half is summed in accumulator columns of its own and the epilogue adds the two, so that a logit does not
 // depend on which half came first (equal rows of the matrix give equal logits wherever they lie).  Rows of 8192 bytes:
 // single-candidate chain at the 13B widths 168.4 -> 161.6 us per draft, 64 sequences at the 34B widths 241 -> 234; more
-// groups of tiles than two are no better.
+// groups of CTAs than two are no better.
 __device__ __forceinline__ int first_half(int num_kb) { return num_kb / 2; }   // K blocks of the first half
 
 __device__ __forceinline__ TilePos pos_of(const GemmJob &j, const TileWalk &w, int t) {

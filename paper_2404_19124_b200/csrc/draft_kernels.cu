@@ -49,7 +49,7 @@ __global__ void __launch_bounds__(kRowThreads, 3) mix_ln_gelu_many_kernel(MixArg
     else mix_ln_gelu_row<kRowThreads, 2, 1, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
 }
 
-// Levels of several waves (their parents are more than 128, so that the projection was not split): throughput counts, and
+// Levels of several waves whose projection was not split (more than 128 parents, or too few K blocks): throughput counts, and
 // a CTA has only as many threads as its row needs with two groups each.  2016 rows of 400 elements 14.7 -> 6.9 us, 1836 of
 // 2296 25.5 -> 21.5.  (Four rows to a CTA, or 128 threads with four groups each, are no better.)
 __global__ void __launch_bounds__(kRowThreads, 3) mix_ln_gelu_waves_kernel(MixArgs m) {

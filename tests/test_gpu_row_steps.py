@@ -85,7 +85,7 @@ def test_merge_lists_round_the_thread_counts(B, V, k, swap):
 @pytest.mark.parametrize("rows", [1, 17, 48])
 @pytest.mark.parametrize("d", [2048, 4096, 2056])
 def test_equal_rows_give_equal_logits_in_every_tile(B, d, rows):
-    """Nodes as MMA columns, rows of 4096 and 8192 bytes: every second weight tile is summed with the halves of its K range
+    """Nodes as MMA columns, rows of 4096 and 8192 bytes: every second CTA sums its weight tiles with the halves of the K range
     in the other order.  Copies of one head row in tiles of either kind must tie exactly, lower token first."""
     V = 20000                                            # 136 rows per CTA: two tiles each
     cfg = small_cfg(d_base=64, d_inner=d, V=V, topk=(8, 2), seed=rows + d)
@@ -277,6 +277,42 @@ def test_a_small_draft_reads_its_weights_in_stream_order(B, d, what):
         torch.cuda.synchronize()
         B.spec_verify(cand, logits, *res, workspace=vws)
         B.spec_next_ctx(state, zero, zero, ctx_state=target)
+        B.spec_draft(h, ctx, tok, cfg.topk, cfg.K, cand_tok=ct, cand_logp=lp, workspace=ws)
+        torch.cuda.synchronize()
+        got = ct.clone(), lp.clone()
+        B.spec_draft(h, ctx, tok, cfg.topk, cfg.K, cand_tok=ct, cand_logp=lp, workspace=ws)
+        torch.cuda.synchronize()
+        assert torch.equal(got[0], ct) and torch.equal(got[1], lp) and not torch.equal(lp, before)
+    B.spec_destroy(h)
+
+
+@pytest.mark.parametrize("e4m3", [False, True])
+def test_weights_rewritten_by_an_ordinary_kernel_are_seen(B, e4m3):
+    """Weights, or the e4m3 copies of heads, rewritten on the stream by kernels that do not let their dependents start early,
+    behind a long verification and directly before the draft."""
+    cfg = small_cfg(d_base=2048, d_inner=2048, V=2048, topk=(4, 2), K=8, B=4, seed=9)
+    gw = weights_to_cuda(synth.make_weights(cfg))
+    ctx, tok = (t.cuda() for t in synth.make_draft_inputs(cfg))
+    h = B.spec_create(gw)
+    if e4m3:
+        B.spec_attach_fp8_heads(h)
+    logits = torch.zeros((16, 8, 4, 128256), dtype=torch.bfloat16, device="cuda")
+    cand = torch.zeros((16, 8, 3), dtype=torch.int32, device="cuda")
+    res = [torch.empty(16, dtype=torch.int32, device="cuda") for _ in range(3)]
+    vws = B.spec_verify(cand, logits)[3]
+    ct, lp, ws = B.spec_draft(h, ctx, tok, cfg.topk, cfg.K)
+    for i in range(10):
+        new = gw.proj[0] * -1.0
+        torch.cuda.synchronize()
+        before = lp.clone()
+        B.spec_verify(cand, logits, *res, workspace=vws)
+        if e4m3:
+            for l in (1, 0):
+                gw.head[l].mul_(-1.0)
+                q, scale = h._fp8[l]
+                assert B._lib.spec_quantize_head(h.ptr, l, q.data_ptr(), scale.data_ptr(), B._stream_ptr(None)) == B.SPEC_OK
+        else:
+            gw.proj[0].copy_(new)
         B.spec_draft(h, ctx, tok, cfg.topk, cfg.K, cand_tok=ct, cand_logp=lp, workspace=ws)
         torch.cuda.synchronize()
         got = ct.clone(), lp.clone()

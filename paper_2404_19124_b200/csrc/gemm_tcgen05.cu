@@ -33,7 +33,7 @@ struct GemmParams {
     int stages, tmem_cols, acc_stride;
     uint32_t slot_bytes;
     int producers;           // TMA-issuing threads: 1 or 2
-    uint32_t tbuf_bytes;     // transposed accumulator tile of a mode-3 job (0: none in this launch)
+    uint32_t tbuf_bytes;     // transposed accumulator tile or column scales (0: neither in this launch), see Pipe
     DraftStart start;        // first kernel of a draft only
     int32_t *err;
 };
@@ -316,6 +316,7 @@ int launch_gemm_tc_jobs(const GemmCall *calls, int n_calls, int32_t *err, cudaSt
             }
             total_tiles += p.job[q].deal_ctas;   // what counts for the grid: the CTAs it occupies
         } else {
+            if (p.job[q].fp8) p.tbuf_bytes = kEpilogueThreads / 32 * kMaxBlockN * sizeof(float);
             total_tiles += (long long)p.job[q].m_tiles * p.job[q].n_tiles * p.job[q].splits;
         }
     }

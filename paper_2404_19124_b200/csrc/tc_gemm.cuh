@@ -37,6 +37,7 @@ constexpr int kThreads = 224;
 constexpr int kEpilogueFirst = 64;     // first epilogue thread
 constexpr int kEpilogueThreads = 128;  // warps 2-5
 constexpr int kMaxStages = 32;         // slots of short weight boxes are small, and what covers the latency is their number
+constexpr int kMaxBlockN = 256;
 constexpr int kABytes = kBlockM * kSlabBytes;
 constexpr int kSmemLimit = 222 * 1024; // leaves room on the SM for the small kernels that overlap with a GEMM
 constexpr uint32_t kSpinFast = 1u << 14;
@@ -84,7 +85,8 @@ struct Pipe {
     int stages;
     uint32_t slot_bytes;
     int acc_stride;        // TMEM columns between the two accumulator slots
-    float *tbuf;           // mode 3: transposed accumulator tile, [nodes][kTPitch] floats (null when not used)
+    float *tbuf;           // mode 3: transposed accumulator tile, [nodes][kTPitch] floats; mode 1 with e4m3 operands: the
+                           // column scales of the tile, a copy per epilogue warp (null when not used)
     int32_t *err;
 };
 
@@ -558,35 +560,38 @@ __device__ __forceinline__ bool mma_job(const Pipe &pp, const GemmJob &j, RingPo
 //           below, so the few columns that reach it hold the answer: they are inserted, in ascending column order, into a
 //           sorted list of kCap.
 // The list leaves the kernel best first (value desc, column asc).
-// e4m3 operands: accumulator -> logit, v[i] * row_scale * col_scale[col0 + c + i] (columns past N untouched).
-__device__ __forceinline__ void scale_chunk(float (&v)[32], float rs, const float *cs, int valid) {
-    if (valid >= 32 && (((uintptr_t)cs) & 15) == 0) {
+// e4m3 operands: accumulator -> logit, v[i] * row_scale * cs[i] (`cs`: the chunk's column scales, in shared memory).
+__device__ __forceinline__ void scale_chunk(float (&v)[32], float rs, const float *cs) {
 #pragma unroll
-        for (int i = 0; i < 32; i += 4) {
-            const float4 q = *(const float4 *)(cs + i);
-            v[i] *= rs * q.x; v[i + 1] *= rs * q.y; v[i + 2] *= rs * q.z; v[i + 3] *= rs * q.w;
-        }
-    } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i)
-            if (i < valid) v[i] *= rs * cs[i];
+    for (int i = 0; i < 32; i += 4) {
+        const float4 q = *(const float4 *)(cs + i);
+        v[i] *= rs * q.x; v[i + 1] *= rs * q.y; v[i + 2] *= rs * q.z; v[i + 3] *= rs * q.w;
     }
+}
+// The column scales of the tile at column col0 (0 past the last column), into the warp's own copy.  They come from DRAM, so
+// they are fetched while the tile's MMAs run: read chunk by chunk behind them they were a chain of seven misses (96 nodes, V
+// 32000, d 4096: 12 us from the last MMA to the last list, the 13B step
+// with e4m3 heads 246.7 -> 244.9 us).
+__device__ __forceinline__ void stage_col_scales(float *cs, const GemmJob &j, int col0) {
+    const int lane = threadIdx.x & 31;
+    __syncwarp();   // the tile before has been read
+    for (int i = lane; i < j.block_n; i += 32) cs[i] = col0 + i < j.N ? j.epi.col_scale[col0 + i] : 0.0f;
+    __syncwarp();
 }
 
 template <int kCap, bool kFp8>
 __device__ __forceinline__ void epilogue_topk(const GemmJob &p, uint32_t taddr, int row, bool row_ok, int col0,
-                                              int n_tile) {
+                                              int n_tile, float rs = 1.0f, const float *cs = nullptr) {
     constexpr float kLog2e = 1.4426950408889634f;
     float best[kCap];
 #pragma unroll
     for (int j = 0; j < kCap; ++j) best[j] = -INFINITY;
     float run_m = -INFINITY, run_s = 0.0f;
-    const float rs = (kFp8 && row_ok) ? p.epi.row_scale[row] : 1.0f;
     for (int c = 0; c < p.block_n; c += 32) {
         float v[32];
         tmem_ld32(taddr + c, v);
         const int valid = p.N - (col0 + c);   // columns of this chunk inside the vocabulary
-        if (kFp8) scale_chunk(v, rs, p.epi.col_scale + col0 + c, valid);
+        if (kFp8) scale_chunk(v, rs, cs + c);
         if (valid < 32) {
 #pragma unroll
             for (int i = 0; i < 32; ++i)
@@ -634,7 +639,7 @@ __device__ __forceinline__ void epilogue_topk(const GemmJob &p, uint32_t taddr, 
         float v[32];
         tmem_ld32(taddr + c, v);
         const int valid = p.N - (col0 + c);
-        if (kFp8) scale_chunk(v, rs, p.epi.col_scale + col0 + c, valid);
+        if (kFp8) scale_chunk(v, rs, cs + c);
         // candidates of this chunk as a bit mask: no per-element branches
         uint32_t mask = 0;
 #pragma unroll
@@ -842,14 +847,14 @@ __device__ __forceinline__ bool epilogue_job_swapped(const Pipe &pp, const GemmJ
     // e4m3: a vocabulary row's scale is applied on the way to shared memory, the node's in the end: it orders nothing
     const float node_scale = j.fp8 && scans ? __ldcg(j.epi.row_scale + node) : 1.0f;
     for (int tile = w.first; tile < w.end; tile += w.step) {
+        const int row0 = w.rel * j.rows_per_cta + tile * kBlockM;   // vocabulary row of TMEM lane 0
+        const bool v_ok = row0 + vrow < row_end;
+        const float v_scale = j.fp8 && v_ok ? j.epi.col_scale[row0 + vrow] : 1.0f;   // (in flight during the wait)
         if (u == 0) bars->epi_ok = mbar_wait(&bars->acc_full[ap.acc], ap.phase, bars, pp.err) ? 1 : 0;
         epi_bar_sync();
         if (!bars->epi_ok) return false;
         tc_fence_after();
         const uint32_t taddr = pp.tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ap.acc * pp.acc_stride);
-        const int row0 = w.rel * j.rows_per_cta + tile * kBlockM;   // vocabulary row of TMEM lane 0
-        const bool v_ok = row0 + vrow < row_end;
-        const float v_scale = j.fp8 && v_ok ? j.epi.col_scale[row0 + vrow] : 1.0f;
         for (int c = 0; c < nodes; c += 16) {
             float v[16];
             tmem_ld16(taddr + c, v);
@@ -920,12 +925,18 @@ __device__ __forceinline__ bool epilogue_job(const Pipe &pp, const GemmJob &j, A
     for (int tile = w.first; tile < w.end; tile += w.step) {
         const TilePos t = pos_of(j, w, tile);
         const int split = t.split, m_tile = t.m_tile, n_tile = t.n_tile;
-        if (!mbar_wait(&bars->acc_full[ap.acc], ap.phase, bars, pp.err)) return false;
-        tc_fence_after();
         const int row = m_tile * kBlockM + row_in_tile;
         const bool row_ok = row < j.M;
-        const uint32_t taddr = pp.tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ap.acc * pp.acc_stride);
         const int col0 = n_tile * j.block_n;
+        float row_scale = 1.0f, *col_scales = nullptr;
+        if (j.fp8) {
+            if (row_ok) row_scale = __ldcg(j.epi.row_scale + row);
+            col_scales = pp.tbuf + quarter * kMaxBlockN;
+            stage_col_scales(col_scales, j, col0);
+        }
+        if (!mbar_wait(&bars->acc_full[ap.acc], ap.phase, bars, pp.err)) return false;
+        tc_fence_after();
+        const uint32_t taddr = pp.tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ap.acc * pp.acc_stride);
         if (j.epi.mode == 0) {
             for (int c = 0; c < j.block_n; c += 32) {
                 float v[32];
@@ -959,7 +970,7 @@ __device__ __forceinline__ bool epilogue_job(const Pipe &pp, const GemmJob &j, A
                 }
             }
         } else {
-            if (j.fp8) epilogue_topk<SPEC_MAX_TOPK, true>(j, taddr, row, row_ok, col0, n_tile);
+            if (j.fp8) epilogue_topk<SPEC_MAX_TOPK, true>(j, taddr, row, row_ok, col0, n_tile, row_scale, col_scales);
             else if (j.epi.topk <= 4) epilogue_topk<4, false>(j, taddr, row, row_ok, col0, n_tile);
             else epilogue_topk<SPEC_MAX_TOPK, false>(j, taddr, row, row_ok, col0, n_tile);
         }

@@ -83,6 +83,19 @@ static __device__ __noinline__ float4 gelu_erf4(float4 y) {
 // differed from one kernel to the next, and with it, now and then, the bf16 value that a state is rounded to.
 __device__ __forceinline__ float mix_element(const MixArgs &m, float p, float z) { return fmaf(m.b, z, __fmul_rn(m.a, p)); }
 
+// Eight floats of a projection, 32-byte aligned (rows are whole groups of eight in the workspace), in one load.  Two 16-byte
+// loads of a warp would each touch every 32-byte sector of the kilobyte and use half of it.
+struct Float8 {
+    float v[8];
+};
+__device__ __forceinline__ Float8 ldcg8(const float *p) {
+    Float8 r;
+    asm volatile("ld.global.cg.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(r.v[0]), "=f"(r.v[1]), "=f"(r.v[2]), "=f"(r.v[3]), "=f"(r.v[4]), "=f"(r.v[5]), "=f"(r.v[6]), "=f"(r.v[7])
+                 : "l"(p));
+    return r;
+}
+
 // The projected parent state (the sum of its partials, added in ascending order) of the groups that thread `tid` owns in
 // mix_ln_gelu_row with one group per thread.
 template <int kThreads>
@@ -93,20 +106,16 @@ __device__ __forceinline__ void parent_state(const MixArgs &m, int parent, int t
     if (i >= m.d) return;
     const float *p = m.P + (size_t)parent * m.d + i;
     for (int s0 = 0; s0 < m.p_splits; s0 += 4) {
-        float4 a[4], b[4];
+        Float8 a[4];
 #pragma unroll
         for (int sp = 0; sp < 4; ++sp) {
-            a[sp] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-            b[sp] = a[sp];
-            if (s0 + sp < m.p_splits) {
-                a[sp] = __ldcg((const float4 *)(p + (s0 + sp) * m.p_split_stride));
-                b[sp] = __ldcg((const float4 *)(p + (s0 + sp) * m.p_split_stride + 4));
-            }
+            a[sp] = Float8{};
+            if (s0 + sp < m.p_splits) a[sp] = ldcg8(p + (s0 + sp) * m.p_split_stride);
         }
 #pragma unroll
         for (int sp = 0; sp < 4; ++sp) {
-            pre[0][0] += a[sp].x; pre[0][1] += a[sp].y; pre[0][2] += a[sp].z; pre[0][3] += a[sp].w;
-            pre[0][4] += b[sp].x; pre[0][5] += b[sp].y; pre[0][6] += b[sp].z; pre[0][7] += b[sp].w;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) pre[0][j] += a[sp].v[j];
         }
     }
 }
@@ -134,18 +143,14 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
     for (int g0 = 0; g0 < kIters; g0 += kGroup) {
         // every load of the group is issued before the first value is used: one round trip per group
         uint4 ev[kGroup];
-        float4 pa[kGroup][kSp], pb[kGroup][kSp];
+        Float8 pa[kGroup][kSp];
 #pragma unroll
         for (int q = 0; q < kGroup; ++q) {
             const int i = ((g0 + q) * nt + tid) * 8;
 #pragma unroll
             for (int sp = 0; sp < kSp; ++sp) {
-                pa[q][sp] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                pb[q][sp] = pa[q][sp];
-                if (pre == nullptr && i < d && sp < m.p_splits) {
-                    pa[q][sp] = __ldcg((const float4 *)(p + sp * m.p_split_stride + i));
-                    pb[q][sp] = __ldcg((const float4 *)(p + sp * m.p_split_stride + i + 4));
-                }
+                pa[q][sp] = Float8{};
+                if (pre == nullptr && i < d && sp < m.p_splits) pa[q][sp] = ldcg8(p + sp * m.p_split_stride + i);
             }
         }
         if (g0 == 0) {   // (only now: everything above is in flight while the token arrives)
@@ -166,18 +171,17 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
             float pv[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
             for (int sp = 0; sp < kSp; ++sp) {      // partials are added in ascending order: reproducible
-                pv[0] += pa[q][sp].x; pv[1] += pa[q][sp].y; pv[2] += pa[q][sp].z; pv[3] += pa[q][sp].w;
-                pv[4] += pb[q][sp].x; pv[5] += pb[q][sp].y; pv[6] += pb[q][sp].z; pv[7] += pb[q][sp].w;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) pv[j] += pa[q][sp].v[j];
             }
             if (pre != nullptr) {
 #pragma unroll
                 for (int j = 0; j < 8; ++j) pv[j] = pre[it][j];
             } else if (i < d) {
                 for (int sp = kSp; sp < m.p_splits; ++sp) {   // more partials than one batch holds (rare)
-                    const float4 p0 = __ldcg((const float4 *)(p + sp * m.p_split_stride + i));
-                    const float4 p1 = __ldcg((const float4 *)(p + sp * m.p_split_stride + i + 4));
-                    pv[0] += p0.x; pv[1] += p0.y; pv[2] += p0.z; pv[3] += p0.w;
-                    pv[4] += p1.x; pv[5] += p1.y; pv[6] += p1.z; pv[7] += p1.w;
+                    const Float8 x = ldcg8(p + sp * m.p_split_stride + i);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) pv[j] += x.v[j];
                 }
             }
             const uint32_t ew[4] = {ev[q].x, ev[q].y, ev[q].z, ev[q].w};
@@ -495,10 +499,9 @@ __device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int f
         if (i < d) {
             const float *p = m.P + (size_t)parent * d + i;
             for (int sp = 0; sp < m.p_splits; ++sp) {
-                const float4 p0 = __ldcg((const float4 *)(p + sp * m.p_split_stride));
-                const float4 p1 = __ldcg((const float4 *)(p + sp * m.p_split_stride + 4));
-                pv[it][0] += p0.x; pv[it][1] += p0.y; pv[it][2] += p0.z; pv[it][3] += p0.w;
-                pv[it][4] += p1.x; pv[it][5] += p1.y; pv[it][6] += p1.z; pv[it][7] += p1.w;
+                const Float8 x = ldcg8(p + sp * m.p_split_stride);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) pv[it][j] += x.v[j];
             }
         }
         const float4 g0 = *(const float4 *)(m.gamma + ic), g1 = *(const float4 *)(m.gamma + ic + 4);

@@ -81,6 +81,7 @@ struct VerifyPlan {
     int rows;          // B * K * (n + 1)
     int vec_per_warp;  // two-kernel form: 16-byte vectors in one warp's contiguous range
     int warps;         // ... ranges, at most (the base at its least aligned)
+    bool pool;         // verify_pool_kernel: the ranges below are CTAs', not warps'
     size_t off_g;      // int32 [rows]
     size_t off_part;   // (fp32 value, int32 index) [warps + min(rows, warps)], see first_piece; early exit: int32 [B * K]
     size_t total;

@@ -8,9 +8,10 @@
 // bf16 the running maximum is taken on packed pairs (max.bf16x2) and the element index is only resolved when a vector
 // beats the lane's current best, so the common case costs about one ALU operation per element.
 //
-// Two forms (one_kernel_form chooses):
+// Three forms (one_kernel_form and pool_form choose):
 //   verify_seq_kernel    one CTA per sequence does the whole job: its warps take equal contiguous ranges of the sequence's
 //                        vectors, fold them into a (value, index) key per row in shared memory, and the CTA accepts.
+//   verify_pool_kernel + verify_accept_kernel    long rows: one range of vectors per SM, shared out among its warps as they go
 //   verify_stream_kernel + verify_accept_kernel    all vectors cut into equal contiguous ranges, one per warp, a single
 //                        wave over the whole GPU; a row that lies in one range is finished there, of the others every
 //                        piece leaves a (value, index) partial; one CTA per sequence folds those and accepts.
@@ -143,6 +144,23 @@ __device__ __forceinline__ void scan_row(const char *base, long long rs, long lo
     }
 }
 
+// (value, first index) as one integer whose maximum is the arg-max: the order-preserving image of the value above the
+// complement of the index.  0 stands for "nothing above -inf".  (+ 0.0f: -0 and +0 are equal.)
+__device__ __forceinline__ uint32_t value_key(float v) {
+    const uint32_t u = __float_as_uint(v + 0.0f);
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+__device__ __forceinline__ unsigned long long argmax_key(float v, int idx) {
+    return idx == kIdxNone ? 0ull : ((unsigned long long)value_key(v) << 32) | (uint32_t)~idx;
+}
+// The index that a key stands for (0 where a row has no value above -inf), and the key as a partial.
+__device__ __forceinline__ int key_index(unsigned long long k) { return k == 0ull ? 0 : (int)~(uint32_t)k; }
+__device__ __forceinline__ float2 key_partial(unsigned long long k) {
+    const uint32_t hi = (uint32_t)(k >> 32);
+    return k == 0ull ? make_float2(-INFINITY, __int_as_float(kIdxNone))
+                     : make_float2(__uint_as_float((hi & 0x80000000u) ? (hi & 0x7fffffffu) : ~hi), __int_as_float(key_index(k)));
+}
+
 // Places of the partials.  A border between two warps is crossed by one row at most, so the pieces behind a border are
 // numbered by their warp; a row's first piece goes to a place of its row or of its warp behind those, whichever are fewer.
 __host__ __device__ __forceinline__ long long first_piece(long long warps, int rows, int row, long long w) {
@@ -174,6 +192,119 @@ verify_stream_kernel(const char *__restrict__ base, int skew, int rows, int V, l
             if (begins && ends) g_out[row] = idx == kIdxNone ? 0 : idx;   // (nothing above -inf, all NaN: 0)
             else part[begins ? first_piece(warps, rows, row, w) : w] = make_float2(best, __int_as_float(idx));
         }
+    }
+}
+
+// Long rows: one CTA per SM takes one range of vectors, and its warps take blocks of it as they get to them.  Bound by DRAM.
+// Of the four CTAs that an SM holds in the form above one is served last, trip after trip (its first loads return after 10 us,
+// the others' after 3), so that in the end it runs on alone; here its warps take fewer blocks instead.  The keys of the
+// rows that a range touches gather in shared memory, so that few pieces are left to the accept kernel, and most trips end with
+// one comparison against their row's key.  28 warps of 64 registers: the accept kernel's CTAs still fit beside them and are there
+// when the last block is read.  us a call, form above -> this one, bf16: V 32000, 16 MB 9.9 -> 8.5, 131 MB 25.1 -> 24.8, 400 MB
+// 65.5 -> 61.4; V 128256, 8 MB 11.4 -> 7.4, 33 MB 13.4 -> 10.8, 131 MB 25.4 -> 24.5; fp32 V 32000, 16 MB 9.7 -> 7.9.
+constexpr int kPoolThreads = 896, kPoolMaxRows = 128;
+
+template <bool kBf16>
+__global__ void __maxnreg__(64)
+verify_pool_kernel(const char *__restrict__ base, int skew, int rows, int V, long long total_vec, int vec_per_cta, int block,
+                   int ctas, int32_t *g_out, float2 *part) {
+    __shared__ unsigned long long keys[kPoolMaxRows];
+    __shared__ int taken;
+    using E = Elem<kBf16>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long beg = (long long)blockIdx.x * vec_per_cta, end = min(total_vec, beg + vec_per_cta);
+    const long long first = (beg << E::kShift) - skew;
+    const int row0 = first > 0 ? (int)(first / V) : 0, n = (int)(end - beg);
+    const int into = (int)(first - (long long)row0 * V);   // the range begins this many elements into row0 (-skew: before it)
+    griddep_launch();
+    for (int i = threadIdx.x; i < kPoolMaxRows; i += kPoolThreads) keys[i] = 0ull;
+    if (threadIdx.x == 0) taken = kPoolThreads / 32 * block;
+    __syncthreads();
+    griddep_wait();
+    // the whole vectors of every row (positions below are relative to the range)
+    for (int a = warp * block; a < n;) {
+        int next = 0;
+        if (lane == 0) next = atomicAdd(&taken, block);
+        const int e = min(a + block, n), at = into + (a << E::kShift);
+        int r = at > 0 ? (int)((uint32_t)at / (uint32_t)V) : 0;
+        for (int re = (r + 1) * V - into;; ++r, re += V) {   // re: where the row ends, in elements from the range's start
+            const int rs = re - V;
+            const int p = max(a, (rs + E::kEpv - 1) >> E::kShift), q = min(e, re >> E::kShift);
+            for (int i = p; i < q; i += 32 * kStreamUnroll) {
+                const uint4 *src = (const uint4 *)base + beg;
+                uint4 v[kStreamUnroll];
+#pragma unroll
+                for (int u = 0; u < kStreamUnroll; ++u) v[u] = ld_stream(src + min(i + 32 * u + lane, q - 1));
+                float mx;
+                if (kBf16) {
+                    uint32_t m[kStreamUnroll];
+#pragma unroll
+                    for (int u = 0; u < kStreamUnroll; ++u) m[u] = max_bf16x2(max_bf16x2(v[u].x, v[u].y), max_bf16x2(v[u].z, v[u].w));
+#pragma unroll
+                    for (int h = kStreamUnroll / 2; h > 0; h >>= 1)
+#pragma unroll
+                        for (int u = 0; u < h; ++u) m[u] = max_bf16x2(m[u], m[u + h]);
+                    mx = fmaxf(__uint_as_float(m[0] << 16), __uint_as_float(m[0] & 0xffff0000u));
+                } else {
+                    float m[kStreamUnroll];
+#pragma unroll
+                    for (int u = 0; u < kStreamUnroll; ++u)
+                        m[u] = fmaxf(fmaxf(__uint_as_float(v[u].x), __uint_as_float(v[u].y)), fmaxf(__uint_as_float(v[u].z), __uint_as_float(v[u].w)));
+#pragma unroll
+                    for (int h = kStreamUnroll / 2; h > 0; h >>= 1)
+#pragma unroll
+                        for (int u = 0; u < h; ++u) m[u] = fmaxf(m[u], m[u + h]);
+                    mx = m[0];
+                }
+                const uint32_t key = mx > -INFINITY ? value_key(mx) : 0u;   // (NaN: nothing)
+                const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+                // most trips find nothing that reaches what their row has already
+                if (top == 0u || top < (uint32_t)(*(volatile unsigned long long *)&keys[r] >> 32)) continue;
+                int pos = kIdxNone;
+                if (key == top) {
+#pragma unroll
+                    for (int u = kStreamUnroll - 1; u >= 0; --u) {
+                        const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+                        const int at_u = min(i + 32 * u + lane, q - 1) << E::kShift;
+#pragma unroll
+                        for (int h = 3; h >= 0; --h) {
+                            if (kBf16) {
+                                if (__uint_as_float(w[h] & 0xffff0000u) == mx) pos = at_u + 2 * h + 1;
+                                if (__uint_as_float(w[h] << 16) == mx) pos = at_u + 2 * h;
+                            } else if (__uint_as_float(w[h]) == mx) {
+                                pos = at_u + h;
+                            }
+                        }
+                    }
+                }
+                pos = __reduce_min_sync(0xffffffffu, pos);
+                if (lane == 0) atomicMax(&keys[r], ((unsigned long long)top << 32) | (uint32_t)~(pos - rs));
+            }
+            if ((re >> E::kShift) >= e || row0 + r + 1 >= rows) break;
+        }
+        a = __shfl_sync(0xffffffffu, next, 0);
+    }
+    // the vectors that rows share: lanes 0 to kEpv - 1 take the row's first elements, the next ones its last
+    for (int r = warp; row0 + r < rows && (r * V - into) >> E::kShift < n; r += kPoolThreads / 32) {
+        const int rs = r * V - into, re = rs + V;
+        const int head = min((rs + E::kEpv - 1) >> E::kShift << E::kShift, re), tail = max(re >> E::kShift << E::kShift, head);
+        const int i = lane < E::kEpv ? rs + lane : tail + lane - E::kEpv;
+        const bool mine = lane < E::kEpv ? i < head : lane < 2 * E::kEpv && i < re;
+        const int vec = i >> E::kShift;
+        const float x = mine && vec >= 0 && vec < n ? E::load(base + (beg << 4), i) : -INFINITY;
+        const uint32_t key = x > -INFINITY ? value_key(x) : 0u;
+        const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+        const int pos = __reduce_min_sync(0xffffffffu, key == top ? i - rs : kIdxNone);
+        if (lane == 0 && top != 0u) atomicMax(&keys[r], ((unsigned long long)top << 32) | (uint32_t)~pos);
+    }
+    __syncthreads();
+    for (int i = threadIdx.x;; i += kPoolThreads) {
+        const int row = row0 + i;
+        const long long rs = skew + (long long)row * V;
+        if (row >= rows || (rs >> E::kShift) >= end) break;
+        const bool begins = (rs >> E::kShift) >= beg, ends = ((rs + V - 1) >> E::kShift) < end;   // in this range
+        if (begins && ends) g_out[row] = key_index(keys[i]);
+        else part[begins ? first_piece(ctas, rows, row, blockIdx.x) : (long long)blockIdx.x] = key_partial(keys[i]);
     }
 }
 
@@ -248,16 +379,13 @@ verify_accept_kernel(const int32_t *cand_tok, const float2 *part, int K, int n, 
         const long long w0 = narrow ? (uint32_t)v0 / (uint32_t)vec_per_warp : v0 / vec_per_warp;
         const int chunks = (int)((narrow ? (uint32_t)v1 / (uint32_t)vec_per_warp : v1 / vec_per_warp) - w0) + 1;
         const float2 *first = part + first_piece(warps, rows, (int)gr, w0), *rest = part + w0;
-        if (chunks == 1) {   // finished by its warp
-            if (g_in_smem) g_s[r] = __ldcg(g_out + gr);
-            continue;
-        }
+        const int whole = __ldcg(g_out + gr);   // (what it says only if the row was finished where it was read)
         float best = -INFINITY;
         int arg = 0;   // a row without any value above -inf (all NaN) yields 0
         for (int c0 = 0; c0 < chunks; c0 += kBatch) {
             float2 v[kBatch];
 #pragma unroll
-            for (int j = 0; j < kBatch; ++j) v[j] = c0 + j < chunks ? __ldcg(c0 + j == 0 ? first : rest + c0 + j) : make_float2(-INFINITY, 0.0f);
+            for (int j = 0; j < kBatch; ++j) v[j] = c0 + j < chunks && chunks > 1 ? __ldcg(c0 + j == 0 ? first : rest + c0 + j) : make_float2(-INFINITY, 0.0f);
 #pragma unroll
             for (int j = 0; j < kBatch; ++j) {
                 const bool take = v[j].x > best;   // chunks ascend, so the first maximum wins
@@ -265,8 +393,9 @@ verify_accept_kernel(const int32_t *cand_tok, const float2 *part, int K, int n, 
                 arg = take ? __float_as_int(v[j].y) : arg;
             }
         }
+        if (chunks == 1) arg = whole;
+        else g_out[gr] = arg;
         if (g_in_smem) g_s[r] = arg;
-        g_out[gr] = arg;
     }
     __syncthreads();
     accept_sequence(cand_tok, g_in_smem ? g_s : g_out + (size_t)b * rows_b, b, K, n, ctok, &key_s, accept_len, best_cand,
@@ -274,13 +403,6 @@ verify_accept_kernel(const int32_t *cand_tok, const float2 *part, int K, int n, 
 }
 
 // ---- one CTA per sequence ---------------------------------------------------------------------------
-// (value, first index) as one integer whose maximum is the arg-max: the order-preserving image of the value above the
-// complement of the index.  0 stands for "nothing above -inf".  (+ 0.0f: -0 and +0 are equal.)
-__device__ __forceinline__ unsigned long long argmax_key(float v, int idx) {
-    const uint32_t u = __float_as_uint(v + 0.0f);
-    const uint32_t hi = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-    return idx == kIdxNone ? 0ull : ((unsigned long long)hi << 32) | (uint32_t)~idx;
-}
 
 template <bool kBf16>
 __global__ void __launch_bounds__(kSeqThreads, 1)
@@ -322,8 +444,7 @@ verify_seq_kernel(const char *__restrict__ base, int skew, const int32_t *cand_t
     }
     __syncthreads();
     for (int r = threadIdx.x; r < rows_b; r += kSeqThreads) {
-        const unsigned long long k = keys[r];
-        const int arg = k == 0ull ? 0 : (int)~(uint32_t)k;
+        const int arg = key_index(keys[r]);
         g_s[r] = arg;
         g_out[(size_t)b * rows_b + r] = arg;
     }
@@ -390,7 +511,7 @@ verify_early_kernel(const char *__restrict__ base, const int32_t *cand_tok, int 
         if (slots > 32) k = max(k, set[lane + 32 < slots ? lane + 32 : lane]);
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) k = max(k, __shfl_xor_sync(0xffffffffu, k, off));
-        const int arg = k == 0ull ? 0 : (int)~(uint32_t)k;   // a row without any value above -inf (all NaN) yields 0
+        const int arg = key_index(k);   // a row without any value above -inf (all NaN) yields 0
         last = arg;
         if (rank == 0 && tid == 0) g[row] = arg;
         if (j < n && tok != arg) {   // uniform over the cluster
@@ -452,6 +573,16 @@ bool one_kernel_form(int B, int rows_b, int V, int dtype) {
            (turns - 1) * V <= 64 * (dtype == SPEC_BF16 ? Elem<true>::kEpv : Elem<false>::kEpv);
 }
 
+// Where verify_pool_kernel takes over from verify_stream_kernel: rows of 48 KB and more, 6 to 512 MB in all.  us a call, stream /
+// pool, bf16: V 2048, 65 MB 17.4 / 20.3, 400 MB 72 / 78; V 8000, 16 MB 9.6 / 9.5, 65 MB 16.0 / 16.7, 131 MB 25.4 / 26.0 (a trip ends at
+// a row's end); V 32000, 2 MB 7.2 / 7.5, 8 MB 8.2 / 7.5.  Above, at the clocks of a long step, the shorter trips of the other form
+// win: V 128256, 5250 MB 765-828 / 765-882.
+constexpr long long kPoolMinRowVec = 3072, kPoolMaxRowVec = 1 << 24, kPoolMinVec = 400000, kPoolMaxVec = 32 << 20;
+bool pool_form(long long total_vec, long long row_vec) {
+    return row_vec >= kPoolMinRowVec && row_vec <= kPoolMaxRowVec && total_vec >= kPoolMinVec && total_vec <= kPoolMaxVec &&
+           (total_vec + num_sms() - 1) / num_sms() / row_vec + 3 <= kPoolMaxRows;
+}
+
 // Resident CTAs per SM of the streaming kernel (launch bound above) times the SM count gives the
 // number of warps of one full wave; every warp gets an equal range of at least one unrolled trip.
 VerifyPlan make_verify_plan(int B, int K, int n, int V, int dtype) {
@@ -465,13 +596,19 @@ VerifyPlan make_verify_plan(int B, int K, int n, int V, int dtype) {
     if (c > (1ll << 30)) c = 1ll << 30;
     p.vec_per_warp = (int)c;
     p.warps = (int)((total + c - 1) / c);
-    p.off_g = kWsAlign;
+    p.off_g = kWsAlign;   // (the scratch is sized for the form that leaves most pieces)
     p.off_part = align_up(p.off_g + sizeof(int32_t) * (size_t)p.rows, kWsAlign);
     // at most a partial behind every border and a first piece for every row that crosses one.  Never less than 4 bytes per
     // candidate, the early-exit form's match lengths.
     const size_t partials = sizeof(float2) * ((size_t)p.warps + (p.rows < p.warps ? p.rows : p.warps));
     const size_t lengths = sizeof(int32_t) * (size_t)B * K;
     p.total = align_up(p.off_part + (partials > lengths ? partials : lengths), kWsAlign);
+    if (pool_form(total, V / epv)) {
+        const long long range = (total + num_sms() - 1) / num_sms();
+        p.pool = true;
+        p.vec_per_warp = (int)range;
+        p.warps = (int)((total + range - 1) / range);
+    }
     return p;
 }
 
@@ -494,9 +631,17 @@ int launch_verify(const int32_t *cand_tok, const void *base_logits, int dtype, i
     float2 *part = (float2 *)(w + plan.off_part);
     const long long total = (skew + (long long)plan.rows * V + (1 << shift) - 1) >> shift;
     const long long warps = (total + plan.vec_per_warp - 1) / plan.vec_per_warp;
-    const unsigned grid = (unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
-    SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_stream_kernel<true> : verify_stream_kernel<false>, dim3(grid), dim3(kArgmaxThreads),
-                             0, st, base, skew, plan.rows, V, total, plan.vec_per_warp, plan.warps, g, part));
+    if (plan.pool) {
+        int block = plan.vec_per_warp / (kPoolThreads / 32 * 8) / (32 * kStreamUnroll) * (32 * kStreamUnroll);
+        block = block < 32 * kStreamUnroll ? 32 * kStreamUnroll : block > 2048 ? 2048 : block;   // about eight blocks a warp
+        SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_pool_kernel<true> : verify_pool_kernel<false>, dim3((unsigned)warps),
+                                 dim3(kPoolThreads), 0, st, base, skew, plan.rows, V, total, plan.vec_per_warp, block, plan.warps, g,
+                                 part));
+    } else {
+        const unsigned grid = (unsigned)((warps + kWarpsPerBlock - 1) / kWarpsPerBlock);
+        SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_stream_kernel<true> : verify_stream_kernel<false>, dim3(grid), dim3(kArgmaxThreads),
+                                 0, st, base, skew, plan.rows, V, total, plan.vec_per_warp, plan.warps, g, part));
+    }
     size_t smem = sizeof(int32_t) * (size_t)rows_b;
     const int g_in_smem = smem <= 40 * 1024;
     if (!g_in_smem) smem = 0;

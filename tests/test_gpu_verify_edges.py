@@ -94,6 +94,47 @@ def test_every_alignment_of_the_base(B, V, dtype):
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("rows,vectors,extra,off", [(130, 3072, 0, 0), (130, 3072, -1, 0), (130, 3072, -1, 3), (131, 3072, 1, 1),
+                                                    (131, 3079, 2, 2), (26, 16032, 0, 0), (26, 16032, 3, 3), (26, 16032, -3, 1),
+                                                    (148, 4096, 0, 0), (149, 4096, 1, 2), (401, 3100, -2, 0), (2, 210001, 1, 1)])
+def test_long_rows_shared_by_the_warps_of_an_sm(B, rows, vectors, extra, off, dtype):
+    """Rows of `vectors` 16-byte vectors plus `extra` elements, the tensor `off` elements past a vector's start: below, at and above
+    the sizes from which an SM's warps share one range, and rows that begin and end inside a vector.  Maxima at the ends of the
+    row, of a trip, of a block and of an SM's range; a second, equal one further right in every third row; rows of -inf, of
+    NaN, and with one NaN before the maximum."""
+    epv = 8 if dtype == torch.bfloat16 else 4
+    V = vectors * epv + extra
+    g = torch.Generator(device="cuda").manual_seed(V + rows + off)
+    buf = torch.randn(rows * V + 2 * epv, generator=g, device="cuda", dtype=torch.float32).clamp_(max=7.0).to(dtype)
+    buf[:off] = 50.0
+    buf[off + rows * V:] = 50.0                           # what lies before and behind the tensor must not be seen
+    flat = buf[off:off + rows * V].view(rows, V)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    span = -(-(rows * V // epv) // sms) * epv             # elements of one SM's range
+    for r in range(rows):
+        start = r * V
+        edge = (-start) % span                            # the first element of a range inside this row, if it has one
+        p = [0, V - 1, 256 * epv - 1, 2048 * epv, min(edge, V - 1), max(0, min(edge, V) - 1), V // 3][r % 7]
+        flat[r, p] = 9.0
+        if r % 3 == 0:
+            flat[r, p + (V - 1 - p) // 2] = 9.0
+        if r % 11 == 5:
+            flat[r] = float("-inf")
+        if r % 11 == 6:
+            flat[r] = float("nan")
+        if r % 11 == 7:
+            flat[r, 0] = float("nan")
+    # two positions per candidate
+    K = 1
+    Bn, n = rows // 2, 1
+    logits = flat[:2 * Bn].view(Bn, K, n + 1, V)
+    cand = torch.randint(0, V, (Bn, K, n), dtype=torch.int64).to(torch.int32)
+    am = logits.float().nan_to_num(nan=float("-inf"), posinf=float("inf"), neginf=float("-inf")).argmax(-1).cpu()
+    cand[::2, 0, 0] = am[::2, 0, 0].to(torch.int32)
+    _check(B, cand, logits)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("Bn,K,n,vectors", [(1, 2, 3, 6143), (1, 2, 3, 6144), (1, 3, 1, 6145), (2, 37, 2, 6150),
                                             (3, 25, 2, 6151), (4, 37, 1, 3073), (149, 1, 1, 3073), (16, 37, 1, 1535),
                                             (16, 37, 1, 1536), (593, 1, 1, 1536), (1, 1, 9, 1537), (7, 3, 3, 1)])

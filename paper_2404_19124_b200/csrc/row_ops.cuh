@@ -35,10 +35,9 @@ struct Scratch {
     int cand_i[kMaxGroupWarps][kMaxRounds];        // ... and token ids
 };
 
-// (`red`: one float per warp, not read by anybody else until the next barrier behind the call.  `in_order`: the warps' sums are
-// added one after the other, as mix_children adds them, instead of in a tree.)
+// (`red`: one float per warp, not read by anybody else until the next barrier behind the call.)
 template <int kThreads, typename Sync>   // (kThreads 0: blockDim.x)
-__device__ __forceinline__ float group_sum(float v, float *red, int tid, bool in_order = false) {
+__device__ __forceinline__ float group_sum(float v, float *red, int tid) {
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     if (kThreads == 32) return v;
@@ -46,16 +45,33 @@ __device__ __forceinline__ float group_sum(float v, float *red, int tid, bool in
     if (l == 0) red[w] = v;
     Sync::sync();
     const int warps = (kThreads > 0 ? kThreads : (int)blockDim.x) / 32;
-    if (in_order) {   // (uniform)
-        float t = 0.0f;
-#pragma unroll
-        for (int q = 0; q < warps; ++q) t += red[q];
-        return t;
-    }
     float t = l < warps ? red[l] : 0.0f;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
     return t;
+}
+
+// The sum over a row of which a thread holds kIters groups of eight.  `in_order`: v[it] is the sum of group it, 256 elements are
+// summed at a time and those sums added one after the other, as mix_children adds them; else v[kIters - 1] is the sum of all
+// of the thread's groups, and the threads' are added in a tree.
+template <int kThreads, int kIters, typename Sync>
+__device__ __forceinline__ float group_sums(const float (&v)[kIters], float *red, int tid, bool in_order) {
+    if (in_order) {   // (uniform)
+        const int warps = (kThreads > 0 ? kThreads : (int)blockDim.x) / 32;
+#pragma unroll
+        for (int it = 0; it < kIters; ++it) {
+            float x = v[it];
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
+            if ((tid & 31) == 0) red[it * warps + (tid >> 5)] = x;
+        }
+        Sync::sync();
+        float t = 0.0f;
+#pragma unroll
+        for (int q = 0; q < kIters * warps; ++q) t += red[q];
+        return t;
+    }
+    return group_sum<kThreads, Sync>(v[kIters - 1], red, tid);
 }
 
 template <int kThreads, typename Sync>
@@ -126,7 +142,7 @@ __device__ __forceinline__ void parent_state(const MixArgs &m, int parent, int t
 // kDepth of those groups, and kSp partial projections of each, have their loads in flight together (registers against
 // latency).
 // `pre`: the projected parent state of this thread's groups (parent_state), if the caller has it already.  `in_order`: see
-// group_sum.
+// group_sums (at most two groups).
 template <int kThreads, int kIters, int kDepth, typename Sync, int kSp = 4>
 __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int parent, int t, int tid, float *red,
                                                 const float (*pre)[8] = nullptr, bool in_order = false) {
@@ -138,7 +154,8 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
     const uint16_t *e = nullptr;
 
     float h[kIters][8];
-    float sum = 0.0f;
+    float sums[kIters];
+    const bool ordered = kIters <= 2 && in_order;
 #pragma unroll
     for (int g0 = 0; g0 < kIters; g0 += kGroup) {
         // every load of the group is issued before the first value is used: one round trip per group
@@ -185,12 +202,14 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
                 }
             }
             const uint32_t ew[4] = {ev[q].x, ev[q].y, ev[q].z, ev[q].w};
+            float sum = it > 0 && !ordered ? sums[it > 0 ? it - 1 : 0] : 0.0f;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
                 const float z = (j & 1) ? __uint_as_float(ew[j >> 1] & 0xffff0000u) : __uint_as_float(ew[j >> 1] << 16);
                 h[it][j] = i < d ? mix_element(m, pv[j], z) : 0.0f;
                 sum += h[it][j];
             }
+            sums[it] = sum;
         }
     }
     // LayerNorm parameters: requested before the two reductions so that they arrive while those run
@@ -209,11 +228,11 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
             bq[it][1] = *(const float4 *)(m.beta + ic + 4);
         }
     }
-    const float mean = group_sum<kThreads, Sync>(sum, red, tid, in_order) / (float)d;
-    float sq = 0.0f;
+    const float mean = group_sums<kThreads, kIters, Sync>(sums, red, tid, ordered) / (float)d;
 #pragma unroll
     for (int it = 0; it < kIters; ++it) {
         const int i = (it * nt + tid) * 8;
+        float sq = it > 0 && !ordered ? sums[it > 0 ? it - 1 : 0] : 0.0f;
         if (i < d) {
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
@@ -221,8 +240,9 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
                 sq += c * c;
             }
         }
+        sums[it] = sq;
     }
-    const float var = group_sum<kThreads, Sync>(sq, red + kMaxGroupWarps, tid, in_order) / (float)d;
+    const float var = group_sums<kThreads, kIters, Sync>(sums, red + kMaxGroupWarps, tid, ordered) / (float)d;
     const float rstd = rsqrtf(var + m.eps);
     float amax = 0.0f;   // largest magnitude of the bf16-rounded state (for the e4m3 copy); h is reused for it
 #pragma unroll
@@ -247,13 +267,15 @@ __device__ __forceinline__ void mix_ln_gelu_row(const MixArgs &m, int r, int par
             y.z = (h[it][j + 2] - mean) * rstd * gv[j + 2] + bv[j + 2];
             y.w = (h[it][j + 3] - mean) * rstd * gv[j + 3] + bv[j + 3];
             y = gelu_erf4(y);
-            packed[j >> 1] = float_to_bf16_bits(y.x) | (float_to_bf16_bits(y.y) << 16);
-            packed[(j >> 1) + 1] = float_to_bf16_bits(y.z) | (float_to_bf16_bits(y.w) << 16);
+            packed[j >> 1] = pack_bf16x2(y.x, y.y);
+            packed[(j >> 1) + 1] = pack_bf16x2(y.z, y.w);
+        }
+        if (m.S8_out != nullptr) {   // (uniform)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const uint32_t w = packed[(j + q) >> 1];
-                h[it][j + q] = i < d ? __uint_as_float((q & 1) ? w & 0xffff0000u : w << 16) : 0.0f;
-                amax = fmaxf(amax, fabsf(h[it][j + q]));
+            for (int j = 0; j < 8; ++j) {
+                const uint32_t w = packed[j >> 1];
+                h[it][j] = i < d ? __uint_as_float((j & 1) ? w & 0xffff0000u : w << 16) : 0.0f;
+                amax = fmaxf(amax, fabsf(h[it][j]));
             }
         }
         if (i < d) *(uint4 *)(m.S_out + (size_t)r * d + i) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
@@ -595,8 +617,8 @@ __device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int f
                     y.z = (h[q][it][j + 2] - mean[q]) * rstd[q] * gv[it][j + 2] + bv[it][j + 2];
                     y.w = (h[q][it][j + 3] - mean[q]) * rstd[q] * gv[it][j + 3] + bv[it][j + 3];
                     y = gelu_erf4(y);
-                    packed[j >> 1] = float_to_bf16_bits(y.x) | (float_to_bf16_bits(y.y) << 16);
-                    packed[(j >> 1) + 1] = float_to_bf16_bits(y.z) | (float_to_bf16_bits(y.w) << 16);
+                    packed[j >> 1] = pack_bf16x2(y.x, y.y);
+                    packed[(j >> 1) + 1] = pack_bf16x2(y.z, y.w);
                 }
                 if (i < d) *(uint4 *)(m.S_out + row * d + i) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
             }

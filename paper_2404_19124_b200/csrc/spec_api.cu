@@ -589,6 +589,7 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
     const bool fold_prune = !h->profile;
     bool proj_done = false;   // the projection of the level about to start ran with the previous head
     bool mix_done = false;    // the states of the level about to start were written by the previous level's merge
+    bool in_order = false;    // ... or would have been by a kernel that takes the LayerNorm sums in another order
     for (int l = 0; l < p.n; ++l) {
         const int rows = p.N[l];
         const int parent_rows = l == 0 ? B : p.N[l - 1];
@@ -611,10 +612,12 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
         // gather + mix + LayerNorm + GELU -> bf16 state of every node of this level
         const bool fp8 = p.use_fp8[l];
         if (!mix_done) {
-            rc = launch_mix_ln_gelu(mix_args(l), rows, st);
+            MixArgs mx = mix_args(l);
+            mx.in_order = in_order ? 1 : 0;
+            rc = launch_mix_ln_gelu(mx, rows, st);
             if (rc != SPEC_OK) return rc;
         }
-        mix_done = false;
+        mix_done = in_order = false;
         SPEC_PROF_MARK();
         // vocabulary head with the fused per-tile top-k / log-sum-exp epilogue.  The next level's
         // projection needs nothing newer than this level's states either, so it rides in the same
@@ -680,8 +683,10 @@ int spec_draft(spec_handle_t h, const void *ctx_state, const int32_t *last_tok, 
             if (proj_done) {
                 // the children's states in the same launch where that pays: their tokens are found here and their
                 // parent projection (this level's rows) ran with the head above
-                rc = launch_merge_mix(g, mix_args(l + 1), rows, st);
+                const MixArgs mx = mix_args(l + 1);
+                rc = launch_merge_mix(g, mx, rows, st);
                 mix_done = rc == SPEC_OK;
+                in_order = !mix_done && mix_sums_in_order(g.topk, mx);
             }
             if (rc == SPEC_ERR_SHAPE) rc = launch_merge_expand(g, rows, st);
         }

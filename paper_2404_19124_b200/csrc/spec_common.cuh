@@ -27,6 +27,13 @@ __device__ __forceinline__ uint32_t float_to_bf16_bits(float f) {
     return u >> 16;
 }
 
+// Two of them, `lo` in the low half, in one instruction (a NaN becomes the canonical one).
+__device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+
 // Programmatic dependent launch: every kernel of the library is enqueued with the
 // "programmatic stream serialization" attribute.  A kernel lets its successor start early
 // (griddep_launch, executed by all threads near the top) so the successor's launch latency,
@@ -164,6 +171,7 @@ struct MixArgs {
     const int32_t *tok;        // [rows]
     const float *gamma, *beta; // fp32 [d]
     int d, V, parent_div;
+    int in_order;              // LayerNorm sums as the kernels take them that compute a parent's one or two children (group_sums)
     float a, b, eps;
     uint16_t *S_out;           // bf16 [rows, d]
     uint8_t *S8_out;           // optional: the same states as e4m3 bytes [rows, d] ...
@@ -222,6 +230,7 @@ int launch_mix_ln_gelu(const MixArgs &m, int rows, cudaStream_t st);
 int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st);
 // merge of one level + mix of the next in one kernel; SPEC_ERR_SHAPE: shape not covered, launch them separately
 int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_t st);
+bool mix_sums_in_order(int topk, const MixArgs &m);   // see launch_merge_mix
 // Cross-shard merge of a vocabulary-parallel head.  Slot g (g < n_ranks, `slot_bytes` apart, starting at
 // `slots`) holds rank g's raw lists: fp32 values [rows, topk], int32 token ids [rows, topk], fp32 lse [rows].
 // Children of every row: the topk best of the n_ranks*topk entries (value desc, token id asc) with

@@ -253,6 +253,29 @@ def test_states_are_the_same_bits_in_every_kernel(B, k, d):
     B.spec_destroy(h)
 
 
+@pytest.mark.parametrize("k", [1, 2])
+@pytest.mark.parametrize("d", [264, 1032, 2048, 2056, 3080, 4096])
+def test_states_are_the_same_bits_above_and_below_one_parent_per_sm(B, k, d):
+    """148 parents of one or two children: one kernel finds and computes these; 150 parents: the merge and the mix are kernels of
+    their own.  The sequences that both batches have get the same states."""
+    topk, n0 = (2, k, 1), 74
+    cfg = small_cfg(d_base=64, d_inner=d, V=600, topk=topk, K=2 * k, B=n0 + 1, seed=d)
+    sw = synth.make_weights(cfg)
+    ctx, tok = synth.make_draft_inputs(cfg)
+    h = B.spec_create(weights_to_cuda(sw))
+    got = []
+    for n in (n0, n0 + 1):
+        _, _, ws = B.spec_draft(h, ctx[:n].cuda(), tok[:n].cuda(), topk, cfg.K)
+        assert B.spec_poll_error(ws) == 0
+        lay = B.spec_draft_layout(h, n, topk, cfg.K)
+        rows = [n0, 2 * n0, 2 * k * n0]
+        got.append([ws[lay.state[l]:lay.state[l] + 2 * rows[l] * d].view(torch.int16) for l in range(3)] +
+                   [ws[lay.tok[l]:lay.tok[l] + 4 * rows[l]].view(torch.int32) for l in (1, 2)])
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
+    B.spec_destroy(h)
+
+
 @pytest.mark.parametrize("d,what", [(256, "ln_gamma"), (256, "ln_beta"), (512, "ln_gamma"), (40, "ln_beta"), (256, "proj"), (256, "head")])
 def test_a_small_draft_reads_its_weights_in_stream_order(B, d, what):
     """spec_next_ctx, whose kernel lets its dependents start at once and waits behind a long verification itself, writes into

@@ -123,6 +123,69 @@ __global__ void __launch_bounds__(kMergeThreads) merge_expand_kernel(MergeArgs g
     prune_if_last<kMergeThreads, BlockSync>(g, blockIdx.x, threadIdx.x, merge_keys, &last_of_sequence);
 }
 
+// The last level's merge and the prune, one CTA per sequence, one warp per row: the leaves' scores meet in shared memory, where
+// with a CTA per row the rows of a sequence were counted in (a fence, an atomic, the scores back from L2: 3.4 us) and 384
+// CTAs took turns on the SMs.  A warp needs longer for a row than five (1.9 us for 143 lists), about 0.2 us per 32 lists beyond the
+// first.  Exposed time, a CTA per row -> this: 12 rows a
+// sequence (7B shape) 6.2 -> 4.7 us, 24 rows of 16 sequences (13B) 9.0 -> 8.2; the batch-1 draft 129.5 -> 126.5, the ragged step 119.8 -> 118.3.
+// At most 48 registers, so that the widest CTA fits beside a resident GEMM CTA.
+struct OneWarp {
+    static __device__ __forceinline__ void sync() { __syncwarp(); }
+};
+constexpr int kPruneRows = 24, kPruneLists = 256;   // at most: rows of a sequence (warps of the CTA), lists of a row
+template <int kLen>
+__global__ void __maxnreg__(48) merge_prune_kernel(MergeArgs g) {
+    __shared__ float4 scores4[kPruneRows * SPEC_MAX_TOPK / 4];
+    __shared__ int toks[kPruneRows * SPEC_MAX_TOPK];
+    float *scores = (float *)scores4;
+    griddep_launch();
+    griddep_wait();
+    const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, L = g.L, topk = g.topk;
+    const int r = b * g.rows_per_seq + warp;
+    const float base = (lane < topk && g.score_in) ? __ldcg(g.score_in + r) : 0.0f;
+    int32_t path[SPEC_MAX_HEADS];
+    const MergeOut o = merge_select<32, kLen, OneWarp>(g, r, lane, nullptr, topk);
+    // the ancestors of leaf `tid`, whose place depends on nothing but its index, on their way until the scores are there
+    if (tid < L) {
+        int idx = tid / topk, per_seq = g.rows_per_seq;
+#pragma unroll
+        for (int l = SPEC_MAX_HEADS - 2; l >= 0; --l) {
+            if (l < g.prune.n - 1) {
+                path[l] = __ldcg(g.prune.tok[l] + (size_t)b * per_seq + idx);
+                idx /= g.prune.topk[l];
+                per_seq /= g.prune.topk[l];
+            }
+        }
+    }
+    if (lane < topk) {
+        const float score = base + (o.val - o.lse);
+        g.tok_out[(size_t)r * topk + lane] = o.id;
+        g.score_out[(size_t)r * topk + lane] = score;
+        scores[warp * topk + lane] = score;
+        toks[warp * topk + lane] = o.id;
+    }
+    if (tid < 3 && L + tid < (L + 3) / 4 * 4) scores[L + tid] = __int_as_float(0x7fffffff);   // (NaN: before nobody)
+    __syncthreads();
+    if (tid >= L) return;
+    const float mine = scores[tid];
+    int rank = 0;   // leaves before this one: a better score, or the same and a lower index
+    for (int j = 0; j < L; j += 4) {
+        const float4 s = scores4[j / 4];
+        rank += (s.x > mine) | ((s.x == mine) & (j < tid));
+        rank += (s.y > mine) | ((s.y == mine) & (j + 1 < tid));
+        rank += (s.z > mine) | ((s.z == mine) & (j + 2 < tid));
+        rank += (s.w > mine) | ((s.w == mine) & (j + 3 < tid));
+    }
+    if (rank >= g.K) return;
+    const size_t c = (size_t)b * g.K + rank;
+    g.cand_logp[c] = mine;
+    int32_t *cand = g.cand_tok + c * g.prune.n;
+#pragma unroll
+    for (int l = 0; l < SPEC_MAX_HEADS - 1; ++l)
+        if (l < g.prune.n - 1) cand[l] = path[l];
+    cand[g.prune.n - 1] = toks[tid];
+}
+
 // Merge of level l and the gather + mix + LayerNorm + GELU of level l + 1 in one launch, for one or two children per row
 // more children than SMs but no more rows: one CTA of 256 threads per row of level l folds the row's partial lists into its children (tokens, scores) and then computes the
 // states of those children, whose tokens it has just found and whose parent projection is this row's.  One
@@ -292,6 +355,11 @@ int launch_draft_init(int32_t *hdr, int words, cudaStream_t st) {
 int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st) {
     const size_t smem = g.seq_done ? prune_smem_bytes(g.L, g.Lpad) : 0;
     const bool four = (g.list_len > 0 ? g.list_len : g.topk) <= 4;
+    if (g.seq_done && g.rows_per_seq <= kPruneRows && g.n_tiles <= kPruneLists) {
+        SPEC_CUDA_TRY(launch_pdl(four ? merge_prune_kernel<4> : merge_prune_kernel<8>, dim3(rows / g.rows_per_seq),
+                                 dim3(32 * g.rows_per_seq), 0, st, g));
+        return SPEC_OK;
+    }
     SPEC_CUDA_TRY(launch_pdl(four ? merge_expand_kernel<4> : merge_expand_kernel<8>, dim3(rows), dim3(kMergeThreads), smem, st, g));
     return SPEC_OK;
 }

@@ -426,6 +426,13 @@ __device__ __forceinline__ MergeOut merge_select(const MergeArgs &g, int r, int 
     float ws = (m > -INFINITY) ? s * __expf(m - wm) : 0.0f;
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) ws += __shfl_xor_sync(0xffffffffu, ws, off);
+    MergeOut out;
+    if constexpr (kWarps == 1) {   // nothing to merge (`sc` is not used)
+        out.val = cv;
+        out.id = ci;
+        out.lse = wm + logf(ws);
+        return out;
+    }
     if (lane < rounds) {
         sc->cand_k[warp][lane] = float_key(cv);
         sc->cand_i[warp][lane] = ci;
@@ -435,7 +442,6 @@ __device__ __forceinline__ MergeOut merge_select(const MergeArgs &g, int r, int 
         sc->red_s[warp] = ws;
     }
     Sync::sync();
-    MergeOut out;
     {
         const float pm = lane < kWarps ? sc->red_m[lane] : -INFINITY;
         const float ps = lane < kWarps ? sc->red_s[lane] : 0.0f;

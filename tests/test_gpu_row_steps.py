@@ -53,6 +53,36 @@ def test_prune_leaves_round_the_thread_counts(B, topk, K, fp8):
     B.spec_destroy(h)
 
 
+@pytest.mark.parametrize("V", [31 * 32, 33 * 32, 256 * 32, 256 * 32 + 1])
+@pytest.mark.parametrize("topk,K,rows", [((1, 1), 1, 1), ((1, 7), 5, 1), ((4, 3, 2), 16, 12), ((6, 4, 3), 72, 24), ((6, 4, 8), 100, 24),
+                                         ((5, 5, 8), 100, 25)])
+def test_last_merge_and_prune_of_a_sequence(B, topk, K, rows, V):
+    """Up to 24 rows a sequence and 256 lists a row the last merge is one CTA per sequence; the kept leaves are the best of the
+    scores that it leaves in the workspace, in order, with the tokens of their paths."""
+    cfg = small_cfg(d_base=48, d_inner=64, V=V, topk=topk, K=K, B=3, seed=K)
+    sw = synth.make_weights(cfg)
+    ctx, tok = synth.make_draft_inputs(cfg)
+    h = B.spec_create(weights_to_cuda(sw))
+    B.spec_set_option(h, B.SPEC_OPT_HEAD_BLOCK_N, 32)
+    ct, lp, ws = B.spec_draft(h, ctx.cuda(), tok.cuda(), topk, K)
+    assert B.spec_poll_error(ws) == 0
+    lay = B.spec_draft_layout(h, cfg.B, topk, K)
+    n, L = cfg.n, cfg.leaves
+    assert L == rows * topk[-1]
+    leaf = ws[lay.score[n]:lay.score[n] + 4 * cfg.B * L].view(torch.float32).view(cfg.B, L)
+    want = torch.sort(leaf, dim=1, descending=True, stable=True)
+    assert torch.equal(lp, want.values[:, :K])
+    per = 1
+    for l in range(n):
+        per *= topk[l]
+        t = ws[lay.tok[l + 1]:lay.tok[l + 1] + 4 * cfg.B * per].view(torch.int32).view(cfg.B, per)
+        assert torch.equal(ct[:, :, l], torch.gather(t, 1, want.indices[:, :K] // (L // per)))
+    chk = DraftChecker(to_oracle_weights(sw), topk, K)
+    for b in range(cfg.B):
+        chk.check(synth.bf16_bits(ctx)[b], int(tok[b]), ct[b].cpu().numpy(), lp[b].cpu().numpy())
+    B.spec_destroy(h)
+
+
 @pytest.mark.parametrize("swap", [0, 128])
 @pytest.mark.parametrize("k", [1, 4, 5, 8])
 @pytest.mark.parametrize("V", [159 * 32, 160 * 32, 161 * 32, 320 * 32 + 1, 80000])

@@ -13,7 +13,7 @@ namespace {
 using namespace rows;
 
 constexpr int kRowThreads = 256;
-constexpr int kFusedMixMaxChildren = 2;
+constexpr int kFusedMixMaxChildren = 2;   // (list_slots(2) below)
 constexpr int kMergeThreads = 160;   // one list per thread up to V = 35000 (a CTA of the head GEMM leaves one)
 
 // Rows of up to 2048 elements: at most 128 registers, so that two CTAs fit beside a resident GEMM CTA.
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) merge_mix_kernel(MergeMixArgs 
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, tid = threadIdx.x;
-    const int tok = merge_expand_row<kRowThreads, 4, BlockSync>(a.merge, r, tid, &sc).id;
+    const int tok = merge_expand_row<kRowThreads, 2, BlockSync>(a.merge, r, tid, &sc).id;
     mix_children<kRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
 }
 
@@ -217,7 +217,7 @@ __global__ void __maxnreg__(72) merge_mix_512_kernel(MergeMixArgs a) {
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, tid = threadIdx.x;
-    const int tok = merge_expand_row<kWideRowThreads, 4, BlockSync>(a.merge, r, tid, &sc).id;
+    const int tok = merge_expand_row<kWideRowThreads, 2, BlockSync>(a.merge, r, tid, &sc).id;
     mix_children<kWideRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
 }
 
@@ -354,13 +354,14 @@ int launch_draft_init(int32_t *hdr, int words, cudaStream_t st) {
 
 int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st) {
     const size_t smem = g.seq_done ? prune_smem_bytes(g.L, g.Lpad) : 0;
-    const bool four = (g.list_len > 0 ? g.list_len : g.topk) <= 4;
+    const int slots = list_slots(g.list_len > 0 ? g.list_len : g.topk);
     if (g.seq_done && g.rows_per_seq <= kPruneRows && g.n_tiles <= kPruneLists) {
-        SPEC_CUDA_TRY(launch_pdl(four ? merge_prune_kernel<4> : merge_prune_kernel<8>, dim3(rows / g.rows_per_seq),
+        SPEC_CUDA_TRY(launch_pdl(slots == 2 ? merge_prune_kernel<2> : slots == 4 ? merge_prune_kernel<4> : merge_prune_kernel<8>, dim3(rows / g.rows_per_seq),
                                  dim3(32 * g.rows_per_seq), 0, st, g));
         return SPEC_OK;
     }
-    SPEC_CUDA_TRY(launch_pdl(four ? merge_expand_kernel<4> : merge_expand_kernel<8>, dim3(rows), dim3(kMergeThreads), smem, st, g));
+    SPEC_CUDA_TRY(launch_pdl(slots == 2 ? merge_expand_kernel<2> : slots == 4 ? merge_expand_kernel<4> : merge_expand_kernel<8>, dim3(rows),
+                             dim3(kMergeThreads), smem, st, g));
     return SPEC_OK;
 }
 
@@ -380,12 +381,16 @@ int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_
     a.merge.next_emb = nullptr;   // the gather follows in the same CTA
     const int children = rows * g.topk;
     if (children <= num_sms()) {
-        const bool four = (g.list_len > 0 ? g.list_len : g.topk) <= 4;
+        const int slots = list_slots(g.list_len > 0 ? g.list_len : g.topk);
         if (m.d > 8 * kRowThreads)
-            SPEC_CUDA_TRY(launch_pdl(four ? merge_mix_child_512_kernel<4> : merge_mix_child_512_kernel<8>, dim3(children),
+            SPEC_CUDA_TRY(launch_pdl(slots == 2   ? merge_mix_child_512_kernel<2>
+                                     : slots == 4 ? merge_mix_child_512_kernel<4>
+                                                  : merge_mix_child_512_kernel<8>, dim3(children),
                                      dim3(kWideRowThreads), 0, st, a));
         else
-            SPEC_CUDA_TRY(launch_pdl(four ? merge_mix_child_kernel<4> : merge_mix_child_kernel<8>, dim3(children),
+            SPEC_CUDA_TRY(launch_pdl(slots == 2   ? merge_mix_child_kernel<2>
+                                     : slots == 4 ? merge_mix_child_kernel<4>
+                                                  : merge_mix_child_kernel<8>, dim3(children),
                                      dim3(kRowThreads), 0, st, a));
         return SPEC_OK;
     }

@@ -254,7 +254,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constan
             const bool row_ok = row < j.M;
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * j.block_n);
             const int col0 = n_tile * j.block_n;
-            if (j.epi.topk <= 4) epilogue_topk<4, false>(j, taddr, row, row_ok, col0, n_tile);
+            if (j.epi.topk <= 2) epilogue_topk<2, false>(j, taddr, row, row_ok, col0, n_tile);
+            else if (j.epi.topk <= 4) epilogue_topk<4, false>(j, taddr, row, row_ok, col0, n_tile);
             else epilogue_topk<SPEC_MAX_TOPK, false>(j, taddr, row, row_ok, col0, n_tile);
             tc_fence_before();
             __syncwarp();

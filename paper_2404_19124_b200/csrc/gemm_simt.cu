@@ -59,8 +59,8 @@ __global__ void partials_from_logits_kernel(const float *__restrict__ logits, in
     const int r = (int)(u / n_tiles), t = (int)(u - (long long)r * n_tiles);
     const float *x = logits + (size_t)r * N;
     const int c0 = t * block_n, c1 = min(N, c0 + block_n);
-    float *pv = part_val + (size_t)u * SPEC_MAX_TOPK;
-    int32_t *pi = part_idx + (size_t)u * SPEC_MAX_TOPK;
+    float *pv = part_val + (size_t)u * list_slots(topk);
+    int32_t *pi = part_idx + (size_t)u * list_slots(topk);
     for (int j = 0; j < topk; ++j) {
         pv[j] = -INFINITY;
         pi[j] = 0x7fffffff;

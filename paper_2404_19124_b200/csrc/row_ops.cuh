@@ -320,8 +320,8 @@ __device__ __forceinline__ void fold_max_sum(float &m, float &s, const float2 &m
 template <int kLen>
 struct TileList {
     float2 ms;
-    float4 v[kLen / 4];
-    int4 i[kLen / 4];
+    float v[kLen];
+    int i[kLen];
 };
 
 template <int kLen>
@@ -329,10 +329,23 @@ __device__ __forceinline__ void load_list(TileList<kLen> &l, const MergeArgs &g,
     l.ms = make_float2(-INFINITY, 0.0f);
     if (valid) {
         l.ms = __ldcg((const float2 *)g.part_ms + tile);
+        if constexpr (kLen == 2) {
+            const float2 v = __ldcg((const float2 *)g.part_val + tile);
+            const int2 i = __ldcg((const int2 *)g.part_idx + tile);
+            l.v[0] = v.x; l.v[1] = v.y;
+            l.i[0] = i.x; l.i[1] = i.y;
+        } else if constexpr (kLen == 4) {
+            const float4 v = __ldcg((const float4 *)g.part_val + tile);
+            const int4 i = __ldcg((const int4 *)g.part_idx + tile);
+            l.v[0] = v.x; l.v[1] = v.y; l.v[2] = v.z; l.v[3] = v.w;
+            l.i[0] = i.x; l.i[1] = i.y; l.i[2] = i.z; l.i[3] = i.w;
+        } else {
+            const Float8 v = ldcg8(g.part_val + 8 * tile), i = ldcg8((const float *)g.part_idx + 8 * tile);
 #pragma unroll
-        for (int q = 0; q < kLen / 4; ++q) {
-            l.v[q] = __ldcg((const float4 *)g.part_val + 2 * tile + q);
-            l.i[q] = __ldcg((const int4 *)g.part_idx + 2 * tile + q);
+            for (int q = 0; q < 8; ++q) {
+                l.v[q] = v.v[q];
+                l.i[q] = __float_as_int(i.v[q]);
+            }
         }
     }
 }
@@ -345,8 +358,8 @@ struct MergeOut {
     float lse;
 };
 
-// The `rounds` best entries (rounds <= kMaxRounds) of row r's partial lists and the row's log-sum-exp.  kLen is 4
-// when a list has at most four valid slots, else 8.
+// The `rounds` best entries (rounds <= kMaxRounds) of row r's partial lists and the row's log-sum-exp.  kLen: the lists' slots
+// (list_slots).
 // The step is a chain of latencies in a kernel that runs for a few microseconds, so it has one barrier and little
 // code: thread t takes the lists t, t + kThreads, ... one at a time (they are sorted best first), and its warp extracts
 // its own `rounds` best with warp-wide integer reductions (redux.sync: maximum of the value keys, then minimum token id
@@ -382,9 +395,9 @@ __device__ __forceinline__ MergeOut merge_select(const MergeArgs &g, int r, int 
         float tv[kLen];
         int ti[kLen];
 #pragma unroll
-        for (int q = 0; q < kLen / 4; ++q) {
-            tv[4 * q] = cur.v[q].x; tv[4 * q + 1] = cur.v[q].y; tv[4 * q + 2] = cur.v[q].z; tv[4 * q + 3] = cur.v[q].w;
-            ti[4 * q] = cur.i[q].x; ti[4 * q + 1] = cur.i[q].y; ti[4 * q + 2] = cur.i[q].z; ti[4 * q + 3] = cur.i[q].w;
+        for (int q = 0; q < kLen; ++q) {
+            tv[q] = cur.v[q];
+            ti[q] = cur.i[q];
         }
 #pragma unroll
         for (int j = 0; j < kLen; ++j) {

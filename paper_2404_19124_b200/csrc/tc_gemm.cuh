@@ -579,6 +579,24 @@ __device__ __forceinline__ void stage_col_scales(float *cs, const GemmJob &j, in
     __syncwarp();
 }
 
+// Partial list number u and its (max, sum-exp).
+template <int kCap>
+__device__ __forceinline__ void store_list(const GemmEpilogue &e, size_t u, const float (&v)[kCap], const int (&id)[kCap], float m, float s) {
+    float *pv = e.part_val + u * kCap;
+    int32_t *pi = e.part_idx + u * kCap;
+    if constexpr (kCap == 2) {
+        *(float2 *)pv = make_float2(v[0], v[1]);
+        *(int2 *)pi = make_int2(id[0], id[1]);
+    } else {
+#pragma unroll
+        for (int q = 0; q < kCap; q += 4) {
+            *(float4 *)(pv + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+            *(int4 *)(pi + q) = make_int4(id[q], id[q + 1], id[q + 2], id[q + 3]);
+        }
+    }
+    *(float2 *)(e.part_ms + 2 * u) = make_float2(m, s);
+}
+
 template <int kCap, bool kFp8>
 __device__ __forceinline__ void epilogue_topk(const GemmJob &p, uint32_t taddr, int row, bool row_ok, int col0,
                                               int n_tile, float rs = 1.0f, const float *cs = nullptr) {
@@ -675,25 +693,18 @@ __device__ __forceinline__ void epilogue_topk(const GemmJob &p, uint32_t taddr, 
         }
     }
     if (row_ok) {
-        const size_t u = (size_t)row * p.n_tiles + n_tile;
-        float4 *pv = (float4 *)(p.epi.part_val + u * SPEC_MAX_TOPK);
-        int4 *pi = (int4 *)(p.epi.part_idx + u * SPEC_MAX_TOPK);
-#pragma unroll
-        for (int q = 0; q < kCap / 4; ++q) {
-            pv[q] = make_float4(lv[4 * q], lv[4 * q + 1], lv[4 * q + 2], lv[4 * q + 3]);
-            pi[q] = make_int4(li[4 * q], li[4 * q + 1], li[4 * q + 2], li[4 * q + 3]);
-        }
-        *(float2 *)(p.epi.part_ms + 2 * u) = make_float2(run_m, run_s);
+        store_list<kCap>(p.epi, (size_t)row * p.n_tiles + n_tile, lv, li, run_m, run_s);
     }
 }
 
 // ---- epilogue, mode 3 (operands swapped: TMEM lanes are vocabulary rows, columns are nodes) ----------
 // What one scan thread carries from tile to tile: the running (max, sum-exp) of its share of a node's
-// logits and the best SPEC_MAX_TOPK of them, best first by (value desc, token id asc).
+// logits and the best kCap of them, best first by (value desc, token id asc).
+template <int kCap>
 struct SwapRun {
     float m, s;
-    float tv[SPEC_MAX_TOPK];
-    int ti[SPEC_MAX_TOPK];
+    float tv[kCap];
+    int ti[kCap];
 };
 
 // (no short-circuit operators: every comparison would be a divergent branch)
@@ -701,12 +712,13 @@ __device__ __forceinline__ bool cand_better(float v, int i, float w, int j) { re
 
 // Branch-free insertion into the sorted list: slot j takes its left neighbour when the newcomer beats that
 // neighbour, the newcomer when it beats only slot j, and keeps its entry otherwise.
-__device__ __forceinline__ void list_insert(SwapRun &r, float x, int id) {
-    bool beats[SPEC_MAX_TOPK];
+template <int kCap>
+__device__ __forceinline__ void list_insert(SwapRun<kCap> &r, float x, int id) {
+    bool beats[kCap];
 #pragma unroll
-    for (int j = 0; j < SPEC_MAX_TOPK; ++j) beats[j] = cand_better(x, id, r.tv[j], r.ti[j]);
+    for (int j = 0; j < kCap; ++j) beats[j] = cand_better(x, id, r.tv[j], r.ti[j]);
 #pragma unroll
-    for (int j = SPEC_MAX_TOPK - 1; j > 0; --j) {
+    for (int j = kCap - 1; j > 0; --j) {
         r.tv[j] = beats[j - 1] ? r.tv[j - 1] : (beats[j] ? x : r.tv[j]);
         r.ti[j] = beats[j - 1] ? r.ti[j - 1] : (beats[j] ? id : r.ti[j]);
     }
@@ -724,7 +736,7 @@ __device__ __forceinline__ void epi_bar_sync() { asm volatile("bar.sync 1, %0;" 
 // the topk-th entry of the running list, into that list.
 template <int kCap>
 __device__ __forceinline__ void swap_scan_tile(const float *col, int len, int valid, int idx0, int topk, float scale,
-                                               SwapRun &r) {
+                                               SwapRun<kCap> &r) {
     const float kLog2e = 1.4426950408889634f * scale;
     float best[kCap];
 #pragma unroll
@@ -789,21 +801,21 @@ __device__ __forceinline__ void swap_scan_tile(const float *col, int len, int va
     }
 }
 
-// The better eight of two lists that are both sorted best first: "the better of a[i] and b[7 - i]" keeps the
-// best eight as a bitonic sequence, which three compare-exchange stages sort.
-__device__ __forceinline__ void merge_sorted8(SwapRun &r, const float (&ov)[SPEC_MAX_TOPK], const int (&oi)[SPEC_MAX_TOPK]) {
-    constexpr int kT = SPEC_MAX_TOPK;
-    static_assert(kT == 8, "three stages sort eight entries");
+// The better kCap of two lists that are both sorted best first: "the better of a[i] and b[kCap - 1 - i]" keeps the
+// best kCap as a bitonic sequence, which log2(kCap) compare-exchange stages sort.
+template <int kCap>
+__device__ __forceinline__ void merge_sorted(SwapRun<kCap> &r, const float (&ov)[kCap], const int (&oi)[kCap]) {
+    static_assert((kCap & (kCap - 1)) == 0, "a bitonic sort");
 #pragma unroll
-    for (int j = 0; j < kT; ++j) {
-        const bool take = cand_better(ov[kT - 1 - j], oi[kT - 1 - j], r.tv[j], r.ti[j]);
-        r.tv[j] = take ? ov[kT - 1 - j] : r.tv[j];
-        r.ti[j] = take ? oi[kT - 1 - j] : r.ti[j];
+    for (int j = 0; j < kCap; ++j) {
+        const bool take = cand_better(ov[kCap - 1 - j], oi[kCap - 1 - j], r.tv[j], r.ti[j]);
+        r.tv[j] = take ? ov[kCap - 1 - j] : r.tv[j];
+        r.ti[j] = take ? oi[kCap - 1 - j] : r.ti[j];
     }
 #pragma unroll
-    for (int stride = kT / 2; stride > 0; stride >>= 1) {
+    for (int stride = kCap / 2; stride > 0; stride >>= 1) {
 #pragma unroll
-        for (int j = 0; j < kT; ++j) {
+        for (int j = 0; j < kCap; ++j) {
             if ((j & stride) == 0) {   // (compile-time condition: the loops are unrolled)
                 const bool sw = cand_better(r.tv[j + stride], r.ti[j + stride], r.tv[j], r.ti[j]);
                 const float hv = sw ? r.tv[j + stride] : r.tv[j], lv = sw ? r.tv[j] : r.tv[j + stride];
@@ -823,6 +835,7 @@ __device__ __forceinline__ void merge_sorted8(SwapRun &r, const float (&ov)[SPEC
 // tile intact until every scan of this one is done.  After the last tile the P threads of a node (neighbouring
 // lanes) combine their lists and (max, sum-exp) pairs with shuffles and the first of them writes the node's
 // partial slot of this CTA.
+template <int kCap>
 __device__ __forceinline__ bool epilogue_job_swapped(const Pipe &pp, const GemmJob &j, AccPos &ap) {
     constexpr float kLog2e = 1.4426950408889634f;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -834,11 +847,11 @@ __device__ __forceinline__ bool epilogue_job_swapped(const Pipe &pp, const GemmJ
     const bool scans = node < nodes;
     const int topk = j.epi.topk;
     Barriers *bars = pp.bars;
-    SwapRun run;
+    SwapRun<kCap> run;
     run.m = -INFINITY;
     run.s = 0.0f;
 #pragma unroll
-    for (int q = 0; q < SPEC_MAX_TOPK; ++q) {
+    for (int q = 0; q < kCap; ++q) {
         run.tv[q] = -INFINITY;
         run.ti[q] = 0x7fffffff;
     }
@@ -877,46 +890,41 @@ __device__ __forceinline__ bool epilogue_job_swapped(const Pipe &pp, const GemmJ
             int valid = row_end - seg_row;
             valid = valid < 0 ? 0 : (valid > len ? len : valid);
             const float *col = pp.tbuf + node * kTPitch + seg * len;
-            if (topk <= 4) swap_scan_tile<4>(col, len, valid, seg_row + j.epi.idx_offset, topk, node_scale, run);
-            else swap_scan_tile<SPEC_MAX_TOPK>(col, len, valid, seg_row + j.epi.idx_offset, topk, node_scale, run);
+            swap_scan_tile<kCap>(col, len, valid, seg_row + j.epi.idx_offset, topk, node_scale, run);
         }
     }
     if (w.first >= w.end) return true;
     run.m *= node_scale;
 #pragma unroll
-    for (int q = 0; q < SPEC_MAX_TOPK; ++q) run.tv[q] *= node_scale;
+    for (int q = 0; q < kCap; ++q) run.tv[q] *= node_scale;
     // the P neighbouring lanes of a node fold their results (every lane of the warp takes part in the shuffles)
     for (int off = 1; off < P; off <<= 1) {
-        float ov[SPEC_MAX_TOPK];
-        int oi[SPEC_MAX_TOPK];
+        float ov[kCap];
+        int oi[kCap];
 #pragma unroll
-        for (int q = 0; q < SPEC_MAX_TOPK; ++q) {
+        for (int q = 0; q < kCap; ++q) {
             ov[q] = __shfl_xor_sync(0xffffffffu, run.tv[q], off);
             oi[q] = __shfl_xor_sync(0xffffffffu, run.ti[q], off);
         }
         const float om = __shfl_xor_sync(0xffffffffu, run.m, off), os = __shfl_xor_sync(0xffffffffu, run.s, off);
-        merge_sorted8(run, ov, oi);
+        merge_sorted(run, ov, oi);
         const float nm = fmaxf(run.m, om);
         if (nm > -INFINITY)
             run.s = run.s * ex2_approx((run.m - nm) * kLog2e) + os * ex2_approx((om - nm) * kLog2e);
         run.m = nm;
     }
-    if (scans && seg == 0) {
-        const size_t slot = (size_t)node * j.epi.n_parts + (size_t)w.rel;
-        float4 *pv = (float4 *)(j.epi.part_val + slot * SPEC_MAX_TOPK);
-        int4 *pi = (int4 *)(j.epi.part_idx + slot * SPEC_MAX_TOPK);
-        pv[0] = make_float4(run.tv[0], run.tv[1], run.tv[2], run.tv[3]);
-        pv[1] = make_float4(run.tv[4], run.tv[5], run.tv[6], run.tv[7]);
-        pi[0] = make_int4(run.ti[0], run.ti[1], run.ti[2], run.ti[3]);
-        pi[1] = make_int4(run.ti[4], run.ti[5], run.ti[6], run.ti[7]);
-        *(float2 *)(j.epi.part_ms + 2 * slot) = make_float2(run.m, run.s);
-    }
+    if (scans && seg == 0) store_list<kCap>(j.epi, (size_t)node * j.epi.n_parts + (size_t)w.rel, run.tv, run.ti, run.m, run.s);
     return true;
 }
 
 // ---- epilogue warps (warps 2-5, all lanes) ----------------------------------------------------------
 __device__ __forceinline__ bool epilogue_job(const Pipe &pp, const GemmJob &j, AccPos &ap) {
-    if (j.epi.mode == 3) return epilogue_job_swapped(pp, j, ap);
+    if (j.epi.mode == 3) {
+        const int slots = list_slots(j.epi.topk);
+        return slots == 2   ? epilogue_job_swapped<2>(pp, j, ap)
+               : slots == 4 ? epilogue_job_swapped<4>(pp, j, ap)
+                            : epilogue_job_swapped<SPEC_MAX_TOPK>(pp, j, ap);
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int quarter = warp & 3;               // TMEM lane quarter this warp may read
     const int row_in_tile = quarter * 32 + lane;
@@ -971,6 +979,7 @@ __device__ __forceinline__ bool epilogue_job(const Pipe &pp, const GemmJob &j, A
             }
         } else {
             if (j.fp8) epilogue_topk<SPEC_MAX_TOPK, true>(j, taddr, row, row_ok, col0, n_tile, row_scale, col_scales);
+            else if (j.epi.topk <= 2) epilogue_topk<2, false>(j, taddr, row, row_ok, col0, n_tile);
             else if (j.epi.topk <= 4) epilogue_topk<4, false>(j, taddr, row, row_ok, col0, n_tile);
             else epilogue_topk<SPEC_MAX_TOPK, false>(j, taddr, row, row_ok, col0, n_tile);
         }

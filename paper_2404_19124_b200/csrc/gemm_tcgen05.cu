@@ -58,10 +58,10 @@ gemm_tc_kernel(const __grid_constant__ GemmMaps maps, const __grid_constant__ Ge
         if (me < p.producers && elect_one()) {
             RingPos rp{0, 0u};
             int issued = 0;
-            bool ok = true;
+            bool ok = true, waited = false;
             // the weights are fetched before the preceding grid is waited for, the states after
             for (int q = 0; ok && q < p.n_jobs; ++q)
-                ok = produce_job(pp, p.job[q], &maps.a[q], &maps.a_short, &maps.b[q], rp, issued, me, p.producers,
+                ok = produce_job(pp, p.job[q], &maps.a[q], &maps.a_short, &maps.b[q], rp, issued, waited, me, p.producers,
                                  [] { griddep_wait(); return true; });
             if (!ok) producer_drain(pp, rp, issued);
         }

@@ -385,14 +385,15 @@ __device__ __forceinline__ void advance(const Pipe &pp, RingPos &rp) {
 // operand only; then `dep_wait()` is called once (it must return true once the states are readable:
 // the preceding grid has completed, or the grid-wide barrier behind which they are written has
 // opened) and the state operand of those slots follows.  A CTA without a tile in the job neither
-// loads nor waits.  `issued` counts slots filled since the kernel started (for the abort path).
+// loads nor waits.  `waited`: it has been called for an earlier job, and the slots are filled both operands together: the states
+// of the first slot would otherwise follow only when the ring has turned (single-candidate chain 156.4 -> 155.0 us).  `issued` counts slots filled since the kernel started (for the abort path).
 // Producer `me` of `n_prod` walks every slot like the others and fills the slots whose running number
 // `issued` (counted over all jobs of the launch) is congruent to `me` (n_prod is a power of two).
 // One loop serves the first fill, its state operands and the rest, again to keep the code small.
 template <typename DepWait>
 __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, const CUtensorMap *tmap_a,
                                             const CUtensorMap *tmap_a_short, const CUtensorMap *tmap_b, RingPos &rp,
-                                            int &issued, int me, int n_prod, DepWait dep_wait) {
+                                            int &issued, bool &waited, int me, int n_prod, DepWait dep_wait) {
     const TileWalk w = walk_of(j);
     if (w.first >= w.end) return true;
     const int ke = slab_elems(j), num_kb = num_k_blocks(j);
@@ -404,12 +405,13 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
     int tile = w.first;
     TilePos t = pos_of(j, w, tile);
     const int n_pre = min(pp.stages, t.kb1 - t.kb0);   // slots of the first fill
-    bool first_fill = true;
+    int fetched_slots = 0;
+    bool first_fill = !waited;
     RingPos q = rp;
     int kb = t.kb0, kx = t.kb0 + t.k_off, done = 0;   // kx: the column block of slot kb
     for (;;) {
         if (((issued + done) & (n_prod - 1)) == me) {
-            const bool fetched = !first_fill && done < n_pre;   // the weights of this slot are already on their way
+            const bool fetched = !first_fill && done < fetched_slots;   // the weights of this slot are already on their way
             uint8_t *slot = pp.tiles + (size_t)q.stage * pp.slot_bytes;
             uint64_t *full = &bars->full[q.stage];
             if (!fetched) {
@@ -430,7 +432,9 @@ __device__ __forceinline__ bool produce_job(const Pipe &pp, const GemmJob &j, co
         ++kb;
         if (first_fill && done == n_pre) {
             if (!dep_wait()) return false;
+            waited = true;
             first_fill = false;
+            fetched_slots = n_pre;
             q = rp;
             done = 0;
             kb = t.kb0;

@@ -573,13 +573,17 @@ bool one_kernel_form(int B, int rows_b, int V, int dtype) {
            (turns - 1) * V <= 64 * (dtype == SPEC_BF16 ? Elem<true>::kEpv : Elem<false>::kEpv);
 }
 
-// Where verify_pool_kernel takes over from verify_stream_kernel: rows of 48 KB and more, 6 to 512 MB in all.  us a call, stream /
-// pool, bf16: V 2048, 65 MB 17.4 / 20.3, 400 MB 72 / 78; V 8000, 16 MB 9.6 / 9.5, 65 MB 16.0 / 16.7, 131 MB 25.4 / 26.0 (a trip ends at
-// a row's end); V 32000, 2 MB 7.2 / 7.5, 8 MB 8.2 / 7.5.  Above, at the clocks of a long step, the shorter trips of the other form
-// win: V 128256, 5250 MB 765-828 / 765-882.
-constexpr long long kPoolMinRowVec = 3072, kPoolMaxRowVec = 1 << 24, kPoolMinVec = 400000, kPoolMaxVec = 32 << 20;
+// Where verify_pool_kernel takes over from verify_stream_kernel: rows of 48 KB and more, 4.8 to 512 MB in all, or from 1.9 MB where a
+// row is 192 KB.  us a call, stream / pool, bf16: V 2048, 65 MB 17.4 / 20.3, 400 MB 72 / 78; V 8000, 16 MB 9.6 / 9.5, 65 MB 16.0 /
+// 16.7, 131 MB 25.4 / 26.0 (a trip ends at a row's end); V 32000, 3 MB 7.2 / 7.4, 5 MB 7.6 / 7.5, 8 MB 8.4 / 7.4; V 50000, 4 MB 7.5 /
+// 7.6, 4.8 MB 8.1 / 7.3; V 128256, 1 MB 7.6 / 7.4 to 7.6, 2 MB 8.0 / 7.6, 4 MB 9.1 / 7.3 (the other form leaves 63 pieces of such a row
+// to the accept kernel; 7.3 is the host's time for two launches); fp32 V 128256, 2 MB 9.7 / 7.3, 8 MB 12.7 / 7.4.  Above, at the clocks
+// of a long step, the shorter trips of the other form win: V 128256, 5250 MB 765-828 / 765-882.
+constexpr long long kPoolMinRowVec = 3072, kPoolMaxRowVec = 1 << 24, kPoolMinVec = 300000, kPoolMaxVec = 32 << 20;
+constexpr long long kPoolLongRowVec = 12000, kPoolLongMinVec = 120000;
 bool pool_form(long long total_vec, long long row_vec) {
-    return row_vec >= kPoolMinRowVec && row_vec <= kPoolMaxRowVec && total_vec >= kPoolMinVec && total_vec <= kPoolMaxVec &&
+    return row_vec >= kPoolMinRowVec && row_vec <= kPoolMaxRowVec &&
+           total_vec >= (row_vec >= kPoolLongRowVec ? kPoolLongMinVec : kPoolMinVec) && total_vec <= kPoolMaxVec &&
            (total_vec + num_sms() - 1) / num_sms() / row_vec + 3 <= kPoolMaxRows;
 }
 

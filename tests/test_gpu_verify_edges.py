@@ -96,7 +96,9 @@ def test_every_alignment_of_the_base(B, V, dtype):
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("rows,vectors,extra,off", [(130, 3072, 0, 0), (130, 3072, -1, 0), (130, 3072, -1, 3), (131, 3072, 1, 1),
                                                     (131, 3079, 2, 2), (26, 16032, 0, 0), (26, 16032, 3, 3), (26, 16032, -3, 1),
-                                                    (148, 4096, 0, 0), (149, 4096, 1, 2), (401, 3100, -2, 0), (2, 210001, 1, 1)])
+                                                    (148, 4096, 0, 0), (149, 4096, 1, 2), (401, 3100, -2, 0), (2, 210001, 1, 1),
+                                                    (96, 3125, 0, 0), (96, 3125, -1, 0), (8, 16032, 0, 0), (8, 16032, 1, 3), (6, 16032, 1, 3),
+                                                    (10, 12000, 0, 0), (10, 12000, -1, 0)])
 def test_long_rows_shared_by_the_warps_of_an_sm(B, rows, vectors, extra, off, dtype):
     """Rows of `vectors` 16-byte vectors plus `extra` elements, the tensor `off` elements past a vector's start: below, at and above
     the sizes from which an SM's warps share one range, and rows that begin and end inside a vector.  Maxima at the ends of the

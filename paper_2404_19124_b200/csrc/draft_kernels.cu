@@ -2,6 +2,7 @@
 //   mix_ln_gelu_kernel   one CTA of 256 threads per tree node
 //   merge_expand_kernel  one CTA of 160 threads per row of the vocabulary head
 //   prune_kernel         one CTA of 256 threads per sequence
+//   merge_prune_kernel   one CTA per sequence, one warp per row: the last level's merge and the prune in one
 // Each is launched with programmatic stream serialization, so its CTAs are usually resident, waiting,
 // while the kernel before it still runs.
 #include "row_ops.cuh"

@@ -235,6 +235,11 @@ verify_pool_kernel(const char *__restrict__ base, int skew, int rows, int V, lon
                 uint4 v[kStreamUnroll];
 #pragma unroll
                 for (int u = 0; u < kStreamUnroll; ++u) v[u] = ld_stream(src + min(i + 32 * u + lane, q - 1));
+                // What the row has already, as one lane sees it: other warps raise the key meanwhile, and whether the warp goes on
+                // to the next reduction must be one decision.  (An old value costs an update, the maximum is taken there.)
+                uint32_t seen = 0u;
+                if (lane == 0) seen = (uint32_t)(*(volatile unsigned long long *)&keys[r] >> 32);
+                seen = __shfl_sync(0xffffffffu, seen, 0);
                 float mx;
                 if (kBf16) {
                     uint32_t m[kStreamUnroll];
@@ -258,8 +263,7 @@ verify_pool_kernel(const char *__restrict__ base, int skew, int rows, int V, lon
                 }
                 const uint32_t key = mx > -INFINITY ? value_key(mx) : 0u;   // (NaN: nothing)
                 const uint32_t top = __reduce_max_sync(0xffffffffu, key);
-                // most trips find nothing that reaches what their row has already
-                if (top == 0u || top < (uint32_t)(*(volatile unsigned long long *)&keys[r] >> 32)) continue;
+                if (top == 0u || top < seen) continue;   // most trips find nothing that reaches what their row has already
                 int pos = kIdxNone;
                 if (key == top) {
 #pragma unroll

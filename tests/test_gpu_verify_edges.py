@@ -137,6 +137,24 @@ def test_long_rows_shared_by_the_warps_of_an_sm(B, rows, vectors, extra, off, dt
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("V", [24577, 128256])
+def test_rows_whose_maximum_rises_trip_by_trip(B, V, dtype):
+    """Rows that rise from end to end, fall, or rise in every 256 vectors: the warps that share such a row raise its key again and
+    again while others compare with it, and some trips of a warp reach it and some do not."""
+    epv = 8 if dtype == torch.bfloat16 else 4
+    Bn, K, n = 6_000_000 // V // 4, 2, 1
+    i = torch.arange(V, device="cuda", dtype=torch.float32)
+    rising, trip = i / V * 64.0, (i % (256 * epv)) / (256 * epv) * 32.0
+    kinds = torch.stack([rising, 64.0 - rising, trip, trip + rising, (i % 2) * rising, -rising])
+    rows = kinds[torch.arange(Bn * K * (n + 1), device="cuda") % len(kinds)]
+    logits = rows.to(dtype).view(Bn, K, n + 1, V).contiguous()
+    g = torch.Generator().manual_seed(V)
+    cand = torch.randint(0, V, (Bn, K, n), generator=g, dtype=torch.int64).to(torch.int32)
+    for _ in range(5):
+        _check(B, cand, logits)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("Bn,K,n,vectors", [(1, 2, 3, 6143), (1, 2, 3, 6144), (1, 3, 1, 6145), (2, 37, 2, 6150),
                                             (3, 25, 2, 6151), (4, 37, 1, 3073), (149, 1, 1, 3073), (16, 37, 1, 1535),
                                             (16, 37, 1, 1536), (593, 1, 1, 1536), (1, 1, 9, 1537), (7, 3, 3, 1)])

@@ -11,7 +11,7 @@
 // Three forms (one_kernel_form and pool_form choose):
 //   verify_seq_kernel    one CTA per sequence does the whole job: its warps take equal contiguous ranges of the sequence's
 //                        vectors, fold them into a (value, index) key per row in shared memory, and the CTA accepts.
-//   verify_pool_kernel + verify_accept_kernel    long rows: one range of vectors per SM, shared out among its warps as they go
+//   verify_pool_kernel + verify_accept_kernel    long rows: two ranges of vectors per SM, each shared out among the warps of a CTA
 //   verify_stream_kernel + verify_accept_kernel    all vectors cut into equal contiguous ranges, one per warp, a single
 //                        wave over the whole GPU; a row that lies in one range is finished there, of the others every
 //                        piece leaves a (value, index) partial; one CTA per sequence folds those and accepts.
@@ -195,14 +195,15 @@ verify_stream_kernel(const char *__restrict__ base, int skew, int rows, int V, l
     }
 }
 
-// Long rows: one CTA per SM takes one range of vectors, and its warps take blocks of it as they get to them.  Bound by DRAM.
-// Of the four CTAs that an SM holds in the form above one is served last, trip after trip (its first loads return after 10 us,
-// the others' after 3), so that in the end it runs on alone; here its warps take fewer blocks instead.  The keys of the
+// Long rows: two CTAs per SM take one range of vectors each, and a CTA's warps take blocks of its range as they get to them.  Bound
+// by DRAM.  Of the four CTAs that an SM holds in the form above one is served last, trip after trip (its first loads return after
+// 10 us, the others' after 3), so that in the end it runs on alone; here its warps take fewer blocks instead.  The keys of the
 // rows that a range touches gather in shared memory, so that few pieces are left to the accept kernel, and most trips end with
-// one comparison against their row's key.  28 warps of 64 registers: the accept kernel's CTAs still fit beside them and are there
-// when the last block is read.  us a call, form above -> this one, bf16: V 32000, 16 MB 9.9 -> 8.5, 131 MB 25.1 -> 24.8, 400 MB
-// 65.5 -> 61.4; V 128256, 8 MB 11.4 -> 7.4, 33 MB 13.4 -> 10.8, 131 MB 25.4 -> 24.5; fp32 V 32000, 16 MB 9.7 -> 7.9.
-constexpr int kPoolThreads = 896, kPoolMaxRows = 128;
+// one comparison against their row's key.  14 warps of 64 registers: one CTA fits beside a CTA of the head GEMM, as a CTA of the
+// form above does, so that a draft on another stream and a verification do not shut each other out (one CTA of 28 warps an SM:
+// the two together at the 7B shape 135.0 us a pair -> 137.0, so 135.1; at batch 4 with fp32 logits the verification 47 -> 64, so
+// 46), and two leave the accept kernel's CTAs their place: they are there when the last block is read.
+constexpr int kPoolThreads = 448, kPoolPerSm = 2, kPoolMaxRows = 128;
 
 template <bool kBf16>
 __global__ void __maxnreg__(64)
@@ -588,7 +589,7 @@ constexpr long long kPoolLongRowVec = 12000, kPoolLongMinVec = 120000;
 bool pool_form(long long total_vec, long long row_vec) {
     return row_vec >= kPoolMinRowVec && row_vec <= kPoolMaxRowVec &&
            total_vec >= (row_vec >= kPoolLongRowVec ? kPoolLongMinVec : kPoolMinVec) && total_vec <= kPoolMaxVec &&
-           (total_vec + num_sms() - 1) / num_sms() / row_vec + 3 <= kPoolMaxRows;
+           (total_vec / (kPoolPerSm * num_sms()) + 1) / row_vec + 3 <= kPoolMaxRows;
 }
 
 // Resident CTAs per SM of the streaming kernel (launch bound above) times the SM count gives the
@@ -612,7 +613,7 @@ VerifyPlan make_verify_plan(int B, int K, int n, int V, int dtype) {
     const size_t lengths = sizeof(int32_t) * (size_t)B * K;
     p.total = align_up(p.off_part + (partials > lengths ? partials : lengths), kWsAlign);
     if (pool_form(total, V / epv)) {
-        const long long range = (total + num_sms() - 1) / num_sms();
+        const long long ctas = (long long)kPoolPerSm * num_sms(), range = (total + ctas - 1) / ctas;
         p.pool = true;
         p.vec_per_warp = (int)range;
         p.warps = (int)((total + range - 1) / range);
@@ -640,8 +641,12 @@ int launch_verify(const int32_t *cand_tok, const void *base_logits, int dtype, i
     const long long total = (skew + (long long)plan.rows * V + (1 << shift) - 1) >> shift;
     const long long warps = (total + plan.vec_per_warp - 1) / plan.vec_per_warp;
     if (plan.pool) {
-        int block = plan.vec_per_warp / (kPoolThreads / 32 * 8) / (32 * kStreamUnroll) * (32 * kStreamUnroll);
-        block = block < 32 * kStreamUnroll ? 32 * kStreamUnroll : block > 2048 ? 2048 : block;   // about eight blocks a warp
+        // Blocks of up to five trips, of which a warp gets a whole number, so that the warps end together; short ones where there
+        // are many of them.  us a call in blocks of one / two / four trips and so, V 32000 in bf16 behind a matrix product: 25 MB
+        // (1.5 trips a warp) 19.1 / 17.6 / 19.4, 17.6; 47 MB 23.0 / 22.1 / 21.6, 21.6; 65 MB 26.8 / 24.6 / 23.6, 23.6; 76 MB
+        // 29.8 / 27.6 / 28.6, 25.7; 131 MB 38.4 / 34.0 / 33.8, 33.8; 400 MB 84.1 / 73.7 / 74.7, 73.7.
+        const int trips = (plan.vec_per_warp / (kPoolThreads / 32) + 32 * kStreamUnroll - 1) / (32 * kStreamUnroll);
+        const int turns = (trips + 4) / 5, block = 32 * kStreamUnroll * (trips > 20 ? 2 : (trips + turns - 1) / turns);
         SPEC_CUDA_TRY(launch_pdl(bf16 ? verify_pool_kernel<true> : verify_pool_kernel<false>, dim3((unsigned)warps),
                                  dim3(kPoolThreads), 0, st, base, skew, plan.rows, V, total, plan.vec_per_warp, block, plan.warps, g,
                                  part));

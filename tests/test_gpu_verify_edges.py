@@ -99,7 +99,8 @@ def test_every_alignment_of_the_base(B, V, dtype):
                                                     (148, 4096, 0, 0), (149, 4096, 1, 2), (401, 3100, -2, 0), (2, 210001, 1, 1),
                                                     (96, 3125, 0, 0), (96, 3125, -1, 0), (8, 16032, 0, 0), (8, 16032, 1, 3), (6, 16032, 1, 3),
                                                     (10, 12000, 0, 0), (10, 12000, -1, 0)])
-def test_long_rows_shared_by_the_warps_of_an_sm(B, rows, vectors, extra, off, dtype):
+@pytest.mark.parametrize("per_sm", [1, 2])
+def test_long_rows_shared_by_the_warps_of_an_sm(B, rows, vectors, extra, off, dtype, per_sm):
     """Rows of `vectors` 16-byte vectors plus `extra` elements, the tensor `off` elements past a vector's start: below, at and above
     the sizes from which an SM's warps share one range, and rows that begin and end inside a vector.  Maxima at the ends of the
     row, of a trip, of a block and of an SM's range; a second, equal one further right in every third row; rows of -inf, of
@@ -112,7 +113,7 @@ def test_long_rows_shared_by_the_warps_of_an_sm(B, rows, vectors, extra, off, dt
     buf[off + rows * V:] = 50.0                           # what lies before and behind the tensor must not be seen
     flat = buf[off:off + rows * V].view(rows, V)
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    span = -(-(rows * V // epv) // sms) * epv             # elements of one SM's range
+    span = -(-(rows * V // epv) // (per_sm * sms)) * epv  # elements of a range, one or two to an SM
     for r in range(rows):
         start = r * V
         edge = (-start) % span                            # the first element of a range inside this row, if it has one
@@ -134,6 +135,28 @@ def test_long_rows_shared_by_the_warps_of_an_sm(B, rows, vectors, extra, off, dt
     am = logits.float().nan_to_num(nan=float("-inf"), posinf=float("inf"), neginf=float("-inf")).argmax(-1).cpu()
     cand[::2, 0, 0] = am[::2, 0, 0].to(torch.int32)
     _check(B, cand, logits)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("trips", [0.4, 1, 1.1, 2.6, 4, 5, 5.1, 9.9, 10.1, 20, 20.1])
+def test_blocks_of_a_shared_range(B, trips, dtype):
+    """Long rows whose warps get `trips` trips of 256 vectors each, on both sides of the sizes where the blocks they take change:
+    every row's maximum is found, wherever in a block, a trip or a warp's lanes it lies."""
+    epv = 8 if dtype == torch.bfloat16 else 4
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    V = 128256 if trips < 1 else 32003
+    rows = int(trips * 256 * 14 * 2 * sms * epv / V) // 4 * 4
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    x = torch.randint(-100, 100, (rows * V,), generator=g, device="cuda", dtype=torch.int8).to(dtype).view(rows, V)
+    r = torch.arange(rows, device="cuda")
+    at = torch.randint(0, V, (rows,), generator=g, device="cuda")
+    x[r, at] = 101.0
+    second = torch.minimum(at + 1 + 37 * (r % 11), torch.full_like(at, V - 1))     # an equal one behind it in every third row
+    x[r[::3], second[::3]] = 101.0
+    Bn, K, n = rows // 4, 2, 1
+    _, _, _, ws = B.spec_verify(torch.zeros(Bn, K, n, dtype=torch.int32, device="cuda"), x.view(Bn, K, n + 1, V))
+    assert B.spec_poll_error(ws) == 0
+    assert torch.equal(ws_view(ws, 256, rows, torch.int32), at.to(torch.int32))
 
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])

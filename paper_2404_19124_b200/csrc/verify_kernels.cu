@@ -578,17 +578,22 @@ bool one_kernel_form(int B, int rows_b, int V, int dtype) {
            (turns - 1) * V <= 64 * (dtype == SPEC_BF16 ? Elem<true>::kEpv : Elem<false>::kEpv);
 }
 
-// Where verify_pool_kernel takes over from verify_stream_kernel: rows of 48 KB and more, 4.8 to 512 MB in all, or from 1.9 MB where a
-// row is 192 KB.  us a call, stream / pool, bf16: V 2048, 65 MB 17.4 / 20.3, 400 MB 72 / 78; V 8000, 16 MB 9.6 / 9.5, 65 MB 16.0 /
-// 16.7, 131 MB 25.4 / 26.0 (a trip ends at a row's end); V 32000, 3 MB 7.2 / 7.4, 5 MB 7.6 / 7.5, 8 MB 8.4 / 7.4; V 50000, 4 MB 7.5 /
-// 7.6, 4.8 MB 8.1 / 7.3; V 128256, 1 MB 7.6 / 7.4 to 7.6, 2 MB 8.0 / 7.6, 4 MB 9.1 / 7.3 (the other form leaves 63 pieces of such a row
-// to the accept kernel; 7.3 is the host's time for two launches); fp32 V 128256, 2 MB 9.7 / 7.3, 8 MB 12.7 / 7.4.  Above, at the clocks
-// of a long step, the shorter trips of the other form win: V 128256, 5250 MB 765-828 / 765-882.
-constexpr long long kPoolMinRowVec = 3072, kPoolMaxRowVec = 1 << 24, kPoolMinVec = 300000, kPoolMaxVec = 32 << 20;
-constexpr long long kPoolLongRowVec = 12000, kPoolLongMinVec = 120000;
+// Where verify_pool_kernel takes over from verify_stream_kernel: up to 1 GB in all; from 25 MB where rows have 48 KB or more, from
+// 4.8 MB for rows of 60 KB, from 1.9 MB for rows of 188 KB, of which the other form leaves dozens of pieces to the accept kernel.
+// Measured behind matrix products that fill the GPU to its power limit, as a base model's last layer does (a call with its
+// launches), and in a loop of calls; pool / stream:
+//   rows, bf16   5 MB   8 MB   16 MB   33 MB   65 MB   131 MB   262 MB   400 MB   800 MB   1.5 GB   3 GB
+//   47-48 KB     1.16   1.02   0.97    0.92    0.92    0.97     0.97     0.97     0.95     1.00     1.00
+//   62 KB        1.02   0.98   0.93    0.92    0.93    0.97     0.97     0.97     0.94     1.00     1.00
+//   98 KB        0.99   0.90   0.87    0.87    0.93    0.96     0.96     0.97     0.89     0.91     1.01
+//   250 KB       0.87   0.81   0.76    0.83    0.90    0.96     0.95     0.93     0.94     0.98     0.99
+// (A loop of calls gains about the same, down to the 8 MB where the host's 7.3 us for two launches are what it takes.)  fp32: 48 KB
+// 1.15 at 8 MB, 1.03 at 16, 0.99 at 33; 125 KB 0.94 to 1.00 up to 16 MB, 0.93 at 33.  Shorter rows, bf16: 31 KB 0.99 at 16 MB,
+// 0.94 at 33 and 65, 1.00 to 1.02 at 131 and 200; 16 KB no better at most sizes (a trip ends at a row's end).
+constexpr long long kPoolMinRowVec = 3072, kPoolMaxRowVec = 1 << 24, kPoolMaxVec = 64 << 20;
+long long pool_min_vec(long long row_vec) { return row_vec >= 12000 ? 120000 : row_vec >= 3840 ? 300000 : 1536 << 10; }
 bool pool_form(long long total_vec, long long row_vec) {
-    return row_vec >= kPoolMinRowVec && row_vec <= kPoolMaxRowVec &&
-           total_vec >= (row_vec >= kPoolLongRowVec ? kPoolLongMinVec : kPoolMinVec) && total_vec <= kPoolMaxVec &&
+    return row_vec >= kPoolMinRowVec && row_vec <= kPoolMaxRowVec && total_vec >= pool_min_vec(row_vec) && total_vec <= kPoolMaxVec &&
            (total_vec / (kPoolPerSm * num_sms()) + 1) / row_vec + 3 <= kPoolMaxRows;
 }
 

@@ -98,7 +98,8 @@ def test_every_alignment_of_the_base(B, V, dtype):
                                                     (131, 3079, 2, 2), (26, 16032, 0, 0), (26, 16032, 3, 3), (26, 16032, -3, 1),
                                                     (148, 4096, 0, 0), (149, 4096, 1, 2), (401, 3100, -2, 0), (2, 210001, 1, 1),
                                                     (96, 3125, 0, 0), (96, 3125, -1, 0), (8, 16032, 0, 0), (8, 16032, 1, 3), (6, 16032, 1, 3),
-                                                    (10, 12000, 0, 0), (10, 12000, -1, 0)])
+                                                    (10, 12000, 0, 0), (10, 12000, -1, 0), (78, 3847, 0, 0), (78, 3846, -1, 2),
+                                                    (512, 3072, 0, 0), (512, 3072, -1, 0), (512, 3080, 1, 1)])
 @pytest.mark.parametrize("per_sm", [1, 2])
 def test_long_rows_shared_by_the_warps_of_an_sm(B, rows, vectors, extra, off, dtype, per_sm):
     """Rows of `vectors` 16-byte vectors plus `extra` elements, the tensor `off` elements past a vector's start: below, at and above

@@ -125,15 +125,15 @@ __global__ void __launch_bounds__(kMergeThreads) merge_expand_kernel(MergeArgs g
 }
 
 // The last level's merge and the prune, one CTA per sequence, one warp per row: the leaves' scores meet in shared memory, where
-// with a CTA per row the rows of a sequence were counted in (a fence, an atomic, the scores back from L2: 3.4 us) and 384
-// CTAs took turns on the SMs.  A warp needs longer for a row than five (1.9 us for 143 lists), about 0.2 us per 32 lists beyond the
-// first.  Exposed time, a CTA per row -> this: 12 rows a
-// sequence (7B shape) 6.2 -> 4.7 us, 24 rows of 16 sequences (13B) 9.0 -> 8.2; the batch-1 draft 129.5 -> 126.5, the ragged step 119.8 -> 118.3.
+// with a CTA per row the rows of a sequence are counted in (a fence, an atomic, the scores back from L2: 3.4 us) and 384 CTAs take
+// turns on the SMs.  A warp needs longer for a row than five (1.9 us for 143 lists), about 0.2 us per 32 lists beyond the first.
+// Exposed time, a CTA per row -> this: 12 rows a sequence (7B shape) 6.2 -> 4.7 us, 24 rows of 16 sequences (13B) 9.0 -> 8.2; the
+// batch-1 draft 129.5 -> 126.5, the ragged step 119.8 -> 118.3.
 // At most 48 registers, so that the widest CTA fits beside a resident GEMM CTA.
 struct OneWarp {
     static __device__ __forceinline__ void sync() { __syncwarp(); }
 };
-constexpr int kPruneRows = 24, kPruneLists = 256;   // at most: rows of a sequence (warps of the CTA), lists of a row
+constexpr int kPruneRows = 24;   // rows of a sequence, at most: warps of the CTA
 template <int kLen>
 __global__ void __maxnreg__(48) merge_prune_kernel(MergeArgs g) {
     __shared__ float4 scores4[kPruneRows * SPEC_MAX_TOPK / 4];
@@ -353,16 +353,41 @@ int launch_draft_init(int32_t *hdr, int words, cudaStream_t st) {
     return SPEC_OK;
 }
 
+// Where the last level takes one warp per row.  A warp selects its lists 32 at a time, in as many rounds each time as a row has
+// children (`rounds` in all), and a sequence's warps share an SM; the five warps of the other form have one to themselves while
+// there are no more rows than SMs.  Draft of d 256 or 512, V 9000 to 128256, 1 to 256 sequences; us, this form less the other:
+//   children  lists     one row a sequence;        2 to 24 rows; in all up to
+//                       up to 48 / more sequences  48 rows        148 rows       592 rows       more
+//   1, 2      36-148    -2.0..+0.1  -1.1..+1.0     -6.8..-1.4     -4.8..-0.6     -4.8..+1.4     -4.5..-0.2
+//   4         36-148    -2.0..-0.2  -1.3..+3.2     -8.7..-0.2     -3.5..-0.2     -4.7..+1.2     -5.4..+1.9
+//   8         71-148    -1.0..+1.5  +0.4..+9.2     -5.3..+2.8 *   -2.8..+5.6     -4.3..+2.9     -6.5..+8.9
+//   1, 2, 4   223-255   --          --             --             -1.5..+2.3 *   -3.1..+1.2     -4.3..+0.1
+//   8         223-255   --          --             --             +0.8..+7.9     -3.1..+4.8 *   -2.7..+1.1
+//   1, 2      501-573   --          +1.4..+3.0     --             -0.3..+2.3     -1.4..+4.1     -2.6..+2.7
+//   4, 8      501-573   --          +1.8..+7.2     --             +0.5..+26.2    -2.1..+19.9    +0.4..+13.1
+// (* Most losses are those of sequences whose rows have more than 480 rounds together.)  Over these 1100 points and 228 of other
+// branching factors (3 and 5 to 7 among them) the rule is 0.15 percent from the better form each time, the limits of 24 rows and
+// 256 lists alone 0.5.
+bool one_warp_per_row(const MergeArgs &g, int rows) {
+    const int rounds = (g.n_tiles + 31) / 32 * g.topk;
+    if (g.rows_per_seq > kPruneRows || g.n_tiles > 256) return false;
+    if (g.rows_per_seq == 1) return rounds <= (rows <= 32 ? 35 : 15);
+    if (rounds <= 24) return true;
+    return (rows <= 48 || rows > num_sms()) && (g.rows_per_seq * rounds <= 480 || rows > 4 * num_sms());
+}
+
 int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st) {
     const size_t smem = g.seq_done ? prune_smem_bytes(g.L, g.Lpad) : 0;
     const int slots = list_slots(g.list_len > 0 ? g.list_len : g.topk);
-    if (g.seq_done && g.rows_per_seq <= kPruneRows && g.n_tiles <= kPruneLists) {
-        SPEC_CUDA_TRY(launch_pdl(slots == 2 ? merge_prune_kernel<2> : slots == 4 ? merge_prune_kernel<4> : merge_prune_kernel<8>, dim3(rows / g.rows_per_seq),
-                                 dim3(32 * g.rows_per_seq), 0, st, g));
+    if (g.seq_done && one_warp_per_row(g, rows)) {
+        SPEC_CUDA_TRY(launch_pdl(slots == 2   ? merge_prune_kernel<2>
+                                 : slots == 4 ? merge_prune_kernel<4>
+                                              : merge_prune_kernel<8>, dim3(rows / g.rows_per_seq), dim3(32 * g.rows_per_seq), 0, st, g));
         return SPEC_OK;
     }
-    SPEC_CUDA_TRY(launch_pdl(slots == 2 ? merge_expand_kernel<2> : slots == 4 ? merge_expand_kernel<4> : merge_expand_kernel<8>, dim3(rows),
-                             dim3(kMergeThreads), smem, st, g));
+    SPEC_CUDA_TRY(launch_pdl(slots == 2   ? merge_expand_kernel<2>
+                             : slots == 4 ? merge_expand_kernel<4>
+                                          : merge_expand_kernel<8>, dim3(rows), dim3(kMergeThreads), smem, st, g));
     return SPEC_OK;
 }
 

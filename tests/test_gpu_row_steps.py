@@ -57,9 +57,23 @@ def test_prune_leaves_round_the_thread_counts(B, topk, K, fp8):
 @pytest.mark.parametrize("topk,K,rows", [((1, 1), 1, 1), ((1, 7), 5, 1), ((4, 3, 2), 16, 12), ((6, 4, 3), 72, 24), ((6, 4, 8), 100, 24),
                                          ((5, 5, 8), 100, 25)])
 def test_last_merge_and_prune_of_a_sequence(B, topk, K, rows, V):
-    """Up to 24 rows a sequence and 256 lists a row the last merge is one CTA per sequence; the kept leaves are the best of the
-    scores that it leaves in the workspace, in order, with the tokens of their paths."""
-    cfg = small_cfg(d_base=48, d_inner=64, V=V, topk=topk, K=K, B=3, seed=K)
+    """The last merge is one CTA per sequence or one per row; the kept leaves are the best of the scores that it leaves in the
+    workspace, in order, with the tokens of their paths."""
+    assert rows * topk[-1] == np.prod(topk)
+    _check_last_merge(B, topk, K, V, 3)
+
+
+@pytest.mark.parametrize("topk,lists,seqs", [((7,), 160, 32), ((7,), 160, 33), ((8,), 160, 1), ((3,), 160, 33), ((4,), 160, 33),
+                                             ((2, 8), 96, 30), ((2, 8), 97, 30), ((3, 4, 8), 160, 4), ((5, 2, 8), 160, 5),
+                                             ((4, 3, 8), 160, 13), ((3, 5, 8), 129, 3), ((8, 2, 6), 160, 3), ((8, 2, 6), 161, 3),
+                                             ((6, 4, 8), 100, 25), ((6, 4, 8), 100, 24)])
+def test_last_merge_on_both_sides_of_its_rule(B, topk, lists, seqs):
+    """Rounds of a row, rows of a sequence and rows in all where the last merge goes from a CTA per sequence to a CTA per row."""
+    _check_last_merge(B, topk, min(12, int(np.prod(topk))), 32 * lists - 5, seqs)
+
+
+def _check_last_merge(B, topk, K, V, seqs):
+    cfg = small_cfg(d_base=48, d_inner=64, V=V, topk=topk, K=K, B=seqs, seed=K)
     sw = synth.make_weights(cfg)
     ctx, tok = synth.make_draft_inputs(cfg)
     h = B.spec_create(weights_to_cuda(sw))
@@ -68,7 +82,6 @@ def test_last_merge_and_prune_of_a_sequence(B, topk, K, rows, V):
     assert B.spec_poll_error(ws) == 0
     lay = B.spec_draft_layout(h, cfg.B, topk, K)
     n, L = cfg.n, cfg.leaves
-    assert L == rows * topk[-1]
     leaf = ws[lay.score[n]:lay.score[n] + 4 * cfg.B * L].view(torch.float32).view(cfg.B, L)
     want = torch.sort(leaf, dim=1, descending=True, stable=True)
     assert torch.equal(lp, want.values[:, :K])
@@ -78,7 +91,7 @@ def test_last_merge_and_prune_of_a_sequence(B, topk, K, rows, V):
         t = ws[lay.tok[l + 1]:lay.tok[l + 1] + 4 * cfg.B * per].view(torch.int32).view(cfg.B, per)
         assert torch.equal(ct[:, :, l], torch.gather(t, 1, want.indices[:, :K] // (L // per)))
     chk = DraftChecker(to_oracle_weights(sw), topk, K)
-    for b in range(cfg.B):
+    for b in range(min(3, seqs)):
         chk.check(synth.bf16_bits(ctx)[b], int(tok[b]), ct[b].cpu().numpy(), lp[b].cpu().numpy())
     B.spec_destroy(h)
 

@@ -46,13 +46,14 @@ __global__ void __launch_bounds__(kRowThreads, 3) mix_ln_gelu_many_kernel(MixArg
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, t = __ldcg(m.tok + r);
-    if (m.d <= 8 * kRowThreads) mix_ln_gelu_row<kRowThreads, 1, 1, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red, nullptr, m.in_order != 0);
-    else mix_ln_gelu_row<kRowThreads, 2, 1, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red, nullptr, m.in_order != 0);
+    if (m.d <= 8 * kRowThreads) mix_ln_gelu_row<kRowThreads, 1, 1, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
+    else mix_ln_gelu_row<kRowThreads, 2, 1, BlockSync>(m, r, r / m.parent_div, t, threadIdx.x, red);
 }
 
 // Levels of several waves whose projection was not split (more than 128 parents, or too few K blocks): throughput counts, and
 // a CTA has only as many threads as its row needs with two groups each.  2016 rows of 400 elements 14.7 -> 6.9 us, 1836 of
 // 2296 25.5 -> 21.5.  (Four rows to a CTA, or 128 threads with four groups each, are no better.)
+// The only one of the separate kernels that takes the LayerNorm sums in order (launch_mix_ln_gelu).
 __global__ void __launch_bounds__(kRowThreads, 3) mix_ln_gelu_waves_kernel(MixArgs m) {
     __shared__ float red[32];
     griddep_launch();
@@ -328,7 +329,8 @@ prune_kernel(const float *leaf_score, PruneArgs pa, int L, int Lpad, int K, int3
 
 int launch_mix_ln_gelu(const MixArgs &m, int rows, cudaStream_t st) {
     const int d_inner = m.d;
-    if (d_inner <= 8 * kRowThreads * 2 && rows > num_sms() && m.p_splits == 1) {
+    // (in_order: set only behind more parents than SMs, whose projection is not split where there are 128 SMs or more)
+    if (d_inner <= 8 * kRowThreads * 2 && rows > num_sms() && (m.p_splits == 1 || m.in_order)) {
         SPEC_CUDA_TRY(launch_pdl(mix_ln_gelu_waves_kernel, dim3(rows), dim3((d_inner + 511) / 512 * 32), 0, st, m));
     } else if (d_inner <= 8 * kRowThreads * 2 && rows > num_sms()) {
         SPEC_CUDA_TRY(launch_pdl(mix_ln_gelu_many_kernel, dim3(rows), dim3(kRowThreads), 0, st, m));

@@ -14,7 +14,7 @@ namespace {
 using namespace rows;
 
 constexpr int kRowThreads = 256;
-constexpr int kFusedMixMaxChildren = 2;   // (list_slots(2) below)
+constexpr int kFusedMixMaxChildren = 2;
 constexpr int kMergeThreads = 160;   // one list per thread up to V = 35000 (a CTA of the head GEMM leaves one)
 
 // Rows of up to 2048 elements: at most 128 registers, so that two CTAs fit beside a resident GEMM CTA.
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(kRowThreads, 2) merge_mix_kernel(MergeMixArgs 
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, tid = threadIdx.x;
-    const int tok = merge_expand_row<kRowThreads, 2, BlockSync>(a.merge, r, tid, &sc).id;
+    const int tok = merge_expand_row<kRowThreads, list_slots(kFusedMixMaxChildren), BlockSync>(a.merge, r, tid, &sc).id;
     mix_children<kRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
 }
 
@@ -219,7 +219,7 @@ __global__ void __maxnreg__(72) merge_mix_512_kernel(MergeMixArgs a) {
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, tid = threadIdx.x;
-    const int tok = merge_expand_row<kWideRowThreads, 2, BlockSync>(a.merge, r, tid, &sc).id;
+    const int tok = merge_expand_row<kWideRowThreads, list_slots(kFusedMixMaxChildren), BlockSync>(a.merge, r, tid, &sc).id;
     mix_children<kWideRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
 }
 
@@ -407,9 +407,8 @@ int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_
     if (m.d > 8 * kRowThreads * 2 || g.lse_out != nullptr || g.seq_done != nullptr) return SPEC_ERR_SHAPE;
     MergeMixArgs a{g, m};
     a.merge.next_emb = nullptr;   // the gather follows in the same CTA
-    const int children = rows * g.topk;
+    const int children = rows * g.topk, slots = list_slots(g.list_len > 0 ? g.list_len : g.topk);
     if (children <= num_sms()) {
-        const int slots = list_slots(g.list_len > 0 ? g.list_len : g.topk);
         if (m.d > 8 * kRowThreads)
             SPEC_CUDA_TRY(launch_pdl(slots == 2   ? merge_mix_child_512_kernel<2>
                                      : slots == 4 ? merge_mix_child_512_kernel<4>
@@ -422,7 +421,8 @@ int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_
                                      dim3(kRowThreads), 0, st, a));
         return SPEC_OK;
     }
-    if (rows > num_sms() || g.topk > kFusedMixMaxChildren || m.S8_out != nullptr) return SPEC_ERR_SHAPE;
+    if (rows > num_sms() || g.topk > kFusedMixMaxChildren || slots != list_slots(kFusedMixMaxChildren) || m.S8_out != nullptr)
+        return SPEC_ERR_SHAPE;
     if (m.d > 8 * kRowThreads) {
         SPEC_CUDA_TRY(launch_pdl(merge_mix_512_kernel, dim3(rows), dim3(kWideRowThreads), 0, st, a));
         return SPEC_OK;

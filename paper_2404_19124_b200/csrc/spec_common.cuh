@@ -102,14 +102,14 @@ int launch_verify_early(const int32_t *cand_tok, const void *base_logits, int dt
                         int32_t *accept_len, int32_t *best_cand, int32_t *next_tok, void *ws, const VerifyPlan &plan,
                         cudaStream_t st);
 
-// ---- tensor-core GEMM (gemm_tcgen05.cu) -------------------------------------------------
-// C[M, N] = A[M, Kd] * B[N, Kd]^T, A and B bf16 row-major (K-major), fp32 accumulation in TMEM.
 // Slots of a partial list that keeps the best `len`; lists lie one behind the other, and what selects, folds and merges them is
 // as long as they are.  (Always eight: half of every 32-byte sector read in vain for up to four, and twice the steps where the
 // threads of a node fold their lists.)  34B step 475.5 -> 470.9 us, batch-1 draft 126.4 -> 125.1, single-candidate chain 159.0 ->
 // 157.9, 13B step with e4m3 heads 239.5 -> 238.6.
-__host__ __device__ inline int list_slots(int len) { return len <= 2 ? 2 : len <= 4 ? 4 : SPEC_MAX_TOPK; }
+__host__ __device__ constexpr int list_slots(int len) { return len <= 2 ? 2 : len <= 4 ? 4 : SPEC_MAX_TOPK; }
 
+// ---- tensor-core GEMM (gemm_tcgen05.cu) -------------------------------------------------
+// C[M, N] = A[M, Kd] * B[N, Kd]^T, A and B bf16 row-major (K-major), fp32 accumulation in TMEM.
 struct GemmEpilogue {
     int mode;          // 0: store fp32 C; 1: per-row partial top-k + (max, sum-exp) per tile;
                        // 2: split-K partials stored transposed, out[split][n][m];

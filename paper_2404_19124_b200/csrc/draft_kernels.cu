@@ -14,7 +14,7 @@ namespace {
 using namespace rows;
 
 constexpr int kRowThreads = 256;
-constexpr int kFusedMixMaxChildren = 2;
+constexpr int kFusedChildren = 2;   // of a row, in merge_mix_kernel
 constexpr int kMergeThreads = 160;   // one list per thread up to V = 35000 (a CTA of the head GEMM leaves one)
 
 // Rows of up to 2048 elements: at most 128 registers, so that two CTAs fit beside a resident GEMM CTA.
@@ -188,10 +188,11 @@ __global__ void __maxnreg__(48) merge_prune_kernel(MergeArgs g) {
     cand[g.prune.n - 1] = toks[tid];
 }
 
-// Merge of level l and the gather + mix + LayerNorm + GELU of level l + 1 in one launch, for one or two children per row
-// more children than SMs but no more rows: one CTA of 256 threads per row of level l folds the row's partial lists into its children (tokens, scores) and then computes the
-// states of those children, whose tokens it has just found and whose parent projection is this row's.  One
-// kernel boundary less between two vocabulary heads.
+// Merge of level l and the gather + mix + LayerNorm + GELU of level l + 1 in one launch, for two children per row where there
+// are more children than SMs but no more rows: one CTA of 256 threads per row of level l folds the row's partial lists into its
+// children (tokens, scores) and then computes the states of those children, whose tokens it has just found and whose parent
+// projection is this row's.  One kernel boundary less between two vocabulary heads.  75 / 128 / 148 rows, V 8000, the whole
+// draft as two kernels -> this: d 1024 52.9 -> 51.4 us, 59.4 -> 56.7, 56.8 -> 54.5; d 2048 64.6 -> 62.8, 71.2 -> 68.4, 76.4 -> 74.5.
 struct MergeMixArgs {
     MergeArgs merge;   // level l
     MixArgs mix;       // level l + 1 (tok and parent_div unused: the tokens come from the merge)
@@ -199,28 +200,27 @@ struct MergeMixArgs {
 
 // At most 128 registers: like the other row kernels its CTAs must fit beside a resident GEMM CTA, or they could
 // not start (and wait, set up) before that kernel ends.
-constexpr int kFusedBatch = 2;
 __global__ void __launch_bounds__(kRowThreads, 2) merge_mix_kernel(MergeMixArgs a) {
     __shared__ Scratch sc;
-    __shared__ float red_a[kRowThreads / 32 * kFusedBatch], red_b[kRowThreads / 32 * kFusedBatch];
+    __shared__ float red_a[kRowThreads / 32 * kFusedChildren], red_b[kRowThreads / 32 * kFusedChildren];
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, tid = threadIdx.x;
-    const int tok = merge_expand_row<kRowThreads, list_slots(kFusedMixMaxChildren), BlockSync>(a.merge, r, tid, &sc).id;
-    mix_children<kRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
+    const int tok = merge_expand_row<kRowThreads, list_slots(kFusedChildren), BlockSync>(a.merge, r, tid, &sc).id;
+    mix_children<kRowThreads, 1, kFusedChildren, BlockSync>(a.mix, r, r * kFusedChildren, tok, red_a, red_b, tid);
 }
 
-// Rows of 2049 to 4096 elements: 512 threads, one 8-element group each, like mix_ln_gelu_512_kernel (single-
-// candidate chain at the 13B widths 210 -> 203 us per draft, at the 34B widths 278 -> 269 us).  72 registers at
-// most, so that the CTA fits beside a resident GEMM CTA.
+// Rows of 2049 to 4096 elements: 512 threads, one 8-element group each, like mix_ln_gelu_512_kernel (d 4096, V 8000, 75 / 128 /
+// 148 rows: 93.3 -> 91.1 us, 102.3 -> 98.1, 125.0 -> 122.0; V 32000 195.8 -> 192.0, 205.0 -> 203.7, 277.3 -> 274.1).  72 registers
+// at most, so that the CTA fits beside a resident GEMM CTA.
 __global__ void __maxnreg__(72) merge_mix_512_kernel(MergeMixArgs a) {
     __shared__ Scratch sc;
-    __shared__ float red_a[kWideRowThreads / 32 * kFusedBatch], red_b[kWideRowThreads / 32 * kFusedBatch];
+    __shared__ float red_a[kWideRowThreads / 32 * kFusedChildren], red_b[kWideRowThreads / 32 * kFusedChildren];
     griddep_launch();
     griddep_wait();
     const int r = blockIdx.x, tid = threadIdx.x;
-    const int tok = merge_expand_row<kWideRowThreads, list_slots(kFusedMixMaxChildren), BlockSync>(a.merge, r, tid, &sc).id;
-    mix_children<kWideRowThreads, 1, kFusedBatch, BlockSync>(a.mix, r, r * a.merge.topk, a.merge.topk, tok, red_a, red_b, tid);
+    const int tok = merge_expand_row<kWideRowThreads, list_slots(kFusedChildren), BlockSync>(a.merge, r, tid, &sc).id;
+    mix_children<kWideRowThreads, 1, kFusedChildren, BlockSync>(a.mix, r, r * kFusedChildren, tok, red_a, red_b, tid);
 }
 
 // The same with one CTA per CHILD, for levels whose children are at most one per SM: every child's CTA repeats its
@@ -237,7 +237,7 @@ __device__ __forceinline__ void merge_mix_child(const MergeMixArgs &a, Scratch *
     const MergeOut o = merge_expand_row<kThreads, kLen, BlockSync>(a.merge, r, tid, sc, c == r * topk,
                                                                    [&] { parent_state<kThreads>(a.mix, r, tid, pre); });
     const int t = __shfl_sync(0xffffffffu, o.id, c - r * topk);
-    const bool in_order = topk <= kFusedMixMaxChildren && a.mix.S8_out == nullptr;
+    const bool in_order = topk <= kFusedChildren && a.mix.S8_out == nullptr;
     mix_ln_gelu_row<kThreads, 1, 1, BlockSync>(a.mix, c, r, t, tid, red, pre, in_order);
 }
 template <int kLen>
@@ -396,13 +396,13 @@ int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st) {
 // Whether the LayerNorm sums of a level with `topk` children per row are taken in order (group_sums) in every kernel that may
 // compute its states, so that these are the same bits whatever the number of rows.
 bool mix_sums_in_order(int topk, const MixArgs &m) {
-    return topk <= kFusedMixMaxChildren && m.S8_out == nullptr && m.d <= 8 * kRowThreads * 2;
+    return topk <= kFusedChildren && m.S8_out == nullptr && m.d <= 8 * kRowThreads * 2;
 }
 
-// Returns SPEC_ERR_SHAPE when no fused form covers the shape (rows wider than 4096 elements; beyond one child per SM also
-// more than two children per row, more rows than SMs, or an e4m3 copy of the states wanted): the caller then launches the merge
-// and the mix separately.  More rows than SMs: the CTAs of a row with 512 threads take turns on the SMs, the separate kernels
-// run in one wave.  384 rows of two children, d 4096: 22.9 us -> 18.0.
+// Returns SPEC_ERR_SHAPE when no fused form covers the shape (rows wider than 4096 elements; beyond one child per SM also other
+// than two children per row, more rows than SMs, or an e4m3 copy of the states wanted): the caller then launches the merge and
+// the mix separately.  More rows than SMs: the CTAs of a row with 512 threads take turns on the SMs, the separate kernels run in
+// one wave.  384 rows of two children, d 4096: 22.9 us -> 18.0.
 int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_t st) {
     if (m.d > 8 * kRowThreads * 2 || g.lse_out != nullptr || g.seq_done != nullptr) return SPEC_ERR_SHAPE;
     MergeMixArgs a{g, m};
@@ -421,7 +421,7 @@ int launch_merge_mix(const MergeArgs &g, const MixArgs &m, int rows, cudaStream_
                                      dim3(kRowThreads), 0, st, a));
         return SPEC_OK;
     }
-    if (rows > num_sms() || g.topk > kFusedMixMaxChildren || slots != list_slots(kFusedMixMaxChildren) || m.S8_out != nullptr)
+    if (rows > num_sms() || g.topk != kFusedChildren || slots != list_slots(kFusedChildren) || m.S8_out != nullptr)
         return SPEC_ERR_SHAPE;
     if (m.d > 8 * kRowThreads) {
         SPEC_CUDA_TRY(launch_pdl(merge_mix_512_kernel, dim3(rows), dim3(kWideRowThreads), 0, st, a));

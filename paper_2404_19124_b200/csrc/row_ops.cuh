@@ -518,16 +518,16 @@ __device__ __forceinline__ MergeOut merge_expand_row(const MergeArgs &g, int r, 
     return o;
 }
 
-// The children of one parent row, all at once: gather + mix + LayerNorm + exact GELU of up to kBatch child
-// nodes per trip (Sec. 3.1: siblings share the projected parent state and differ in the token embedding).
+// The kBatch children of one parent row, all at once: gather + mix + LayerNorm + exact GELU (Sec. 3.1: siblings share the
+// projected parent state and differ in the token embedding).
 // Lane j of every warp holds child j's token (`tok`, as merge_select returns it), `first_child` is the row of child 0
 // in the next level.  The projected parent state (sum of the split-K partials, added in
-// ascending order) and the LayerNorm parameters are loaded once; per trip the embedding rows of the batch
-// are requested together and the two LayerNorm reductions are done for the whole batch with one barrier
-// each (red_a / red_b: kThreads / 32 x kBatch floats each; kBatch children per trip).  d <= 8 * kThreads * kIters, d % 8 == 0.
+// ascending order) and the LayerNorm parameters are loaded once; the children's embedding rows
+// are requested together and the two LayerNorm reductions are done for all of them with one barrier
+// each (red_a / red_b: kThreads / 32 x kBatch floats each).  d <= 8 * kThreads * kIters, d % 8 == 0.
 template <int kThreads, int kIters, int kBatch, typename Sync>
-__device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int first_child, int n_child, int tok,
-                                             float *red_a, float *red_b, int tid) {
+__device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int first_child, int tok, float *red_a, float *red_b,
+                                             int tid) {
     constexpr int kWarps = kThreads / 32;
     const int d = m.d, lane = tid & 31, warp = tid >> 5;
     float pv[kIters][8], gv[kIters][8], bv[kIters][8];
@@ -552,95 +552,92 @@ __device__ __forceinline__ void mix_children(const MixArgs &m, int parent, int f
         bv[it][0] = b0.x; bv[it][1] = b0.y; bv[it][2] = b0.z; bv[it][3] = b0.w;
         bv[it][4] = b1.x; bv[it][5] = b1.y; bv[it][6] = b1.z; bv[it][7] = b1.w;
     }
-    for (int c0 = 0; c0 < n_child; c0 += kBatch) {
-        float h[kBatch][kIters][8];
-        float part[kBatch];
-        uint4 ev[kBatch][kIters];
+    float h[kBatch][kIters][8];
+    float part[kBatch];
+    uint4 ev[kBatch][kIters];
 #pragma unroll
-        for (int q = 0; q < kBatch; ++q) {
-            const int t = c0 + q < n_child ? __shfl_sync(0xffffffffu, tok, c0 + q) : -1;
-            const bool tok_ok = t >= 0 && t < m.V;
-            if (c0 + q < n_child && !tok_ok && tid == 0) report_error(m.err, SPEC_ERR_TOKEN_RANGE);
+    for (int q = 0; q < kBatch; ++q) {
+        const int t = __shfl_sync(0xffffffffu, tok, q);
+        const bool tok_ok = t >= 0 && t < m.V;
+        if (!tok_ok && tid == 0) report_error(m.err, SPEC_ERR_TOKEN_RANGE);
 #pragma unroll
-            for (int it = 0; it < kIters; ++it) {
-                const int i = (it * kThreads + tid) * 8;
-                ev[q][it] = make_uint4(0u, 0u, 0u, 0u);
-                if (tok_ok && i < d) ev[q][it] = *(const uint4 *)(m.emb + (size_t)t * d + i);
+        for (int it = 0; it < kIters; ++it) {
+            const int i = (it * kThreads + tid) * 8;
+            ev[q][it] = make_uint4(0u, 0u, 0u, 0u);
+            if (tok_ok && i < d) ev[q][it] = *(const uint4 *)(m.emb + (size_t)t * d + i);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < kBatch; ++q) {
+        part[q] = 0.0f;
+#pragma unroll
+        for (int it = 0; it < kIters; ++it) {
+            const int i = (it * kThreads + tid) * 8;
+            const uint32_t ew[4] = {ev[q][it].x, ev[q][it].y, ev[q][it].z, ev[q][it].w};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float z = (j & 1) ? __uint_as_float(ew[j >> 1] & 0xffff0000u) : __uint_as_float(ew[j >> 1] << 16);
+                h[q][it][j] = i < d ? mix_element(m, pv[it][j], z) : 0.0f;
+                part[q] += h[q][it][j];
             }
         }
+    }
+    // batch-wide reductions: warp shuffles, one slot per (warp, child), then every thread adds the warps' slots
+    float mean[kBatch], rstd[kBatch];
+#pragma unroll
+    for (int pass = 0; pass < 2; ++pass) {
+        float *red = pass == 0 ? red_a : red_b;
 #pragma unroll
         for (int q = 0; q < kBatch; ++q) {
-            part[q] = 0.0f;
+            float v = part[q];
 #pragma unroll
-            for (int it = 0; it < kIters; ++it) {
-                const int i = (it * kThreads + tid) * 8;
-                const uint32_t ew[4] = {ev[q][it].x, ev[q][it].y, ev[q][it].z, ev[q][it].w};
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float z = (j & 1) ? __uint_as_float(ew[j >> 1] & 0xffff0000u) : __uint_as_float(ew[j >> 1] << 16);
-                    h[q][it][j] = i < d ? mix_element(m, pv[it][j], z) : 0.0f;
-                    part[q] += h[q][it][j];
-                }
-            }
+            for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+            if (lane == 0) red[warp * kBatch + q] = v;
         }
-        // batch-wide reductions: warp shuffles, one slot per (warp, child), then every thread adds the warps' slots
-        float mean[kBatch], rstd[kBatch];
+        Sync::sync();
 #pragma unroll
-        for (int pass = 0; pass < 2; ++pass) {
-            float *red = pass == 0 ? red_a : red_b;
+        for (int q = 0; q < kBatch; ++q) {
+            float t = 0.0f;
 #pragma unroll
-            for (int q = 0; q < kBatch; ++q) {
-                float v = part[q];
+            for (int w = 0; w < kWarps; ++w) t += red[w * kBatch + q];
+            if (pass == 0) {
+                mean[q] = t / (float)d;
+                part[q] = 0.0f;
 #pragma unroll
-                for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-                if (lane == 0) red[warp * kBatch + q] = v;
-            }
-            Sync::sync();
+                for (int it = 0; it < kIters; ++it) {
+                    const int i = (it * kThreads + tid) * 8;
+                    if (i < d) {
 #pragma unroll
-            for (int q = 0; q < kBatch; ++q) {
-                float t = 0.0f;
-#pragma unroll
-                for (int w = 0; w < kWarps; ++w) t += red[w * kBatch + q];
-                if (pass == 0) {
-                    mean[q] = t / (float)d;
-                    part[q] = 0.0f;
-#pragma unroll
-                    for (int it = 0; it < kIters; ++it) {
-                        const int i = (it * kThreads + tid) * 8;
-                        if (i < d) {
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const float c = h[q][it][j] - mean[q];
-                                part[q] += c * c;
-                            }
+                        for (int j = 0; j < 8; ++j) {
+                            const float c = h[q][it][j] - mean[q];
+                            part[q] += c * c;
                         }
                     }
-                } else {
-                    rstd[q] = rsqrtf(t / (float)d + m.eps);
                 }
+            } else {
+                rstd[q] = rsqrtf(t / (float)d + m.eps);
             }
         }
+    }
 #pragma unroll
-        for (int q = 0; q < kBatch; ++q) {
-            if (c0 + q >= n_child) continue;
-            const size_t row = (size_t)first_child + c0 + q;
+    for (int q = 0; q < kBatch; ++q) {
+        const size_t row = (size_t)first_child + q;
 #pragma unroll
-            for (int it = 0; it < kIters; ++it) {
-                const int i = (it * kThreads + tid) * 8;
-                uint32_t packed[4];
+        for (int it = 0; it < kIters; ++it) {
+            const int i = (it * kThreads + tid) * 8;
+            uint32_t packed[4];
 #pragma unroll
-                for (int j = 0; j < 8; j += 4) {
-                    float4 y;
-                    y.x = (h[q][it][j] - mean[q]) * rstd[q] * gv[it][j] + bv[it][j];
-                    y.y = (h[q][it][j + 1] - mean[q]) * rstd[q] * gv[it][j + 1] + bv[it][j + 1];
-                    y.z = (h[q][it][j + 2] - mean[q]) * rstd[q] * gv[it][j + 2] + bv[it][j + 2];
-                    y.w = (h[q][it][j + 3] - mean[q]) * rstd[q] * gv[it][j + 3] + bv[it][j + 3];
-                    y = gelu_erf4(y);
-                    packed[j >> 1] = pack_bf16x2(y.x, y.y);
-                    packed[(j >> 1) + 1] = pack_bf16x2(y.z, y.w);
-                }
-                if (i < d) *(uint4 *)(m.S_out + row * d + i) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+            for (int j = 0; j < 8; j += 4) {
+                float4 y;
+                y.x = (h[q][it][j] - mean[q]) * rstd[q] * gv[it][j] + bv[it][j];
+                y.y = (h[q][it][j + 1] - mean[q]) * rstd[q] * gv[it][j + 1] + bv[it][j + 1];
+                y.z = (h[q][it][j + 2] - mean[q]) * rstd[q] * gv[it][j + 2] + bv[it][j + 2];
+                y.w = (h[q][it][j + 3] - mean[q]) * rstd[q] * gv[it][j + 3] + bv[it][j + 3];
+                y = gelu_erf4(y);
+                packed[j >> 1] = pack_bf16x2(y.x, y.y);
+                packed[(j >> 1) + 1] = pack_bf16x2(y.z, y.w);
             }
+            if (i < d) *(uint4 *)(m.S_out + row * d + i) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
         }
     }
 }

@@ -108,7 +108,10 @@ typedef struct {
     uint64_t state[SPEC_MAX_HEADS];       /* bf16  [N_l, d_inner]: post-GELU state of level l */
     uint64_t proj;                        /* fp32  [max rows, d_inner]: projected parent states */
     uint64_t state8, state8_scale;        /* e4m3 [rows, d_inner] + fp32 [rows]: states of an e4m3 level */
-    uint64_t part_val, part_idx, part_ms; /* per-tile partial top-k lists and (max, sum-exp)  */
+    /* per-tile partial top-k lists and (max, sum-exp) of the level that ran last: entry j of row r and tile t at
+     * (r * n_tiles + t) * slots + j, slots = 2, 4 or 8, the least that holds topk (8 behind an e4m3 head); part_ms at
+     * (r * n_tiles + t) * 2 */
+    uint64_t part_val, part_idx, part_ms;
     uint64_t logits;                      /* fp32 [max N_l, V]; only with SPEC_OPT_GEMM_IMPL=1 */
     int32_t block_n[SPEC_MAX_HEADS];      /* vocabulary columns per head-GEMM tile            */
     int32_t n_tiles[SPEC_MAX_HEADS];      /* vocabulary tiles per row of the head GEMM        */

@@ -192,7 +192,8 @@ __global__ void __maxnreg__(48) merge_prune_kernel(MergeArgs g) {
 // are more children than SMs but no more rows: one CTA of 256 threads per row of level l folds the row's partial lists into its
 // children (tokens, scores) and then computes the states of those children, whose tokens it has just found and whose parent
 // projection is this row's.  One kernel boundary less between two vocabulary heads.  75 / 128 / 148 rows, V 8000, the whole
-// draft as two kernels -> this: d 1024 52.9 -> 51.4 us, 59.4 -> 56.7, 56.8 -> 54.5; d 2048 64.6 -> 62.8, 71.2 -> 68.4, 76.4 -> 74.5.
+// draft as two kernels -> this: d 1024 52.9 -> 51.4 us, 59.4 -> 56.7, 56.8 -> 54.5; d 2048 64.6 -> 62.8, 71.2 -> 68.4, 76.4 ->
+// 74.5.
 struct MergeMixArgs {
     MergeArgs merge;   // level l
     MixArgs mix;       // level l + 1 (tok and parent_div unused: the tokens come from the merge)
@@ -384,7 +385,8 @@ int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st) {
     if (g.seq_done && one_warp_per_row(g, rows)) {
         SPEC_CUDA_TRY(launch_pdl(slots == 2   ? merge_prune_kernel<2>
                                  : slots == 4 ? merge_prune_kernel<4>
-                                              : merge_prune_kernel<8>, dim3(rows / g.rows_per_seq), dim3(32 * g.rows_per_seq), 0, st, g));
+                                              : merge_prune_kernel<8>, dim3(rows / g.rows_per_seq),
+                                 dim3(32 * g.rows_per_seq), 0, st, g));
         return SPEC_OK;
     }
     SPEC_CUDA_TRY(launch_pdl(slots == 2   ? merge_expand_kernel<2>
@@ -393,8 +395,10 @@ int launch_merge_expand(const MergeArgs &g, int rows, cudaStream_t st) {
     return SPEC_OK;
 }
 
-// Whether the LayerNorm sums of a level with `topk` children per row are taken in order (group_sums) in every kernel that may
-// compute its states, so that these are the same bits whatever the number of rows.
+// Whether the LayerNorm sums of a level with `topk` children per row, behind a bf16 head, are taken in order (group_sums) in every
+// kernel that may compute its states, so that these are the same bits whatever the number of rows.  In a tree, whose shape goes
+// by the kernel and so by the number of rows, they are taken at the first level, behind three children and more or an e4m3 head,
+// in a level that has an e4m3 copy, in rows of more than 4096 elements, of split vocabularies and with per-kernel profiling.
 bool mix_sums_in_order(int topk, const MixArgs &m) {
     return topk <= kFusedChildren && m.S8_out == nullptr && m.d <= 8 * kRowThreads * 2;
 }

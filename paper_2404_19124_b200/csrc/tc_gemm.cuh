@@ -385,8 +385,9 @@ __device__ __forceinline__ void advance(const Pipe &pp, RingPos &rp) {
 // operand only; then `dep_wait()` is called once (it must return true once the states are readable:
 // the preceding grid has completed, or the grid-wide barrier behind which they are written has
 // opened) and the state operand of those slots follows.  A CTA without a tile in the job neither
-// loads nor waits.  `waited`: it has been called for an earlier job, and the slots are filled both operands together: the states
-// of the first slot would otherwise follow only when the ring has turned (single-candidate chain 156.4 -> 155.0 us).  `issued` counts slots filled since the kernel started (for the abort path).
+// loads nor waits.  `waited`: it has been called for an earlier job, and the slots are filled both operands together: the
+// states of the first slot would otherwise follow only when the ring has turned (single-candidate chain 156.4 -> 155.0 us).
+// `issued` counts slots filled since the kernel started (for the abort path).
 // Producer `me` of `n_prod` walks every slot like the others and fills the slots whose running number
 // `issued` (counted over all jobs of the launch) is congruent to `me` (n_prod is a power of two).
 // One loop serves the first fill, its state operands and the rest, again to keep the code small.
@@ -574,8 +575,7 @@ __device__ __forceinline__ void scale_chunk(float (&v)[32], float rs, const floa
 }
 // The column scales of the tile at column col0 (0 past the last column), into the warp's own copy.  They come from DRAM, so
 // they are fetched while the tile's MMAs run: read chunk by chunk behind them they were a chain of seven misses (96 nodes, V
-// 32000, d 4096: 12 us from the last MMA to the last list, the 13B step
-// with e4m3 heads 246.7 -> 244.9 us).
+// 32000, d 4096: 12 us from the last MMA to the last list, the 13B step with e4m3 heads 246.7 -> 244.9 us).
 __device__ __forceinline__ void stage_col_scales(float *cs, const GemmJob &j, int col0) {
     const int lane = threadIdx.x & 31;
     __syncwarp();   // the tile before has been read
